@@ -22,7 +22,7 @@ using wd::status_t;
 
 namespace {
 
-constexpr int ROWS_PER_CTA = 256;  // one thread per front row (gather / apply_L)
+constexpr int ROWS_PER_CTA = 32;   // front rows per apply_L item
 
 enum LaunchKind {
     K_INIT, K_PANEL, K_UPDATE, K_SYRK, K_UPDATE_TC, K_SYRK_TC, K_DIAG,      // factor
