@@ -157,6 +157,7 @@ struct wd_ctx {
     // words of every supernode (offsets chain_flagoff), then one task counter
     // per level and the launch-wide abort word; zeroed before each factor
     bool chain = false;
+    int *d_diag_cnt = nullptr;        // FP64 fronts: arrivals at each front's next diagonal block (zero between launches)
     std::vector<int8_t> level_step;   // per level: 1 keeps the launch pairs (wd_set_level_schedule)
     unsigned *d_chain_flags = nullptr;
     int64_t *d_chain_flagoff = nullptr;
@@ -792,6 +793,7 @@ static wd_status reset_analysis(wd_handle h) {
     h->d_chain_flags = nullptr;
     h->d_chain_flagoff = nullptr;
     h->d_chain_lpack = nullptr;
+    h->d_diag_cnt = nullptr;
     h->chain_words = h->chain_ctr = 0;
     h->splan = Plan();
     h->aplan = Plan();
@@ -1149,6 +1151,8 @@ static wd_status finish_analysis(wd_handle h, std::chrono::steady_clock::time_po
         if (st != WD_OK) return st;
     }
     CK(h->mem.alloc((void **)&h->d_tstatus, sizeof(status_t)), "status alloc");
+    CK(h->mem.alloc((void **)&h->d_diag_cnt, ns * sizeof(int)), "arrival counters alloc");
+    CK(cudaMemset(h->d_diag_cnt, 0, ns * sizeof(int)), "arrival counters clear");
     if (h->opt.test_closed_gate) {
         CK(h->mem.alloc((void **)&h->d_gate, sizeof(unsigned)), "gate alloc");
         CK(cudaMemset(h->d_gate, 0, sizeof(unsigned)), "gate clear");
@@ -1325,6 +1329,11 @@ static void enqueue_factor_plan(wd_handle h, cudaStream_t st, bool prof) {
     oa.status = h->d_status;
     oa.tstatus = h->d_tstatus;
     oa.wait_limit = ta.wait_limit;
+    wd::F64Args fa{};
+    fa.f = reinterpret_cast<double *>(F);
+    fa.di = reinterpret_cast<double *>(Dv);
+    fa.cnt = h->d_diag_cnt;
+    fa.status = h->d_status;
     wd::ChainArgs ca{};
     ca.dinv = reinterpret_cast<float *>(Dv);
     ca.lpack = h->d_chain_lpack;
@@ -1348,11 +1357,18 @@ static void enqueue_factor_plan(wd_handle h, cudaStream_t st, bool prof) {
                 break;
             case K_INIT: wd::launch_front_init<T>(d, F, it, L.count, st); break;
             case K_DIAG:
-                wd::launch_diag_factor<T>(d, F, Dv, it, L.count, h->opt.diag64_min_k, h->d_status, st);
+                if (fp32)
+                    wd::launch_diag_factor<float>(d, reinterpret_cast<float *>(F), ta.dinv, it, L.count,
+                                                  h->opt.diag64_min_k, h->d_status, st);
+                else wd::launch_diag64(d, fa, it, L.count, st);
                 break;
-            case K_PANEL: wd::launch_panel<T>(d, F, Dv, pk, it, L.count, L.arg, st); break;
-            case K_UPDATE: wd::launch_schur<T>(d, F, Dv, it, L.count, L.arg, 0, h->d_status, st); break;
-            case K_SYRK: wd::launch_schur<T>(d, F, Dv, it, L.count, 0, 1, h->d_status, st); break;
+            case K_PANEL:
+                if (fp32)
+                    wd::launch_panel<float>(d, reinterpret_cast<float *>(F), ta.dinv, pk, it, L.count, L.arg, st);
+                else wd::launch_panel64(d, fa, it, L.count, L.arg, st);
+                break;
+            case K_UPDATE: wd::launch_update64(d, fa, it, L.count, L.arg, 0, st); break;
+            case K_SYRK: wd::launch_update64(d, fa, it, L.count, 0, 1, st); break;
             case K_UPDATE_TC:
                 wd::launch_tc_schur(d, reinterpret_cast<float *>(F), pk, it, L.count, L.arg, 0, ta, st);
                 break;
@@ -1367,7 +1383,11 @@ static void enqueue_factor_plan(wd_handle h, cudaStream_t st, bool prof) {
                 break;
             case K_OZ_SYRK: wd::launch_oz_schur(d, reinterpret_cast<double *>(F), it, L.count, 0, 1, oa, st); break;
             case K_SBINV_DIAG:
-                wd::launch_sbinv_diag<T>(d, Dv, static_cast<T *>(h->d_xs), h->d_xsoff, it, L.count, st);
+                if (fp32)
+                    wd::launch_sbinv_diag(d, ta.dinv, static_cast<float *>(h->d_xs), h->d_xsoff, it, L.count, st);
+                else
+                    wd::launch_sbinv_diag64(d, fa.f, fa.di, static_cast<double *>(h->d_xs), h->d_xsoff, it, L.count,
+                                            st);
                 break;
             case K_SBINV_STAGE:
                 wd::launch_sbinv_stage<T>(d, F, Dv, static_cast<T *>(h->d_xs), h->d_xsoff, it, L.count, L.arg,

@@ -49,6 +49,7 @@ void init_tc_solve_attributes();
 void init_lu_attributes();
 void init_oz_attributes();
 void init_chain_attributes();
+void init_front64_attributes();
 inline void init_kernel_attributes() {
     init_front_attributes();
     init_solve_attributes();
@@ -58,6 +59,7 @@ inline void init_kernel_attributes() {
     init_lu_attributes();
     init_oz_attributes();
     init_chain_attributes();
+    init_front64_attributes();
 }
 
 
@@ -75,13 +77,29 @@ void launch_diag_factor(const DevSym &d, T *front, T *dinv, const int4 *items, i
 template <class T>
 void launch_panel(const DevSym &d, T *front, const T *dinv, unsigned char *pk, const int4 *items, int count,
                   int kb, cudaStream_t st);
-// mode 0: pivot-column update of step kb, then the CTA of tile (0, 0) factors
-// diagonal block kb + NB (into the front and dinv); mode 1: final update
-// matrix (syrk)
-template <class T>
-void launch_schur(const DevSym &d, T *front, T *dinv, const int4 *items, int count, int kb,
-                  int mode, status_t *status, cudaStream_t st);
+// tile of the plans' FP64 update items
 constexpr int SCHUR_BM = 128, SCHUR_BN = 64;
+
+// FP64 fronts (front64.cu): Cholesky (g = nullptr), or LU with the fronts of
+// U^T beside those of L
+struct F64Args {
+    double *f;          // fronts: L
+    double *g;          // LU: fronts of U^T
+    double *di, *du;    // inverses of the diagonal blocks of L and U^T: the 16 x 16 diagonal sub-blocks
+                        // (the diagonal's entries are the reciprocal pivots), completed by sbinv_diag64
+    int sym;            // LU of a symmetric matrix: U^T = L D comes out of L's panels, g is not assembled
+    int *cnt;           // per supernode: arrivals at the next diagonal block (zero between launches)
+    status_t *status;
+};
+void init_front64_attributes();
+void launch_diag64(const DevSym &d, const F64Args &a, const int4 *items, int count, cudaStream_t st);
+void launch_panel64(const DevSym &d, const F64Args &a, const int4 *items, int count, int kb, cudaStream_t st);
+// mode 0: pivot-column update of step kb, then the last CTA at the next
+// diagonal block factors it; mode 1: final update matrix
+void launch_update64(const DevSym &d, const F64Args &a, const int4 *items, int count, int kb, int mode,
+                     cudaStream_t st);
+void launch_sbinv_diag64(const DevSym &d, const double *front, double *dinv, double *xpool, const int64_t *xsoff,
+                         const int4 *items, int count, cudaStream_t st);
 
 // Packed tf32 operand lines of a supernode's L panel (FP32 fronts, tensor-core
 // Schur updates): for each chunk kc of 32 pivot columns and plane p (0 = hi,
@@ -267,8 +285,7 @@ void launch_sym_outer(const DevSym &d, const int32_t *prow, const int32_t *psrc,
 // its transpose XT) at xsoff[s] + sb * SB * SB, column-major with leading
 // dimension wp = roundup(width, NB).
 constexpr int SB = 512;
-template <class T>
-void launch_sbinv_diag(const DevSym &d, const T *dinv, T *xpool, const int64_t *xsoff, const int4 *items,
+void launch_sbinv_diag(const DevSym &d, const float *dinv, float *xpool, const int64_t *xsoff, const int4 *items,
                        int count, cudaStream_t st);
 template <class T>
 void launch_sbinv_stage(const DevSym &d, const T *front, const T *dinv, T *xpool, const int64_t *xsoff,

@@ -35,9 +35,6 @@ namespace wd {
 namespace {
 
 constexpr int THREADS = 256;
-constexpr int BM = SCHUR_BM;   // rows of a Schur tile
-constexpr int BN = SCHUR_BN;   // columns of a Schur tile
-constexpr int BK = 32;         // inner-dimension chunk
 
 using blk::load4;
 // four consecutive shared-memory elements (16-byte aligned for float,
@@ -258,105 +255,8 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2) panel_kernel(
     }
 }
 
-// ---------------------------------------------------------------------------
-// Schur tile: C(rows [r0, r0+BM), cols [c0, c0+BN)) -= A(rows, ka:ka+K) A(cols, ka:ka+K)^T
-// restricted to r >= c, r < mp, c < cmax.  thread (tx, ty): rows tx + 16 i,
-// columns ty + 16 j (i < 8, j < 4).
-//   mode 0 (step):  base = kb + NB, ka = kb, K = NB, cmax = k
-//   mode 1 (syrk):  base = kp, ka = 0, K = k, cmax = mp
-// In mode 0 the CTA of tile (0, 0), which holds the whole next diagonal
-// block, then factors that block (L11 and L11^-1 of step kb + NB).
-// ---------------------------------------------------------------------------
-template <class T>
-__global__ void __launch_bounds__(THREADS) schur_kernel(DevSym d, T *__restrict__ front,
-                                                        T *__restrict__ dinv,
-                                                        const int4 *__restrict__ items, int kb,
-                                                        int mode, status_t *status) {
-    static_assert(BM >= NB && BN >= NB, "tile (0, 0) covers the next diagonal block");
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    T *As[2] = {sm, sm + BK * (BM + BN)};
-    T *Bs[2] = {sm + BK * BM, sm + BK * (BM + BN) + BK * BM};
-    const int4 it = items[blockIdx.x];
-    const int s = it.x, ti = it.y, tj = it.z;
-    const Dims z = dims(d, s);
-    int base, ka, K, cmax;
-    if (mode == 0) {
-        base = kb + NB;
-        ka = kb;
-        K = NB;
-        cmax = z.k;
-    } else {
-        base = z.kp;
-        ka = 0;
-        K = z.k;
-        cmax = z.mp;
-    }
-    const int r0 = base + ti * BM, c0 = base + tj * BN;
-    T *F = front + d.foff[s];
-    const T *Ar = F + (int64_t)ka * z.ld + r0;
-    const T *Bc = F + (int64_t)ka * z.ld + c0;
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    T acc[8][4];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-    const int nk = (K + BK - 1) / BK;
-    stage_tile<T, THREADS>(As[0], BM, Ar, z.ld, BM, BK, z.mp - r0, min(BK, K));
-    stage_tile<T, THREADS>(Bs[0], BN, Bc, z.ld, BN, BK, cmax - c0, min(BK, K));
-    cp_async_commit();
-    for (int kt = 0; kt < nk; ++kt) {
-        const int cur = kt & 1;
-        if (kt + 1 < nk) {
-            const int k1 = (kt + 1) * BK;
-            stage_tile<T, THREADS>(As[cur ^ 1], BM, Ar + (int64_t)k1 * z.ld, z.ld, BM, BK, z.mp - r0,
-                                   min(BK, K - k1));
-            stage_tile<T, THREADS>(Bs[cur ^ 1], BN, Bc + (int64_t)k1 * z.ld, z.ld, BN, BK, cmax - c0,
-                                   min(BK, K - k1));
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const T *A = As[cur];
-        const T *B = Bs[cur];
-#pragma unroll 8
-        for (int kk = 0; kk < BK; ++kk) {
-            T a[8], b[4];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) a[i] = A[kk * BM + tx + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = B[kk * BN + ty + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = c0 + ty + 16 * j;
-        if (c >= cmax) continue;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = r0 + tx + 16 * i;
-            if (r < z.mp && r >= c) F[(int64_t)c * z.ld + r] -= acc[i][j];
-        }
-    }
-    if (mode == 0 && ti == 0 && tj == 0 && kb + NB < z.k) {
-        __syncthreads();   // the block's updated entries, written above, visible to the CTA
-        blk::factor_diag_block<T, T, THREADS>(d, front, dinv, s, kb + NB, status, smem_raw);
-    }
-}
-
 template <class T>
 constexpr size_t panel_smem() { return sizeof(T) * (NB * XLD + NB * RB); }
-constexpr size_t cmax_size(size_t a, size_t b) { return a > b ? a : b; }
-template <class T>
-constexpr size_t schur_smem() { return cmax_size(2 * sizeof(T) * BK * (BM + BN), blk::block_smem_bytes<T>()); }
 constexpr size_t diag_smem() { return blk::block_smem_bytes<double>(); }
 
 template <class T>
@@ -365,8 +265,6 @@ void set_smem_attrs() {
     if (done) return;
     cudaFuncSetAttribute(panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)panel_smem<T>());
-    cudaFuncSetAttribute(schur_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)schur_smem<T>());
     cudaFuncSetAttribute(diag_factor_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)diag_smem());
     cudaFuncSetAttribute(diag_factor_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -377,7 +275,6 @@ void set_smem_attrs() {
 }  // namespace
 
 void init_front_attributes() {
-    set_smem_attrs<double>();
     set_smem_attrs<float>();
 }
 
@@ -407,24 +304,11 @@ void launch_panel(const DevSym &d, T *front, const T *dinv, unsigned char *pk, c
     panel_kernel<T><<<count, THREADS, panel_smem<T>(), st>>>(d, front, dinv, pk, items, kb);
 }
 
-template <class T>
-void launch_schur(const DevSym &d, T *front, T *dinv, const int4 *items, int count, int kb,
-                  int mode, status_t *status, cudaStream_t st) {
-    if (count <= 0) return;
-    set_smem_attrs<T>();
-    schur_kernel<T><<<count, THREADS, schur_smem<T>(), st>>>(d, front, dinv, items, kb, mode, status);
-}
-
-#define WD_INST(T)                                                                               \
-    template void launch_front_init<T>(const DevSym &, T *, const int4 *, int, cudaStream_t);    \
-    template void launch_diag_factor<T>(const DevSym &, T *, T *, const int4 *, int, int, status_t *, \
-                                        cudaStream_t);                                           \
-    template void launch_panel<T>(const DevSym &, T *, const T *, unsigned char *, const int4 *, int, \
-                                  int, cudaStream_t);                                            \
-    template void launch_schur<T>(const DevSym &, T *, T *, const int4 *, int, int, int,         \
-                                  status_t *, cudaStream_t);
-WD_INST(double)
-WD_INST(float)
-#undef WD_INST
+template void launch_front_init<double>(const DevSym &, double *, const int4 *, int, cudaStream_t);
+template void launch_front_init<float>(const DevSym &, float *, const int4 *, int, cudaStream_t);
+template void launch_diag_factor<float>(const DevSym &, float *, float *, const int4 *, int, int, status_t *,
+                                        cudaStream_t);
+template void launch_panel<float>(const DevSym &, float *, const float *, unsigned char *, const int4 *, int, int,
+                                  cudaStream_t);
 
 }  // namespace wd

@@ -43,7 +43,7 @@
 
 #include "dev_common.cuh"
 #include "engine.h"
-#include "front_block.cuh"
+#include "front64.cuh"
 #include "tc_common.cuh"
 
 namespace wd {
@@ -58,7 +58,7 @@ constexpr int STAGE = NSL * (A_PLANE + B_PLANE); // 192 KB
 constexpr int OZ_THREADS = 320;
 constexpr uint32_t WAIT_LIMIT = 1u << 26;
 constexpr uint32_t DRAIN_LIMIT = 1u << 26;
-static_assert(STAGE >= (int)blk::block_smem_bytes<double>(), "the stage holds the block factorization");
+static_assert(STAGE >= f64::BLOCK_ELEMS * (int)sizeof(double), "the stage holds the block factorization");
 
 __device__ __forceinline__ void bulk_copy(void *dst_smem, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile(
@@ -312,7 +312,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_schur_kernel(DevSym d, doubl
     }
     if (mode == 0 && ti == 0 && tj == 0 && kb + NB < k) {
         // the next diagonal block lies inside this tile, written above
-        blk::factor_diag_block<double, double, OZ_THREADS>(d, front, a.dinv, s, kb + NB, a.status, sm);
+        F64Args fa{};
+        fa.f = front;
+        fa.di = a.dinv;
+        fa.status = a.status;
+        f64::factor_block<OZ_THREADS>(d, fa, s, kb + NB, reinterpret_cast<double *>(sm));
     }
 }
 

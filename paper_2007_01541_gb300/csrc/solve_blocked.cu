@@ -26,18 +26,18 @@ constexpr int THREADS = 256;
 // ---------------------------------------------------------------------------
 // super-block inverses
 // ---------------------------------------------------------------------------
-// X(t, t) = Dinv of pivot block sb*8 + t; item = (s, sb, t)
-template <class T>
-__global__ void __launch_bounds__(THREADS) sbinv_diag_kernel(DevSym d, const T *__restrict__ dinv,
-                                                             T *__restrict__ xpool,
+// X(t, t) = Dinv of pivot block sb*8 + t; item = (s, sb, t) (FP32 fronts;
+// FP64: sbinv_diag64 in front64.cu)
+__global__ void __launch_bounds__(THREADS) sbinv_diag_kernel(DevSym d, const float *__restrict__ dinv,
+                                                             float *__restrict__ xpool,
                                                              const int64_t *__restrict__ xsoff,
                                                              const int4 *__restrict__ items) {
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y, t = it.z;
     const int k = d.sk[s];
     const int w = min(SB, k - sb * SB), wp = (w + NB - 1) / NB * NB;
-    const T *D = dinv + d.dinvoff[s] + (int64_t)(sb * (SB / NB) + t) * NB * NB;
-    T *X = xpool + xsoff[s] + (int64_t)sb * SB * SB + (int64_t)(t * NB) * wp + t * NB;
+    const float *D = dinv + d.dinvoff[s] + (int64_t)(sb * (SB / NB) + t) * NB * NB;
+    float *X = xpool + xsoff[s] + (int64_t)sb * SB * SB + (int64_t)(t * NB) * wp + t * NB;
     for (int idx = threadIdx.x; idx < NB * NB; idx += THREADS) {
         const int r = idx % NB, c = idx / NB;
         X[(int64_t)c * wp + r] = D[idx];
@@ -773,10 +773,9 @@ int solve_tile_rows(int large) { return large == 1 ? TileTc::ROWS : TileS::ROWS;
 int solve_tile_rhs(int large) { return large == 1 ? TileTc::RHS : TileS::RHS; }
 int solve_update_rows(int large) { return large == 2 ? NRW : solve_tile_rows(large); }
 
-template <class T>
-void launch_sbinv_diag(const DevSym &d, const T *dinv, T *xpool, const int64_t *xsoff, const int4 *items,
+void launch_sbinv_diag(const DevSym &d, const float *dinv, float *xpool, const int64_t *xsoff, const int4 *items,
                        int count, cudaStream_t st) {
-    if (count > 0) sbinv_diag_kernel<T><<<count, THREADS, 0, st>>>(d, dinv, xpool, xsoff, items);
+    if (count > 0) sbinv_diag_kernel<<<count, THREADS, 0, st>>>(d, dinv, xpool, xsoff, items);
 }
 template <class T>
 void launch_sbinv_stage(const DevSym &d, const T *front, const T *dinv, T *xpool, const int64_t *xsoff,
@@ -870,8 +869,6 @@ void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const
 }
 
 #define WD_BLOCKED_INST(T)                                                                              \
-    template void launch_sbinv_diag<T>(const DevSym &, const T *, T *, const int64_t *, const int4 *, int, \
-                                       cudaStream_t);                                                   \
     template void launch_sbinv_stage<T>(const DevSym &, const T *, const T *, T *, const int64_t *,      \
                                         const int4 *, int, int, cudaStream_t);                          \
     template void launch_sbinv_transpose<T>(const DevSym &, const T *, T *, const int64_t *, const int4 *, \

@@ -33,3 +33,39 @@ def test_apply_L_column_tiles(wdlib, cuda, dim, J, ncols):
     s = wdlib.Solver().analyze(cp, ri, b)
     for prec, tol in (("fp64", 1e-12), ("mixed", 1e-5)):   # mixed: the FP32 factor
         assert np.abs(s.factor(v, prec).apply_L(Z) - ref).max() <= tol * np.abs(ref).max()
+
+
+def _lower_csc(A):
+    n = A.shape[0]
+    cp = np.concatenate([[0], np.cumsum(np.arange(n, 0, -1))]).astype(np.int64)
+    ri = np.concatenate([np.arange(j, n) for j in range(n)]).astype(np.int32)
+    return cp, ri, np.concatenate([A[j:, j] for j in range(n)])
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 31, 33, 48, 63, 64, 65, 97, 128, 131, 200])
+def test_fp64_block_edges(wdlib, cuda, n):
+    """One dense front: pivot blocks and update tiles cut at every remainder."""
+    rng = np.random.default_rng(n)
+    M = rng.standard_normal((n, n))
+    A = M @ M.T + n * np.eye(n)
+    cp, ri, v = _lower_csc(A)
+    s = wdlib.Solver().analyze(cp, ri).factor(v, "fp64")
+    L = np.zeros((n, n))
+    L[np.concatenate([np.arange(j, n) for j in range(n)]), np.repeat(np.arange(n), np.arange(n, 0, -1))] = \
+        s.L_csc_like(cp, ri)
+    ref = np.linalg.cholesky(A)
+    assert np.linalg.norm(L - ref, axis=0).max() <= 1e-12 * np.linalg.norm(ref)
+    B = rhs(n, 3, seed=1)
+    assert oracle.backward_error(cp, ri, v, s.solve(B), B).max() <= 1e-14
+
+
+@pytest.mark.parametrize("bad", [0, 15, 16, 40, 63, 64, 99])
+def test_fp64_pivot_status(wdlib, cuda, bad):
+    n = 100
+    A = np.eye(n) * 2.0 + 0.001
+    A[bad, bad] = -1.0
+    cp, ri, v = _lower_csc(A)
+    s = wdlib.Solver().analyze(cp, ri)
+    with pytest.raises(wdlib.WdError) as e:
+        s.factor(v, "fp64")
+    assert e.value.status == wdlib.WD_ERR_NOT_SPD and e.value.column == bad
