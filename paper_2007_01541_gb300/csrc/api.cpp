@@ -30,8 +30,6 @@ enum LaunchKind {
     K_FWD_GATHER, K_FWD_XAPPLY, K_FWD_BUPDATE,                 // forward solve
     K_BWD_REDUCE, K_BWD_FINISH, K_BWD_XAPPLY,                  // backward solve
     K_APPLY_L,
-    K_LU_INIT, K_LU_DIAG, K_LU_PANEL, K_LU_UPDATE,               // LU factor
-    K_LU_GATHER, K_LU_FWD, K_LU_BWD,                             // LU substitutions
     K_OZ_SLICE, K_OZ_UPDATE, K_OZ_SYRK,                          // FP64 updates on the tensor cores
     K_CHAIN_TC                                                   // pivot columns of a level, one launch
 };
@@ -51,9 +49,7 @@ const char *kind_name(int k) {
                                   "tc_schur_update", "tc_schur_syrk", "diag_factor", "sbinv_diag",
                                   "sbinv_stage", "sbinv_transpose", "fwd_gather", "fwd_xapply",
                                   "fwd_bupdate", "bwd_reduce", "bwd_finish", "bwd_xapply",
-                                  "apply_L", "lu_init", "lu_diag", "lu_panel", "lu_update",
-                                  "lu_gather", "lu_fwd", "lu_bwd", "oz_slice", "oz_schur_update",
-                                  "oz_schur_syrk", "tc_chain"};
+                                  "apply_L", "oz_slice", "oz_schur_update", "oz_schur_syrk", "tc_chain"};
     return names[k];
 }
 
@@ -125,15 +121,16 @@ struct wd_ctx {
     int32_t *d_csr_src = nullptr;
     double *d_csr_val = nullptr;
     // LU without pivoting (wd_factor_lu, FP64): position codes of the full
-    // CSR, both values per position, U11^-1 blocks, plans
+    // CSR, both values per position, the fronts of U^T and the inverses of
+    // their diagonal blocks
     bool lu_factored = false;
     bool ldlt = false;          // the LU factor is that of a symmetric matrix (wd_factor_ldlt)
-    bool front_dirty = false;   // the fronts' upper parts hold an LU factor
+    void *d_front_u = nullptr;
+    GraphCache g_lu;
     std::vector<int8_t> h_csr_code;
     int8_t *d_lu_code = nullptr;
     double *d_vrow = nullptr, *d_vcol = nullptr, *d_uinv = nullptr, *d_lu_part = nullptr;
     double *d_upper_stage = nullptr;
-    Plan fplan_lu, splan_lu_f, splan_lu_b;
     double *d_gcsr = nullptr;   // mass matrix G on the full CSR (wd_set_mass; nullptr: G = I)
     double *mass_buf = nullptr; // its storage (analysis lifetime)
     float *d_csr_vh = nullptr, *d_csr_vl = nullptr;   // double-float split of csr_val
@@ -337,6 +334,7 @@ void wd_destroy(wd_handle h) {
             if (e) cudaEventDestroy(e);
         h->g_factor.reset();
         h->g_solve.reset();
+        h->g_lu.reset();
         if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
         h->work.free_all();
         h->mem.free_all();
@@ -805,12 +803,11 @@ static wd_status reset_analysis(wd_handle h) {
     h->d_front = nullptr;
     h->d_dinv = nullptr;
     h->d_gcsr = h->mass_buf = nullptr;
-    h->lu_factored = h->front_dirty = false;
+    h->lu_factored = false;
+    h->d_front_u = nullptr;
+    h->g_lu.reset();
     h->d_lu_code = nullptr;
     h->d_vrow = h->d_vcol = h->d_uinv = h->d_lu_part = h->d_upper_stage = nullptr;
-    h->fplan_lu = Plan();
-    h->splan_lu_f = Plan();
-    h->splan_lu_b = Plan();
     h->d_xs = h->d_xts = nullptr;
     h->d_xsoff = nullptr;
     h->d_oz_sl = nullptr;
@@ -1456,20 +1453,15 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
     wait_export(h);   // a pending allocation-free export still reads the fronts
     h->factored = false;
     h->lu_factored = false;
-    if (h->front_dirty && h->d_front) {
-        // an LU factor filled the upper parts that the Cholesky kernels keep zero
-        CK(cudaMemsetAsync(h->d_front, 0, h->front_elems * sizeof(double), st), "front pool clear");
-        h->front_dirty = false;
-    }
     const int64_t nnzl = h->S.pcp[h->S.n];
     if (!h->d_front) {
         CK(h->mem.alloc(&h->d_front, h->front_elems * sizeof(double)), "front pool alloc");
-        CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
-        CK(h->mem.alloc(&h->d_xs, h->xs_elems * sizeof(double)), "super-block inverse alloc");
-        CK(h->mem.alloc(&h->d_xts, h->xs_elems * sizeof(double)), "super-block inverse alloc");
         // padding rows stay zero forever: no kernel writes them
         CK(cudaMemsetAsync(h->d_front, 0, h->front_elems * sizeof(double), st), "front pool clear");
     }
+    if (!h->d_dinv) CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
+    if (!h->d_xs) CK(h->mem.alloc(&h->d_xs, h->xs_elems * sizeof(double)), "super-block inverse alloc");
+    if (!h->d_xts) CK(h->mem.alloc(&h->d_xts, h->xs_elems * sizeof(double)), "super-block inverse alloc");
     if (prec == WD_FP64 && h->opt.fp64_tc_schur && !h->d_oz_sl) {
         CK(h->mem.alloc((void **)&h->d_oz_sl, h->oz_sl_bytes), "slice planes alloc");
         CK(h->mem.alloc((void **)&h->d_oz_ex, h->oz_ex_elems * sizeof(int16_t)), "slice scales alloc");
@@ -1570,9 +1562,12 @@ static wd_status ensure_solve_ws(wd_handle h, int64_t nrhs) {
     return WD_OK;
 }
 
+// lu: the backward pass reads the fronts of U^T (and d_xts their super-block
+// inverses) in the place of L's
 template <class T>
-static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, bool prof) {
+static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, bool prof, bool lu) {
     const T *F = static_cast<const T *>(h->d_front);
+    const T *Fb = lu ? static_cast<const T *>(h->d_front_u) : F;
     const T *Xs = static_cast<const T *>(h->d_xs);
     const T *XTs = static_cast<const T *>(h->d_xts);
     T *W = static_cast<T *>(h->d_W);
@@ -1630,7 +1625,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.out = reinterpret_cast<float *>(P);
                     wd::launch_tc_breduce(d, a, it, L.count, st);
                 } else {
-                    wd::launch_breduce<T>(d, F, Y, P, it, L.count, lg, nrhs, st);
+                    wd::launch_breduce<T>(d, Fb, Y, P, it, L.count, lg, nrhs, st);
                 }
                 break;
             case K_BWD_FINISH: wd::launch_breduce_finish<T>(d, Y, Tt, P, it, L.count, lg, nrhs, st); break;
@@ -1653,11 +1648,11 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
 }
 
 template <class T>
-static wd_status run_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st) {
+static wd_status run_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, bool lu = false) {
     const bool prof = prof_begin(h, h->splan.launches.size());
-    const int64_t key = ((int64_t)nrhs << 8) + (sizeof(T) == 8 ? 1 : 2) + (prof ? 10 : 0);
+    const int64_t key = ((int64_t)nrhs << 8) + (sizeof(T) == 8 ? 1 : 2) + (prof ? 10 : 0) + (lu ? 100 : 0);
     wd_status s = run_graph(h, h->g_solve, key, st,
-                            [&](cudaStream_t cs) { enqueue_solve_plan<T>(h, Y, nrhs, cs, prof); });
+                            [&](cudaStream_t cs) { enqueue_solve_plan<T>(h, Y, nrhs, cs, prof, lu); });
     if (s != WD_OK) return s;
     h->launches += (int64_t)h->splan.launches.size();
     if (prof) prof_end(h, h->splan, sizeof(T), sizeof(T) == 8 ? "_fp64" : "_fp32");
@@ -1749,14 +1744,14 @@ static wd_status backward_errors(wd_handle h, const double *X, int64_t nrhs, cud
 }
 
 // workspaces and the launch plan of solves with nrhs right-hand sides
-static wd_status prepare_solve(wd_handle h, int64_t nrhs) {
+static wd_status prepare_solve(wd_handle h, int64_t nrhs, bool mixed) {
     wd_status s = ensure_solve_ws(h, nrhs);
     if (s != WD_OK) return s;
     // tiles of 64 rows x 32 right-hand sides; FP32 with more than 8
     // right-hand sides: tensor-core tiles of 128 rows x 64 right-hand sides
     // (unless wd_options.solve_simt); up to 8 right-hand sides:
     // matrix-vector shaped kernels, lanes over rows
-    const int large = nrhs <= 8 ? 2 : (h->prec == WD_MIXED && !h->opt.solve_simt ? 1 : 0);
+    const int large = nrhs <= 8 ? 2 : (mixed && !h->opt.solve_simt ? 1 : 0);
     if (h->splan_nrhs != nrhs || h->splan.large != large) {
         build_solve_plan(h->S, (int)nrhs, large, h->sms, h->splan);
         s = upload_plan(h, h->work, h->splan);
@@ -1883,7 +1878,7 @@ extern "C" wd_status wd_solve(wd_handle h, double *B, int64_t nrhs, int64_t ldb,
     if (nrhs == 0) return WD_OK;
     CK(cudaSetDevice(h->device), "set device");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    wd_status s = prepare_solve(h, nrhs);
+    wd_status s = prepare_solve(h, nrhs, h->prec == WD_MIXED);
     if (s != WD_OK) return s;
     double *Bd = B;
     int64_t ld = ldb;
@@ -1919,7 +1914,7 @@ extern "C" wd_status wd_theta_step(wd_handle h, double *U, const double *F, int6
     if (nrhs == 0) return WD_OK;
     CK(cudaSetDevice(h->device), "set device");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    wd_status s = prepare_solve(h, nrhs);
+    wd_status s = prepare_solve(h, nrhs, h->prec == WD_MIXED);
     if (s != WD_OK) return s;
     double *Ud = U;
     const double *Fd = F;
@@ -2459,98 +2454,77 @@ extern "C" wd_status wd_value_gradient(wd_handle h, double g_logdet, const doubl
 // ---------------------------------------------------------------------------
 // LU without pivoting (FP64)
 // ---------------------------------------------------------------------------
-static void build_lu_plans(const wd::Symbolic &S, Plan &fp, Plan &sf, Plan &sb) {
-    fp = Plan();
-    sf = Plan();
-    sb = Plan();
-    constexpr int TL = 64;
-    for (int l = 0; l < S.nlevels; ++l) {
-        const int b = S.level_ptr[l], e = S.level_ptr[l + 1];
-        size_t f0 = fp.items.size();
-        double el = 0;
-        for (int i = b; i < e; ++i) {
-            const int s = S.level_nodes[i];
-            const int mp = front_order(S, s);
-            for (int q = 0; q < (mp + 7) / 8 * 8; ++q) fp.items.push_back({s, q < mp ? q : -1, 0, 0});
-            el += (double)mp * mp;
-        }
-        add_launch(fp, K_LU_INIT, f0, 0, 0, el, 0);
-        int kmax = 0;
-        for (int i = b; i < e; ++i) kmax = std::max(kmax, S.k(S.level_nodes[i]));
-        for (int kb = 0; kb < kmax; kb += NB) {
-            f0 = fp.items.size();
-            double fl = 0;
-            for (int i = b; i < e; ++i) {
-                const int s = S.level_nodes[i];
-                if (S.k(s) <= kb) continue;
-                const double nb = std::min(NB, S.k(s) - kb);
-                fp.items.push_back({s, 0, 0, 0});
-                fl += 2.0 * nb * nb * nb / 3 + 2.0 * nb * nb * nb / 3;
+// the factorization of enqueue_factor_plan for LU: the FP64 plan's launches on
+// the fronts of L and (unless sym) U^T, then both sides' super-block inverses,
+// U^T's through d_xs into its transposed place d_xts before L's take d_xs
+static void enqueue_lu_plan(wd_handle h, cudaStream_t st, bool sym) {
+    const DevSym &d = h->dsym;
+    const Plan &P = h->fplan;
+    wd::F64Args fa{};
+    fa.f = static_cast<double *>(h->d_front);
+    fa.g = static_cast<double *>(h->d_front_u);
+    fa.di = static_cast<double *>(h->d_dinv);
+    fa.du = h->d_uinv;
+    fa.sym = sym ? 1 : 0;
+    fa.cnt = h->d_diag_cnt;
+    fa.status = h->d_status;
+    double *xs = static_cast<double *>(h->d_xs), *xts = static_cast<double *>(h->d_xts);
+    for (const Launch &L : P.launches) {
+        const int4 *it = P.d_items + L.off;
+        switch (L.kind) {
+            case K_INIT: {
+                DevSym dv = d;
+                dv.csr_val = h->d_vcol;
+                wd::launch_front_init<double>(dv, fa.f, it, L.count, st);
+                if (sym) break;
+                dv.csr_val = h->d_vrow;
+                wd::launch_front_init<double>(dv, fa.g, it, L.count, st);
+                break;
             }
-            add_launch(fp, K_LU_DIAG, f0, kb, fl, 0, 0);
-            f0 = fp.items.size();
-            fl = 0;
-            for (int i = b; i < e; ++i) {
-                const int s = S.level_nodes[i], k = S.k(s);
-                if (k <= kb) continue;
-                const int nb = std::min(NB, k - kb), t0 = kb + nb, mp = front_order(S, s);
-                const int start = (t0 == k) ? kpad(k) : t0;
-                const int nblk = (mp - start + TL - 1) / TL;
-                for (int side = 0; side < 2; ++side)
-                    for (int q = 0; q < nblk; ++q) fp.items.push_back({s, q, side, 0});
-                fl += 2.0 * (double)(S.m(s) - t0) * nb * nb;
-            }
-            add_launch(fp, K_LU_PANEL, f0, kb, fl, 0, 0);
-            f0 = fp.items.size();
-            fl = 0;
-            for (int i = b; i < e; ++i) {
-                const int s = S.level_nodes[i], k = S.k(s);
-                if (k <= kb) continue;
-                const int nb = std::min(NB, k - kb), base = kb + nb, mp = front_order(S, s);
-                const int T = (mp - base + TL - 1) / TL;
-                for (int tj = 0; tj < T; ++tj)
-                    for (int ti = 0; ti < T; ++ti) fp.items.push_back({s, ti, tj, 0});
-                const double r = S.m(s) - base;
-                fl += 2.0 * r * r * nb;
-            }
-            add_launch(fp, K_LU_UPDATE, f0, kb, fl, 0, 0);
-        }
-        // substitutions: gather, then the pivot blocks of the level in order
-        f0 = sf.items.size();
-        for (int i = b; i < e; ++i) {
-            const int s = S.level_nodes[i];
-            for (int rc = 0; rc * 32 < S.m(s); ++rc) sf.items.push_back({s, rc, 0, 0});
-        }
-        add_launch(sf, K_LU_GATHER, f0, 0, 0, 0, 0);
-        for (int kb = 0; kb < kmax; kb += NB) {
-            f0 = sf.items.size();
-            for (int i = b; i < e; ++i) {
-                const int s = S.level_nodes[i], k = S.k(s);
-                if (k <= kb) continue;
-                const int t0 = kb + std::min(NB, k - kb);
-                const int nblk = 1 + (S.m(s) - t0 + TL - 1) / TL;
-                for (int q = 0; q < nblk; ++q) sf.items.push_back({s, q, 0, 0});
-            }
-            add_launch(sf, K_LU_FWD, f0, kb, 0, 0, 0);
+            case K_DIAG: wd::launch_diag64(d, fa, it, L.count, st); break;
+            case K_PANEL: wd::launch_panel64(d, fa, it, L.count, L.arg, st); break;
+            case K_UPDATE:
+            case K_OZ_UPDATE: wd::launch_update64(d, fa, it, L.count, L.arg, 0, st); break;
+            case K_SYRK:
+            case K_OZ_SYRK: wd::launch_update64(d, fa, it, L.count, 0, 1, st); break;
         }
     }
-    for (int l = S.nlevels - 1; l >= 0; --l) {
-        const int b = S.level_ptr[l], e = S.level_ptr[l + 1];
-        int kmax = 0;
-        for (int i = b; i < e; ++i) kmax = std::max(kmax, S.k(S.level_nodes[i]));
-        for (int kb = (kmax - 1) / NB * NB; kb >= 0; kb -= NB) {
-            const size_t f0 = sb.items.size();
-            for (int i = b; i < e; ++i) {
-                const int s = S.level_nodes[i];
-                if (S.k(s) > kb) sb.items.push_back({s, 0, 0, 0});
+    for (int side = 1; side >= 0; --side)
+        for (const Launch &L : P.launches) {
+            const int4 *it = P.d_items + L.off;
+            const double *F = side ? fa.g : fa.f;
+            double *D = side ? fa.du : fa.di;
+            switch (L.kind) {
+                case K_SBINV_DIAG: wd::launch_sbinv_diag64(d, F, D, xs, h->d_xsoff, it, L.count, st); break;
+                case K_SBINV_STAGE:
+                    wd::launch_sbinv_stage<double>(d, F, D, xs, h->d_xsoff, it, L.count, L.arg, st);
+                    break;
+                case K_SBINV_T:
+                    if (side) wd::launch_sbinv_transpose<double>(d, xs, xts, h->d_xsoff, it, L.count, st);
+                    break;
             }
-            add_launch(sb, K_LU_BWD, f0, kb, 0, 0, 0);
         }
-    }
 }
+
+static int64_t lu_launches(const Plan &P, bool sym) {
+    int64_t n = 0;
+    for (const Launch &L : P.launches) {
+        if (L.kind == K_OZ_SLICE) continue;
+        n += (L.kind == K_INIT && !sym) || L.kind == K_SBINV_DIAG || L.kind == K_SBINV_STAGE ? 2 : 1;
+    }
+    return n;
+}
+
+static wd_status factor_lu(wd_handle h, const double *lower, const double *upper, int on_device, bool sym,
+                           void *stream);
 
 extern "C" wd_status wd_factor_lu(wd_handle h, const double *lower, const double *upper, int on_device,
                                   void *stream) {
+    return factor_lu(h, lower, upper, on_device, false, stream);
+}
+
+static wd_status factor_lu(wd_handle h, const double *lower, const double *upper, int on_device, bool sym,
+                           void *stream) {
     if (!h) return WD_ERR_INVALID_ARG;
     if (!h->analyzed || h->opt.symbolic_only)
         return fail(h, WD_ERR_STATE, "wd_factor_lu before wd_analyze (or on a host-only handle)");
@@ -2565,25 +2539,24 @@ extern "C" wd_status wd_factor_lu(wd_handle h, const double *lower, const double
     const int64_t nnzl = h->S.pcp[h->S.n];
     if (!h->d_front) {
         CK(h->mem.alloc(&h->d_front, h->front_elems * sizeof(double)), "front pool alloc");
-        CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
-        CK(h->mem.alloc(&h->d_xs, h->xs_elems * sizeof(double)), "super-block inverse alloc");
-        CK(h->mem.alloc(&h->d_xts, h->xs_elems * sizeof(double)), "super-block inverse alloc");
         CK(cudaMemsetAsync(h->d_front, 0, h->front_elems * sizeof(double), st), "front pool clear");
     }
-    if (!h->d_uinv) {
-        CK(h->mem.alloc((void **)&h->d_uinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
-        CK(h->mem.alloc((void **)&h->d_vrow, h->nnz_full * sizeof(double)), "values alloc");
-        CK(h->mem.alloc((void **)&h->d_vcol, h->nnz_full * sizeof(double)), "values alloc");
-        CK(h->mem.alloc((void **)&h->d_lu_part, 2 * 64 * sizeof(double)), "logdet alloc");
+    if (!h->d_dinv) CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
+    if (!h->d_xs) CK(h->mem.alloc(&h->d_xs, h->xs_elems * sizeof(double)), "super-block inverse alloc");
+    if (!h->d_xts) CK(h->mem.alloc(&h->d_xts, h->xs_elems * sizeof(double)), "super-block inverse alloc");
+    if (!h->d_front_u) {
+        CK(h->mem.alloc(&h->d_front_u, h->front_elems * sizeof(double)), "front pool alloc");
+        CK(cudaMemsetAsync(h->d_front_u, 0, h->front_elems * sizeof(double), st), "front pool clear");
+    }
+    if (!h->d_uinv) CK(h->mem.alloc((void **)&h->d_uinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
+    if (!h->d_vrow) CK(h->mem.alloc((void **)&h->d_vrow, h->nnz_full * sizeof(double)), "values alloc");
+    if (!h->d_vcol) CK(h->mem.alloc((void **)&h->d_vcol, h->nnz_full * sizeof(double)), "values alloc");
+    if (!h->d_lu_part) CK(h->mem.alloc((void **)&h->d_lu_part, 2 * 64 * sizeof(double)), "logdet alloc");
+    if (!h->d_lu_code) {
         const int8_t *p = nullptr;
         wd_status us = upload(h, h->h_csr_code, &p);
         if (us != WD_OK) return us;
         h->d_lu_code = const_cast<int8_t *>(p);
-        build_lu_plans(h->S, h->fplan_lu, h->splan_lu_f, h->splan_lu_b);
-        for (Plan *P : {&h->fplan_lu, &h->splan_lu_f, &h->splan_lu_b}) {
-            wd_status ps = upload_plan(h, h->mem, *P);
-            if (ps != WD_OK) return ps;
-        }
     }
     const double *lo = lower, *up = upper;
     if (!on_device) {
@@ -2598,21 +2571,12 @@ extern "C" wd_status wd_factor_lu(wd_handle h, const double *lower, const double
     }
     wd::launch_lu_gather(h->d_csr_src, h->d_lu_code, lo, up, h->d_vrow, h->d_vcol, h->nnz_full, st);
     CK(cudaMemsetAsync(h->d_status, 0xFF, sizeof(status_t), st), "status reset");
-    h->front_dirty = true;
-    double *F = static_cast<double *>(h->d_front);
-    double *Li = static_cast<double *>(h->d_dinv);
-    const DevSym &d = h->dsym;
-    const Plan &P = h->fplan_lu;
-    for (const Launch &L : P.launches) {
-        const int4 *it = P.d_items + L.off;
-        switch (L.kind) {
-            case K_LU_INIT: wd::launch_lu_init(d, F, h->d_vrow, h->d_vcol, it, L.count, st); break;
-            case K_LU_DIAG: wd::launch_lu_diag(d, F, Li, h->d_uinv, it, L.count, L.arg, h->d_status, st); break;
-            case K_LU_PANEL: wd::launch_lu_panel(d, F, Li, h->d_uinv, it, L.count, L.arg, st); break;
-            case K_LU_UPDATE: wd::launch_lu_update(d, F, it, L.count, L.arg, st); break;
-        }
+    {
+        const wd_status fs =
+            run_graph(h, h->g_lu, sym ? 2 : 1, st, [&](cudaStream_t cs) { enqueue_lu_plan(h, cs, sym); });
+        if (fs != WD_OK) return fs;
     }
-    h->launches += 1 + (int64_t)P.launches.size();
+    h->launches += 1 + lu_launches(h->fplan, sym);
     CK(cudaGetLastError(), "LU factor launch");
     status_t status = 0;
     CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
@@ -2654,8 +2618,8 @@ extern "C" wd_status wd_get_level_schedule(wd_handle h, int8_t *step, int32_t nl
 extern "C" wd_status wd_factor_ldlt(wd_handle h, const double *values, int on_device, void *stream) {
     if (!h) return WD_ERR_INVALID_ARG;
     // the LU decomposition without pivoting of the symmetric matrix: L, and
-    // U = D L^T (the same values for both triangles)
-    const wd_status s = wd_factor_lu(h, values, values, on_device, stream);
+    // U = D L^T, which comes out of L's panels
+    const wd_status s = factor_lu(h, values, values, on_device, true, stream);
     h->ldlt = s == WD_OK;
     return s;
 }
@@ -2698,42 +2662,37 @@ extern "C" wd_status wd_solve_lu(wd_handle h, double *B, int64_t nrhs, int64_t l
     if (nrhs == 0) return WD_OK;
     CK(cudaSetDevice(h->device), "set device");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    constexpr int CH = 16;                      // right-hand sides per pass
-    wd_status s = ensure_solve_ws(h, CH);
+    // passes of at most CH columns, cut evenly, all with the plan (and graph)
+    // of the first; a shorter last pass solves zero columns beside its own
+    constexpr int64_t CH = 64;
+    const int64_t npass = (nrhs + CH - 1) / CH;
+    const int nc = (int)((nrhs + npass - 1) / npass);
+    wd_status s = prepare_solve(h, nc, false);
     if (s != WD_OK) return s;
-    double *Bd = B;          // host arrays go through d_B in chunks of CH columns
-    const int64_t ld = ldb;
-    double *Y = static_cast<double *>(h->d_Y), *Tt = static_cast<double *>(h->d_T);
-    double *W = static_cast<double *>(h->d_W);
-    const double *F = static_cast<const double *>(h->d_front);
-    const double *Li = static_cast<const double *>(h->d_dinv);
+    double *Y = static_cast<double *>(h->d_Y);
     const DevSym &d = h->dsym;
-    for (int64_t c0 = 0; c0 < nrhs; c0 += CH) {
-        const int nc = (int)std::min<int64_t>(CH, nrhs - c0);
-        if (B_on_device) {
-            wd::launch_permute_in<double>(Bd + c0 * ld, ld, Y, d.perm, n, nc, st);
-        } else {
+    for (int64_t c0 = 0; c0 < nrhs; c0 += nc) {
+        const int64_t mine = std::min<int64_t>(nc, nrhs - c0);
+        double *Bd = B + c0 * ldb;
+        int64_t ld = ldb;
+        if (!B_on_device) {   // host arrays go through d_B
             CK(cudaMemcpy2DAsync(h->d_B, n * sizeof(double), B + c0 * ldb, ldb * sizeof(double), n * sizeof(double),
-                                 nc, cudaMemcpyHostToDevice, st),
+                                 mine, cudaMemcpyHostToDevice, st),
                "B H2D");
-            wd::launch_permute_in<double>(h->d_B, n, Y, d.perm, n, nc, st);
+            Bd = h->d_B;
+            ld = n;
         }
-        for (const Launch &L : h->splan_lu_f.launches) {
-            const int4 *it = h->splan_lu_f.d_items + L.off;
-            if (L.kind == K_LU_GATHER) wd::launch_bfwd_gather<double>(d, Y, Tt, W, it, L.count, 16, nc, st);
-            else wd::launch_lu_fwd(d, F, Li, Y, Tt, W, it, L.count, L.arg, nc, st);
-        }
-        for (const Launch &L : h->splan_lu_b.launches)
-            wd::launch_lu_bwd(d, F, h->d_uinv, Y, h->splan_lu_b.d_items + L.off, L.count, L.arg, nc, st);
-        if (B_on_device) {
-            wd::launch_permute_out<double>(Y, Bd + c0 * ld, ld, d.perm, n, nc, st);
-        } else {
-            wd::launch_permute_out<double>(Y, h->d_B, n, d.perm, n, nc, st);
+        wd::launch_permute_in<double>(Bd, ld, Y, d.perm, n, mine, st);
+        if (mine < nc)
+            CK(cudaMemsetAsync(Y + n * mine, 0, n * (nc - mine) * sizeof(double), st), "empty columns");
+        s = run_solve_plan<double>(h, Y, nc, st, true);
+        if (s != WD_OK) return s;
+        wd::launch_permute_out<double>(Y, Bd, ld, d.perm, n, mine, st);
+        h->launches += 2;
+        if (!B_on_device)
             CK(cudaMemcpy2DAsync(B + c0 * ldb, ldb * sizeof(double), h->d_B, n * sizeof(double), n * sizeof(double),
-                                 nc, cudaMemcpyDeviceToHost, st),
+                                 mine, cudaMemcpyDeviceToHost, st),
                "B D2H");
-        }
-        h->launches += 2 + (int64_t)h->splan_lu_f.launches.size() + (int64_t)h->splan_lu_b.launches.size();
     }
     CK(cudaGetLastError(), "LU solve launch");
     CK(cudaStreamSynchronize(st), "LU solve");
@@ -2769,7 +2728,8 @@ extern "C" wd_status wd_export_LU(wd_handle h, double *lpanels, double *utpanels
         return cuda_fail(h, cudaErrorMemoryAllocation, "export alloc");
     }
     cudaMemcpy(d_poff, poff.data(), S.ns * sizeof(int64_t), cudaMemcpyHostToDevice);
-    wd::launch_lu_export(h->dsym, static_cast<const double *>(h->d_front), d_out, d_out + tot, d_poff, 0);
+    wd::launch_lu_export(h->dsym, static_cast<const double *>(h->d_front),
+                         static_cast<const double *>(h->d_front_u), d_out, d_out + tot, d_poff, 0);
     cudaError_t e = cudaMemcpy(lpanels, d_out, tot * sizeof(double), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(utpanels, d_out + tot, tot * sizeof(double), cudaMemcpyDeviceToHost);
     cudaFree(d_out);

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(T64) diag64_kernel(DevSym d, F64Args a, const 
 constexpr int PR = 16;           // rows per CTA
 constexpr int PLD = NB + 2;      // row stride of the staged T (16-byte multiple)
 constexpr int PXL = PR + 2;      // column stride of the staged rows
-constexpr int PANEL_ELEMS = NB * PLD + NB * PXL + PR * (PR + 1) + NB;
+constexpr int PANEL_ELEMS = NB * PLD + NB * PXL + PR * (PR + 1) + 2 * NB;
 
 __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const int4 *__restrict__ items, int kb,
                                                       int sides) {
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
     double *Ts = reinterpret_cast<double *>(smem_raw);   // [p][c]: T(c, p), the diagonal 16 x 16 blocks inverted
     double *Xs = Ts + NB * PLD;                            // [p][r]
     double *Bs = Xs + NB * PXL;                            // [r][c] of the current block
-    double *rd = Bs + PR * (PR + 1);                       // symmetric LU: 1 / d
+    double *rd = Bs + PR * (PR + 1);                       // symmetric LU: 1 / d, then d
     const int side = blockIdx.x % sides, q = (blockIdx.x / sides) % (RB / PR);
     const int4 it = items[blockIdx.x / (sides * (RB / PR))];
     const int s = it.x, rb = it.y;
@@ -109,7 +109,11 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
         cp_async16(Xs + p * PXL + r, valid ? C + (int64_t)(kb + p) * z.ld + r0 + r : Dv, 8 * valid);
     }
     cp_async_commit();
-    if (a.sym && tid < nb) rd[tid] = 1.0 / T[(int64_t)tid * z.ld + tid];
+    if (a.sym && tid < nb) {
+        const double dv = T[(int64_t)tid * z.ld + tid];
+        rd[tid] = 1.0 / dv;
+        rd[NB + tid] = dv;
+    }
     cp_async_wait<0>();
     __syncthreads();
     const int c = tid % 16, ra = tid / 16;      // rows ra, ra + 8
@@ -144,8 +148,10 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
         const double v = Xs[p * PXL + r];
         const int64_t o = (int64_t)(kb + p) * z.ld + r0 + r;
         if (a.sym) {
+            // v / d to half an ulp, by the reciprocal and one correction
+            const double r = rd[p], x = v * r;
             a.g[d.foff[s] + o] = v;
-            C[o] = v * rd[p];
+            C[o] = fma(fma(-x, rd[NB + p], v), r, x);
         } else {
             C[o] = v;
         }

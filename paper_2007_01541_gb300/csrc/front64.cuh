@@ -101,10 +101,16 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
                 if (lane == c) dl = dc, rl = r, v[c] = dc;
                 __syncwarp();
                 if (lane > c) {
-                    const double x = v[c] * r;
+                    double x = v[c] * r;
+                    if (lu) {
+                        // the quotient to half an ulp: x stays in the factor
+                        x = fma(fma(-x, dc, v[c]), r, x);
+                        // symmetric: U12 = D L21^T is w itself
+                        if (a.sym && lane >= S16 && act) A[jb + c][row] = v[c];
+                        v[c] = x;
+                    }
 #pragma unroll
                     for (int q = c + 1; q < S16; ++q) v[q] -= x * ub[q];
-                    if (lu) v[c] = x;
                 }
                 __syncwarp();
             }
@@ -155,13 +161,6 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
                 for (int q = 1; q < S16; ++q) A[jb + q][c] = y[q];
             }
             __syncthreads();
-        } else if (lu && rem > 0) {
-            // symmetric: U12 = D L21^T
-            for (int idx = tid; idx < rem * S16; idx += NT) {
-                const int c = t0 + idx % rem, q = jb + idx / rem;
-                A[q][c] = A[c][q] * A[q][q];
-            }
-            __syncthreads();
         }
         // trailing part (Cholesky and symmetric LU: lower), 2 x 2 tiles; the
         // block beyond nb is the identity and stays so
@@ -193,8 +192,8 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
     }
     // inverses of the 16 x 16 diagonal sub-blocks
     double *Di = a.di + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB;
-    double *Du = nonsym ? a.du + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB : nullptr;
-    if (warp < 4 && S16 * warp < nb && (nonsym || lane < S16)) {
+    double *Du = lu ? a.du + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB : nullptr;
+    if (warp < 4 && S16 * warp < nb && (lu || lane < S16)) {
         const int b0 = S16 * warp, c = lane & 15;
         const bool up = lane >= S16;        // U^T's
         double x[S16];

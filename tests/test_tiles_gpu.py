@@ -69,3 +69,45 @@ def test_fp64_pivot_status(wdlib, cuda, bad):
     with pytest.raises(wdlib.WdError) as e:
         s.factor(v, "fp64")
     assert e.value.status == wdlib.WD_ERR_NOT_SPD and e.value.column == bad
+
+
+@pytest.mark.parametrize("kind", ["lu", "ldlt"])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 33, 63, 64, 65, 97, 131, 200])
+def test_lu_block_edges(wdlib, cuda, kind, n):
+    """One dense front, nonsymmetric or symmetric indefinite, diagonally
+    dominant (so that no pivot is small); per-column tolerance 1e-10 as in
+    test_lu.py."""
+    rng = np.random.default_rng(n)
+    A = rng.standard_normal((n, n))
+    if kind == "ldlt":
+        A = A + A.T
+    A += np.diag(np.where(rng.random(n) < 0.5, -2.0, 2.0) * n)
+    cp, ri, lo = _lower_csc(A)
+    up = _lower_csc(np.ascontiguousarray(A.T))[2]
+    o = oracle.Oracle(cp, ri)
+    assert o.factor_lu(lo, up) == 0
+    s = wdlib.Solver().analyze(cp, ri)
+    s.factor_lu(lo, up) if kind == "lu" else s.factor_ldlt(lo)
+    for got, ref in zip(s.export_LU(), o.lu_values()):
+        got = s.L_csc_like(o.Lp, o.Li, got)
+        for j in range(n):
+            a, e = o.Lp[j], o.Lp[j + 1]
+            assert np.linalg.norm(got[a:e] - ref[a:e]) <= 1e-10 * np.linalg.norm(ref[a:e]), j
+    assert s.logdet_lu()[1] == o.logdet_lu()[1]
+    if kind == "ldlt":
+        assert s.inertia()[1] == int((np.linalg.eigvalsh(A) < 0).sum())
+
+
+@pytest.mark.parametrize("nrhs", [64, 65, 130])
+def test_lu_solve_passes(wdlib, cuda, nrhs):
+    """More right-hand sides than one pass takes: even and uneven passes."""
+    rng = np.random.default_rng(nrhs)
+    n = 150
+    A = rng.standard_normal((n, n)) + np.diag(np.full(n, 2.0 * n))
+    cp, ri, lo = _lower_csc(A)
+    up = _lower_csc(np.ascontiguousarray(A.T))[2]
+    s = wdlib.Solver().analyze(cp, ri).factor_lu(lo, up)
+    B = rhs(n, nrhs, seed=0)
+    for _ in range(2):                       # the second time with the kept plan
+        X = s.solve_lu(B)
+        assert oracle.nonsym_backward_error(cp, ri, lo, up, X, B).max() <= 1e-13
