@@ -19,7 +19,8 @@ SOURCES = ["csrc/symbolic.cpp", "csrc/api.cpp", "csrc/front_kernels.cu", "csrc/f
            "csrc/noalloc.cu", "csrc/batch.cu", "csrc/solve_blocked.cu", "csrc/tc_solve.cu",
            "csrc/lu.cu", "csrc/oz_schur.cu"]
 HEADERS = ["csrc/symbolic.h", "csrc/engine.h", "csrc/dev_common.cuh", "csrc/tc_common.cuh",
-           "csrc/front_block.cuh", "csrc/front64.cuh"]
+           "csrc/front_block.cuh", "csrc/front64.cuh",
+           "csrc/tile32.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -200,7 +200,7 @@ struct wd_ctx {
     double normA = 0.0;
     // selected inverse (built on first use; pointers into mem)
     struct SelStep {
-        int kind;  // 0 trinv, 1 gemm, 2 zgather
+        int kind;  // 0 super-block inverses, 1 gemm, 2 zgather
         int64_t off;
         int count;
     };
@@ -542,19 +542,24 @@ static void build_factor_plan(const wd::Symbolic &S, Plan &p, bool tc, bool oz =
                 }
         add_launch(p, K_SBINV_DIAG, f0, 0, 0, el, 0);
     }
-    for (int t = 1; t < BPS; ++t) {
+    // doublings: pairs of hb-block neighbours, 32 x 32 tiles (two per block),
+    // the same tiles in both phases
+    for (int hb = 1; hb < BPS; hb *= 2) {
         const size_t f0 = p.items.size();
         double fl = 0, el = 0;
-        for (int s = 0; s < S.ns; ++s)
+        for (int s = S.ns - 1; s >= 0; --s)
             for (int sb = 0; sb * wd::SB < S.k(s); ++sb) {
-                if (nblk_of(s, sb) <= t) continue;
-                for (int bj = 0; bj < t; ++bj) {
-                    p.items.push_back({s, sb, bj, 0});
-                    fl += 2.0 * NB * NB * NB * (t - bj) + (double)NB * NB * NB;
-                    el += 2.0 * NB * NB * (t - bj) + 2.0 * NB * NB;
+                const int nb = nblk_of(s, sb);
+                for (int g = 0; (2 * g + 1) * hb < nb; ++g) {
+                    const int rows = std::min(hb, nb - (2 * g + 1) * hb);
+                    for (int ti = 2 * rows - 1; ti >= 0; --ti)
+                        for (int tj = 0; tj < 2 * hb; ++tj) p.items.push_back({s, sb, g, ti | (tj << 16)});
+                    fl += 1.0 * rows * hb * hb * NB * NB * NB;
+                    el += 2.0 * rows * hb * NB * NB;
                 }
             }
-        add_launch(p, K_SBINV_STAGE, f0, t, fl, el, 0);
+        add_launch(p, K_SBINV_STAGE, f0, 2 * hb, fl, el, 0);
+        add_launch(p, K_SBINV_STAGE, f0, 2 * hb + 1, fl, el, 0);
     }
     {
         const size_t f0 = p.items.size();
@@ -1387,8 +1392,8 @@ static void enqueue_factor_plan(wd_handle h, cudaStream_t st, bool prof) {
                                             st);
                 break;
             case K_SBINV_STAGE:
-                wd::launch_sbinv_stage<T>(d, F, Dv, static_cast<T *>(h->d_xs), h->d_xsoff, it, L.count, L.arg,
-                                          st);
+                wd::launch_sbinv_double<T>(d, F, static_cast<T *>(h->d_xs), static_cast<T *>(h->d_xts), h->d_xsoff,
+                                           it, L.count, L.arg / 2, L.arg % 2, st);
                 break;
             case K_SBINV_T:
                 wd::launch_sbinv_transpose<T>(d, static_cast<const T *>(h->d_xs), static_cast<T *>(h->d_xts),
@@ -2221,16 +2226,11 @@ static wd_status build_selinv(wd_handle h) {
         if (end > off) steps.push_back({kind, off, (int)(end - off)});
     };
     auto tiles = [](int x) { return (x + 63) / 64; };
-    // 1) X = L_JJ^-1 by block rows
-    int maxblk = 0;
-    for (int s = 0; s < ns; ++s) maxblk = std::max(maxblk, tiles(S.k(s)));
-    for (int t = 0; t < maxblk; ++t) {
-        const int64_t o = (int64_t)items.size();
-        for (int s = 0; s < ns; ++s)
-            if (tiles(S.k(s)) > t)
-                for (int bj = 0; bj <= t; ++bj) items.push_back({s, t, bj, 0});
-        push_step(0, o, (int64_t)items.size());
-    }
+    // 1) X = L_JJ^-1: the factor's super-block inverses on its diagonal, then
+    //    doublings, X21 = -X22 (L21 X11), with L21 X11 kept where Z_JJ will be
+    for (int s = ns - 1; s >= 0; --s)
+        for (int sb = 0; sb * wd::SB < S.k(s); ++sb) items.push_back({s, sb, 0, 0});
+    push_step(0, 0, (int64_t)items.size());
     auto gi = [](const double *A, int64_t ars, int64_t acs, const double *B, int64_t brs, int64_t bcs,
                  double *C, int64_t crs, int64_t ccs, int M, int N, int p0, int p1, int i0, int j0,
                  int flags, double alpha) {
@@ -2255,11 +2255,35 @@ static wd_status build_selinv(wd_handle h) {
         g.alpha = alpha;
         return g;
     };
+    int maxk = 0;
+    for (int s = 0; s < ns; ++s) maxk = std::max(maxk, S.k(s));
+    for (int hw = wd::SB; hw < maxk; hw *= 2)
+        for (int phase = 0; phase < 2; ++phase) {
+            const int64_t o = (int64_t)gemm.size();
+            for (int s = ns - 1; s >= 0; --s) {
+                const int k = S.k(s), ld = h->h_sld[s];
+                const int64_t fo = h->h_foff[s];
+                double *X = XW + xoff[s], *T = Z + fo;
+                for (int g0 = 0; g0 + hw < k; g0 += 2 * hw) {
+                    const int mid = g0 + hw, end = std::min(k, mid + hw);
+                    for (int i0 = mid; i0 < end; i0 += 64)
+                        for (int j0 = g0; j0 < mid; j0 += 64) {
+                            if (phase == 0)
+                                gemm.push_back(gi(F + fo, 1, ld, X, k, 1, T, 1, ld, end, mid, j0, mid, i0, j0, 0, 1.0));
+                            else
+                                gemm.push_back(gi(X, 1, k, T, ld, 1, X, 1, k, end, mid, mid, std::min(end, i0 + 64), i0,
+                                                  j0, 0, -1.0));
+                        }
+                    flops += (double)(end - mid) * hw * hw;
+                }
+            }
+            push_step(1, o, (int64_t)gemm.size());
+        }
     // 2) W = L_RJ X (X lower triangular: p from the tile's first column) and
     //    Z_JJ = X^T X (lower tiles, p from the tile's first row)
     {
         const int64_t o = (int64_t)gemm.size();
-        for (int s = 0; s < ns; ++s) {
+        for (int s = ns - 1; s >= 0; --s) {
             const int k = S.k(s), r = S.m(s) - S.k(s), kp = kpad(k), ld = h->h_sld[s];
             const int64_t fo = h->h_foff[s];
             double *X = XW + xoff[s], *W = X + (int64_t)k * k;
@@ -2339,13 +2363,12 @@ static wd_status selinv_enqueue(wd_handle h, double *dst, cudaStream_t st) {
         if (s != WD_OK) return s;
     }
     const DevSym &d = h->dsym;
-    const double *F = static_cast<const double *>(h->d_front);
-    const double *Dv = static_cast<const double *>(h->d_dinv);
     prof_single(h, "selinv_fp64", 0, 0, st, true);
     for (const auto &sp : h->sel_steps) {
         switch (sp.kind) {
             case 0:
-                wd::launch_trinv(d, F, Dv, h->d_xw, h->d_xoff, h->d_sel_items + sp.off, sp.count, st);
+                wd::launch_xcopy(d, static_cast<const double *>(h->d_xs), h->d_xsoff, h->d_xw, h->d_xoff,
+                                 h->d_sel_items + sp.off, sp.count, st);
                 break;
             case 1: wd::launch_gemm_items(h->d_sel_gemm + sp.off, sp.count, st); break;
             case 2:
@@ -2497,7 +2520,8 @@ static void enqueue_lu_plan(wd_handle h, cudaStream_t st, bool sym) {
             switch (L.kind) {
                 case K_SBINV_DIAG: wd::launch_sbinv_diag64(d, F, D, xs, h->d_xsoff, it, L.count, st); break;
                 case K_SBINV_STAGE:
-                    wd::launch_sbinv_stage<double>(d, F, D, xs, h->d_xsoff, it, L.count, L.arg, st);
+                    wd::launch_sbinv_double<double>(d, F, xs, xts, h->d_xsoff, it, L.count, L.arg / 2, L.arg % 2,
+                                                    st);
                     break;
                 case K_SBINV_T:
                     if (side) wd::launch_sbinv_transpose<double>(d, xs, xts, h->d_xsoff, it, L.count, st);

@@ -266,8 +266,9 @@ struct GemmItem {
     double alpha;
 };
 void launch_gemm_items(const GemmItem *items, int count, cudaStream_t st);
-void launch_trinv(const DevSym &d, const double *front, const double *dinv, double *xpool,
-                  const int64_t *xoff, const int4 *items, int count, cudaStream_t st);
+// item = (s, super-block): its inverse (d_xs) into the diagonal of X_s
+void launch_xcopy(const DevSym &d, const double *xs, const int64_t *xsoff, double *xpool, const int64_t *xoff,
+                  const int4 *items, int count, cudaStream_t st);
 void launch_zgather(const DevSym &d, double *zpool, const int32_t *upmap, const int64_t *upoff,
                     const int4 *items, int count, cudaStream_t st);
 void launch_zextract(const DevSym &d, const double *zpool, const int32_t *col2s, const int32_t *psrc,
@@ -285,9 +286,11 @@ void launch_sym_outer(const DevSym &d, const int32_t *prow, const int32_t *psrc,
 constexpr int SB = 512;
 void launch_sbinv_diag(const DevSym &d, const float *dinv, float *xpool, const int64_t *xsoff, const int4 *items,
                        int count, cudaStream_t st);
+// one half step of a doubling of the super-block inverses: blocks of hb x 64
+// columns in place; tpool: the transposes' store (scratch in its lower blocks)
 template <class T>
-void launch_sbinv_stage(const DevSym &d, const T *front, const T *dinv, T *xpool, const int64_t *xsoff,
-                        const int4 *items, int count, int t, cudaStream_t st);
+void launch_sbinv_double(const DevSym &d, const T *front, T *xpool, T *tpool, const int64_t *xsoff,
+                         const int4 *items, int count, int hb, int phase, cudaStream_t st);
 template <class T>
 void launch_sbinv_transpose(const DevSym &d, const T *xpool, T *xtpool, const int64_t *xsoff,
                             const int4 *items, int count, cudaStream_t st);

@@ -9,139 +9,89 @@
 // Z_RR (the rows of R are a clique of L's graph, all owned by ancestors) is
 // gathered from the parent's Z front through the extend-add row maps.  Every
 // supernode stores its whole Z front (rows x rows, lower), laid out like its
-// factor front.  L_JJ^-1 is built by blocked inversion from the stored
-// inverses of the 64 x 64 diagonal blocks:
-//   X(bi, bj) = -D(bi)^-1 sum_{p in blocks bj .. bi-1} L(bi, p) X(p, bj).
+// factor front.  L_JJ^-1 starts from the factor's super-block inverses and
+// doubles: X21 = -X22 (L21 X11).
 #include "dev_common.cuh"
 #include "engine.h"
+#include "tile32.cuh"
 
 namespace wd {
 namespace {
 
 constexpr int THREADS = 256;
-constexpr int TM = 64, TN = 64, TK = 16;
 
-// C(i, j) (+)= alpha sum_p A(i, p) B(j, p) on one 64 x 64 tile.  a_pfast /
-// b_pfast: the operand is contiguous along p (load p-fastest for coalescing).
-template <class FA, class FB>
-__device__ __forceinline__ void tile_acc(FA a_at, FB b_at, bool a_pfast, bool b_pfast, int M, int N,
-                                         int p0, int p1, int i0, int j0, double (&acc)[4][4],
-                                         double *smem) {
-    double(*As)[TM + 1] = reinterpret_cast<double(*)[TM + 1]>(smem);
-    double(*Bs)[TN + 1] = reinterpret_cast<double(*)[TN + 1]>(smem + TK * (TM + 1));
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    for (int k0 = p0; k0 < p1; k0 += TK) {
-        for (int idx = tid; idx < TK * TM; idx += THREADS) {
-            const int kk = a_pfast ? idx % TK : idx / TM, r = a_pfast ? idx / TK : idx % TM;
-            const int p = k0 + kk;
-            As[kk][r] = (p < p1 && i0 + r < M) ? a_at(i0 + r, p) : 0.0;
+// One 64 x 64 item is four CTAs of 32 x 32 (tile32.cuh).  Each operand is
+// read along its contiguous index: rows (x_rs == 1) or the inner one; a
+// symmetric A is read below its diagonal.  Bound: the FP64 pipe.
+// Square, 16,384 unknowns: the products 28.1 -> 20.7 ms against 64 x 64 tiles
+// of 256 threads, now with the inversion's, which took 23.0 ms as block rows
+// one after the other.
+__global__ void __launch_bounds__(t32::TH) gemm_items_kernel(const GemmItem *__restrict__ items) {
+    __shared__ double As[2][t32::TK * t32::LD], Bs[2][t32::TK * t32::LD];
+    const GemmItem &g = items[blockIdx.x >> 2];
+    const int i0 = g.i0 + 32 * (blockIdx.x & 1), j0 = g.j0 + 32 * ((blockIdx.x >> 1) & 1);
+    const int M = g.M, N = g.N, p1 = g.p1, flags = g.flags;
+    if (i0 >= M || j0 >= N || ((flags & GEMM_C_LOWER) && i0 + 31 < j0)) return;
+    const double *A = g.A, *B = g.B;
+    const int64_t ars = g.a_rs, acs = g.a_cs, brs = g.b_rs, bcs = g.b_cs;
+    double acc[4][2] = {};
+    t32::product(acc, As, Bs, g.p0, p1, [&](int buf, int p) {
+        if (flags & GEMM_A_SYM_LOWER) {
+            if (p + t32::TK <= i0) {
+                t32::stage_rows(As[buf], A + (int64_t)p * acs + i0, acs, M - i0, p1 - p);
+            } else if (p >= i0 + t32::TT) {
+                t32::stage_inner(As[buf], A + (int64_t)i0 * acs + p, acs, M - i0, p1 - p);
+            } else {
+                for (int idx = threadIdx.x; idx < t32::TT * t32::TK; idx += t32::TH) {
+                    const int i = i0 + idx % t32::TT, q = p + idx / t32::TT;
+                    const bool v = i < M && q < p1;
+                    const int hi = max(i, q), lo = min(i, q);
+                    cp_async_elem(&As[buf][(q - p) * t32::LD + i - i0], v ? A + (int64_t)lo * acs + hi : A, v);
+                }
+            }
+        } else if (ars == 1) {
+            t32::stage_rows(As[buf], A + (int64_t)p * acs + i0, acs, M - i0, p1 - p);
+        } else {
+            t32::stage_inner(As[buf], A + (int64_t)i0 * ars + p, ars, M - i0, p1 - p);
         }
-        for (int idx = tid; idx < TK * TN; idx += THREADS) {
-            const int kk = b_pfast ? idx % TK : idx / TN, r = b_pfast ? idx / TK : idx % TN;
-            const int p = k0 + kk;
-            Bs[kk][r] = (p < p1 && j0 + r < N) ? b_at(j0 + r, p) : 0.0;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < TK; ++kk) {
-            double a[4], b[4];
+        if (bcs == 1) t32::stage_inner(Bs[buf], B + (int64_t)j0 * brs + p, brs, N - j0, p1 - p);
+        else t32::stage_rows(Bs[buf], B + (int64_t)p * bcs + j0, bcs, N - j0, p1 - p);
+    });
+    const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
+    const double alpha = g.alpha;
+    const int64_t crs = g.c_rs, ccs = g.c_cs;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][tx + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][ty + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
-        }
-        __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(THREADS) gemm_items_kernel(const GemmItem *__restrict__ items) {
-    __shared__ double smem[TK * (TM + 1) + TK * (TN + 1)];
-    const GemmItem g = items[blockIdx.x];
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    const bool asym = g.flags & GEMM_A_SYM_LOWER;
-    auto a_at = [&](int i, int p) -> double {
-        if (asym) {
-            const int hi = i > p ? i : p, lo = i > p ? p : i;
-            return g.A[(int64_t)hi * g.a_rs + (int64_t)lo * g.a_cs];
-        }
-        return g.A[(int64_t)i * g.a_rs + (int64_t)p * g.a_cs];
-    };
-    auto b_at = [&](int j, int p) -> double { return g.B[(int64_t)j * g.b_rs + (int64_t)p * g.b_cs]; };
-    tile_acc(a_at, b_at, !asym && g.a_cs == 1, g.b_cs == 1, g.M, g.N, g.p0, g.p1, g.i0, g.j0, acc,
-             smem);
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = g.j0 + ty + 16 * j;
-        if (c >= g.N) continue;
+    for (int j = 0; j < 2; ++j) {
+        const int c = j0 + ty + 16 * j;
+        if (c >= N) continue;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int r = g.i0 + tx + 16 * i;
-            if (r >= g.M) continue;
-            if ((g.flags & GEMM_C_LOWER) && r < c) continue;
-            double *cp = g.C + (int64_t)r * g.c_rs + (int64_t)c * g.c_cs;
-            const double v = g.alpha * acc[i][j];
-            *cp = (g.flags & GEMM_ACCUMULATE) ? *cp + v : v;
+            const int r = i0 + tx + 8 * i;
+            if (r >= M || ((flags & GEMM_C_LOWER) && r < c)) continue;
+            double *cp = g.C + (int64_t)r * crs + (int64_t)c * ccs;
+            const double v = alpha * acc[i][j];
+            *cp = (flags & GEMM_ACCUMULATE) ? *cp + v : v;
         }
     }
 }
 
-// X(bi, bj) = -D(bi)^-1 T with T = sum_{p in [bj*64, bi*64)} L(bi*64 + r, p) X(p, bj*64 + c),
-// or X(bi, bi) = D(bi)^-1 when bj == bi.  item = (supernode, bi, bj)
-__global__ void __launch_bounds__(THREADS) trinv_kernel(DevSym d, const double *__restrict__ front,
-                                                        const double *__restrict__ dinv,
+// the super-block's inverse into the diagonal of X_s (k x k, ld k);
+// item = (s, super-block)
+__global__ void __launch_bounds__(THREADS) xcopy_kernel(DevSym d, const double *__restrict__ xs,
+                                                        const int64_t *__restrict__ xsoff,
                                                         double *__restrict__ xpool,
                                                         const int64_t *__restrict__ xoff,
                                                         const int4 *__restrict__ items) {
-    // the tile product's staging buffers, then (after it) the 64 x 64 result
-    __shared__ double smem[NB * (NB + 1)];
-    static_assert(TK * (TM + 1) + TK * (TN + 1) <= NB * (NB + 1), "staging fits");
-    double(*Ts)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(smem);
     const int4 it = items[blockIdx.x];
-    const int s = it.x, bi = it.y, bj = it.z;
-    const int k = d.sk[s], ld = d.sld[s];
-    const double *L = front + d.foff[s];
-    double *X = xpool + xoff[s];  // k x k, ld k
-    const double *Db = dinv + d.dinvoff[s] + (int64_t)bi * NB * NB;
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int r0 = bi * NB, c0 = bj * NB;
-    if (bi == bj) {
-        for (int idx = tid; idx < NB * NB; idx += THREADS) {
-            const int r = idx % NB, c = idx / NB;
-            if (r0 + r < k && c0 + c < k) X[(int64_t)(c0 + c) * k + r0 + r] = Db[idx];
-        }
-        return;
-    }
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    auto a_at = [&](int i, int p) -> double { return L[(int64_t)p * ld + i]; };
-    auto b_at = [&](int j, int p) -> double { return X[(int64_t)j * k + p]; };
-    tile_acc(a_at, b_at, false, true, k, k, c0, r0, r0, c0, acc, smem);
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) Ts[tx + 16 * i][ty + 16 * j] = acc[i][j];
-    __syncthreads();
-    // X(bi, bj) = -Db Ts  (Db lower triangular, column-major NB x NB; rows of a
-    // partial last block beyond k are not used)
-    const int kv = min(NB, k - r0);
-    for (int idx = tid; idx < NB * NB; idx += THREADS) {
-        const int r = idx % NB, c = idx / NB;
-        double v = 0.0;
-        if (r < kv)
-            for (int p = 0; p <= r; ++p) v += Db[(int64_t)p * NB + r] * Ts[p][c];
-        if (r0 + r < k && c0 + c < k) X[(int64_t)(c0 + c) * k + r0 + r] = -v;
+    const int s = it.x, sb = it.y, k = d.sk[s], c0 = sb * SB;
+    const int w = min(SB, k - c0), wp = (w + NB - 1) / NB * NB;
+    const double *S = xs + xsoff[s] + (int64_t)sb * SB * SB;
+    double *X = xpool + xoff[s] + (int64_t)c0 * k + c0;
+    // 64-row stripes of the launch's second grid dimension
+    const int r0 = blockIdx.y * NB;
+    for (int idx = threadIdx.x; idx < NB * (r0 + NB); idx += THREADS) {
+        const int r = r0 + idx % NB, c = idx / NB;
+        if (r < w && c <= r) X[(int64_t)c * k + r] = S[(int64_t)c * wp + r];
     }
 }
 
@@ -217,13 +167,13 @@ __global__ void sym_outer_kernel(DevSym d, const int32_t *__restrict__ prow,
 
 void launch_gemm_items(const GemmItem *items, int count, cudaStream_t st) {
     if (count <= 0) return;
-    gemm_items_kernel<<<count, THREADS, 0, st>>>(items);
+    gemm_items_kernel<<<4 * count, t32::TH, 0, st>>>(items);
 }
 
-void launch_trinv(const DevSym &d, const double *front, const double *dinv, double *xpool,
-                  const int64_t *xoff, const int4 *items, int count, cudaStream_t st) {
+void launch_xcopy(const DevSym &d, const double *xs, const int64_t *xsoff, double *xpool, const int64_t *xoff,
+                  const int4 *items, int count, cudaStream_t st) {
     if (count <= 0) return;
-    trinv_kernel<<<count, THREADS, 0, st>>>(d, front, dinv, xpool, xoff, items);
+    xcopy_kernel<<<dim3(count, SB / NB), THREADS, 0, st>>>(d, xs, xsoff, xpool, xoff, items);
 }
 
 void launch_zgather(const DevSym &d, double *zpool, const int32_t *upmap, const int64_t *upoff,
