@@ -63,7 +63,7 @@ struct Plan {
     std::vector<Launch> launches;
     int4 *d_items = nullptr;
     int rgt = 16;            // solve plans: right-hand sides per gather CTA
-    int large = 0;           // solve plans: product mode (0: 64 x 32 tiles, 2: few right-hand sides)
+    int large = 0;           // solve plans: product mode (0: 32 x 32 tiles, 1: tensor cores, 2: few right-hand sides)
     int64_t slots = 0;       // solve plans: partial-sum slots of the largest split step
     int64_t ksplit = 0;      // solve plans: CTAs of the largest launch split over the inner dimension
 };
@@ -182,12 +182,12 @@ struct wd_ctx {
     void *d_Y = nullptr, *d_W = nullptr, *d_T = nullptr;
     void *d_part = nullptr;        // partial sums of the backward split reduction
     int64_t part_elems = 0;
-    // tensor-core solve products split over the inner dimension: one partial
+    // solve products split over the inner dimension: one partial
     // tile per CTA and one arrival counter per output tile (kept at zero
     // between launches)
-    float *d_ksw = nullptr;
+    void *d_ksw = nullptr;
     int *d_kcnt = nullptr;
-    int64_t ksw_items = 0;
+    int64_t ksw_bytes = 0, ksw_items = 0;
     int sms = 152;                 // multiprocessors of the device
     double *d_B = nullptr, *d_Bp = nullptr, *d_X = nullptr, *d_R = nullptr, *d_cm = nullptr;
     float2 *d_Xp = nullptr;   // double-float split of the refinement vectors, (hi, lo) pairs
@@ -598,6 +598,28 @@ static void split_inner(Plan &p, size_t f0, int sms) {
     p.ksplit = std::max<int64_t>(p.ksplit, (int64_t)split.size());
 }
 
+// The same for the 32 x 32 tiles (mode 0): up to eight CTAs per tile, at least
+// 64 of the inner dimension each (nch: a tile's 64-wide chunks), until the
+// launch has two CTAs per SM: below that a tile's whole inner dimension on
+// one SM sets the launch's time, above it the splits only add traffic.
+static void split_tiles(Plan &p, size_t f0, const std::vector<int> &nch, int sms) {
+    const int64_t tiles = (int64_t)(p.items.size() - f0);
+    if (tiles <= 0 || tiles >= 2 * sms) return;
+    const int want = (int)std::min<int64_t>(8, (2 * sms + tiles - 1) / tiles);
+    std::vector<int4> split;
+    for (int64_t i = 0; i < tiles; ++i) {
+        const int nks = std::max(1, std::min(want, nch[i]));
+        for (int ks = 0; ks < nks; ++ks) {
+            int4 q = p.items[f0 + i];
+            q.z = q.z | (ks << 16) | (nks << 24);
+            split.push_back(q);
+        }
+    }
+    p.items.resize(f0);
+    p.items.insert(p.items.end(), split.begin(), split.end());
+    p.ksplit = std::max<int64_t>(p.ksplit, (int64_t)split.size());
+}
+
 static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms, Plan &p) {
     p.items.clear();
     p.launches.clear();
@@ -615,6 +637,12 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
     auto nsb = [&](int s) { return (S.k(s) + SBW - 1) / SBW; };
     auto width = [&](int s, int sb) { return std::min(SBW, S.k(s) - sb * SBW); };
     auto wpad = [&](int s, int sb) { return (width(s, sb) + NB - 1) / NB * NB; };
+    std::vector<int> nch;      // mode 0: 64-wide chunks of each tile's inner dimension
+    auto split = [&](size_t f0) {
+        if (large == 1) split_inner(p, f0, sms);
+        else if (large == 0) split_tiles(p, f0, nch, sms);
+        nch.clear();
+    };
     for (int l = 0; l < S.nlevels; ++l) {
         const int b = S.level_ptr[l], e = S.level_ptr[l + 1];
         size_t f0 = p.items.size();
@@ -637,12 +665,15 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
                 const int s = S.level_nodes[i];
                 if (nsb(s) <= sb) continue;
                 const int w = width(s, sb), wp = wpad(s, sb);
-                for (int rb = 0; rb * TRX < wp; ++rb)
-                    for (int g = 0; g < ng; ++g) p.items.push_back({s, sb, rb, g});
+                for (int rb = (wp + TRX - 1) / TRX - 1; rb >= 0; --rb)   // the longest inner ranges first
+                    for (int g = 0; g < ng; ++g) {
+                        p.items.push_back({s, sb, rb, g});
+                        nch.push_back((std::min(w, (rb + 1) * TRX) + 63) / 64);
+                    }
                 fl += (double)w * (w + 1) * R;
                 el += (double)w * (w + 1) / 2 + 2.0 * w * R;
             }
-            if (large == 1) split_inner(p, f0, sms);
+            split(f0);
             add_launch(p, K_FWD_XAPPLY, f0, sb, fl, el, 0);
             f0 = p.items.size();
             el = fl = 0;
@@ -655,10 +686,11 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
                     for (int g = 0; g < ng; ++g) p.items.push_back({s, sb, rb, g});
                 for (int rb = 0; rb * TRX < nR; ++rb)
                     for (int g = 0; g < ng; ++g) p.items.push_back({s, sb, rb, g + 65536});
+                nch.resize(p.items.size() - f0, (w + 63) / 64);
                 fl += 2.0 * (nJ + nR) * w * R;
                 el += (double)(nJ + nR) * w + 2.0 * (nJ + nR) * R + w * R;
             }
-            if (large == 1) split_inner(p, f0, sms);
+            split(f0);
             add_launch(p, K_FWD_BUPDATE, f0, sb, fl, el, 0);
         }
     }
@@ -677,16 +709,17 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
                 if (nsb(s) <= sb) continue;
                 const int m = S.m(s), w = width(s, sb);
                 const int below = m - (sb * SBW + w);
-                // tensor-core splits run over the front's storage rows from the
-                // 32-row boundary at or above the super-block's end
-                const int kbeg = (sb * SBW + w) & ~31;
-                const int nsplit = large == 1 ? (below > 0 ? (front_order(S, s) - kbeg + KSR - 1) / KSR : 0)
-                                              : (below + KSR - 1) / KSR;
+                // the splits run over the front's storage rows (tensor cores:
+                // from the 32-row boundary at or above the super-block's end),
+                // the narrow kernels' over the rows below
+                const int kbeg = large == 1 ? (sb * SBW + w) & ~31 : sb * SBW + w;
+                const int nsplit = large == 2 ? (below + KSR - 1) / KSR
+                                              : (below > 0 ? (front_order(S, s) - kbeg + KSR - 1) / KSR : 0);
                 for (int cb = 0; cb * TRW < w; ++cb)
                     for (int g = 0; g < ng; ++g) {
-                        fin.push_back({s, sb * 8 + cb, g + 65536 * nsplit, slot});
+                        fin.push_back({s, sb * 16 + cb, g + 65536 * nsplit, slot});
                         for (int ks = 0; ks < nsplit; ++ks)
-                            p.items.push_back({s, sb * 8 + cb, g + 65536 * ks, slot++});
+                            p.items.push_back({s, sb * 16 + cb, g + 65536 * ks, slot++});
                     }
                 fl += 2.0 * below * w * R;
                 el += (double)below * w + below * R;
@@ -707,11 +740,14 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
                 if (nsb(s) <= sb) continue;
                 const int w = width(s, sb), wp = wpad(s, sb);
                 for (int rb = 0; rb * TRX < wp; ++rb)
-                    for (int g = 0; g < ng; ++g) p.items.push_back({s, sb, rb, g});
+                    for (int g = 0; g < ng; ++g) {
+                        p.items.push_back({s, sb, rb, g});
+                        nch.push_back((std::max(1, w - rb * TRX) + 63) / 64);
+                    }
                 fl += (double)w * (w + 1) * R;
                 el += (double)w * (w + 1) / 2 + 2.0 * w * R;
             }
-            if (large == 1) split_inner(p, f0, sms);
+            split(f0);
             add_launch(p, K_BWD_XAPPLY, f0, sb, fl, el, 0);
         }
     }
@@ -804,7 +840,7 @@ static wd_status reset_analysis(wd_handle h) {
     h->ws_cols = 0;
     h->d_ksw = nullptr;
     h->d_kcnt = nullptr;
-    h->ksw_items = 0;
+    h->ksw_items = h->ksw_bytes = 0;
     h->d_front = nullptr;
     h->d_dinv = nullptr;
     h->d_gcsr = h->mass_buf = nullptr;
@@ -1543,7 +1579,7 @@ static wd_status ensure_solve_ws(wd_handle h, int64_t nrhs) {
     h->d_Xp = nullptr;
     h->d_ksw = nullptr;
     h->d_kcnt = nullptr;
-    h->ksw_items = 0;
+    h->ksw_items = h->ksw_bytes = 0;
     h->splan = Plan();
     h->aplan = Plan();
     h->splan_nrhs = h->aplan_nrhs = -1;
@@ -1578,6 +1614,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
     T *W = static_cast<T *>(h->d_W);
     T *Tt = static_cast<T *>(h->d_T);
     T *P = static_cast<T *>(h->d_part);
+    T *ksw = static_cast<T *>(h->d_ksw);
     const DevSym &d = h->dsym;
     const int rgt = h->splan.rgt;
     const int lg = h->splan.large;
@@ -1591,7 +1628,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
     ta.tstatus = h->d_tstatus;
     ta.nrhs = nrhs;
     ta.wait_limit = (uint32_t)std::max(0, h->opt.wait_limit);
-    ta.ksw = h->d_ksw;
+    ta.ksw = static_cast<float *>(h->d_ksw);
     ta.kcnt = h->d_kcnt;
     ta.sms = h->sms;
     const bool tc = lg == 1 && sizeof(T) == 4;
@@ -1610,7 +1647,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.upper = 0;
                     wd::launch_tc_xapply(d, a, it, L.count, st);
                 } else {
-                    wd::launch_xapply<T>(d, Xs, h->d_xsoff, Tt, Y, it, L.count, 0, lg, nrhs, st);
+                    wd::launch_xapply<T>(d, Xs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 0, lg, nrhs, st);
                 }
                 break;
             case K_FWD_BUPDATE:
@@ -1620,7 +1657,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.out = reinterpret_cast<float *>(Tt);
                     wd::launch_tc_bupdate(d, a, it, L.count, st);
                 } else {
-                    wd::launch_bupdate<T>(d, F, Y, Tt, W, it, L.count, lg, nrhs, st);
+                    wd::launch_bupdate<T>(d, F, Y, Tt, W, ksw, h->d_kcnt, it, L.count, lg, nrhs, st);
                 }
                 break;
             case K_BWD_REDUCE:
@@ -1643,7 +1680,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.upper = 1;
                     wd::launch_tc_xapply(d, a, it, L.count, st);
                 } else {
-                    wd::launch_xapply<T>(d, XTs, h->d_xsoff, Tt, Y, it, L.count, 1, lg, nrhs, st);
+                    wd::launch_xapply<T>(d, XTs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 1, lg, nrhs, st);
                 }
                 break;
         }
@@ -1752,7 +1789,7 @@ static wd_status backward_errors(wd_handle h, const double *X, int64_t nrhs, cud
 static wd_status prepare_solve(wd_handle h, int64_t nrhs, bool mixed) {
     wd_status s = ensure_solve_ws(h, nrhs);
     if (s != WD_OK) return s;
-    // tiles of 64 rows x 32 right-hand sides; FP32 with more than 8
+    // tiles of 32 rows x 32 right-hand sides; FP32 with more than 8
     // right-hand sides: tensor-core tiles of 128 rows x 64 right-hand sides
     // (unless wd_options.solve_simt); up to 8 right-hand sides:
     // matrix-vector shaped kernels, lanes over rows
@@ -1761,13 +1798,18 @@ static wd_status prepare_solve(wd_handle h, int64_t nrhs, bool mixed) {
         build_solve_plan(h->S, (int)nrhs, large, h->sms, h->splan);
         s = upload_plan(h, h->work, h->splan);
         if (s != WD_OK) return s;
-        if (h->splan.ksplit > h->ksw_items) {
+        const int64_t kb = h->splan.ksplit * (large == 1 ? wd::TC_SOLVE_TILE * sizeof(float) : 32 * 32 * sizeof(double));
+        if (kb > h->ksw_bytes) {
             if (h->d_ksw) h->work.release(h->d_ksw);
-            if (h->d_kcnt) h->work.release(h->d_kcnt);
             h->d_ksw = nullptr;
+            h->ksw_bytes = 0;
+            CK(h->work.alloc(&h->d_ksw, kb), "solve ws");
+            h->ksw_bytes = kb;
+        }
+        if (h->splan.ksplit > h->ksw_items) {
+            if (h->d_kcnt) h->work.release(h->d_kcnt);
             h->d_kcnt = nullptr;
             h->ksw_items = 0;
-            CK(h->work.alloc((void **)&h->d_ksw, h->splan.ksplit * wd::TC_SOLVE_TILE * sizeof(float)), "solve ws");
             CK(h->work.alloc((void **)&h->d_kcnt, h->splan.ksplit * sizeof(int)), "solve ws");
             CK(cudaMemset(h->d_kcnt, 0, h->splan.ksplit * sizeof(int)), "solve ws clear");
             h->ksw_items = h->splan.ksplit;

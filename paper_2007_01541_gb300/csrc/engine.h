@@ -44,7 +44,6 @@ struct DevSym {
 void init_front_attributes();
 void init_solve_attributes();
 void init_tc_attributes();
-void init_blocked_attributes();
 void init_tc_solve_attributes();
 void init_oz_attributes();
 void init_chain_attributes();
@@ -53,7 +52,6 @@ inline void init_kernel_attributes() {
     init_front_attributes();
     init_solve_attributes();
     init_tc_attributes();
-    init_blocked_attributes();
     init_tc_solve_attributes();
     init_oz_attributes();
     init_chain_attributes();
@@ -298,22 +296,23 @@ void launch_sbinv_transpose(const DevSym &d, const T *xpool, T *xtpool, const in
 template <class T>
 void launch_bfwd_gather(const DevSym &d, const T *Y, T *Tt, T *W, const int4 *items, int count, int rgt,
                         int nrhs, cudaStream_t st);
-// xapply / bupdate / breduce modes ("large"): 0 -> tiles of 64 rows x 32
+// xapply / bupdate / breduce modes ("large"): 0 -> tiles of 32 rows x 32
 // right-hand sides per CTA; 1 -> FP32 on the tensor cores, tiles of 128 rows
 // x 64 right-hand sides (tc_solve.cu); 2 -> up to 8 right-hand sides, matrix-vector
-// shaped (32 rows per xapply / bupdate CTA, lanes over rows; breduce keeps the
-// 64-column items and the 64 x 32 partial layout of mode 0); the partial-sum
-// tile sizes (the same for both modes):
+// shaped (32 rows per xapply / bupdate CTA, lanes over rows; breduce has
+// 64-column items and 64 x 32 partial tiles); the partial-sum tile sizes:
 int solve_tile_rows(int large);
 int solve_tile_rhs(int large);
-// rows per CTA of the xapply / bupdate items (mode 0: 64, mode 2: 32)
+// rows per CTA of the xapply / bupdate items
 int solve_update_rows(int large);
+// split inner dimension (mode 0): ksw one 32 x 32 partial tile per CTA, kcnt
+// one arrival counter per CTA (zero between launches)
 template <class T>
-void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out,
+void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out, T *ksw, int *kcnt,
                    const int4 *items, int count, int upper, int large, int nrhs, cudaStream_t st);
 template <class T>
-void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, const int4 *items, int count,
-                    int large, int nrhs, cudaStream_t st);
+void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, T *ksw, int *kcnt,
+                    const int4 *items, int count, int large, int nrhs, cudaStream_t st);
 // split reduction of the backward pass: partial sums of KSR-row splits into
 // P (rows x rhs of the tile per slot), then Tt = y - sum over the splits in order
 constexpr int SOLVE_KSR = 128;

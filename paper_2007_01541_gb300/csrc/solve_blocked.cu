@@ -123,39 +123,6 @@ __global__ void __launch_bounds__(THREADS) sbinv_transpose_kernel(DevSym d, cons
 // ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
-// Right-hand-side tiles: RGT (64 or 16) columns per CTA; 256 threads = 64 rows
-// (or pivot columns) x 4 groups of NPT = RGT / 4 right-hand sides.  Operand
-// rows of right-hand sides are staged RHS-contiguous, so a thread reads its
-// NPT values with 16-byte shared-memory loads.
-
-// 16-byte vector of T
-template <class T>
-struct Vec16;
-template <>
-struct Vec16<float> {
-    using type = float4;
-    static constexpr int n = 4;
-};
-template <>
-struct Vec16<double> {
-    using type = double2;
-    static constexpr int n = 2;
-};
-
-// acc[j] += a * v[j], j < NPT, v 16-byte aligned in shared memory
-template <class T, int NPT>
-__device__ __forceinline__ void axpy_row(T (&acc)[NPT], T a, const T *v) {
-    using V = typename Vec16<T>::type;
-    constexpr int E = Vec16<T>::n;
-#pragma unroll
-    for (int j = 0; j < NPT; j += E) {
-        const V q = *reinterpret_cast<const V *>(v + j);
-        const T *e = reinterpret_cast<const T *>(&q);
-#pragma unroll
-        for (int u = 0; u < E; ++u) acc[j + u] += a * e[u];
-    }
-}
-
 // pivot rows: Tt = b_J + children's update vectors; rows below: W_s = the
 // children's update vectors.  item = (s, 32-row block, rhs tile); lane = row,
 // warp w takes right-hand sides w, w + 8, ... of the tile.
@@ -202,227 +169,133 @@ __global__ void __launch_bounds__(THREADS) bfwd_gather_kernel(DevSym d, const T 
     }
 }
 
-// Tiles of the dependent solve products: ROWS rows (or pivot columns) x RHS
-// right-hand sides per CTA; warp w owns RPW consecutive rows, lane l the
-// right-hand sides l, l + 32, ... (RPL of them).  The matrix tile is staged
-// with rows contiguous (A[p * lda + row]) and read by a whole warp at once
-// (broadcast 16-byte loads), the right-hand-side tile is staged right-hand-
-// side major with an odd stride (R[c * LDR + p]), so both the staging writes
-// and the reads are free of bank conflicts.  The shape in use is 64 x 32 (8
-// rows per warp, one right-hand side per lane); 128 x 64 tiles measured slower
-// on the 2D 256^2 case (half the CTAs on the narrow tree levels).
-template <int RPW_, int RPL_>
-struct TileCfg {
-    static constexpr int RPW = RPW_;
-    static constexpr int RPL = RPL_;
-    static constexpr int ROWS = 8 * RPW;
-    static constexpr int RHS = 32 * RPL;
-    static constexpr int LDO = ROWS + 1;     // stride of the staged result
-    static constexpr int MINB = RPW * RPL > 8 ? 2 : 4;   // resident CTAs per SM (register budget)
-};
-using TileS = TileCfg<8, 1>;
-constexpr int LDR = NB + 1;                  // stride of a staged right-hand side
-
-template <class T, class C, int LDA>
-__device__ __forceinline__ void tile_accumulate(T (&acc)[C::RPW][C::RPL], const T *A, const T *R, int np) {
-    using V = typename Vec16<T>::type;
-    constexpr int E = Vec16<T>::n;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const T *a = A + C::RPW * w;
-    const T *r = R + lane * LDR;
-#pragma unroll 2
-    for (int p = 0; p < np; ++p) {
-        T x[C::RPL];
+// Products with more than 8 right-hand sides on the FP64 (or, by option, the
+// FP32) pipes: 32 x 32 tiles (tile32.cuh).  A tile's time is that of its inner
+// dimension on one SM (150 us for 512 in FP64), so a launch with few tiles
+// splits the inner dimension over up to eight CTAs per tile: each stores its
+// partial tile and counts itself in, and the last to arrive (no CTA waits)
+// adds the partials in split order.  The plan's item carries the split (row
+// block | split << 16 | splits << 24).  Against 64 x 32 tiles of 256 threads,
+// unsplit: square, 16,384 unknowns, 130 right-hand sides, FP64: xapply 3.9 ->
+// 1.8 ms, bupdate 3.7 -> 2.8, breduce 3.3 -> 3.0 (the last two at 0.9 TFLOP/s
+// of the FP64 pipe's 1.06); 32 right-hand sides: xapply 3.6 -> 0.6 ms a solve.
+template <class T>
+__device__ bool split_sum(T (&acc)[4][2], T *ksw, int *kcnt, int z) {
+    const int ks = (z >> 16) & 0xFF, nks = z >> 24;
+    if (nks <= 1) return true;
+    __shared__ int last;
+    constexpr int TILE = t32::TT * t32::TT;
+    T *mine = ksw + (int64_t)blockIdx.x * TILE + threadIdx.x;
 #pragma unroll
-        for (int q = 0; q < C::RPL; ++q) x[q] = r[q * 32 * LDR + p];
-#pragma unroll
-        for (int j = 0; j < C::RPW; j += E) {
-            const V v = *reinterpret_cast<const V *>(a + p * LDA + j);
-            const T *e = reinterpret_cast<const T *>(&v);
-#pragma unroll
-            for (int u = 0; u < E; ++u)
-#pragma unroll
-                for (int q = 0; q < C::RPL; ++q) acc[j + u][q] += e[u] * x[q];
-        }
+    for (int e = 0; e < 8; ++e) mine[e * t32::TH] = acc[e >> 1][e & 1];
+    __threadfence();
+    __syncthreads();
+    const int first = blockIdx.x - ks;
+    if (threadIdx.x == 0) {
+        last = atomicAdd(kcnt + first, 1) == nks - 1;
+        if (last) kcnt[first] = 0;      // for the next launch
     }
-}
-
-template <class T, class C>
-__device__ __forceinline__ void tile_zero(T (&acc)[C::RPW][C::RPL]) {
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    const T *from = ksw + (int64_t)first * TILE + threadIdx.x;
 #pragma unroll
-    for (int i = 0; i < C::RPW; ++i)
+    for (int e = 0; e < 8; ++e) acc[e >> 1][e & 1] = T(0);
+    for (int q = 0; q < nks; ++q)
 #pragma unroll
-        for (int q = 0; q < C::RPL; ++q) acc[i][q] = T(0);
+        for (int e = 0; e < 8; ++e) acc[e >> 1][e & 1] += __ldcg(from + (int64_t)q * TILE + e * t32::TH);
+    return true;
 }
 
-// the CTA's result into O[c * LDO + r] (r = row of the tile, c = right-hand
-// side), so that it can be written out with rows contiguous
-template <class T, class C>
-__device__ __forceinline__ void tile_to_smem(const T (&acc)[C::RPW][C::RPL], T *O) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int i = 0; i < C::RPW; ++i)
-#pragma unroll
-        for (int q = 0; q < C::RPL; ++q) O[(lane + 32 * q) * C::LDO + C::RPW * w + i] = acc[i][q];
+// this CTA's part [pa, pb) of the inner range [p0, p1)
+__device__ __forceinline__ void split_range(int z, int p0, int p1, int &pa, int &pb) {
+    const int ks = (z >> 16) & 0xFF, nks = max(1, z >> 24);
+    const int per = ((p1 - p0 + t32::TK - 1) / t32::TK + nks - 1) / nks * t32::TK;
+    pa = min(p1, p0 + ks * per);
+    pb = min(p1, pa + per);
 }
 
-// rows [p0, p0 + 64) of right-hand sides c0 .. c0 + RHS - 1 (column-major,
-// ld n, first row `row0`) into R[c * LDR + p]; rows >= valid (and columns
-// >= nc) zero
-template <class T, class C>
-__device__ __forceinline__ void stage_rhs(T *R, const T *src, int64_t row0, int p0, int valid, int c0,
-                                          int nc, int64_t n) {
-    for (int idx = threadIdx.x; idx < NB * C::RHS; idx += THREADS) {
-        const int p = idx % NB, c = idx / NB;
-        const bool v = p0 + p < valid && c < nc;
-        cp_async_elem(R + c * LDR + p, v ? src + row0 + p0 + p + (int64_t)(c0 + c) * n : src, v);
-    }
-}
-
-template <class T, class C>
-constexpr int tile_smem_elems() {
-    return 2 * NB * C::ROWS + 2 * C::RHS * LDR + 8;
-}
-
-// out(B rows ROWS rb .. +ROWS) = X_B in_B (upper = 0) or X_B^T in_B (upper =
-// 1, using the stored transpose); item = (s, sb, rb, rhs tile)
-template <class T, class C>
-__global__ void __launch_bounds__(THREADS, C::MINB) xapply_kernel(DevSym d, const T *__restrict__ xp,
+// out(B rows 32 rb .. +32) = X_B in_B (upper = 0) or X_B^T in_B (upper = 1,
+// using the stored transpose); item = (s, sb, rb | split, rhs tile)
+template <class T>
+__global__ void __launch_bounds__(t32::TH) xapply_kernel(DevSym d, const T *__restrict__ xp,
                                                          const int64_t *__restrict__ xsoff,
-                                                         const T *__restrict__ in, T *__restrict__ out,
-                                                         const int4 *__restrict__ items, int upper,
+                                                         const T *__restrict__ in, T *__restrict__ out, T *ksw,
+                                                         int *kcnt, const int4 *__restrict__ items, int upper,
                                                          int nrhs) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    T *Xs[2] = {sm, sm + NB * C::ROWS};                                    // [p][r], ld ROWS
-    T *Rs[2] = {sm + 2 * NB * C::ROWS, sm + 2 * NB * C::ROWS + C::RHS * LDR};  // [c][p], ld LDR
+    __shared__ T As[2][t32::TK * t32::LD], Bs[2][t32::TK * t32::LD];
     const int4 it = items[blockIdx.x];
-    const int s = it.x, sb = it.y, rb = it.z, c0 = it.w * C::RHS;
-    const int k = d.sk[s];
-    const int b0 = sb * SB;
-    const int w = min(SB, k - b0), wp = (w + NB - 1) / NB * NB;
-    const int nb = wp / NB;
-    const int nc = min(C::RHS, nrhs - c0);
-    const int64_t n = d.n;
-    const int64_t row0 = d.sfirst[s] + b0;
-    const T *X = xp + xsoff[s] + (int64_t)sb * SB * SB;
-    const int r0 = rb * C::ROWS, rvalid = wp - r0;
-    const int q0 = upper ? r0 / NB : 0, q1 = upper ? nb : min(nb, (r0 + C::ROWS) / NB);
-    auto stage = [&](int buf, int q) {
-        stage_tile<T, THREADS>(Xs[buf], C::ROWS, X + (int64_t)(q * NB) * wp + r0, wp, C::ROWS, NB, rvalid, NB);
-        stage_rhs<T, C>(Rs[buf], in, row0, q * NB, w, c0, nc, n);
-        cp_async_commit();
-    };
-    T acc[C::RPW][C::RPL];
-    tile_zero<T, C>(acc);
-    stage(0, q0);
-    for (int q = q0; q < q1; ++q) {
-        const int cur = (q - q0) & 1;
-        if (q + 1 < q1) {
-            stage(cur ^ 1, q + 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
+    const int s = it.x, sb = it.y, r0 = (it.z & 0xFFFF) * t32::TT, c0 = it.w * t32::TT;
+    const int b0 = sb * SB, w = min(SB, d.sk[s] - b0), wp = (w + NB - 1) / NB * NB;
+    const int nc = min(t32::TT, nrhs - c0);
+    const int64_t n = d.n, row0 = d.sfirst[s] + b0;
+    const T *X = xp + xsoff[s] + (int64_t)sb * SB * SB + r0;
+    const T *R = in + row0 + (int64_t)c0 * n;
+    int pa, pb;
+    split_range(it.z, upper ? r0 : 0, upper ? w : min(w, r0 + t32::TT), pa, pb);
+    T acc[4][2] = {};
+    t32::product(acc, As, Bs, pa, pb, [&](int buf, int p) {
+        t32::stage_rows(As[buf], X + (int64_t)p * wp, wp, t32::TT, pb - p);
+        t32::stage_inner(Bs[buf], R + p, n, nc, pb - p);
+    }, nc <= 16);
+    if (!split_sum(acc, ksw, kcnt, it.z)) return;
+    const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + tx + 8 * i, c = ty + 16 * j;
+            if (r < w && c < nc) out[row0 + r + (int64_t)(c0 + c) * n] = acc[i][j];
         }
-        __syncthreads();
-        tile_accumulate<T, C, C::ROWS>(acc, Xs[cur], Rs[cur], min(NB, w - q * NB));
-        __syncthreads();
-    }
-    T *O = sm;
-    tile_to_smem<T, C>(acc, O);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < C::ROWS * C::RHS; idx += THREADS) {
-        const int r = idx % C::ROWS, c = idx / C::ROWS;
-        const int rr = r0 + r;
-        if (rr < w && c < nc) out[row0 + rr + (int64_t)(c0 + c) * n] = O[c * C::LDO + r];
-    }
 }
 
-// rows below super-block B: target -= L(rows, B) y_B.  item = (s, sb, rb,
-// tile + 65536 * seg): seg 0 = pivot rows after B (target Tt), seg 1 = rows
-// of R (target the update vector W_s)
-template <class T, class C>
-__global__ void __launch_bounds__(THREADS, C::MINB) bupdate_kernel(DevSym d, const T *__restrict__ front,
+// rows below super-block B: target -= L(rows, B) y_B.  item = (s, sb, rb |
+// split, tile + 65536 * seg): seg 0 = pivot rows after B (target Tt), seg 1 =
+// rows of R (target the update vector W_s)
+template <class T>
+__global__ void __launch_bounds__(t32::TH) bupdate_kernel(DevSym d, const T *__restrict__ front,
                                                           const T *__restrict__ Y, T *__restrict__ Tt,
-                                                          T *__restrict__ W, const int4 *__restrict__ items,
-                                                          int nrhs) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    T *Ls[2] = {sm, sm + NB * C::ROWS};
-    T *Rs[2] = {sm + 2 * NB * C::ROWS, sm + 2 * NB * C::ROWS + C::RHS * LDR};
+                                                          T *__restrict__ W, T *ksw, int *kcnt,
+                                                          const int4 *__restrict__ items, int nrhs) {
+    __shared__ T As[2][t32::TK * t32::LD], Bs[2][t32::TK * t32::LD];
     const int4 it = items[blockIdx.x];
-    const int s = it.x, sb = it.y, rb = it.z, g = it.w & 0xFFFF, seg = it.w >> 16;
-    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s];
+    const int s = it.x, sb = it.y, rb = it.z & 0xFFFF, g = it.w & 0xFFFF, seg = it.w >> 16;
+    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s], f = d.sfirst[s];
     const int b0 = sb * SB, w = min(SB, k - b0);
-    const int c0 = g * C::RHS, nc = min(C::RHS, nrhs - c0);
+    const int c0 = g * t32::TT, nc = min(t32::TT, nrhs - c0);
     const int64_t n = d.n;
-    const int f = d.sfirst[s];
-    const int i0 = seg == 0 ? b0 + w + rb * C::ROWS : rb * C::ROWS;     // seg 1: index into R
-    const int nrow = seg == 0 ? k - i0 : (m - k) - i0;
-    const int mrow = seg == 0 ? i0 : kp + i0;
-    const T *F = front + d.foff[s] + mrow;
-    auto stage = [&](int buf, int p0) {
-        stage_tile<T, THREADS>(Ls[buf], C::ROWS, F + (int64_t)(b0 + p0) * ld, ld, C::ROWS, NB, nrow, w - p0);
-        stage_rhs<T, C>(Rs[buf], Y, f + b0, p0, w, c0, nc, n);
-        cp_async_commit();
-    };
-    T *dst;
-    int64_t ldd;
-    if (seg == 0) {
-        dst = Tt + f + i0;
-        ldd = n;
-    } else {
-        dst = W + d.woff[s] * nrhs + i0;
-        ldd = m - k;
-    }
-    constexpr int PE = C::ROWS * C::RHS / THREADS;   // target elements per thread
-    // FP32 with the small tile has the registers to hold the target early
-    constexpr bool PRE = sizeof(T) == 4 && C::RPW * C::RPL <= 8;
-    T acc[C::RPW][C::RPL];
-    tile_zero<T, C>(acc);
-    const int nchunk = (w + NB - 1) / NB;
-    stage(0, 0);
-    // the target tile is read now, while the staging copies are in flight
-    // (same element order as the write-back below: rows contiguous)
-    T tpre[PE];
+    const int i0 = (seg == 0 ? b0 + w : 0) + rb * t32::TT;              // seg 1: index into R
+    const int nrow = (seg == 0 ? k : m - k) - i0;
+    const T *F = front + d.foff[s] + (int64_t)b0 * ld + (seg == 0 ? i0 : kp + i0);
+    const T *R = Y + f + b0 + (int64_t)c0 * n;
+    int pa, pb;
+    split_range(it.z, 0, w, pa, pb);
+    T acc[4][2] = {};
+    t32::product(acc, As, Bs, pa, pb, [&](int buf, int p) {
+        t32::stage_rows(As[buf], F + (int64_t)p * ld, ld, nrow, pb - p);
+        t32::stage_inner(Bs[buf], R + p, n, nc, pb - p);
+    }, nc <= 16);
+    if (!split_sum(acc, ksw, kcnt, it.z)) return;
+    T *dst = seg == 0 ? Tt + f + i0 + (int64_t)c0 * n : W + d.woff[s] * nrhs + i0 + (int64_t)c0 * (m - k);
+    const int64_t ldd = seg == 0 ? n : m - k;
+    const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
+    // every old value is read before the first store: a store may alias a
+    // later load through the runtime stride
+    T old[4][2];
 #pragma unroll
-    for (int e = 0; e < PE; ++e) {
-        const int idx = threadIdx.x + e * THREADS;
-        const int r = idx % C::ROWS, c = idx / C::ROWS;
-        tpre[e] = (PRE && r < nrow && c < nc) ? dst[r + (int64_t)(c0 + c) * ldd] : T(0);
-    }
-    for (int ch = 0; ch < nchunk; ++ch) {
-        const int cur = ch & 1;
-        if (ch + 1 < nchunk) {
-            stage(cur ^ 1, (ch + 1) * NB);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = tx + 8 * i, c = ty + 16 * j;
+            old[i][j] = r < nrow && c < nc ? dst[r + c * ldd] : T(0);
         }
-        __syncthreads();
-        tile_accumulate<T, C, C::ROWS>(acc, Ls[cur], Rs[cur], min(NB, w - ch * NB));
-        __syncthreads();
-    }
-    T *O = sm;
-    tile_to_smem<T, C>(acc, O);
-    if (!PRE) {
-        // every old target value is read before the first store: a store may
-        // alias a later element's load through the runtime stride, which
-        // would make each read-modify-write a memory round trip of its own
 #pragma unroll
-        for (int e = 0; e < PE; ++e) {
-            const int idx = threadIdx.x + e * THREADS;
-            const int r = idx % C::ROWS, c = idx / C::ROWS;
-            tpre[e] = (r < nrow && c < nc) ? dst[r + (int64_t)(c0 + c) * ldd] : T(0);
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = tx + 8 * i, c = ty + 16 * j;
+            if (r < nrow && c < nc) dst[r + c * ldd] = old[i][j] - acc[i][j];
         }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < PE; ++e) {
-        const int idx = threadIdx.x + e * THREADS;
-        const int r = idx % C::ROWS, c = idx / C::ROWS;
-        if (r < nrow && c < nc) dst[r + (int64_t)(c0 + c) * ldd] = tpre[e] - O[c * C::LDO + r];
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -430,105 +303,68 @@ __global__ void __launch_bounds__(THREADS, C::MINB) bupdate_kernel(DevSym d, con
 // ---------------------------------------------------------------------------
 constexpr int KSR = SOLVE_KSR;    // rows below B per split of the reduction
 
-template <class C>
-struct ReduceCfg {
-    static constexpr int LDT = C::ROWS + 4;   // row stride of the staged L^T tile (16-byte multiple)
-};
-
-template <class T, class C>
-constexpr int breduce_smem_elems() {
-    return 2 * (64 * ReduceCfg<C>::LDT + C::RHS * LDR) + 8;
-}
-
 // Partial reduction of t_B = y_B - L(rows below B, B)^T x(rows below) over the
-// rows [ks * KSR, (ks + 1) * KSR) of the "rows below" list (pivot rows after B,
-// then the rows of R; x of a front row read at its global row):
-// P[slot] (RHS x ROWS, [rhs][c]) = sum_i L(i, j0 + c) x(i, rhs), j0 = b0 +
-// ROWS cb.  item = (s, sb * 8 + cb, tile + 65536 * ks, slot)
-template <class T, class C>
-__global__ void __launch_bounds__(THREADS, C::MINB) breduce_kernel(DevSym d, const T *__restrict__ front,
+// storage rows [b0 + w + ks KSR, ... + KSR) of the front (pivot rows after B,
+// zero padding, the rows of R; x of a front row read at its global row), 32
+// columns from j0 = b0 + 32 cb: P[slot] ([rhs][c]) = sum_i L(i, j0 + c) x(i,
+// rhs).  item = (s, sb * 16 + cb, tile + 65536 * ks, slot)
+template <class T>
+__global__ void __launch_bounds__(t32::TH) breduce_kernel(DevSym d, const T *__restrict__ front,
                                                           const T *__restrict__ Y, T *__restrict__ P,
                                                           const int4 *__restrict__ items, int nrhs) {
-    constexpr int LDT = ReduceCfg<C>::LDT;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    T *Ls[2] = {sm, sm + 64 * LDT};                                          // [rr][c], ld LDT
-    T *Rs[2] = {sm + 2 * 64 * LDT, sm + 2 * 64 * LDT + C::RHS * LDR};        // [rhs][rr], ld LDR
+    __shared__ T As[2][t32::TK * t32::LD], Bs[2][t32::TK * t32::LD];
     const int4 it = items[blockIdx.x];
-    const int s = it.x, sb = it.y >> 3, cb = it.y & 7, g = it.z & 0xFFFF, ks = it.z >> 16;
-    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s];
+    const int s = it.x, sb = it.y >> 4, cb = it.y & 15, g = it.z & 0xFFFF, ks = it.z >> 16;
+    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s], mp = kp + m - k;
     const int b0 = sb * SB, w = min(SB, k - b0);
-    const int j0 = b0 + cb * C::ROWS, nb = min(C::ROWS, k - j0);
-    const int c0 = g * C::RHS, nc = min(C::RHS, nrhs - c0);
+    const int j0 = b0 + cb * t32::TT, nb = min(t32::TT, b0 + w - j0);
+    const int c0 = g * t32::TT, nc = min(t32::TT, nrhs - c0);
     const int64_t n = d.n;
     const T *F = front + d.foff[s] + (int64_t)j0 * ld;
     const int32_t *rows = d.rows + d.rowptr[s];
-    const int tid = threadIdx.x;
-    const int nJ = k - (b0 + w), nbelow = nJ + (m - k);
-    const int u0 = ks * KSR, u1 = min(nbelow, u0 + KSR);
-    auto stage = [&](int buf, int ua) {
-        for (int idx = tid; idx < 64 * C::ROWS; idx += THREADS) {
-            const int rr = idx % 64, c = idx / 64;
-            const int u = ua + rr;
-            const bool v = u < u1 && c < nb;
-            const int mrow = u < nJ ? b0 + w + u : kp + (u - nJ);
-            cp_async_elem(Ls[buf] + rr * LDT + c, v ? F + (int64_t)c * ld + mrow : F, v);
+    const int q0 = b0 + w + ks * KSR, q1 = min(mp, q0 + KSR);
+    T acc[4][2] = {};
+    t32::product(acc, As, Bs, q0, q1, [&](int buf, int q) {
+        t32::stage_inner(As[buf], F + q, ld, nb, q1 - q);
+        // a thread's rows of x are the same for all its right-hand sides
+        const int pp = threadIdx.x % t32::TK, row = q + pp;
+        const bool vr = row < q1 && (row < k || row >= kp);
+        const T *x = Y + (vr ? rows[row < k ? row : row - (kp - k)] : 0) + (int64_t)c0 * n;
+#pragma unroll
+        for (int u = 0; u < t32::TT * t32::TK / t32::TH; ++u) {
+            const int c = threadIdx.x / t32::TK + u * (t32::TH / t32::TK);
+            const bool v = vr && c < nc;
+            cp_async_elem(&Bs[buf][pp * t32::LD + c], v ? x + (int64_t)c * n : Y, v);
         }
-        for (int idx = tid; idx < 64 * C::RHS; idx += THREADS) {
-            const int rr = idx % 64, c = idx / 64;
-            const int u = ua + rr;
-            const bool v = u < u1 && c < nc;
-            const int lr = u < nJ ? b0 + w + u : k + (u - nJ);
-            cp_async_elem(Rs[buf] + c * LDR + rr, v ? Y + rows[lr] + (int64_t)(c0 + c) * n : Y, v);
-        }
-        cp_async_commit();
-    };
-    T acc[C::RPW][C::RPL];
-    tile_zero<T, C>(acc);
-    const int nchunk = (u1 - u0 + 63) / 64;
-    stage(0, u0);
-    for (int ch = 0; ch < nchunk; ++ch) {
-        const int cur = ch & 1;
-        if (ch + 1 < nchunk) {
-            stage(cur ^ 1, u0 + (ch + 1) * 64);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        tile_accumulate<T, C, LDT>(acc, Ls[cur], Rs[cur], min(64, u1 - u0 - ch * 64));
-        __syncthreads();
-    }
-    T *O = sm;
-    tile_to_smem<T, C>(acc, O);
-    __syncthreads();
-    T *Pt = P + (int64_t)it.w * C::RHS * C::ROWS;
-    for (int idx = tid; idx < C::ROWS * C::RHS; idx += THREADS) {
-        const int r = idx % C::ROWS, c = idx / C::ROWS;
-        Pt[c * C::ROWS + r] = O[c * C::LDO + r];
-    }
+    }, nc <= 16);
+    T *Pt = P + (int64_t)it.w * t32::TT * t32::TT;
+    const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Pt[(ty + 16 * j) * t32::TT + tx + 8 * i] = acc[i][j];
 }
 
 // Tt(B columns) = y - sum of the splits' partial sums, in split order; one
 // element of the ROWS x RHS tile per thread.
-// item = (s, sb * 8 + cb, tile + 65536 * nsplit, first slot)
-template <class T, class C>
+// item = (s, sb * 16 + cb, tile + 65536 * nsplit, first slot)
+template <class T, int ROWS, int RHS>
 __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const T *__restrict__ Y,
                                                                  T *__restrict__ Tt, const T *__restrict__ P,
                                                                  const int4 *__restrict__ items, int nrhs) {
-    constexpr int PER = C::ROWS * C::RHS / THREADS;   // CTAs per item
+    constexpr int PER = ROWS * RHS / THREADS;   // CTAs per item
     const int4 it = items[blockIdx.x / PER];
-    const int s = it.x, sb = it.y >> 3, cb = it.y & 7, g = it.z & 0xFFFF, nsplit = it.z >> 16;
+    const int s = it.x, sb = it.y >> 4, cb = it.y & 15, g = it.z & 0xFFFF, nsplit = it.z >> 16;
     const int k = d.sk[s];
-    const int j0 = sb * SB + cb * C::ROWS, nb = min(C::ROWS, k - j0);
-    const int c0 = g * C::RHS, nc = min(C::RHS, nrhs - c0);
+    const int j0 = sb * SB + cb * ROWS, nb = min(ROWS, k - j0);
+    const int c0 = g * RHS, nc = min(RHS, nrhs - c0);
     const int64_t n = d.n;
     const int f = d.sfirst[s];
     const int idx = (blockIdx.x % PER) * THREADS + threadIdx.x;
-    const int cl = idx % C::ROWS, c = idx / C::ROWS;
+    const int cl = idx % ROWS, c = idx / ROWS;
     if (cl >= nb || c >= nc) return;
     T sum = T(0);
-    for (int q = 0; q < nsplit; ++q) sum += P[((int64_t)(it.w + q) * C::RHS + c) * C::ROWS + cl];
+    for (int q = 0; q < nsplit; ++q) sum += P[((int64_t)(it.w + q) * RHS + c) * ROWS + cl];
     const int64_t o = f + j0 + cl + (int64_t)(c0 + c) * n;
     Tt[o] = Y[o] - sum;
 }
@@ -542,6 +378,7 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // NR = nrhs rounded up to 1, 2, 4 or 8; columns c >= nrhs are zero.
 // ---------------------------------------------------------------------------
 constexpr int NRW = 32;
+constexpr int NARROW_COLS = 64, NARROW_RHS = 32;   // partial-sum tile of the backward reduction
 constexpr int NWARP = THREADS / 32;
 
 // acc[c] += sum over p in [pa, pb) with p = warp (mod NWARP) of A[p * lda] V[p * NR + c]
@@ -674,15 +511,15 @@ __global__ void __launch_bounds__(THREADS) bupdate_narrow_kernel(DevSym d, const
 // rows [ks KSR, (ks + 1) KSR) of the "rows below" list, for the 64 columns
 // j0 = b0 + 64 cb ...: one warp per column (8 columns per warp), lanes over
 // rows; P[slot] holds the sums in the 64 x 32 tile layout ([rhs][column]).
-// item = (s, sb * 8 + cb, 65536 * ks, slot)
+// item = (s, sb * 16 + cb, 65536 * ks, slot)
 template <class T, int NR>
 __global__ void __launch_bounds__(THREADS) breduce_narrow_kernel(DevSym d, const T *__restrict__ front,
                                                                  const T *__restrict__ Y, T *__restrict__ P,
                                                                  const int4 *__restrict__ items, int nrhs) {
-    constexpr int RC = TileS::ROWS, RR = TileS::RHS;     // P tile: RR right-hand sides x RC columns
+    constexpr int RC = NARROW_COLS, RR = NARROW_RHS;     // P tile: RR right-hand sides x RC columns
     __shared__ T xs[KSR * NR];
     const int4 it = items[blockIdx.x];
-    const int s = it.x, sb = it.y >> 3, cb = it.y & 7, ks = it.z >> 16;
+    const int s = it.x, sb = it.y >> 4, cb = it.y & 15, ks = it.z >> 16;
     const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s];
     const int b0 = sb * SB, w = min(SB, k - b0);
     const int j0 = b0 + cb * RC, nb = min(RC, k - j0);
@@ -728,29 +565,10 @@ __global__ void __launch_bounds__(THREADS) breduce_narrow_kernel(DevSym d, const
 
 }  // namespace
 
-template <class T, class C>
-void set_blocked_attributes() {
-    cudaFuncSetAttribute(xapply_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(tile_smem_elems<T, C>() * sizeof(T)));
-    cudaFuncSetAttribute(bupdate_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(tile_smem_elems<T, C>() * sizeof(T)));
-    cudaFuncSetAttribute(breduce_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(breduce_smem_elems<T, C>() * sizeof(T)));
-}
-
-void init_blocked_attributes() {
-    static bool done = false;
-    if (done) return;
-    set_blocked_attributes<float, TileS>();
-    set_blocked_attributes<double, TileS>();
-    done = true;
-}
-
-// the partial-sum tile of the tensor-core backward products (128 columns x 64
-// right-hand sides); only its ROWS and RHS are used
-using TileTc = TileCfg<16, 2>;
-int solve_tile_rows(int large) { return large == 1 ? TileTc::ROWS : TileS::ROWS; }
-int solve_tile_rhs(int large) { return large == 1 ? TileTc::RHS : TileS::RHS; }
+// partial-sum tiles: mode 0 the 32 x 32 product tiles, mode 1 the tensor-core
+// tiles (128 columns x 64 right-hand sides), mode 2 the narrow kernels' items
+int solve_tile_rows(int large) { return large == 1 ? 128 : (large == 2 ? NARROW_COLS : t32::TT); }
+int solve_tile_rhs(int large) { return large == 1 ? 64 : (large == 2 ? NARROW_RHS : t32::TT); }
 int solve_update_rows(int large) { return large == 2 ? NRW : solve_tile_rows(large); }
 
 void launch_sbinv_diag(const DevSym &d, const float *dinv, float *xpool, const int64_t *xsoff, const int4 *items,
@@ -775,34 +593,15 @@ void launch_bfwd_gather(const DevSym &d, const T *Y, T *Tt, T *W, const int4 *it
     if (rgt == 64) bfwd_gather_kernel<T, 64><<<count, THREADS, 0, st>>>(d, Y, Tt, W, items, nrhs);
     else bfwd_gather_kernel<T, 16><<<count, THREADS, 0, st>>>(d, Y, Tt, W, items, nrhs);
 }
-template <class T, class C>
-static void xapply_go(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out,
-                      const int4 *items, int count, int upper, int nrhs, cudaStream_t st) {
-    xapply_kernel<T, C><<<count, THREADS, tile_smem_elems<T, C>() * sizeof(T), st>>>(d, xp, xsoff, in, out,
-                                                                                   items, upper, nrhs);
-}
-template <class T, class C>
-static void bupdate_go(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, const int4 *items,
-                       int count, int nrhs, cudaStream_t st) {
-    bupdate_kernel<T, C><<<count, THREADS, tile_smem_elems<T, C>() * sizeof(T), st>>>(d, front, Y, Tt, W,
-                                                                                    items, nrhs);
-}
-template <class T, class C>
-static void breduce_go(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count,
-                       int nrhs, cudaStream_t st) {
-    breduce_kernel<T, C><<<count, THREADS, breduce_smem_elems<T, C>() * sizeof(T), st>>>(d, front, Y, P,
-                                                                                       items, nrhs);
-}
-template <class T, class C>
+template <class T, int ROWS, int RHS>
 static void finish_go(const DevSym &d, const T *Y, T *Tt, const T *P, const int4 *items, int count, int nrhs,
                       cudaStream_t st) {
-    constexpr int PER = C::ROWS * C::RHS / THREADS;
-    breduce_finish_kernel<T, C><<<count * PER, THREADS, 0, st>>>(d, Y, Tt, P, items, nrhs);
+    constexpr int PER = ROWS * RHS / THREADS;
+    breduce_finish_kernel<T, ROWS, RHS><<<count * PER, THREADS, 0, st>>>(d, Y, Tt, P, items, nrhs);
 }
 
-// large = 1 selects the 128 x 64 tiles (FP32 only)
 template <class T>
-void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out,
+void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out, T *ksw, int *kcnt,
                    const int4 *items, int count, int upper, int large, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
     if (large == 2) {
@@ -812,11 +611,11 @@ void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *
         else xapply_narrow_kernel<T, 8><<<count, THREADS, 0, st>>>(d, xp, xsoff, in, out, items, upper, nrhs);
         return;
     }
-    xapply_go<T, TileS>(d, xp, xsoff, in, out, items, count, upper, nrhs, st);
+    xapply_kernel<T><<<count, t32::TH, 0, st>>>(d, xp, xsoff, in, out, ksw, kcnt, items, upper, nrhs);
 }
 template <class T>
-void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, const int4 *items, int count,
-                    int large, int nrhs, cudaStream_t st) {
+void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, T *ksw, int *kcnt,
+                    const int4 *items, int count, int large, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
     if (large == 2) {
         if (nrhs == 1) bupdate_narrow_kernel<T, 1><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
@@ -825,7 +624,7 @@ void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, co
         else bupdate_narrow_kernel<T, 8><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
         return;
     }
-    bupdate_go<T, TileS>(d, front, Y, Tt, W, items, count, nrhs, st);
+    bupdate_kernel<T><<<count, t32::TH, 0, st>>>(d, front, Y, Tt, W, ksw, kcnt, items, nrhs);
 }
 template <class T>
 void launch_breduce(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count,
@@ -838,14 +637,15 @@ void launch_breduce(const DevSym &d, const T *front, const T *Y, T *P, const int
         else breduce_narrow_kernel<T, 8><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
         return;
     }
-    breduce_go<T, TileS>(d, front, Y, P, items, count, nrhs, st);
+    breduce_kernel<T><<<count, t32::TH, 0, st>>>(d, front, Y, P, items, nrhs);
 }
 template <class T>
 void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const int4 *items, int count,
                            int large, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
-    if (large == 1) finish_go<T, TileTc>(d, Y, Tt, P, items, count, nrhs, st);
-    else finish_go<T, TileS>(d, Y, Tt, P, items, count, nrhs, st);
+    if (large == 1) finish_go<T, 128, 64>(d, Y, Tt, P, items, count, nrhs, st);
+    else if (large == 2) finish_go<T, NARROW_COLS, NARROW_RHS>(d, Y, Tt, P, items, count, nrhs, st);
+    else finish_go<T, t32::TT, t32::TT>(d, Y, Tt, P, items, count, nrhs, st);
 }
 
 #define WD_BLOCKED_INST(T)                                                                              \
@@ -855,10 +655,10 @@ void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const
                                             int, cudaStream_t);                                         \
     template void launch_bfwd_gather<T>(const DevSym &, const T *, T *, T *, const int4 *, int, int, int, \
                                         cudaStream_t);                                                  \
-    template void launch_xapply<T>(const DevSym &, const T *, const int64_t *, const T *, T *,           \
+    template void launch_xapply<T>(const DevSym &, const T *, const int64_t *, const T *, T *, T *, int *, \
                                    const int4 *, int, int, int, int, cudaStream_t);                     \
-    template void launch_bupdate<T>(const DevSym &, const T *, const T *, T *, T *, const int4 *, int,   \
-                                    int, int, cudaStream_t);                                            \
+    template void launch_bupdate<T>(const DevSym &, const T *, const T *, T *, T *, T *, int *,          \
+                                    const int4 *, int, int, int, cudaStream_t);                         \
     template void launch_breduce<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
                                     int, cudaStream_t);                                                 \
     template void launch_breduce_finish<T>(const DevSym &, const T *, T *, const T *, const int4 *, int, \

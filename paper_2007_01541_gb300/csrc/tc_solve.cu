@@ -95,7 +95,7 @@ __device__ __forceinline__ Geo geometry(const DevSym &d, const TcSolveArgs &a, i
     g.mp = g.kp + g.m - g.k;
     g.ld = d.sld[g.s];
     g.f = d.sfirst[g.s];
-    const int sb = OP == OP_BREDUCE ? (it.y >> 3) : it.y;
+    const int sb = OP == OP_BREDUCE ? (it.y >> 4) : it.y;
     g.b0 = sb * SB;
     g.w = min(SB, g.k - g.b0);
     g.wp = (g.w + NB - 1) / NB * NB;
@@ -129,7 +129,7 @@ __device__ __forceinline__ Geo geometry(const DevSym &d, const TcSolveArgs &a, i
         g.kc0 = g.b0 / TK;
         g.nchunk = (g.w + TK - 1) / TK;
     } else {
-        const int cb = it.y & 7, ks = it.z >> 16;
+        const int cb = it.y & 15, ks = it.z >> 16;
         g.j0 = g.b0 + cb * TM;
         g.nb = min(TM, g.b0 + g.w - g.j0);
         const int kbeg = (g.b0 + g.w) & ~(TK - 1);   // storage rows below B, from a 32-row boundary

@@ -32,28 +32,29 @@ __device__ __forceinline__ void stage_inner(T *s, const T *g, int64_t ld, int rv
     }
 }
 
-template <class T>
+// NJ = 1: the tile's first 16 columns only
+template <int NJ, class T>
 __device__ __forceinline__ void accumulate(T (&acc)[4][2], const T *A, const T *B, int np) {
     const T *a = A + threadIdx.x % 8, *b = B + threadIdx.x / 8;
 #pragma unroll 4
     for (int p = 0; p < np; ++p) {
-        T x[4], y[2];
+        T x[4], y[NJ];
 #pragma unroll
         for (int i = 0; i < 4; ++i) x[i] = a[p * LD + 8 * i];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) y[j] = b[p * LD + 16 * j];
+        for (int j = 0; j < NJ; ++j) y[j] = b[p * LD + 16 * j];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) acc[i][j] += x[i] * y[j];
+            for (int j = 0; j < NJ; ++j) acc[i][j] += x[i] * y[j];
     }
 }
 
 // acc += sum_{p in [p0, p1)} A(i, p) B(j, p); stage(buffer, p) issues both
-// operands' chunk from p on
+// operands' chunk from p on; half: the tile has at most 16 columns
 template <class T, class F>
 __device__ __forceinline__ void product(T (&acc)[4][2], T (&As)[2][TK * LD], T (&Bs)[2][TK * LD], int p0, int p1,
-                                        F stage) {
+                                        F stage, bool half = false) {
     if (p0 >= p1) return;
     stage(0, p0);
     cp_async_commit();
@@ -66,7 +67,8 @@ __device__ __forceinline__ void product(T (&acc)[4][2], T (&As)[2][TK * LD], T (
             cp_async_wait<0>();
         }
         __syncthreads();
-        accumulate(acc, As[cur], Bs[cur], min(TK, p1 - p));
+        if (half) accumulate<1>(acc, As[cur], Bs[cur], min(TK, p1 - p));
+        else accumulate<2>(acc, As[cur], Bs[cur], min(TK, p1 - p));
         __syncthreads();
     }
 }

@@ -111,3 +111,20 @@ def test_lu_solve_passes(wdlib, cuda, nrhs):
     for _ in range(2):                       # the second time with the kept plan
         X = s.solve_lu(B)
         assert oracle.nonsym_backward_error(cp, ri, lo, up, X, B).max() <= 1e-13
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(solve_simt=True)])
+@pytest.mark.parametrize("nrhs", [9, 16, 17, 32, 33, 49])
+def test_solve_tiles(wdlib, cuda, opts, nrhs):
+    """The 32 x 32 tiles of the solves, split and not, in FP64 and (by option)
+    FP32: a tree of fronts and one dense front wider than a super-block."""
+    b, cp, ri, v, o = _case(2, 5)
+    n = 600
+    rng = np.random.default_rng(n)
+    M = rng.standard_normal((n, n))
+    dense = _lower_csc(M @ M.T + n * np.eye(n))
+    prec = "mixed" if opts else "fp64"
+    for c, r, vals, basis in ((cp, ri, v, b), dense + (None,)):
+        B = rhs(c.size - 1, nrhs, seed=nrhs)
+        s = wdlib.Solver(**opts).analyze(c, r, basis).factor(vals, prec)
+        assert oracle.backward_error(c, r, vals, s.solve(B), B).max() <= 1e-12
