@@ -633,7 +633,8 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
     const int TRX = wd::solve_update_rows(large);   // rows per CTA of the xapply / bupdate items
     const int ng = (nrhs + TNW - 1) / TNW;
     const double R = nrhs;
-    const int SBW = wd::SB, KSR = large == 1 ? wd::SOLVE_KSR_TC : wd::SOLVE_KSR;
+    const int SBW = wd::SB;
+    const int KSR = large == 1 ? wd::SOLVE_KSR_TC : (large == 2 ? wd::SOLVE_KSR_NARROW : wd::SOLVE_KSR);
     auto nsb = [&](int s) { return (S.k(s) + SBW - 1) / SBW; };
     auto width = [&](int s, int sb) { return std::min(SBW, S.k(s) - sb * SBW); };
     auto wpad = [&](int s, int sb) { return (width(s, sb) + NB - 1) / NB * NB; };
@@ -650,7 +651,8 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
         double el = 0, fl = 0;
         for (int i = b; i < e; ++i) {
             const int s = S.level_nodes[i];
-            for (int rc = 0; rc * 32 < S.m(s); ++rc)
+            // (mode 2: the kernels that use the gathered values gather them)
+            for (int rc = 0; large != 2 && rc * 32 < S.m(s); ++rc)
                 for (int g = 0; g < ngg; ++g) p.items.push_back({s, rc, g, 0});
             maxsb = std::max(maxsb, nsb(s));
             el += R * (S.m(s) + S.k(s));
@@ -704,17 +706,18 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
             double el = 0, fl = 0;
             int slot = 0;
             std::vector<int4> fin;
+            std::vector<int> first_slot;   // of each front with this super-block
             for (int i = b; i < e; ++i) {
                 const int s = S.level_nodes[i];
                 if (nsb(s) <= sb) continue;
                 const int m = S.m(s), w = width(s, sb);
                 const int below = m - (sb * SBW + w);
-                // the splits run over the front's storage rows (tensor cores:
-                // from the 32-row boundary at or above the super-block's end),
-                // the narrow kernels' over the rows below
-                const int kbeg = large == 1 ? (sb * SBW + w) & ~31 : sb * SBW + w;
-                const int nsplit = large == 2 ? (below + KSR - 1) / KSR
-                                              : (below > 0 ? (front_order(S, s) - kbeg + KSR - 1) / KSR : 0);
+                // the splits run over the front's storage rows (tensor cores and
+                // few right-hand sides: from the 32-row boundary at or above
+                // the super-block's end)
+                const int kbeg = large == 0 ? sb * SBW + w : (sb * SBW + w) & ~31;
+                const int nsplit = below > 0 ? (front_order(S, s) - kbeg + KSR - 1) / KSR : 0;
+                first_slot.push_back(slot);
                 for (int cb = 0; cb * TRW < w; ++cb)
                     for (int g = 0; g < ng; ++g) {
                         fin.push_back({s, sb * 16 + cb, g + 65536 * nsplit, slot});
@@ -729,19 +732,21 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
             f0 = p.items.size();
             el = 0;
             for (const int4 &q : fin) {
+                if (large == 2) break;     // part of xnarrow
                 p.items.push_back(q);
                 el += 2.0 * TRW * R + (double)(q.z >> 16) * TRW * TNW;
             }
             add_launch(p, K_BWD_FINISH, f0, sb, 0, el, 0);
             f0 = p.items.size();
             el = fl = 0;
+            size_t with = 0;
             for (int i = b; i < e; ++i) {
                 const int s = S.level_nodes[i];
                 if (nsb(s) <= sb) continue;
-                const int w = width(s, sb), wp = wpad(s, sb);
+                const int w = width(s, sb), wp = wpad(s, sb), slot0 = first_slot[with++];
                 for (int rb = 0; rb * TRX < wp; ++rb)
                     for (int g = 0; g < ng; ++g) {
-                        p.items.push_back({s, sb, rb, g});
+                        p.items.push_back({s, sb, rb, large == 2 ? slot0 : g});
                         nch.push_back((std::max(1, w - rb * TRX) + 63) / 64);
                     }
                 fl += (double)w * (w + 1) * R;
@@ -1646,8 +1651,10 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.out = reinterpret_cast<float *>(Y);
                     a.upper = 0;
                     wd::launch_tc_xapply(d, a, it, L.count, st);
+                } else if (lg == 2) {
+                    wd::launch_xnarrow<T>(d, Xs, h->d_xsoff, Y, Tt, W, P, it, L.count, true, nrhs, st);
                 } else {
-                    wd::launch_xapply<T>(d, Xs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 0, lg, nrhs, st);
+                    wd::launch_xapply<T>(d, Xs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 0, nrhs, st);
                 }
                 break;
             case K_FWD_BUPDATE:
@@ -1656,8 +1663,10 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.in = reinterpret_cast<const float *>(Y);
                     a.out = reinterpret_cast<float *>(Tt);
                     wd::launch_tc_bupdate(d, a, it, L.count, st);
+                } else if (lg == 2) {
+                    wd::launch_bnarrow<T>(d, F, Y, Tt, W, it, L.count, nrhs, st);
                 } else {
-                    wd::launch_bupdate<T>(d, F, Y, Tt, W, ksw, h->d_kcnt, it, L.count, lg, nrhs, st);
+                    wd::launch_bupdate<T>(d, F, Y, Tt, W, ksw, h->d_kcnt, it, L.count, nrhs, st);
                 }
                 break;
             case K_BWD_REDUCE:
@@ -1666,8 +1675,10 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.in = reinterpret_cast<const float *>(Y);
                     a.out = reinterpret_cast<float *>(P);
                     wd::launch_tc_breduce(d, a, it, L.count, st);
+                } else if (lg == 2) {
+                    wd::launch_rnarrow<T>(d, Fb, Y, P, it, L.count, nrhs, st);
                 } else {
-                    wd::launch_breduce<T>(d, Fb, Y, P, it, L.count, lg, nrhs, st);
+                    wd::launch_breduce<T>(d, Fb, Y, P, it, L.count, nrhs, st);
                 }
                 break;
             case K_BWD_FINISH: wd::launch_breduce_finish<T>(d, Y, Tt, P, it, L.count, lg, nrhs, st); break;
@@ -1679,8 +1690,10 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.out = reinterpret_cast<float *>(Y);
                     a.upper = 1;
                     wd::launch_tc_xapply(d, a, it, L.count, st);
+                } else if (lg == 2) {
+                    wd::launch_xnarrow<T>(d, XTs, h->d_xsoff, Y, Tt, W, P, it, L.count, false, nrhs, st);
                 } else {
-                    wd::launch_xapply<T>(d, XTs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 1, lg, nrhs, st);
+                    wd::launch_xapply<T>(d, XTs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 1, nrhs, st);
                 }
                 break;
         }

@@ -299,8 +299,9 @@ void launch_bfwd_gather(const DevSym &d, const T *Y, T *Tt, T *W, const int4 *it
 // xapply / bupdate / breduce modes ("large"): 0 -> tiles of 32 rows x 32
 // right-hand sides per CTA; 1 -> FP32 on the tensor cores, tiles of 128 rows
 // x 64 right-hand sides (tc_solve.cu); 2 -> up to 8 right-hand sides, matrix-vector
-// shaped (32 rows per xapply / bupdate CTA, lanes over rows; breduce has
-// 64-column items and 64 x 32 partial tiles); the partial-sum tile sizes:
+// shaped kernels of their own (xnarrow, bnarrow: 32 rows per CTA; rnarrow: 64
+// columns and SOLVE_KSR_NARROW storage rows per CTA, from the 32-row boundary
+// at or above the super-block's end); the partial-sum tile sizes:
 int solve_tile_rows(int large);
 int solve_tile_rhs(int large);
 // rows per CTA of the xapply / bupdate items
@@ -309,16 +310,28 @@ int solve_update_rows(int large);
 // one arrival counter per CTA (zero between launches)
 template <class T>
 void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out, T *ksw, int *kcnt,
-                   const int4 *items, int count, int upper, int large, int nrhs, cudaStream_t st);
+                   const int4 *items, int count, int upper, int nrhs, cudaStream_t st);
 template <class T>
 void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, T *ksw, int *kcnt,
-                    const int4 *items, int count, int large, int nrhs, cudaStream_t st);
+                    const int4 *items, int count, int nrhs, cudaStream_t st);
+// mode 2: y_B (forward: Y and the children's into Tt) or x_B (backward: Tt and
+// the partial sums P into Y); the rows below; the partial sums
+constexpr int SOLVE_KSR_NARROW = 256;
+template <class T>
+void launch_xnarrow(const DevSym &d, const T *xp, const int64_t *xsoff, T *Y, T *Tt, const T *W, const T *P,
+                    const int4 *items, int count, bool forward, int nrhs, cudaStream_t st);
+template <class T>
+void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, const int4 *items, int count, int nrhs,
+                    cudaStream_t st);
+template <class T>
+void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
+                    cudaStream_t st);
 // split reduction of the backward pass: partial sums of KSR-row splits into
 // P (rows x rhs of the tile per slot), then Tt = y - sum over the splits in order
 constexpr int SOLVE_KSR = 128;
 template <class T>
 void launch_breduce(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count,
-                    int large, int nrhs, cudaStream_t st);
+                    int nrhs, cudaStream_t st);
 template <class T>
 void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const int4 *items, int count,
                            int large, int nrhs, cudaStream_t st);

@@ -19,6 +19,8 @@
 #include "engine.h"
 #include "tile32.cuh"
 
+#include <type_traits>
+
 namespace wd {
 namespace {
 
@@ -370,102 +372,202 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 }
 
 // ---------------------------------------------------------------------------
-// Few right-hand sides (nrhs <= 8): the products are matrix-vector shaped, so
-// lanes run over rows (coalesced columns of L or X) instead of right-hand
-// sides.  A CTA covers NRW = 32 rows; its 8 warps split the columns (column p
-// to warp p mod 8), the right-hand-side block is staged in shared memory
-// (V[p * NR + c]), and the warps' partial sums are added in a fixed order.
-// NR = nrhs rounded up to 1, 2, 4 or 8; columns c >= nrhs are zero.
+// Few right-hand sides (nrhs <= 8): matrix-vector shaped products, four
+// dependent launches per super-block (two forward, two backward).  Bound: the
+// latency of the chain of launches and, inside each, of its loads (the bytes,
+// L once per direction, would take a tenth of the time).  So
+//   * a CTA covers 32 rows and all its columns (or 64 columns and 256 rows) with
+//     16-byte loads, up to sixteen of them in flight per lane, most often all;
+//   * the forward gather of the children's update vectors is part of the two
+//     kernels that use it (xnarrow for the super-block's own rows, repeated by
+//     its CTAs, bnarrow for the rows it writes), and the backward sum of the
+//     partial reductions part of the kernel that uses it.
+// NR = nrhs rounded up to 1, 2, 4 or 8; columns c >= nrhs are zero.  Sums are
+// taken in a fixed order.  Buffers: Y holds b and the pending right-hand side,
+// then x; Tt holds y.
+// Against one 4-byte load per lane and column, four in flight, and launches of
+// their own for the gather and the sum: 256 x 256, one right-hand side against
+// a kept factor 2.30 -> 1.67 ms; 128 x 128, a theta step 0.84 -> 0.68 ms.
 // ---------------------------------------------------------------------------
 constexpr int NRW = 32;
-constexpr int NARROW_COLS = 64, NARROW_RHS = 32;   // partial-sum tile of the backward reduction
 constexpr int NWARP = THREADS / 32;
+constexpr int NARROW_COLS = 64, NARROW_RHS = 8;   // partial-sum tile of the backward reduction
+constexpr int NKSR = SOLVE_KSR_NARROW;             // rows per split of the backward reduction
 
-// acc[c] += sum over p in [pa, pb) with p = warp (mod NWARP) of A[p * lda] V[p * NR + c]
-// (A already offset to this lane's row; ok = the row is valid)
+template <class T>
+struct Vec16;
+template <>
+struct Vec16<float> {
+    using type = float4;
+};
+template <>
+struct Vec16<double> {
+    using type = double2;
+};
+
+// the children's update vectors, staged per CTA in groups of CHG
+constexpr int CHG = 16;
+struct Children {
+    int64_t map[CHG], w[CHG];
+    int ld[CHG];
+};
+static_assert(sizeof(Children) <= NWARP * NRW * sizeof(float), "fits the product's reduction buffer");
+// t[c] += the children's values of local row r (ok: r exists); all threads of
+// the CTA call it
 template <class T, int NR>
-__device__ __forceinline__ void narrow_accumulate(T (&acc)[NR], const T *__restrict__ A, int64_t lda, bool ok,
-                                                  const T *V, int pa, int pb) {
-    const int warp = threadIdx.x >> 5;
-    constexpr int U = 4;
-    for (int p0 = pa + warp; p0 < pb; p0 += NWARP * U) {
-        T a[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int p = p0 + NWARP * u;
-            a[u] = (ok && p < pb) ? A[(int64_t)p * lda] : T(0);
+__device__ __forceinline__ void add_children(const DevSym &d, int s, const T *__restrict__ W, int nrhs, Children &ch,
+                                             int r, bool ok, T (&t)[NR]) {
+    const int cb = d.child_ptr[s], ce = d.child_ptr[s + 1];
+    for (int g0 = cb; g0 < ce; g0 += CHG) {
+        const int ng = min(CHG, ce - g0);
+        __syncthreads();
+        if (threadIdx.x < ng) {
+            const int c = d.children[g0 + threadIdx.x];
+            ch.map[threadIdx.x] = d.mapoff[c];
+            ch.w[threadIdx.x] = d.woff[c] * nrhs;
+            ch.ld[threadIdx.x] = d.sm[c] - d.sk[c];
         }
+        __syncthreads();
+        if (!ok) continue;
+        for (int i = 0; i < ng; i += 4) {
+            int ic[4];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int p = min(p0 + NWARP * u, pb - 1);
+            for (int u = 0; u < 4; ++u) ic[u] = i + u < ng ? d.relmap[ch.map[i + u] + r] : -1;
 #pragma unroll
-            for (int c = 0; c < NR; ++c) acc[c] += a[u] * V[p * NR + c];
+            for (int u = 0; u < 4; ++u) {
+                if (ic[u] < 0) continue;
+                const T *w = W + ch.w[i + u] + ic[u];
+                const int ldc = ch.ld[i + u];
+#pragma unroll
+                for (int c = 0; c < NR; ++c)
+                    if (c < nrhs) t[c] += w[(int64_t)c * ldc];
+            }
         }
     }
 }
 
-// the warps' sums of row (tid % 32), column (tid / 32) in warp order, for
-// tid < 32 NR (red: [NWARP][NRW][NR]); call after narrow_accumulate by all threads
+// The product of rows [0, 32) at A (row offset included; column-major, lda,
+// 16-byte aligned, all 32 rows readable) and columns [pa, pb) with V[p * NR +
+// c]: the sum of row tid % 32 and right-hand side tid / 32 for tid < 32 NR.
+// red: NWARP * 32 * NR.  Called by all threads after V is visible.
 template <class T, int NR>
-__device__ __forceinline__ T narrow_reduce(const T (&acc)[NR], T *red) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__device__ __forceinline__ T narrow_product(const T *__restrict__ A, int64_t lda, const T *V, int pa, int pb, T *red) {
+    using VT = typename Vec16<T>::type;
+    constexpr int VR = 16 / sizeof(T), LR = NRW / VR, CPW = 32 / LR;   // rows per lane, lanes per column, columns per load
+    constexpr int U = 16;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane % LR, lc = lane / LR;
+    T acc[VR][NR];
 #pragma unroll
-    for (int c = 0; c < NR; ++c) red[(warp * NRW + lane) * NR + c] = acc[c];
+    for (int i = 0; i < VR; ++i)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) acc[i][c] = T(0);
+    const T *a = A + VR * lr;
+    for (int p0 = pa + warp * CPW + lc; p0 < pb; p0 += U * NWARP * CPW) {
+        VT x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + u * NWARP * CPW;
+            if (p < pb) x[u] = *reinterpret_cast<const VT *>(a + (int64_t)p * lda);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + u * NWARP * CPW;
+            if (p < pb) {
+                const T *e = reinterpret_cast<const T *>(&x[u]);
+#pragma unroll
+                for (int c = 0; c < NR; ++c) {
+                    const T v = V[p * NR + c];
+#pragma unroll
+                    for (int i = 0; i < VR; ++i) acc[i][c] += e[i] * v;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < VR; ++i)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+#pragma unroll
+            for (int o = LR; o < 32; o *= 2) acc[i][c] += __shfl_xor_sync(0xffffffffu, acc[i][c], o);
+            if (lc == 0) red[(warp * NR + c) * NRW + VR * lr + i] = acc[i][c];
+        }
     __syncthreads();
     T sum = T(0);
-    if (threadIdx.x < NRW * NR) {
-        const int r = threadIdx.x % NRW, c = threadIdx.x / NRW;
-        for (int g = 0; g < NWARP; ++g) sum += red[(g * NRW + r) * NR + c];
-    }
+    if (threadIdx.x < NRW * NR)
+        for (int g = 0; g < NWARP; ++g) sum += red[g * NR * NRW + threadIdx.x];
     return sum;
 }
 
-// y_B rows [32 rb, 32 rb + 32) = X_B in_B (upper = 0) or X_B^T in_B (upper =
-// 1, the stored transpose); item = (s, sb, rb, 0)
-template <class T, int NR>
-__global__ void __launch_bounds__(THREADS) xapply_narrow_kernel(DevSym d, const T *__restrict__ xp,
-                                                                const int64_t *__restrict__ xsoff,
-                                                                const T *__restrict__ in, T *__restrict__ out,
-                                                                const int4 *__restrict__ items, int upper,
-                                                                int nrhs) {
-    __shared__ T V[SB * NR];
-    __shared__ T red[NWARP * NRW * NR];
-    const int4 it = items[blockIdx.x];
-    const int s = it.x, sb = it.y, rb = it.z;
-    const int k = d.sk[s];
-    const int b0 = sb * SB, w = min(SB, k - b0), wp = (w + NB - 1) / NB * NB;
-    const int64_t n = d.n;
-    const int64_t row0 = d.sfirst[s] + b0;
-    const T *X = xp + xsoff[s] + (int64_t)sb * SB * SB;
-    for (int idx = threadIdx.x; idx < w * NR; idx += THREADS) {
-        const int q = idx / NR, c = idx % NR;
-        V[idx] = c < nrhs ? in[row0 + q + (int64_t)c * n] : T(0);
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, r0 = rb * NRW, r = r0 + lane;
-    T acc[NR];
-#pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = T(0);
-    // lower: columns q <= r; upper: q >= r (the stored blocks are zero outside)
-    const int qa = upper ? r0 : 0, qb = upper ? w : min(w, r0 + NRW);
-    narrow_accumulate<T, NR>(acc, X + r, wp, r < w, V, qa, qb);
-    const T sum = narrow_reduce<T, NR>(acc, red);
-    if (threadIdx.x < NRW * NR) {
-        const int rr = r0 + threadIdx.x % NRW, c = threadIdx.x / NRW;
-        if (rr < w && c < nrhs) out[row0 + rr + (int64_t)c * n] = sum;
-    }
+// first storage row and number of splits of the reduction below super-block sb
+__device__ __forceinline__ int narrow_first_row(int b0, int w) { return (b0 + w) & ~31; }
+__device__ __forceinline__ int narrow_splits(int b0, int w, int m, int mp) {
+    return b0 + w < m ? (mp - narrow_first_row(b0, w) + NKSR - 1) / NKSR : 0;
 }
 
-// rows below super-block B: target -= L(rows, B) y_B, 32 rows per CTA; item =
-// (s, sb, rb, 65536 * seg): seg 0 = pivot rows after B (target Tt), seg 1 =
-// rows of R (target the update vector W_s)
-template <class T, int NR>
-__global__ void __launch_bounds__(THREADS) bupdate_narrow_kernel(DevSym d, const T *__restrict__ front,
-                                                                 const T *__restrict__ Y, T *__restrict__ Tt,
-                                                                 T *__restrict__ W, const int4 *__restrict__ items,
-                                                                 int nrhs) {
+// FWD: y_B = X_B t_B, t_B = b_B + the children's (sb = 0) or the pending
+// right-hand side, from Y into Tt.  else: x_B = X_B^T t_B (xp: the stored
+// transposes), t_B = y_B - the splits' partial sums, from Tt into Y; 32 rows
+// per CTA.  item = (s, sb, row block, backward: first slot)
+template <class T, int NR, bool FWD>
+__global__ void __launch_bounds__(THREADS) xnarrow_kernel(DevSym d, const T *__restrict__ xp,
+                                                          const int64_t *__restrict__ xsoff, T *Y, T *Tt,
+                                                          const T *__restrict__ W, const T *__restrict__ P,
+                                                          const int4 *__restrict__ items, int nrhs) {
     __shared__ T V[SB * NR];
-    __shared__ T red[NWARP * NRW * NR];
+    __shared__ __align__(16) T red[NWARP * NRW * NR];
+    Children &ch = *reinterpret_cast<Children *>(red);    // done with before the product writes red
+    const int4 it = items[blockIdx.x];
+    const int s = it.x, sb = it.y, r0 = it.z * NRW;
+    const int k = d.sk[s];
+    const int b0 = sb * SB, w = min(SB, k - b0), wp = (w + NB - 1) / NB * NB;
+    const int64_t n = d.n, row0 = d.sfirst[s] + b0;
+    // lower: columns up to the rows' last; upper: from the rows' first
+    const int pa = FWD ? 0 : r0, pb = FWD ? min(w, r0 + NRW) : w;
+    const T *in = FWD ? Y : Tt;
+    T *out = FWD ? Tt : Y;
+    const int m = d.sm[s], nsplit = FWD ? 0 : narrow_splits(b0, w, m, d.skp[s] + m - k);
+    for (int p0 = pa; p0 < pb; p0 += THREADS) {
+        const int p = p0 + threadIdx.x;
+        const bool ok = p < pb;
+        T t[NR];
+#pragma unroll
+        for (int c = 0; c < NR; ++c) t[c] = ok && c < nrhs ? in[row0 + p + (int64_t)c * n] : T(0);
+        if (FWD) {
+            if (sb == 0) add_children<T, NR>(d, s, W, nrhs, ch, p, ok, t);
+        } else if (ok) {
+            const T *Pp = P + ((int64_t)(it.w + (p / NARROW_COLS) * nsplit) * NR) * NARROW_COLS + p % NARROW_COLS;
+            T sum[NR];
+#pragma unroll
+            for (int c = 0; c < NR; ++c) sum[c] = T(0);
+#pragma unroll 4
+            for (int q = 0; q < nsplit; ++q)
+#pragma unroll
+                for (int c = 0; c < NR; ++c) sum[c] += Pp[(int64_t)(q * NR + c) * NARROW_COLS];
+#pragma unroll
+            for (int c = 0; c < NR; ++c) t[c] -= sum[c];
+        }
+        if (ok) {
+#pragma unroll
+            for (int c = 0; c < NR; ++c) V[p * NR + c] = t[c];
+        }
+    }
+    __syncthreads();
+    const T sum = narrow_product<T, NR>(xp + xsoff[s] + (int64_t)sb * SB * SB + r0, wp, V, pa, pb, red);
+    const int r = r0 + threadIdx.x % NRW, c = threadIdx.x / NRW;
+    if (threadIdx.x < NRW * NR && r < w && c < nrhs) out[row0 + r + (int64_t)c * n] = sum;
+}
+
+// rows below super-block B: target = pending - L(rows, B) y_B, 32 rows per
+// CTA; for the first super-block the pending values are b (pivot rows) plus
+// the children's.  item = (s, sb, rb, 65536 * seg): seg 0 = pivot rows after B
+// (in Y), seg 1 = rows of R (the update vector W_s)
+template <class T, int NR>
+__global__ void __launch_bounds__(THREADS) bnarrow_kernel(DevSym d, const T *__restrict__ front, T *Y,
+                                                          const T *__restrict__ Tt, T *W,
+                                                          const int4 *__restrict__ items, int nrhs) {
+    __shared__ T V[SB * NR];
+    __shared__ __align__(16) T red[NWARP * NRW * NR];
+    Children &ch = *reinterpret_cast<Children *>(red);    // done with before the product writes red
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y, rb = it.z, seg = it.w >> 16;
     const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s];
@@ -474,91 +576,104 @@ __global__ void __launch_bounds__(THREADS) bupdate_narrow_kernel(DevSym d, const
     const int f = d.sfirst[s];
     const int i0 = seg == 0 ? b0 + w + rb * NRW : rb * NRW;
     const int nrow = seg == 0 ? k - i0 : (m - k) - i0;
-    const int mrow = seg == 0 ? i0 : kp + i0;
-    T *dst;
-    int64_t ldd;
-    if (seg == 0) {
-        dst = Tt + f + i0;
-        ldd = n;
-    } else {
-        dst = W + d.woff[s] * nrhs + i0;
-        ldd = m - k;
-    }
+    T *dst = seg == 0 ? Y + f + i0 : W + d.woff[s] * nrhs + i0;
+    const int64_t ldd = seg == 0 ? n : m - k;
     for (int idx = threadIdx.x; idx < w * NR; idx += THREADS) {
         const int p = idx / NR, c = idx % NR;
-        V[idx] = c < nrhs ? Y[f + b0 + p + (int64_t)c * n] : T(0);
+        V[idx] = c < nrhs ? Tt[f + b0 + p + (int64_t)c * n] : T(0);
     }
-    // the target is read while the columns stream in
-    T tpre = T(0);
-    if (threadIdx.x < NRW * NR) {
-        const int r = threadIdx.x % NRW, c = threadIdx.x / NRW;
-        if (r < nrow && c < nrhs) tpre = dst[r + (int64_t)c * ldd];
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    T acc[NR];
+    // pending values: warp 0, one row per lane
+    const bool own = threadIdx.x < NRW && threadIdx.x < nrow;
+    T t[NR];
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = T(0);
-    narrow_accumulate<T, NR>(acc, front + d.foff[s] + (int64_t)b0 * ld + mrow + lane, ld, lane < nrow, V, 0, w);
-    const T sum = narrow_reduce<T, NR>(acc, red);
-    if (threadIdx.x < NRW * NR) {
-        const int r = threadIdx.x % NRW, c = threadIdx.x / NRW;
-        if (r < nrow && c < nrhs) dst[r + (int64_t)c * ldd] = tpre - sum;
+    for (int c = 0; c < NR; ++c)
+        t[c] = own && c < nrhs && (seg == 0 || sb > 0) ? dst[threadIdx.x + (int64_t)c * ldd] : T(0);
+    if (sb == 0)
+        add_children<T, NR>(d, s, W, nrhs, ch, (seg == 0 ? i0 : k + i0) + (int)threadIdx.x, own, t);
+    __syncthreads();
+    const T sum = narrow_product<T, NR>(front + d.foff[s] + (int64_t)b0 * ld + (seg == 0 ? i0 : kp + i0), ld, V, 0, w,
+                                        red);
+    // the sums, (row, right-hand side) over threads, to the pending values' lanes
+    __syncthreads();
+    if (threadIdx.x < NRW * NR) red[threadIdx.x] = sum;
+    __syncthreads();
+    if (own) {
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+            if (c < nrhs) dst[threadIdx.x + (int64_t)c * ldd] = t[c] - red[c * NRW + threadIdx.x];
     }
 }
 
 // Partial reduction of t_B = y_B - L(rows below B, B)^T x(rows below) over the
-// rows [ks KSR, (ks + 1) KSR) of the "rows below" list, for the 64 columns
-// j0 = b0 + 64 cb ...: one warp per column (8 columns per warp), lanes over
-// rows; P[slot] holds the sums in the 64 x 32 tile layout ([rhs][column]).
+// storage rows [q0, q0 + NKSR) from the 32-row boundary at or above the super-
+// block's end, for the 64 columns b0 + 64 cb ...: 8 columns per warp, lanes
+// over rows (x zero at rows that do not count); P[slot] ([rhs][column]).
 // item = (s, sb * 16 + cb, 65536 * ks, slot)
 template <class T, int NR>
-__global__ void __launch_bounds__(THREADS) breduce_narrow_kernel(DevSym d, const T *__restrict__ front,
-                                                                 const T *__restrict__ Y, T *__restrict__ P,
-                                                                 const int4 *__restrict__ items, int nrhs) {
-    constexpr int RC = NARROW_COLS, RR = NARROW_RHS;     // P tile: RR right-hand sides x RC columns
-    __shared__ T xs[KSR * NR];
+__global__ void __launch_bounds__(THREADS) rnarrow_kernel(DevSym d, const T *__restrict__ front,
+                                                          const T *__restrict__ Y, T *__restrict__ P,
+                                                          const int4 *__restrict__ items, int nrhs) {
+    using VT = typename Vec16<T>::type;
+    constexpr int VR = 16 / sizeof(T), H = NKSR / (32 * VR);   // vectors of a lane per column
+    constexpr int CG = 16 / H;                                 // columns whose loads are in flight together
+    __shared__ T xs[NKSR * NR];
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y >> 4, cb = it.y & 15, ks = it.z >> 16;
-    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s];
+    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s], mp = kp + m - k;
     const int b0 = sb * SB, w = min(SB, k - b0);
-    const int j0 = b0 + cb * RC, nb = min(RC, k - j0);
+    const int j0 = b0 + cb * NARROW_COLS, nb = min(NARROW_COLS, b0 + w - j0);
     const int64_t n = d.n;
-    const T *F = front + d.foff[s] + (int64_t)j0 * ld;
     const int32_t *rows = d.rows + d.rowptr[s];
-    const int nJ = k - (b0 + w), nbelow = nJ + (m - k);
-    const int u0 = ks * KSR, nu = min(nbelow, u0 + KSR) - u0;
-    for (int idx = threadIdx.x; idx < nu * NR; idx += THREADS) {
-        const int rr = idx / NR, c = idx % NR;
-        const int u = u0 + rr;
-        const int lr = u < nJ ? b0 + w + u : k + (u - nJ);
-        xs[idx] = c < nrhs ? Y[rows[lr] + (int64_t)c * n] : T(0);
+    const int q0 = narrow_first_row(b0, w) + ks * NKSR;
+    for (int idx = threadIdx.x; idx < NKSR; idx += THREADS) {
+        const int q = q0 + idx;
+        const bool ok = q >= b0 + w && q < mp && (q < k || q >= kp);
+        const int64_t g = ok ? rows[q < k ? q : q - (kp - k)] : 0;
+#pragma unroll
+        for (int c = 0; c < NR; ++c) xs[c * NKSR + idx] = ok && c < nrhs ? Y[g + (int64_t)c * n] : T(0);
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    T *Pt = P + (int64_t)it.w * RR * RC;
-    for (int q = 0; q < RC / NWARP; ++q) {
-        const int cl = warp * (RC / NWARP) + q;
-        if (cl >= nb) break;
-        T acc[NR];
+    const T *F = front + d.foff[s] + (int64_t)j0 * ld;
+    constexpr int CW = NARROW_COLS / NWARP;
+    for (int c0 = 0; c0 < CW; c0 += CG) {
+        VT x[CG][H];
 #pragma unroll
-        for (int c = 0; c < NR; ++c) acc[c] = T(0);
-        const T *col = F + (int64_t)cl * ld;
+        for (int u = 0; u < CG; ++u)
 #pragma unroll
-        for (int rr = lane; rr < KSR; rr += 32) {
-            if (rr < nu) {
-                const int u = u0 + rr;
-                const T a = col[u < nJ ? b0 + w + u : kp + (u - nJ)];
-#pragma unroll
-                for (int c = 0; c < NR; ++c) acc[c] += a * xs[rr * NR + c];
+            for (int h = 0; h < H; ++h) {
+                const int cl = warp * CW + c0 + u, q = q0 + (h * 32 + lane) * VR;
+                // q < mp: the 16 bytes lie inside the column (ld is a multiple of 32)
+                if (c0 + u < CW && cl < nb && q < mp) x[u][h] = *reinterpret_cast<const VT *>(F + (int64_t)cl * ld + q);
             }
-        }
 #pragma unroll
-        for (int c = 0; c < NR; ++c) {
-            T v = acc[c];
+        for (int u = 0; u < CG; ++u) {
+            const int cl = warp * CW + c0 + u;
+            if (c0 + u >= CW || cl >= nb) break;
+            T acc[NR];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0 && c < nrhs) Pt[c * RC + cl] = v;
+            for (int c = 0; c < NR; ++c) acc[c] = T(0);
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const int r = (h * 32 + lane) * VR;
+                if (q0 + r >= mp) continue;
+                const T *e = reinterpret_cast<const T *>(&x[u][h]);
+#pragma unroll
+                for (int i = 0; i < VR; ++i) {
+                    // rows of the super-block itself (above its diagonal
+                    // anything) and past the end of the front do not count
+                    const T v = q0 + r + i >= b0 + w && q0 + r + i < mp ? e[i] : T(0);
+#pragma unroll
+                    for (int c = 0; c < NR; ++c) acc[c] += v * xs[c * NKSR + r + i];
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NR; ++c) {
+                T v = acc[c];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == 0) P[((int64_t)it.w * NR + c) * NARROW_COLS + cl] = v;
+            }
         }
     }
 }
@@ -602,41 +717,20 @@ static void finish_go(const DevSym &d, const T *Y, T *Tt, const T *P, const int4
 
 template <class T>
 void launch_xapply(const DevSym &d, const T *xp, const int64_t *xsoff, const T *in, T *out, T *ksw, int *kcnt,
-                   const int4 *items, int count, int upper, int large, int nrhs, cudaStream_t st) {
+                   const int4 *items, int count, int upper, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
-    if (large == 2) {
-        if (nrhs == 1) xapply_narrow_kernel<T, 1><<<count, THREADS, 0, st>>>(d, xp, xsoff, in, out, items, upper, nrhs);
-        else if (nrhs == 2) xapply_narrow_kernel<T, 2><<<count, THREADS, 0, st>>>(d, xp, xsoff, in, out, items, upper, nrhs);
-        else if (nrhs <= 4) xapply_narrow_kernel<T, 4><<<count, THREADS, 0, st>>>(d, xp, xsoff, in, out, items, upper, nrhs);
-        else xapply_narrow_kernel<T, 8><<<count, THREADS, 0, st>>>(d, xp, xsoff, in, out, items, upper, nrhs);
-        return;
-    }
     xapply_kernel<T><<<count, t32::TH, 0, st>>>(d, xp, xsoff, in, out, ksw, kcnt, items, upper, nrhs);
 }
 template <class T>
 void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, T *ksw, int *kcnt,
-                    const int4 *items, int count, int large, int nrhs, cudaStream_t st) {
+                    const int4 *items, int count, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
-    if (large == 2) {
-        if (nrhs == 1) bupdate_narrow_kernel<T, 1><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
-        else if (nrhs == 2) bupdate_narrow_kernel<T, 2><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
-        else if (nrhs <= 4) bupdate_narrow_kernel<T, 4><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
-        else bupdate_narrow_kernel<T, 8><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
-        return;
-    }
     bupdate_kernel<T><<<count, t32::TH, 0, st>>>(d, front, Y, Tt, W, ksw, kcnt, items, nrhs);
 }
 template <class T>
 void launch_breduce(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count,
-                    int large, int nrhs, cudaStream_t st) {
+                    int nrhs, cudaStream_t st) {
     if (count <= 0) return;
-    if (large == 2) {
-        if (nrhs == 1) breduce_narrow_kernel<T, 1><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
-        else if (nrhs == 2) breduce_narrow_kernel<T, 2><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
-        else if (nrhs <= 4) breduce_narrow_kernel<T, 4><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
-        else breduce_narrow_kernel<T, 8><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
-        return;
-    }
     breduce_kernel<T><<<count, t32::TH, 0, st>>>(d, front, Y, P, items, nrhs);
 }
 template <class T>
@@ -644,8 +738,42 @@ void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const
                            int large, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
     if (large == 1) finish_go<T, 128, 64>(d, Y, Tt, P, items, count, nrhs, st);
-    else if (large == 2) finish_go<T, NARROW_COLS, NARROW_RHS>(d, Y, Tt, P, items, count, nrhs, st);
     else finish_go<T, t32::TT, t32::TT>(d, Y, Tt, P, items, count, nrhs, st);
+}
+
+// f<NR>() for nrhs <= 8
+template <class F>
+static void by_width(int nrhs, F f) {
+    if (nrhs == 1) f(std::integral_constant<int, 1>());
+    else if (nrhs == 2) f(std::integral_constant<int, 2>());
+    else if (nrhs <= 4) f(std::integral_constant<int, 4>());
+    else f(std::integral_constant<int, 8>());
+}
+template <class T>
+void launch_xnarrow(const DevSym &d, const T *xp, const int64_t *xsoff, T *Y, T *Tt, const T *W, const T *P,
+                    const int4 *items, int count, bool forward, int nrhs, cudaStream_t st) {
+    if (count <= 0) return;
+    by_width(nrhs, [&](auto nr) {
+        if (forward)
+            xnarrow_kernel<T, nr.value, true><<<count, THREADS, 0, st>>>(d, xp, xsoff, Y, Tt, W, P, items, nrhs);
+        else xnarrow_kernel<T, nr.value, false><<<count, THREADS, 0, st>>>(d, xp, xsoff, Y, Tt, W, P, items, nrhs);
+    });
+}
+template <class T>
+void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, const int4 *items, int count, int nrhs,
+                    cudaStream_t st) {
+    if (count <= 0) return;
+    by_width(nrhs, [&](auto nr) {
+        bnarrow_kernel<T, nr.value><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
+    });
+}
+template <class T>
+void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
+                    cudaStream_t st) {
+    if (count <= 0) return;
+    by_width(nrhs, [&](auto nr) {
+        rnarrow_kernel<T, nr.value><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
+    });
 }
 
 #define WD_BLOCKED_INST(T)                                                                              \
@@ -656,11 +784,17 @@ void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const
     template void launch_bfwd_gather<T>(const DevSym &, const T *, T *, T *, const int4 *, int, int, int, \
                                         cudaStream_t);                                                  \
     template void launch_xapply<T>(const DevSym &, const T *, const int64_t *, const T *, T *, T *, int *, \
-                                   const int4 *, int, int, int, int, cudaStream_t);                     \
+                                   const int4 *, int, int, int, cudaStream_t);                          \
     template void launch_bupdate<T>(const DevSym &, const T *, const T *, T *, T *, T *, int *,          \
-                                    const int4 *, int, int, int, cudaStream_t);                         \
-    template void launch_breduce<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
+                                    const int4 *, int, int, cudaStream_t);                              \
+    template void launch_xnarrow<T>(const DevSym &, const T *, const int64_t *, T *, T *, const T *,     \
+                                    const T *, const int4 *, int, bool, int, cudaStream_t);             \
+    template void launch_bnarrow<T>(const DevSym &, const T *, T *, const T *, T *, const int4 *, int,   \
                                     int, cudaStream_t);                                                 \
+    template void launch_rnarrow<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
+                                    cudaStream_t);                                                      \
+    template void launch_breduce<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
+                                    cudaStream_t);                                                 \
     template void launch_breduce_finish<T>(const DevSym &, const T *, T *, const T *, const int4 *, int, \
                                            int, int, cudaStream_t);
 WD_BLOCKED_INST(float)

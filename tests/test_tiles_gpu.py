@@ -128,3 +128,30 @@ def test_solve_tiles(wdlib, cuda, opts, nrhs):
         B = rhs(c.size - 1, nrhs, seed=nrhs)
         s = wdlib.Solver(**opts).analyze(c, r, basis).factor(vals, prec)
         assert oracle.backward_error(c, r, vals, s.solve(B), B).max() <= 1e-12
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 8])
+def test_narrow_solve_edges(wdlib, cuda, prec, nrhs):
+    """Up to 8 right-hand sides: dense fronts around the widths of blocks and
+    super-blocks, and trees with many children and rows below."""
+    rng = np.random.default_rng(nrhs)
+    cases = []
+    for n in (1, 31, 33, 64, 511, 513, 600):
+        M = rng.standard_normal((n, n))
+        cases.append(_lower_csc(M @ M.T + n * np.eye(n)) + (None,))
+    for dim, J in ((1, 3), (1, 9), (2, 5)):
+        b, cp, ri, v, _ = _case(dim, J)
+        cases.append((cp, ri, v, b))
+    n = 70                                   # an arrow: 69 children of one root
+    A = np.eye(n) * 4.0
+    A[-1, :-1] = A[:-1, -1] = 0.3
+    A[-1, -1] = n
+    cp = np.arange(0, 2 * n, 2)
+    cp = np.concatenate([cp, [2 * n - 1]]).astype(np.int64)
+    ri = np.array([x for j in range(n - 1) for x in (j, n - 1)] + [n - 1], np.int32)
+    cases.append((cp, ri, A[ri, np.repeat(np.arange(n), np.diff(cp))], None))
+    for cp, ri, v, basis in cases:
+        B = rhs(cp.size - 1, nrhs, seed=nrhs)
+        s = wdlib.Solver(relax_k=0, relax_pct=0).analyze(cp, ri, basis).factor(v, prec)
+        assert oracle.backward_error(cp, ri, v, s.solve(B), B).max() <= 1e-12
