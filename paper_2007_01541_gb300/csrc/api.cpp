@@ -1538,13 +1538,14 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
         wd_status fs = (prec == WD_FP64) ? run_factor_plan<double>(h, st) : run_factor_plan<float>(h, st);
         if (fs != WD_OK) return fs;
     }
-    wd::launch_norm_inf_rows(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin, h->n_spmv_fin,
-                             h->d_norm_part, h->d_scalars, st);
+    // ||A||_inf, or every instance's own (all that a batch uses)
     h->launches += h->n_spmv_fin > 0 ? 2 : 1;
-    if (h->batch_count > 0) {
+    if (h->batch_count == 0) {
+        wd::launch_norm_inf_rows(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin, h->n_spmv_fin,
+                                 h->d_norm_part, h->d_scalars, st);
+    } else {
         wd::launch_seg_norm_inf(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin, h->n_spmv_fin,
                                 h->d_norm_part, h->d_batch_coff, h->batch_count, h->d_batch_norm, st);
-        h->launches += 1;
         h->batch_normA.resize(h->batch_count);
         CK(cudaMemcpyAsync(h->batch_normA.data(), h->d_batch_norm, h->batch_count * sizeof(double),
                            cudaMemcpyDeviceToHost, st),
@@ -1554,7 +1555,8 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
     status_t status = 0, tstatus = 0;
     CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
     CK(cudaMemcpyAsync(&tstatus, h->d_tstatus, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
-    CK(cudaMemcpyAsync(&h->normA, h->d_scalars, sizeof(double), cudaMemcpyDeviceToHost, st), "norm D2H");
+    if (h->batch_count == 0)
+        CK(cudaMemcpyAsync(&h->normA, h->d_scalars, sizeof(double), cudaMemcpyDeviceToHost, st), "norm D2H");
     CK(cudaStreamSynchronize(st), "factor");
     if (tstatus != 0) return fail(h, WD_ERR_TIMEOUT, "a bounded wait of the tensor-core update expired");
     if (status != ~0ULL) {

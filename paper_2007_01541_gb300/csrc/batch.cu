@@ -2,6 +2,7 @@
 // block-diagonal matrix (wd_analyze_batch): instance i owns the permuted rows
 // [coff[i], coff[i+1]) and the supernodes [soff[i], soff[i+1]).  One block per
 // instance, fixed reduction order (deterministic).
+#include "dev_common.cuh"
 #include "engine.h"
 
 namespace wd {
@@ -9,14 +10,14 @@ namespace {
 
 constexpr int THREADS = 256;
 
-__device__ __forceinline__ double block_max(double v, double *red) {
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+__device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long *red) {
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __syncthreads();
     if (lane == 0) red[w] = v;
     __syncthreads();
-    v = lane < THREADS / 32 ? red[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    v = lane < THREADS / 32 ? red[lane] : 0ull;
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
@@ -48,20 +49,23 @@ __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v) {
 }
 
 // out[inst] = max over the instance's rows of sum_j |a_ij|: the chunk items of
-// the residual product (row, first entry, end, slot), one warp each; rows cut
+// the residual product (row, first entry, end, slot), NL lanes each; rows cut
 // into several chunks leave their partial sums in partial[slot] for the finish
 // kernel.  out must be zeroed; the maximum is order-independent.
+constexpr int NL = 8;
 __global__ void __launch_bounds__(THREADS) seg_norm_chunks_kernel(DevSym d, const int4 *__restrict__ items,
                                                                   int nchunks, double *__restrict__ partial,
                                                                   const int64_t *__restrict__ coff, int count,
                                                                   double *__restrict__ out) {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / NL;
+    const int lane = threadIdx.x % NL;
+    const unsigned mask = (0xFFu << (threadIdx.x & 24));
     if (w >= nchunks) return;
     const int4 it = items[w];
     double acc = 0.0;
-    for (int e = it.y + lane; e < it.z; e += 32) acc += fabs(d.csr_val[e]);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+#pragma unroll 4
+    for (int e = it.y + lane; e < it.z; e += NL) acc += fabs(d.csr_val[e]);
+    for (int o = NL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(mask, acc, o);
     if (lane == 0) {
         if (it.w < 0) atomic_max_nonneg(out + instance_of(coff, count, it.x), acc);
         else partial[it.w] = acc;
@@ -85,23 +89,24 @@ __global__ void __launch_bounds__(THREADS) seg_colmax3_kernel(const double *__re
                                                               const double *__restrict__ B,
                                                               const int64_t *__restrict__ coff, int nrhs,
                                                               double *__restrict__ out) {
-    __shared__ double red[THREADS / 32];
+    __shared__ unsigned long long red[THREADS / 32];
     const int inst = blockIdx.x;
     for (int c = 0; c < nrhs; ++c) {
-        double a = 0.0, b = 0.0, e = 0.0;
+        unsigned long long a = 0, b = 0, e = 0;
+#pragma unroll 4
         for (int64_t r = coff[inst] + threadIdx.x; r < coff[inst + 1]; r += THREADS) {
-            a = fmax(a, fabs(R[r * nrhs + c]));
-            b = fmax(b, fabs(X[r * nrhs + c]));
-            e = fmax(e, fabs(B[r * nrhs + c]));
+            a = max(a, abs_key(R[r * nrhs + c]));
+            b = max(b, abs_key(X[r * nrhs + c]));
+            e = max(e, abs_key(B[r * nrhs + c]));
         }
         a = block_max(a, red);
         b = block_max(b, red);
         e = block_max(e, red);
         if (threadIdx.x == 0) {
             double *o = out + ((int64_t)inst * nrhs + c) * 3;
-            o[0] = a;
-            o[1] = b;
-            o[2] = e;
+            o[0] = __longlong_as_double((long long)a);
+            o[1] = __longlong_as_double((long long)b);
+            o[2] = __longlong_as_double((long long)e);
         }
     }
 }
@@ -138,7 +143,7 @@ __global__ void __launch_bounds__(THREADS) seg_sum_kernel(const double *__restri
 void launch_seg_norm_inf(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin, int nfin,
                          double *partial, const int64_t *coff, int count, double *out, cudaStream_t st) {
     cudaMemsetAsync(out, 0, count * sizeof(double), st);
-    seg_norm_chunks_kernel<<<(int)(((int64_t)nchunks * 32 + THREADS - 1) / THREADS), THREADS, 0, st>>>(
+    seg_norm_chunks_kernel<<<(int)(((int64_t)nchunks * NL + THREADS - 1) / THREADS), THREADS, 0, st>>>(
         d, chunks, nchunks, partial, coff, count, out);
     if (nfin > 0) seg_norm_finish_kernel<<<(nfin + 127) / 128, 128, 0, st>>>(fin, nfin, partial, coff, count, out);
 }

@@ -2,6 +2,8 @@
 #pragma once
 #include <cstdint>
 
+#include "engine.h"
+
 namespace wd {
 
 // Asynchronous global -> shared copies (cp.async): the copy does not occupy a
@@ -26,6 +28,23 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
+}
+
+// |x| as a key that orders like the value; NaN counts as 0 (fmax ignores it)
+__device__ __forceinline__ unsigned long long abs_key(double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+    return u > 0x7FF0000000000000ull ? 0ull : u;
+}
+
+// the supernode of column j
+__device__ __forceinline__ int supernode_of(const DevSym &d, int j) {
+    int lo = 0, hi = d.ns - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (d.sfirst[mid] <= j) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
 }
 
 // Copy one element of type T with zero fill (valid = false -> zero).

@@ -4,6 +4,8 @@
 #include "dev_common.cuh"
 #include "engine.h"
 
+#include <algorithm>
+
 namespace wd {
 namespace {
 
@@ -32,6 +34,30 @@ __global__ void permute_out_kernel(const T *__restrict__ Y, double *__restrict__
     }
 }
 
+// x = h + l, h = x rounded to FP32, l = the rest rounded to FP32, on x's bits:
+// the conversions between the formats and the subtraction would each take the
+// FP64 pipe (64 cycles per warp and SM quarter), which bounded the gather of
+// A's values (22 million: 163 us against 80 us of memory traffic; a batch of
+// 64 instances: 581 -> 405 us).  Same
+// results (nearest, ties to even).  Exponents near the ends of FP32's range,
+// zeros, infinities and NaN take the conversions.
+__device__ __forceinline__ void split_bits(double x, float &h, float &l) {
+    const uint64_t u = (uint64_t)__double_as_longlong(x);
+    const int e = (int)((u >> 52) & 0x7FF) - 1023;
+    if (e < -70 || e > 126) {
+        h = __double2float_rn(x);
+        l = __double2float_rn(x - (double)h);
+        return;
+    }
+    const uint32_t top = (uint32_t)(u >> 29) & 0x7FFFFFu, low = (uint32_t)u & 0x1FFFFFFFu;
+    const uint32_t up = low > 0x10000000u || (low == 0x10000000u && (top & 1u)) ? 1u : 0u;
+    const uint32_t sign = (uint32_t)(u >> 32) & 0x80000000u;
+    h = __uint_as_float(sign | ((((uint32_t)(e + 127) << 23) | top) + up));
+    // the rest, an integer of at most 29 bits times 2^(e - 52)
+    const float r = __int2float_rn((int)low - (int)(up << 29));
+    l = r * __uint_as_float(sign | ((uint32_t)(e - 52 + 127) << 23));
+}
+
 // out = values in CSR order; hi / lo (optional): the double-float split
 // out = hi + lo (hi = out rounded to FP32, lo = the rest rounded to FP32)
 __global__ void gather_values_kernel(const int32_t *__restrict__ src, const double *__restrict__ v,
@@ -41,11 +67,7 @@ __global__ void gather_values_kernel(const int32_t *__restrict__ src, const doub
          e += (int64_t)gridDim.x * blockDim.x) {
         const double x = v[src[e]];
         out[e] = x;
-        if (hi) {
-            const float h = __double2float_rn(x);
-            hi[e] = h;
-            lo[e] = __double2float_rn(x - (double)h);
-        }
+        if (hi) split_bits(x, hi[e], lo[e]);
     }
 }
 
@@ -54,9 +76,9 @@ __global__ void gather_values_kernel(const int32_t *__restrict__ src, const doub
 __global__ void split_df_kernel(const double *__restrict__ X, float2 *__restrict__ Xp, int64_t cnt) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const double x = X[t];
-        const float h = __double2float_rn(x);
-        Xp[t] = make_float2(h, __double2float_rn(x - (double)h));
+        float2 q;
+        split_bits(X[t], q.x, q.y);
+        Xp[t] = q;
     }
 }
 
@@ -295,6 +317,20 @@ __global__ void transpose_kernel(Tc *__restrict__ C, double *__restrict__ Rm, in
                 Rm[i * nrhs + c] = accumulate ? Rm[i * nrhs + c] + v : v;
             }
         }
+    }
+}
+
+// the same for few right-hand sides, one row per thread (the 32 x 32 tiles
+// would be almost empty)
+template <class Tc>
+__global__ void transpose_narrow_kernel(Tc *__restrict__ C, double *__restrict__ Rm, int64_t n, int nrhs, int dir,
+                                        int accumulate) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    for (int c = 0; c < nrhs; ++c) {
+        const int64_t r = i * nrhs + c;
+        if (dir == 0) C[i + c * n] = (Tc)Rm[r];
+        else Rm[r] = accumulate ? Rm[r] + (double)C[i + c * n] : (double)C[i + c * n];
     }
 }
 
@@ -669,7 +705,11 @@ __global__ void xupdate_kernel(const float *__restrict__ Y, double *__restrict__
     }
 }
 
-// Few right-hand sides (<= 8): lanes over the entries of the chunk, NR (the
+// Few right-hand sides (<= 8): SPL = 8 lanes per chunk over its entries (a whole
+// warp per chunk spends five FP64 warp additions on the sum of one row, as many
+// as it spends on 160 entries, and the FP64 pipe is the bound here; with 8
+// lanes it is three for four rows: 256 x 256 problem, one right-hand side, 93
+// -> 84 us; a batch of 64 instances 427 -> 278), NR (the
 // number of right-hand sides rounded up to 1, 2, 4 or 8) accumulators per
 // lane and U = 4 entries per lane in flight (their values, columns and x loads
 // are all issued before the first product), which hides the dependent
@@ -679,6 +719,7 @@ __global__ void xupdate_kernel(const float *__restrict__ Y, double *__restrict__
 // first entry with weight 0, accumulators past nrhs read right-hand side 0
 // (never written out), and a column index outside [0, n) is skipped and its
 // CSR position recorded in *bad (atomic minimum; the host clears and reads it).
+constexpr int SPL = 8;
 template <int NR>
 __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const int4 *__restrict__ items,
                                                               int count, const double *__restrict__ X,
@@ -686,8 +727,9 @@ __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const in
                                                               double *__restrict__ R,
                                                               double *__restrict__ P, int nrhs,
                                                               unsigned long long *__restrict__ bad) {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / SPL;
+    const int lane = threadIdx.x % SPL;
+    const unsigned mask = (0xFFu << (threadIdx.x & 24));    // this chunk's lanes
     if (w >= count) return;
     const int4 it = items[w];
     const int64_t row = it.x;
@@ -696,12 +738,12 @@ __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const in
     double acc[NR];
 #pragma unroll
     for (int c = 0; c < NR; ++c) acc[c] = 0.0;
-    for (int e0 = it.y + lane; e0 < it.z; e0 += 32 * U) {
+    for (int e0 = it.y + lane; e0 < it.z; e0 += SPL * U) {
         double v[U];
         int64_t xo[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int e = e0 + 32 * u;
+            const int e = e0 + SPL * u;
             const bool in = e < it.z;
             const int ec = in ? e : e0;
             double val = __ldcs(d.csr_val + ec);
@@ -726,7 +768,7 @@ __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const in
     for (int c = 0; c < NR; ++c) {
         double a = acc[c];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        for (int o = SPL / 2; o > 0; o >>= 1) a += __shfl_xor_sync(mask, a, o);
         if (lane == 0 && c < nrhs) {
             if (slot < 0) R[row * nrhs + c] = Bp[row * nrhs + c] - a;
             else P[(int64_t)slot * nrhs + c] = a;
@@ -749,6 +791,24 @@ __global__ void spmv_finish_kernel(const int4 *__restrict__ items, int count,
     }
 }
 
+// the same for few right-hand sides: one warp per row and right-hand side,
+// lanes over the slots, a fixed shuffle tree
+__global__ void __launch_bounds__(THREADS) spmv_finish_narrow_kernel(const int4 *__restrict__ items, int count,
+                                                                     const double *__restrict__ Bp,
+                                                                     double *__restrict__ R,
+                                                                     const double *__restrict__ P, int nrhs) {
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= (int64_t)count * nrhs) return;
+    const int4 it = items[w / nrhs];
+    const int c = (int)(w % nrhs);
+    double acc = 0.0;
+    for (int q = lane; q < it.z; q += 32) acc += P[(int64_t)(it.y + q) * nrhs + c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) R[(int64_t)it.x * nrhs + c] = Bp[(int64_t)it.x * nrhs + c] - acc;
+}
+
 __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v) {
     // non-negative doubles order like their bit patterns
     atomicMax(reinterpret_cast<unsigned long long *>(addr), (unsigned long long)__double_as_longlong(v));
@@ -758,14 +818,16 @@ __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v) {
 // (single-chunk rows go straight to the maximum, cut rows through partial[])
 __global__ void norm_inf_chunks_kernel(DevSym d, const int4 *__restrict__ items, int count,
                                        double *__restrict__ partial, double *out) {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / SPL;   // 8 lanes per chunk, as the residual
+    const int lane = threadIdx.x % SPL;
+    const unsigned mask = (0xFFu << (threadIdx.x & 24));
     if (w >= count) return;
     const int4 it = items[w];
     double acc = 0.0;
-    for (int e = it.y + lane; e < it.z; e += 32) acc += fabs(d.csr_val[e]);
+#pragma unroll 4
+    for (int e = it.y + lane; e < it.z; e += SPL) acc += fabs(d.csr_val[e]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    for (int o = SPL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(mask, acc, o);
     if (lane == 0) {
         if (it.w < 0) atomic_max_nonneg(out, acc);
         else partial[it.w] = acc;
@@ -782,22 +844,63 @@ __global__ void norm_inf_finish_kernel(const int4 *__restrict__ fin, int nfin,
 }
 
 // per column c: out[3c] = max|R|, out[3c+1] = max|X|, out[3c+2] = max|B|
-// (row-major arrays; out must be zeroed; blocks take chunks of rows)
-__global__ void colmax3_rm_kernel(const double *__restrict__ R, const double *__restrict__ X,
-                                  const double *__restrict__ B, int64_t n, int nrhs,
-                                  int64_t rows_per_block, double *out) {
+// (row-major arrays; out must be zeroed; blocks take chunks of rows), on the
+// bits of |x| (abs_key: NaN does not count): an FP64 comparison takes the FP64
+// pipe.  256 threads are 64 columns x 4 rows; one atomic per block and column
+// (a block of 32 rows with its own atomics spent its time on them: 65,536
+// rows, 64 columns, with it the 256 x
+// 256 step 11.70 -> 11.56 ms).
+__global__ void __launch_bounds__(256) colmax3_rm_kernel(const double *__restrict__ R, const double *__restrict__ X,
+                                                         const double *__restrict__ B, int64_t n, int nrhs,
+                                                         int64_t rows_per_block, double *out) {
+    __shared__ unsigned long long red[3][4][64];
     const int64_t r0 = blockIdx.x * rows_per_block;
     const int64_t r1 = min(n, r0 + rows_per_block);
-    for (int c = threadIdx.x; c < nrhs; c += blockDim.x) {
-        double a = 0, b = 0, e = 0;
-        for (int64_t i = r0; i < r1; ++i) {
-            a = fmax(a, fabs(R[i * nrhs + c]));
-            b = fmax(b, fabs(X[i * nrhs + c]));
-            e = fmax(e, fabs(B[i * nrhs + c]));
+    const int cl = threadIdx.x & 63, g = threadIdx.x >> 6;
+    for (int c0 = 0; c0 < nrhs; c0 += 64) {
+        const int c = c0 + cl;
+        unsigned long long a = 0, b = 0, e = 0;
+        if (c < nrhs) {
+#pragma unroll 4
+            for (int64_t i = r0 + g; i < r1; i += 4) {
+                a = max(a, abs_key(R[i * nrhs + c]));
+                b = max(b, abs_key(X[i * nrhs + c]));
+                e = max(e, abs_key(B[i * nrhs + c]));
+            }
         }
-        atomic_max_nonneg(out + 3 * c, a);
-        atomic_max_nonneg(out + 3 * c + 1, b);
-        atomic_max_nonneg(out + 3 * c + 2, e);
+        red[0][g][cl] = a;
+        red[1][g][cl] = b;
+        red[2][g][cl] = e;
+        __syncthreads();
+        for (int t = threadIdx.x; t < 192; t += 256) {
+            const int q = t / 64, cc = t % 64;
+            const unsigned long long v = max(max(red[q][0][cc], red[q][1][cc]), max(red[q][2][cc], red[q][3][cc]));
+            if (c0 + cc < nrhs)
+                atomicMax(reinterpret_cast<unsigned long long *>(out + 3 * (int64_t)(c0 + cc) + q), v);
+        }
+        __syncthreads();
+    }
+}
+// few right-hand sides: lanes over rows
+__global__ void __launch_bounds__(256) colmax3_narrow_kernel(const double *__restrict__ R,
+                                                             const double *__restrict__ X,
+                                                             const double *__restrict__ B, int64_t n, int nrhs,
+                                                             double *out) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int c = 0; c < nrhs; ++c) {
+        unsigned long long m[3] = {0, 0, 0};
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += step) {
+            m[0] = max(m[0], abs_key(R[i * nrhs + c]));
+            m[1] = max(m[1], abs_key(X[i * nrhs + c]));
+            m[2] = max(m[2], abs_key(B[i * nrhs + c]));
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m[q] = max(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
+            if ((threadIdx.x & 31) == 0)
+                atomicMax(reinterpret_cast<unsigned long long *>(out + 3 * (int64_t)c + q), m[q]);
+        }
     }
 }
 
@@ -816,15 +919,15 @@ __global__ void cast_kernel(const double *__restrict__ src, T *__restrict__ dst,
         dst[t] = (T)src[t];
 }
 
-// block-wise pairwise sums of 2 log L_jj (fixed order, deterministic)
+// block-wise pairwise sums of 2 log L_jj (fixed order, deterministic), pivots
+// over all threads of the grid (a pivot's supernode by bisection)
 template <class T>
 __global__ void logdet_partial_kernel(DevSym d, const T *__restrict__ front, double *partial) {
     __shared__ double red[THREADS];
     double acc = 0.0;
-    for (int s = blockIdx.x; s < d.ns; s += gridDim.x) {
-        const int k = d.sk[s], ld = d.sld[s];
-        const T *F = front + d.foff[s];
-        for (int j = threadIdx.x; j < k; j += THREADS) acc += 2.0 * log((double)F[(int64_t)j * ld + j]);
+    for (int64_t j = blockIdx.x * (int64_t)THREADS + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * THREADS) {
+        const int s = supernode_of(d, (int)j);
+        acc += 2.0 * log((double)front[d.foff[s] + (j - d.sfirst[s]) * (d.sld[s] + (int64_t)1)]);
     }
     red[threadIdx.x] = acc;
     __syncthreads();
@@ -923,6 +1026,10 @@ void launch_permute_out_rm(const double *X, double *B, int64_t ldb, const int32_
 template <class Tc>
 void launch_transpose(Tc *C, double *Rm, int64_t n, int64_t nrhs, int dir, int accumulate,
                       cudaStream_t st) {
+    if (nrhs <= 8) {
+        transpose_narrow_kernel<Tc><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(C, Rm, n, (int)nrhs, dir, accumulate);
+        return;
+    }
     dim3 grid((unsigned)((n + 31) / 32), (unsigned)((nrhs + 31) / 32));
     transpose_kernel<Tc><<<grid, dim3(32, 8), 0, st>>>(C, Rm, n, nrhs, dir, accumulate);
 }
@@ -930,7 +1037,8 @@ void launch_transpose(Tc *C, double *Rm, int64_t n, int64_t nrhs, int dir, int a
 void launch_spmv_residual(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, const double *X, const double *Bp, double *R, double *P,
                           int64_t nrhs, unsigned long long *bad, cudaStream_t st) {
-    const int blocks = (int)(((int64_t)nchunks * 32 + THREADS - 1) / THREADS);
+    const int lanes = nrhs <= 8 ? SPL : 32;    // per chunk
+    const int blocks = (int)(((int64_t)nchunks * lanes + THREADS - 1) / THREADS);
     const int nr = (int)nrhs;
     if (nrhs == 1)
         spmv_narrow_kernel<1><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad);
@@ -942,7 +1050,9 @@ void launch_spmv_residual(const DevSym &d, const int4 *chunks, int nchunks, cons
         spmv_narrow_kernel<8><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad);
     else
         spmv_wide_kernel<<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, (int)nrhs);
-    if (nfin > 0) spmv_finish_kernel<<<nfin, 64, 0, st>>>(fin, nfin, Bp, R, P, (int)nrhs);
+    if (nfin > 0 && nrhs <= 8)
+        spmv_finish_narrow_kernel<<<(nfin * nr + 7) / 8, THREADS, 0, st>>>(fin, nfin, Bp, R, P, nr);
+    else if (nfin > 0) spmv_finish_kernel<<<nfin, 64, 0, st>>>(fin, nfin, Bp, R, P, (int)nrhs);
 }
 
 void launch_spmv_residual_df(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin, int nfin,
@@ -975,7 +1085,7 @@ void launch_xupdate(const float *Y, double *X, float *Xf, int64_t n, int64_t nrh
 void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, double *partial, double *out, cudaStream_t st) {
     cudaMemsetAsync(out, 0, sizeof(double), st);
-    norm_inf_chunks_kernel<<<(int)(((int64_t)nchunks * 32 + THREADS - 1) / THREADS), THREADS, 0, st>>>(
+    norm_inf_chunks_kernel<<<(int)(((int64_t)nchunks * SPL + THREADS - 1) / THREADS), THREADS, 0, st>>>(
         d, chunks, nchunks, partial, out);
     if (nfin > 0) norm_inf_finish_kernel<<<(nfin + 127) / 128, 128, 0, st>>>(fin, nfin, partial, out);
 }
@@ -983,8 +1093,13 @@ void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, cons
 void launch_colmax3(const double *R, const double *X, const double *Bp, int64_t n, int64_t nrhs,
                     double *out3, cudaStream_t st) {
     cudaMemsetAsync(out3, 0, 3 * nrhs * sizeof(double), st);
-    const int64_t rpb = 32;
-    colmax3_rm_kernel<<<(int)((n + rpb - 1) / rpb), 64, 0, st>>>(R, X, Bp, n, (int)nrhs, rpb, out3);
+    if (nrhs <= 8) {
+        const int blocks = (int)std::min<int64_t>((n + 1023) / 1024, 152);
+        colmax3_narrow_kernel<<<blocks, 256, 0, st>>>(R, X, Bp, n, (int)nrhs, out3);
+        return;
+    }
+    const int64_t rpb = std::max<int64_t>(16, (n + 607) / 608);    // four blocks per SM
+    colmax3_rm_kernel<<<(int)((n + rpb - 1) / rpb), 256, 0, st>>>(R, X, Bp, n, (int)nrhs, rpb, out3);
 }
 
 template <class T>
