@@ -163,6 +163,11 @@ struct wd_ctx {
     status_t *d_tstatus = nullptr;    // nonzero: a bounded device wait expired
     unsigned *d_gate = nullptr;       // a device word that stays zero (wd_options.test_closed_gate)
     cudaStream_t cap_stream = nullptr;
+    // pinned host words for what the calls read back (status words, norms, the
+    // column maxima of the residual): a copy to pageable memory makes the host
+    // wait for it, one after the other; these are all in flight before one wait
+    double *pin = nullptr;
+    int64_t pin_elems = 0;
     // wd_export_L_noalloc returns without waiting; this event, recorded on its
     // stream, orders that read of the fronts before the next call that
     // rewrites or frees them (wd_factor, wd_analyze, wd_destroy)
@@ -336,6 +341,7 @@ void wd_destroy(wd_handle h) {
         h->g_solve.reset();
         h->g_lu.reset();
         if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+        if (h->pin) cudaFreeHost(h->pin);
         h->work.free_all();
         h->mem.free_all();
         cudaSetDevice(prev);
@@ -815,6 +821,24 @@ static void fill_info(wd_handle h, int64_t nnzl, int maxm, int maxk,
         std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
 }
 
+// pinned words: PIN_* of their own, then room for the column maxima
+enum { PIN_STATUS, PIN_TSTATUS, PIN_NORM, PIN_BAD, PIN_BAD_STEP, PIN_CM = 8 };
+static wd_status ensure_pin(wd_handle h, int64_t elems) {
+    elems += PIN_CM;
+    if (h->pin_elems >= elems) return WD_OK;
+    if (h->pin) cudaFreeHost(h->pin);
+    h->pin = nullptr;
+    h->pin_elems = 0;
+    CK(cudaHostAlloc((void **)&h->pin, elems * sizeof(double), cudaHostAllocDefault), "pinned alloc");
+    h->pin_elems = elems;
+    return WD_OK;
+}
+static status_t pin_word(wd_handle h, int i) {
+    status_t v;
+    std::memcpy(&v, h->pin + i, sizeof(v));
+    return v;
+}
+
 // drop everything of a previous analysis; set up the device and stream
 static wd_status reset_analysis(wd_handle h) {
     const bool host_only = h->opt.symbolic_only != 0;
@@ -1211,6 +1235,11 @@ static wd_status finish_analysis(wd_handle h, std::chrono::steady_clock::time_po
         CK(h->mem.alloc((void **)&h->d_batch_ld, h->batch_count * sizeof(double)), "batch alloc");
         CK(h->mem.alloc((void **)&h->d_batch_sdl, std::max(ns, 1) * sizeof(double)), "batch alloc");
     }
+    {
+        // enough for the column maxima of 128 right-hand sides (and instances)
+        const wd_status ps = ensure_pin(h, 3 * 128);
+        if (ps != WD_OK) return ps;
+    }
     fill_info(h, nnzl, maxm, maxk, t0);
     h->analyzed = true;
     return WD_OK;
@@ -1546,18 +1575,22 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
     } else {
         wd::launch_seg_norm_inf(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin, h->n_spmv_fin,
                                 h->d_norm_part, h->d_batch_coff, h->batch_count, h->d_batch_norm, st);
-        h->batch_normA.resize(h->batch_count);
-        CK(cudaMemcpyAsync(h->batch_normA.data(), h->d_batch_norm, h->batch_count * sizeof(double),
+        const wd_status ps = ensure_pin(h, h->batch_count);
+        if (ps != WD_OK) return ps;
+        CK(cudaMemcpyAsync(h->pin + PIN_CM, h->d_batch_norm, h->batch_count * sizeof(double),
                            cudaMemcpyDeviceToHost, st),
            "norm D2H");
     }
     CK(cudaGetLastError(), "factor launch");
-    status_t status = 0, tstatus = 0;
-    CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
-    CK(cudaMemcpyAsync(&tstatus, h->d_tstatus, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
+    CK(cudaMemcpyAsync(h->pin + PIN_STATUS, h->d_status, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
+    CK(cudaMemcpyAsync(h->pin + PIN_TSTATUS, h->d_tstatus, sizeof(status_t), cudaMemcpyDeviceToHost, st),
+       "status D2H");
     if (h->batch_count == 0)
-        CK(cudaMemcpyAsync(&h->normA, h->d_scalars, sizeof(double), cudaMemcpyDeviceToHost, st), "norm D2H");
+        CK(cudaMemcpyAsync(h->pin + PIN_NORM, h->d_scalars, sizeof(double), cudaMemcpyDeviceToHost, st), "norm D2H");
     CK(cudaStreamSynchronize(st), "factor");
+    const status_t status = pin_word(h, PIN_STATUS), tstatus = pin_word(h, PIN_TSTATUS);
+    h->normA = h->pin[PIN_NORM];
+    if (h->batch_count > 0) h->batch_normA.assign(h->pin + PIN_CM, h->pin + PIN_CM + h->batch_count);
     if (tstatus != 0) return fail(h, WD_ERR_TIMEOUT, "a bounded wait of the tensor-core update expired");
     if (status != ~0ULL) {
         std::string where = "pivot not positive at column " + std::to_string(status);
@@ -1606,6 +1639,11 @@ static wd_status ensure_solve_ws(wd_handle h, int64_t nrhs) {
     if (h->batch_count > 0)
         CK(h->work.alloc((void **)&h->d_batch_cm, 3 * (int64_t)h->batch_count * nrhs * sizeof(double)),
            "solve ws");
+    {
+        // before anything of the call is in flight
+        const wd_status ps = ensure_pin(h, 3 * (int64_t)std::max(1, h->batch_count) * nrhs);
+        if (ps != WD_OK) return ps;
+    }
     h->ws_cols = nrhs;
     return WD_OK;
 }
@@ -1750,54 +1788,53 @@ static wd_status launch_residual(wd_handle h, const double *X, int64_t nrhs, cud
     return WD_OK;
 }
 
-// R = Bp - A X (FP64, row-major n x nrhs) and the largest normwise backward
-// error over the columns
-static wd_status backward_errors(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st,
-                                 double *be_max, const float *Xf = nullptr, const double *S = nullptr) {
-    const int64_t n = h->S.n;
-    unsigned long long bad = ~0ULL;
-    wd_status rs = launch_residual(h, X, nrhs, st, Xf, S);
-    if (rs != WD_OK) return rs;
-    if (h->batch_count > 0) {
-        // per instance and column: each instance is its own system
-        const int cnt = h->batch_count;
-        wd::launch_seg_colmax3(h->d_R, X, h->d_Bp, h->d_batch_coff, cnt, (int)nrhs, h->d_batch_cm, st);
-        h->launches += 2;
-        std::vector<double> cm(3 * (size_t)cnt * nrhs);
-        if (nrhs <= 8)
-            CK(cudaMemcpyAsync(&bad, h->d_spmv_bad, sizeof(bad), cudaMemcpyDeviceToHost, st), "spmv check");
-        CK(cudaMemcpyAsync(cm.data(), h->d_batch_cm, cm.size() * sizeof(double), cudaMemcpyDeviceToHost, st),
-           "be D2H");
-        CK(cudaStreamSynchronize(st), "backward error");
-        if (bad != ~0ULL)
-            return fail(h, WD_ERR_CUDA, "residual: column index out of range at CSR position " + std::to_string(bad));
-        double mx = 0.0;
-        for (int i = 0; i < cnt; ++i)
-            for (int64_t c = 0; c < nrhs; ++c) {
-                const double *q = cm.data() + ((size_t)i * nrhs + c) * 3;
-                const double den = h->batch_normA[i] * q[1] + q[2];
-                mx = std::max(mx, den > 0 ? q[0] / den : 0.0);
-            }
-        *be_max = mx;
-        return WD_OK;
-    }
-    wd::launch_colmax3(h->d_R, X, h->d_Bp, n, nrhs, h->d_cm, st);
+static wd_status bad_column(wd_handle h, status_t at) {
+    return fail(h, WD_ERR_CUDA, "residual: column index out of range at CSR position " + std::to_string(at));
+}
+
+// R = Bp - A X (FP64, row-major n x nrhs) and its column maxima (per instance
+// for a batch, each its own system), enqueued with their copies to h->pin
+static wd_status enqueue_backward_errors(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st,
+                                         const float *Xf = nullptr, const double *S = nullptr) {
+    const int64_t cnt = h->batch_count > 0 ? h->batch_count : 1;
+    wd_status s = launch_residual(h, X, nrhs, st, Xf, S);
+    if (s != WD_OK) return s;
+    double *cm = h->batch_count > 0 ? h->d_batch_cm : h->d_cm;
+    if (h->batch_count > 0)
+        wd::launch_seg_colmax3(h->d_R, X, h->d_Bp, h->d_batch_coff, (int)cnt, (int)nrhs, cm, st);
+    else
+        wd::launch_colmax3(h->d_R, X, h->d_Bp, h->S.n, nrhs, cm, st);
     h->launches += 2;
-    std::vector<double> cm(3 * nrhs);
     if (nrhs <= 8)
-        CK(cudaMemcpyAsync(&bad, h->d_spmv_bad, sizeof(bad), cudaMemcpyDeviceToHost, st), "spmv check");
-    CK(cudaMemcpyAsync(cm.data(), h->d_cm, cm.size() * sizeof(double), cudaMemcpyDeviceToHost, st), "be D2H");
-    CK(cudaStreamSynchronize(st), "backward error");
-    if (bad != ~0ULL)
-        return fail(h, WD_ERR_CUDA, "residual: column index out of range at CSR position " + std::to_string(bad));
+        CK(cudaMemcpyAsync(h->pin + PIN_BAD, h->d_spmv_bad, sizeof(status_t), cudaMemcpyDeviceToHost, st),
+           "spmv check");
+    CK(cudaMemcpyAsync(h->pin + PIN_CM, cm, 3 * cnt * nrhs * sizeof(double), cudaMemcpyDeviceToHost, st), "be D2H");
+    return WD_OK;
+}
+
+// the largest normwise backward error over columns (and instances), after the
+// copies have landed
+static wd_status read_backward_errors(wd_handle h, int64_t nrhs, double *be_max) {
+    if (nrhs <= 8 && pin_word(h, PIN_BAD) != ~0ULL) return bad_column(h, pin_word(h, PIN_BAD));
+    const int64_t cnt = h->batch_count > 0 ? h->batch_count : 1;
     double mx = 0.0;
-    for (int64_t c = 0; c < nrhs; ++c) {
-        const double den = h->normA * cm[3 * c + 1] + cm[3 * c + 2];
-        const double be = den > 0 ? cm[3 * c] / den : 0.0;
-        mx = std::max(mx, be);
+    for (int64_t i = 0; i < cnt; ++i) {
+        const double nrm = h->batch_count > 0 ? h->batch_normA[i] : h->normA;
+        for (int64_t c = 0; c < nrhs; ++c) {
+            const double *q = h->pin + PIN_CM + (i * nrhs + c) * 3;
+            const double den = nrm * q[1] + q[2];
+            mx = std::max(mx, den > 0 ? q[0] / den : 0.0);
+        }
     }
     *be_max = mx;
     return WD_OK;
+}
+
+static wd_status backward_errors(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st, double *be_max) {
+    wd_status s = enqueue_backward_errors(h, X, nrhs, st);
+    if (s != WD_OK) return s;
+    CK(cudaStreamSynchronize(st), "backward error");
+    return read_backward_errors(h, nrhs, be_max);
 }
 
 // workspaces and the launch plan of solves with nrhs right-hand sides
@@ -1862,10 +1899,8 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
         if (info) {
             wd::launch_transpose<double>(Y, h->d_X, n, nrhs, 1, 0, st);
             h->launches += 1;
-            double be;
-            s = backward_errors(h, h->d_X, nrhs, st, &be);
+            s = enqueue_backward_errors(h, h->d_X, nrhs, st);
             if (s != WD_OK) return s;
-            info->backward_error = be;
         }
         wd::launch_permute_out<double>(Y, Bd, ld, h->dsym.perm, n, nrhs, st);
         h->launches += 1;
@@ -1887,9 +1922,28 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
         double be = 1.0;
         int it = 0;
         for (;;) {
-            s = backward_errors(h, h->d_X, nrhs, st, &be, Xf, it == 0 ? h->d_Bp : h->d_R);
+            s = enqueue_backward_errors(h, h->d_X, nrhs, st, Xf, it == 0 ? h->d_Bp : h->d_R);
             if (s != WD_OK) return s;
-            if (be <= h->opt.ir_tol || it >= h->opt.ir_max_iter) break;
+            // one wait per step: after a refinement x is most often the
+            // result, so it goes out (again, if not) before the wait
+            const bool last = it > 0 || it >= h->opt.ir_max_iter;
+            if (last) {
+                wd::launch_permute_out_rm(h->d_X, Bd, ld, h->dsym.perm, n, nrhs, st);
+                h->launches += 1;
+            }
+            CK(cudaMemcpyAsync(h->pin + PIN_TSTATUS, h->d_tstatus, sizeof(status_t), cudaMemcpyDeviceToHost, st),
+               "status D2H");
+            CK(cudaStreamSynchronize(st), "backward error");
+            s = read_backward_errors(h, nrhs, &be);
+            if (s != WD_OK) return s;
+            if (be <= h->opt.ir_tol || it >= h->opt.ir_max_iter) {
+                if (!last) {
+                    wd::launch_permute_out_rm(h->d_X, Bd, ld, h->dsym.perm, n, nrhs, st);
+                    h->launches += 1;
+                    CK(cudaStreamSynchronize(st), "solve");
+                }
+                break;
+            }
             wd::launch_transpose<float>(Y, h->d_R, n, nrhs, 0, 0, st);
             s = run_solve_plan<float>(h, Y, nr, st);
             if (s != WD_OK) return s;
@@ -1903,12 +1957,7 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
             info->iterations = it;
             info->backward_error = be;
         }
-        wd::launch_permute_out_rm(h->d_X, Bd, ld, h->dsym.perm, n, nrhs, st);
-        h->launches += 1;
-        status_t tstatus = 0;
-        CK(cudaMemcpyAsync(&tstatus, h->d_tstatus, sizeof(status_t), cudaMemcpyDeviceToHost, st), "status D2H");
-        CK(cudaStreamSynchronize(st), "solve");
-        if (tstatus != 0) return fail(h, WD_ERR_TIMEOUT, "a bounded wait of a tensor-core solve product expired");
+        if (pin_word(h, PIN_TSTATUS) != 0) return fail(h, WD_ERR_TIMEOUT, "a bounded wait of a tensor-core solve product expired");
         if (be > h->opt.ir_tol) {
             if (!B_on_device)
                 cudaMemcpy2DAsync(B, ldb * sizeof(double), h->d_B, n * sizeof(double), n * sizeof(double),
@@ -1923,7 +1972,8 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
         CK(cudaMemcpy2DAsync(B, ldb * sizeof(double), h->d_B, n * sizeof(double), n * sizeof(double), nrhs,
                              cudaMemcpyDeviceToHost, st),
            "B D2H");
-    CK(cudaStreamSynchronize(st), "solve");
+    if (h->prec == WD_FP64 || !B_on_device) CK(cudaStreamSynchronize(st), "solve");
+    if (h->prec == WD_FP64 && info) return read_backward_errors(h, nrhs, &info->backward_error);
     return WD_OK;
 }
 
@@ -2010,14 +2060,17 @@ extern "C" wd_status wd_theta_step(wd_handle h, double *U, const double *F, int6
     if (theta < 1.0) {
         s = launch_residual(h, h->d_X, nrhs, st);
         if (s != WD_OK) return s;
-        unsigned long long bad = ~0ULL;
+        // the product's check of the column indices is read after the solve's wait
+        h->pin[PIN_BAD_STEP] = 0.0;
         if (nrhs <= 8)
-            CK(cudaMemcpyAsync(&bad, h->d_spmv_bad, sizeof(bad), cudaMemcpyDeviceToHost, st), "spmv check");
+            CK(cudaMemcpyAsync(h->pin + PIN_BAD_STEP, h->d_spmv_bad, sizeof(status_t), cudaMemcpyDeviceToHost, st),
+               "spmv check");
         CK(cudaMemcpyAsync(h->d_Bp, h->d_R, n * nrhs * sizeof(double), cudaMemcpyDeviceToDevice, st),
            "step right-hand side");
-        CK(cudaStreamSynchronize(st), "theta step");
-        if (bad != ~0ULL)
-            return fail(h, WD_ERR_CUDA, "residual: column index out of range at CSR position " + std::to_string(bad));
+        s = solve_core(h, Ud, ldd, U, ld, on_device, nrhs, st, info);
+        if (nrhs <= 8 && (s == WD_OK || s == WD_ERR_NO_CONVERGENCE) && pin_word(h, PIN_BAD_STEP) != ~0ULL)
+            return bad_column(h, pin_word(h, PIN_BAD_STEP));
+        return s;
     }
     return solve_core(h, Ud, ldd, U, ld, on_device, nrhs, st, info);
 }

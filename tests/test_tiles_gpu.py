@@ -155,3 +155,19 @@ def test_narrow_solve_edges(wdlib, cuda, prec, nrhs):
         B = rhs(cp.size - 1, nrhs, seed=nrhs)
         s = wdlib.Solver(relax_k=0, relax_pct=0).analyze(cp, ri, basis).factor(v, prec)
         assert oracle.backward_error(cp, ri, v, s.solve(B), B).max() <= 1e-12
+
+
+@pytest.mark.parametrize("ncols", [1, 3, 8, 9, 12, 32, 33, 64, 66, 130])
+def test_residual_chunks(wdlib, cuda, ncols):
+    """The residual products' rows and rows cut into chunks, through the
+    backward error of a given X.  The residual's
+    double-float arithmetic (about 48 bits) leaves the estimate within 5e-15
+    of the FP64 one."""
+    for dim, J in ((2, 5), (1, 9), (2, 2)):
+        b, cp, ri, v, o = _case(dim, J)
+        s = wdlib.Solver().analyze(cp, ri, b).factor(v, "fp64")
+        rng = np.random.default_rng(ncols)
+        B = rhs(o.n, ncols, seed=ncols)
+        X = o.solve(B) * (1.0 + 1e-7 * rng.standard_normal(B.shape))
+        ref = oracle.backward_error(cp, ri, v, X, B).max()
+        assert abs(s.backward_error(X, B) - ref) <= 5e-15 + 1e-9 * ref
