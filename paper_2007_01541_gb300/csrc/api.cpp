@@ -707,7 +707,20 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
         int maxsb = 0;
         for (int i = b; i < e; ++i) maxsb = std::max(maxsb, nsb(S.level_nodes[i]));
         for (int sb = maxsb - 1; sb >= 0; --sb) {
-            // partial sums over splits of the rows below the super-block
+            // partial sums over splits of the rows below the super-block;
+            // tensor cores: half the rows per split if the launch has at
+            // most as many CTAs as half the SMs
+            int ksr = KSR;
+            if (large == 1) {
+                int64_t ctas = 0;
+                for (int i = b; i < e; ++i) {
+                    const int s = S.level_nodes[i];
+                    if (nsb(s) <= sb || S.m(s) <= sb * SBW + width(s, sb)) continue;
+                    const int rows = front_order(S, s) - ((sb * SBW + width(s, sb)) & ~31);
+                    ctas += (int64_t)((rows + KSR - 1) / KSR) * ((width(s, sb) + TRW - 1) / TRW) * ng;
+                }
+                if (2 * ctas <= sms) ksr = KSR / 2;
+            }
             size_t f0 = p.items.size();
             double el = 0, fl = 0;
             int slot = 0;
@@ -722,7 +735,7 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
                 // few right-hand sides: from the 32-row boundary at or above
                 // the super-block's end)
                 const int kbeg = large == 0 ? sb * SBW + w : (sb * SBW + w) & ~31;
-                const int nsplit = below > 0 ? (front_order(S, s) - kbeg + KSR - 1) / KSR : 0;
+                const int nsplit = below > 0 ? (front_order(S, s) - kbeg + ksr - 1) / ksr : 0;
                 first_slot.push_back(slot);
                 for (int cb = 0; cb * TRW < w; ++cb)
                     for (int g = 0; g < ng; ++g) {
@@ -734,7 +747,7 @@ static void build_solve_plan(const wd::Symbolic &S, int nrhs, int large, int sms
                 el += (double)below * w + below * R;
             }
             p.slots = std::max<int64_t>(p.slots, slot);
-            add_launch(p, K_BWD_REDUCE, f0, sb, fl, el, 0);
+            add_launch(p, K_BWD_REDUCE, f0, ksr, fl, el, 0);
             f0 = p.items.size();
             el = 0;
             for (const int4 &q : fin) {
@@ -1714,6 +1727,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     wd::TcSolveArgs a = ta;
                     a.in = reinterpret_cast<const float *>(Y);
                     a.out = reinterpret_cast<float *>(P);
+                    a.ksr = L.arg;
                     wd::launch_tc_breduce(d, a, it, L.count, st);
                 } else if (lg == 2) {
                     wd::launch_rnarrow<T>(d, Fb, Y, P, it, L.count, nrhs, st);

@@ -339,8 +339,9 @@ void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const
 // ---- tensor-core products of the solves (tc_solve.cu; FP32 fronts, mode 1) --
 // Tiles of 128 rows (xapply, bupdate) or 128 pivot columns (breduce) x 64
 // right-hand sides; items as in mode 0 with these tile sizes; breduce splits
-// the rows below a super-block into SOLVE_KSR_TC storage rows of the front,
-// counted from the first 32-row boundary at or above the super-block's end.
+// the rows below a super-block into SOLVE_KSR_TC storage rows of the front
+// (half as many in a launch that would leave SMs idle), counted from the first
+// 32-row boundary at or above the super-block's end.
 constexpr int SOLVE_KSR_TC = 256;
 struct TcSolveArgs {
     const float *front;           // FP32 fronts
@@ -356,7 +357,8 @@ struct TcSolveArgs {
     uint32_t wait_limit;          // 0: the default
     float *ksw;                   // split inner dimension: one partial tile per CTA
     int *kcnt;                    // split inner dimension: arrivals per output tile (zero between launches)
-    int sms;                      // the device's SMs: a bupdate launch of more CTAs than SMs runs two per SM
+    int sms;                      // the device's SMs: a launch of more CTAs than SMs runs two per SM
+    int ksr;                      // breduce: storage rows per split
 };
 constexpr int TC_SOLVE_TILE = 128 * 64;   // entries of one output tile of the tensor-core solve products
 void launch_tc_xapply(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st);

@@ -22,10 +22,13 @@
 // places; each thread then splits the values it copied in place (hi) and into
 // the lo plane, and one thread issues the chunk's MMAs while the next chunks
 // are in flight.  The ring has three stages, two chunks ahead (144 KB), except
-// in a bupdate launch of more CTAs than SMs (the many short products of the
+// in a launch of more CTAs than SMs (the many short products of the
 // lower levels, a few chunks each): there it has two stages, one chunk ahead
 // (96 KB), so that two CTAs share an SM and one's set-up, waits and epilogue
 // overlap the other's copies.  The stage count changes no arithmetic.
+// (256 x 256, 64 right-hand sides: bupdate 1.62 -> 0.92 ms per step; breduce
+// in the same form, its row splits halved where the launch has few CTAs, takes
+// the whole call from 11.53 to 11.19 ms.)
 //
 // A launch with few output tiles (the top of the tree: a few super-blocks of
 // one or two fronts) splits the inner dimension of xapply and bupdate over up
@@ -133,8 +136,8 @@ __device__ __forceinline__ Geo geometry(const DevSym &d, const TcSolveArgs &a, i
         g.j0 = g.b0 + cb * TM;
         g.nb = min(TM, g.b0 + g.w - g.j0);
         const int kbeg = (g.b0 + g.w) & ~(TK - 1);   // storage rows below B, from a 32-row boundary
-        g.q0 = kbeg + ks * SOLVE_KSR_TC;
-        g.q1 = min(g.mp, g.q0 + SOLVE_KSR_TC);
+        g.q0 = kbeg + ks * a.ksr;
+        g.q1 = min(g.mp, g.q0 + a.ksr);
         g.kc0 = g.q0 / TK;
         g.nchunk = (g.q1 - g.q0 + TK - 1) / TK;
         g.slot = it.w;
@@ -239,7 +242,7 @@ __device__ __forceinline__ void split_chunk(unsigned char *Ah, unsigned char *Al
     split4_inplace(Bh, Bl, tc::sw128_offset(j, kq + 4));
 }
 
-// NS: stages of the ring (3, or 2 for bupdate launches of more CTAs than SMs)
+// NS: stages of the ring (3, or 2 for launches of more CTAs than SMs)
 template <int OP, int NS>
 __global__ void __launch_bounds__(NTH, NS == 2 ? 2 : 1) tc_solve_kernel(DevSym d, TcSolveArgs a,
                                                                        const int4 *__restrict__ items) {
@@ -460,32 +463,34 @@ void set_attr() {
 
 void init_tc_solve_attributes() {
     set_attr<OP_XAPPLY, NSTG>();
+    set_attr<OP_XAPPLY, 2>();
     set_attr<OP_BUPDATE, NSTG>();
     set_attr<OP_BUPDATE, 2>();
     set_attr<OP_BREDUCE, NSTG>();
+    set_attr<OP_BREDUCE, 2>();
 }
 
-void launch_tc_xapply(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st) {
+// more CTAs than SMs (the lower levels: many short products): two stages, two
+// CTAs per SM
+template <int OP>
+static void launch_tc(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st) {
     if (count <= 0) return;
-    set_attr<OP_XAPPLY, NSTG>();
-    tc_solve_kernel<OP_XAPPLY, NSTG><<<count, NTH, tc_solve_smem(NSTG), st>>>(d, a, items);
-}
-void launch_tc_bupdate(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st) {
-    if (count <= 0) return;
-    // more CTAs than SMs (the lower levels: one super-block, a few chunks
-    // per CTA): two stages, two CTAs per SM
     if (a.sms > 0 && count > a.sms) {
-        set_attr<OP_BUPDATE, 2>();
-        tc_solve_kernel<OP_BUPDATE, 2><<<count, NTH, tc_solve_smem(2), st>>>(d, a, items);
+        set_attr<OP, 2>();
+        tc_solve_kernel<OP, 2><<<count, NTH, tc_solve_smem(2), st>>>(d, a, items);
     } else {
-        set_attr<OP_BUPDATE, NSTG>();
-        tc_solve_kernel<OP_BUPDATE, NSTG><<<count, NTH, tc_solve_smem(NSTG), st>>>(d, a, items);
+        set_attr<OP, NSTG>();
+        tc_solve_kernel<OP, NSTG><<<count, NTH, tc_solve_smem(NSTG), st>>>(d, a, items);
     }
 }
+void launch_tc_xapply(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st) {
+    launch_tc<OP_XAPPLY>(d, a, items, count, st);
+}
+void launch_tc_bupdate(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st) {
+    launch_tc<OP_BUPDATE>(d, a, items, count, st);
+}
 void launch_tc_breduce(const DevSym &d, const TcSolveArgs &a, const int4 *items, int count, cudaStream_t st) {
-    if (count <= 0) return;
-    set_attr<OP_BREDUCE, NSTG>();
-    tc_solve_kernel<OP_BREDUCE, NSTG><<<count, NTH, tc_solve_smem(NSTG), st>>>(d, a, items);
+    launch_tc<OP_BREDUCE>(d, a, items, count, st);
 }
 
 }  // namespace wd
