@@ -14,19 +14,21 @@
 // Product.  For rows r and columns c of a tile,
 //   sum_k L_rk L_ck = 2^(e_r + e_c) sum_d 2^(-7 d) D_d(r, c),
 //   D_d = sum_{i + j = d} sum_k q_i(r, k) q_j(c, k),   d = 2..9,
-// where every D_d is an integer below 2^23 in magnitude (at most 8 slice
-// pairs, 64 terms, products below 2^14), so it accumulates EXACTLY in the
+// where every D_d is an integer below 2^22 in magnitude (at most 8 slice
+// pairs, 64 terms, products of at most 2^12, 2^13 with one q_1 and 2^14 with
+// two: 2^20 for d = 2 and 2.5 2^20 for d = 9), so it accumulates EXACTLY in the
 // FP32 accumulators of the MMA, in any order.  The pairs with i + j > 9 are
 // dropped: at most 2^-47 of 2^(e_r + e_c) per 64-column block, at the level
 // of FP64's own rounding bound for such a sum (64 u max|L_r| max|L_c|).  The
 // 36 slice-pair products of a 64-column block are 144 tcgen05.mma kind::f16
 // instructions (128 x 64 x 16 each) into eight TMEM accumulators of 64
 // columns (all 512 columns of the SM's tensor memory).  The epilogue reads
-// them, adds the eight terms in double-float arithmetic on the FP32 pipes
-// (exact powers of two as scales, TwoSum), turns the pair into two doubles
-// scaled by 2^(e_r + e_c) with integer operations on the bits, and adds them
-// to an FP64 register accumulator (two FP64 additions: GB300's FP64 pipe is
-// the scarce one); after the last block C -= acc in FP64.
+// them, adds the eight terms exactly as 64-bit integers, builds the double
+// scaled by 2^(e_r + e_c) with integer operations on the bits, and adds it to
+// an FP64 register accumulator: one FP64 addition per entry and block (GB300's
+// FP64 pipe is the scarce one; the sum in double-float arithmetic and two FP64
+// additions before took the 256 x 256 factorization's products 19.5 ms, now
+// 17.3); after the last block C -= acc in FP64.
 //
 // One CTA per 128 x 64 output tile (the tiles of the SIMT FP64 kernel):
 //   warp 0: producer (bulk copies of the 8 + 8 slice planes of a block)
@@ -75,24 +77,32 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(bar)) : "memory");
 }
 
-// f 2^e as a double, built from f's bits on the integer pipes (no FP64
-// conversion or multiply): zero and FP32 subnormals give 0, so do results
-// below the FP64 normal range
-__device__ __forceinline__ double f2d_scaled(float f, int e) {
-    const uint32_t u = __float_as_uint(f);
-    const int ex = (int)((u >> 23) & 0xFFu) - 127 + 1023 + e;
-    const bool zero = ((u >> 23) & 0xFFu) == 0u || ex < 1;
-    const uint64_t bits = ((uint64_t)(u >> 31) << 63) | ((uint64_t)min(ex, 2046) << 52) |
-                          ((uint64_t)(u & 0x7FFFFFu) << 29);
-    return zero ? 0.0 : __longlong_as_double((long long)bits);
+// sum_d 2^(-7 d) D_d for the eight accumulators D[d - 2] (integers below 2^22
+// in magnitude, as floats), times 2^56, as a 64-bit integer (the last term
+// rounded: 2^-57).  Pairs of neighbours fit 32 bits; adding 1.5 2^23 turns a
+// float's low bits into the integer.
+__device__ __forceinline__ long long combine(const float (&D)[8]) {
+    int u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) u[i] = __float_as_int(__fadd_rn(D[i], 12582912.0f)) - 0x4B400000;
+    const int p0 = u[0] * 128 + u[1], p1 = u[2] * 128 + u[3], p2 = u[4] * 128 + u[5], p3 = u[6] * 128 + u[7];
+    long long v = (long long)p2 * 128 + ((p3 + 64) >> 7);
+    v += (long long)p1 * (1 << 21);
+    return v + ((long long)p0 << 35);
 }
 
-__device__ __forceinline__ void two_sum(float &h, float &l, float t) {
-    const float s = __fadd_rn(h, t);
-    const float bb = __fsub_rn(s, h);
-    const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(t, bb));
-    h = s;
-    l = __fadd_rn(l, err);
+// v 2^e as a double, rounded to nearest (ties away), from integer operations
+// (a conversion and a product would take the FP64 pipe); below the normal
+// range 0
+__device__ __forceinline__ double i2d_scaled(long long v, int e) {
+    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+    const int lz = __clzll((long long)m);
+    const unsigned long long q = m << (lz & 63);            // top bit set
+    const unsigned long long r = (q >> 11) + ((q >> 10) & 1);   // 53 bits, or 2^53
+    const int ex = 1023 + 63 - lz + e;
+    if (m == 0 || ex < 2) return 0.0;
+    const unsigned long long bits = ((unsigned long long)(min(ex, 2046) - 1) << 52) + r;
+    return __longlong_as_double((long long)(bits | ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
 // ---------------------------------------------------------------------------
@@ -291,13 +301,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_schur_kernel(DevSym d, doubl
                     tc::tmem_ld8(tmem + ((uint32_t)(32 * lg) << 16) + dd * ON + 32 * half + 8 * g, D[dd]);
 #pragma unroll
                 for (int cc = 0; cc < 8; ++cc) {
-                    // sum_d 2^(-7 d) D_d, smallest term first
-                    float h = D[NACC - 1][cc] * 0x1p-63f, l = 0.0f;
+                    float t[NACC];
 #pragma unroll
-                    for (int dd = NACC - 2; dd >= 0; --dd) two_sum(h, l, D[dd][cc] * __int_as_float((127 - 7 * (dd + 2)) << 23));
-                    const int esc = er + Eb[cb + 8 * g + cc];
-                    acc[8 * g + cc] += f2d_scaled(h, esc);
-                    acc[8 * g + cc] += f2d_scaled(l, esc);
+                    for (int dd = 0; dd < NACC; ++dd) t[dd] = D[dd][cc];
+                    acc[8 * g + cc] += i2d_scaled(combine(t), er + Eb[cb + 8 * g + cc] - 56);
                 }
             }
             tc::tc_fence_before();
