@@ -30,6 +30,30 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
 
+// Programmatic dependent launch: a kernel started with launch_dependent (on a
+// stream or into a captured graph) may begin while the one before it still
+// runs, once all CTAs of that one have called allow_dependents or ended; it
+// sees that kernel's (and so every earlier one's) results only after
+// wait_prerequisites, which every thread calls before it reads or writes
+// anything that an earlier kernel of the chain writes or reads.
+__device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+template <class... P, class... A>
+inline void launch_dependent(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st,
+                             A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // |x| as a key that orders like the value; NaN counts as 0 (fmax ignores it)
 __device__ __forceinline__ unsigned long long abs_key(double x) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;

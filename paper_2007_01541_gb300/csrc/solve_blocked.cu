@@ -378,6 +378,10 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // L once per direction, would take a tenth of the time).  So
 //   * a CTA covers 32 rows and all its columns (or 64 columns and 256 rows) with
 //     16-byte loads, up to sixteen of them in flight per lane, most often all;
+//   * the kernels of launches that are not large (NARROW_DEEP) are launched
+//     dependent on one another programmatically: while one finishes, the next
+//     one's CTAs start, read their items and sizes and load their part of L or
+//     X, which no solve writes, and only then wait;
 //   * the forward gather of the children's update vectors is part of the two
 //     kernels that use it (xnarrow for the super-block's own rows, repeated by
 //     its CTAs, bnarrow for the rows it writes), and the backward sum of the
@@ -388,8 +392,20 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // Against one 4-byte load per lane and column, four in flight, and launches of
 // their own for the gather and the sum: 256 x 256, one right-hand side against
 // a kept factor 2.30 -> 1.67 ms; 128 x 128, a theta step 0.84 -> 0.68 ms.
+// Dependent launches and the deep and shallow forms: 1.57 -> 1.05 ms, 0.655 ->
+// 0.490 ms, the batch of 64 instances 12.47 -> 11.72.
 // ---------------------------------------------------------------------------
 constexpr int NRW = 32;
+// DEEP launches, at most NARROW_DEEP CTAs (four per SM): sixteen loads in flight
+// per lane, the first of them before the wait.  Larger launches (the lower
+// levels of large trees and of batches) have other CTAs to overlap with: four
+// loads (eight in the reduction), two to four CTAs per SM, ordinary launches.
+// All launches deep / up to 2,432 CTAs / up to 608: 256 x 256, one right-hand
+// side 1.17 / 1.08 / 1.05 ms; 16 theta steps at 128 x 128 8.01 / 7.92 / 7.85;
+// batch of 64 instances 12.87 / 11.83 / 11.72.  The arithmetic is the same.
+constexpr int NARROW_DEEP = 608;
+template <bool DEEP, int NR>
+constexpr int narrow_ctas() { return DEEP ? 1 : (NR <= 2 ? 4 : NR == 4 ? 3 : 2); }
 constexpr int NWARP = THREADS / 32;
 constexpr int NARROW_COLS = 64, NARROW_RHS = 8;   // partial-sum tile of the backward reduction
 constexpr int NKSR = SOLVE_KSR_NARROW;             // rows per split of the backward reduction
@@ -448,55 +464,72 @@ __device__ __forceinline__ void add_children(const DevSym &d, int s, const T *__
 
 // The product of rows [0, 32) at A (row offset included; column-major, lda,
 // 16-byte aligned, all 32 rows readable) and columns [pa, pb) with V[p * NR +
-// c]: the sum of row tid % 32 and right-hand side tid / 32 for tid < 32 NR.
-// red: NWARP * 32 * NR.  Called by all threads after V is visible.
-template <class T, int NR>
-__device__ __forceinline__ T narrow_product(const T *__restrict__ A, int64_t lda, const T *V, int pa, int pb, T *red) {
+// c].  load: the first U columns' loads of each lane (before the CTA waits for
+// its predecessors: the matrix is not theirs); finish: the rest and the sum of
+// row tid % 32 and right-hand side tid / 32 for tid < 32 NR, called by all
+// threads after V is visible.  red: NWARP * 32 * NR.
+template <class T, int NR, int U>
+struct NarrowProduct {
     using VT = typename Vec16<T>::type;
-    constexpr int VR = 16 / sizeof(T), LR = NRW / VR, CPW = 32 / LR;   // rows per lane, lanes per column, columns per load
-    constexpr int U = 16;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane % LR, lc = lane / LR;
-    T acc[VR][NR];
+    static constexpr int VR = 16 / sizeof(T), LR = NRW / VR, CPW = 32 / LR;   // rows per lane, lanes per column, columns per load
+    static constexpr int STEP = NWARP * CPW;
+    VT x[U];
+    const T *a;
+    int64_t lda;
+    int p0, pb;
+
+    __device__ __forceinline__ void fetch() {
 #pragma unroll
-    for (int i = 0; i < VR; ++i)
+        for (int u = 0; u < U; ++u)
+            if (p0 + u * STEP < pb) x[u] = *reinterpret_cast<const VT *>(a + (int64_t)(p0 + u * STEP) * lda);
+    }
+    __device__ __forceinline__ void load(const T *A, int64_t lda_, int pa, int pb_) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        a = A + VR * (lane % LR);
+        lda = lda_;
+        p0 = pa + warp * CPW + lane / LR;
+        pb = pb_;
+        fetch();
+    }
+    __device__ __forceinline__ T finish(const T *V, T *red) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane % LR, lc = lane / LR;
+        T acc[VR][NR];
 #pragma unroll
-        for (int c = 0; c < NR; ++c) acc[i][c] = T(0);
-    const T *a = A + VR * lr;
-    for (int p0 = pa + warp * CPW + lc; p0 < pb; p0 += U * NWARP * CPW) {
-        VT x[U];
+        for (int i = 0; i < VR; ++i)
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int p = p0 + u * NWARP * CPW;
-            if (p < pb) x[u] = *reinterpret_cast<const VT *>(a + (int64_t)p * lda);
-        }
+            for (int c = 0; c < NR; ++c) acc[i][c] = T(0);
+        while (p0 < pb) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int p = p0 + u * NWARP * CPW;
-            if (p < pb) {
-                const T *e = reinterpret_cast<const T *>(&x[u]);
+            for (int u = 0; u < U; ++u) {
+                const int p = p0 + u * STEP;
+                if (p < pb) {
+                    const T *e = reinterpret_cast<const T *>(&x[u]);
 #pragma unroll
-                for (int c = 0; c < NR; ++c) {
-                    const T v = V[p * NR + c];
+                    for (int c = 0; c < NR; ++c) {
+                        const T v = V[p * NR + c];
 #pragma unroll
-                    for (int i = 0; i < VR; ++i) acc[i][c] += e[i] * v;
+                        for (int i = 0; i < VR; ++i) acc[i][c] += e[i] * v;
+                    }
                 }
             }
+            p0 += U * STEP;
+            fetch();
         }
+#pragma unroll
+        for (int i = 0; i < VR; ++i)
+#pragma unroll
+            for (int c = 0; c < NR; ++c) {
+#pragma unroll
+                for (int o = LR; o < 32; o *= 2) acc[i][c] += __shfl_xor_sync(0xffffffffu, acc[i][c], o);
+                if (lc == 0) red[(warp * NR + c) * NRW + VR * lr + i] = acc[i][c];
+            }
+        __syncthreads();
+        T sum = T(0);
+        if (threadIdx.x < NRW * NR)
+            for (int g = 0; g < NWARP; ++g) sum += red[g * NR * NRW + threadIdx.x];
+        return sum;
     }
-#pragma unroll
-    for (int i = 0; i < VR; ++i)
-#pragma unroll
-        for (int c = 0; c < NR; ++c) {
-#pragma unroll
-            for (int o = LR; o < 32; o *= 2) acc[i][c] += __shfl_xor_sync(0xffffffffu, acc[i][c], o);
-            if (lc == 0) red[(warp * NR + c) * NRW + VR * lr + i] = acc[i][c];
-        }
-    __syncthreads();
-    T sum = T(0);
-    if (threadIdx.x < NRW * NR)
-        for (int g = 0; g < NWARP; ++g) sum += red[g * NR * NRW + threadIdx.x];
-    return sum;
-}
+};
 
 // first storage row and number of splits of the reduction below super-block sb
 __device__ __forceinline__ int narrow_first_row(int b0, int w) { return (b0 + w) & ~31; }
@@ -508,8 +541,8 @@ __device__ __forceinline__ int narrow_splits(int b0, int w, int m, int mp) {
 // right-hand side, from Y into Tt.  else: x_B = X_B^T t_B (xp: the stored
 // transposes), t_B = y_B - the splits' partial sums, from Tt into Y; 32 rows
 // per CTA.  item = (s, sb, row block, backward: first slot)
-template <class T, int NR, bool FWD>
-__global__ void __launch_bounds__(THREADS) xnarrow_kernel(DevSym d, const T *__restrict__ xp,
+template <class T, int NR, bool DEEP, bool FWD>
+__global__ void __launch_bounds__(THREADS, narrow_ctas<DEEP, NR>()) xnarrow_kernel(DevSym d, const T *__restrict__ xp,
                                                           const int64_t *__restrict__ xsoff, T *Y, T *Tt,
                                                           const T *__restrict__ W, const T *__restrict__ P,
                                                           const int4 *__restrict__ items, int nrhs) {
@@ -526,6 +559,10 @@ __global__ void __launch_bounds__(THREADS) xnarrow_kernel(DevSym d, const T *__r
     const T *in = FWD ? Y : Tt;
     T *out = FWD ? Tt : Y;
     const int m = d.sm[s], nsplit = FWD ? 0 : narrow_splits(b0, w, m, d.skp[s] + m - k);
+    NarrowProduct<T, NR, DEEP ? 16 : 4> prod;
+    prod.load(xp + xsoff[s] + (int64_t)sb * SB * SB + r0, wp, pa, pb);
+    allow_dependents();
+    wait_prerequisites();
     for (int p0 = pa; p0 < pb; p0 += THREADS) {
         const int p = p0 + threadIdx.x;
         const bool ok = p < pb;
@@ -552,7 +589,7 @@ __global__ void __launch_bounds__(THREADS) xnarrow_kernel(DevSym d, const T *__r
         }
     }
     __syncthreads();
-    const T sum = narrow_product<T, NR>(xp + xsoff[s] + (int64_t)sb * SB * SB + r0, wp, V, pa, pb, red);
+    const T sum = prod.finish(V, red);
     const int r = r0 + threadIdx.x % NRW, c = threadIdx.x / NRW;
     if (threadIdx.x < NRW * NR && r < w && c < nrhs) out[row0 + r + (int64_t)c * n] = sum;
 }
@@ -561,8 +598,8 @@ __global__ void __launch_bounds__(THREADS) xnarrow_kernel(DevSym d, const T *__r
 // CTA; for the first super-block the pending values are b (pivot rows) plus
 // the children's.  item = (s, sb, rb, 65536 * seg): seg 0 = pivot rows after B
 // (in Y), seg 1 = rows of R (the update vector W_s)
-template <class T, int NR>
-__global__ void __launch_bounds__(THREADS) bnarrow_kernel(DevSym d, const T *__restrict__ front, T *Y,
+template <class T, int NR, bool DEEP>
+__global__ void __launch_bounds__(THREADS, narrow_ctas<DEEP, NR>()) bnarrow_kernel(DevSym d, const T *__restrict__ front, T *Y,
                                                           const T *__restrict__ Tt, T *W,
                                                           const int4 *__restrict__ items, int nrhs) {
     __shared__ T V[SB * NR];
@@ -578,6 +615,10 @@ __global__ void __launch_bounds__(THREADS) bnarrow_kernel(DevSym d, const T *__r
     const int nrow = seg == 0 ? k - i0 : (m - k) - i0;
     T *dst = seg == 0 ? Y + f + i0 : W + d.woff[s] * nrhs + i0;
     const int64_t ldd = seg == 0 ? n : m - k;
+    NarrowProduct<T, NR, DEEP ? 16 : 4> prod;
+    prod.load(front + d.foff[s] + (int64_t)b0 * ld + (seg == 0 ? i0 : kp + i0), ld, 0, w);
+    allow_dependents();
+    wait_prerequisites();
     for (int idx = threadIdx.x; idx < w * NR; idx += THREADS) {
         const int p = idx / NR, c = idx % NR;
         V[idx] = c < nrhs ? Tt[f + b0 + p + (int64_t)c * n] : T(0);
@@ -591,8 +632,7 @@ __global__ void __launch_bounds__(THREADS) bnarrow_kernel(DevSym d, const T *__r
     if (sb == 0)
         add_children<T, NR>(d, s, W, nrhs, ch, (seg == 0 ? i0 : k + i0) + (int)threadIdx.x, own, t);
     __syncthreads();
-    const T sum = narrow_product<T, NR>(front + d.foff[s] + (int64_t)b0 * ld + (seg == 0 ? i0 : kp + i0), ld, V, 0, w,
-                                        red);
+    const T sum = prod.finish(V, red);
     // the sums, (row, right-hand side) over threads, to the pending values' lanes
     __syncthreads();
     if (threadIdx.x < NRW * NR) red[threadIdx.x] = sum;
@@ -609,13 +649,13 @@ __global__ void __launch_bounds__(THREADS) bnarrow_kernel(DevSym d, const T *__r
 // block's end, for the 64 columns b0 + 64 cb ...: 8 columns per warp, lanes
 // over rows (x zero at rows that do not count); P[slot] ([rhs][column]).
 // item = (s, sb * 16 + cb, 65536 * ks, slot)
-template <class T, int NR>
-__global__ void __launch_bounds__(THREADS) rnarrow_kernel(DevSym d, const T *__restrict__ front,
+template <class T, int NR, bool DEEP>
+__global__ void __launch_bounds__(THREADS, narrow_ctas<DEEP, NR>()) rnarrow_kernel(DevSym d, const T *__restrict__ front,
                                                           const T *__restrict__ Y, T *__restrict__ P,
                                                           const int4 *__restrict__ items, int nrhs) {
     using VT = typename Vec16<T>::type;
     constexpr int VR = 16 / sizeof(T), H = NKSR / (32 * VR);   // vectors of a lane per column
-    constexpr int CG = 16 / H;                                 // columns whose loads are in flight together
+    constexpr int CG = (DEEP ? 16 : 8) / H;                    // columns whose loads are in flight together
     __shared__ T xs[NKSR * NR];
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y >> 4, cb = it.y & 15, ks = it.z >> 16;
@@ -625,19 +665,11 @@ __global__ void __launch_bounds__(THREADS) rnarrow_kernel(DevSym d, const T *__r
     const int64_t n = d.n;
     const int32_t *rows = d.rows + d.rowptr[s];
     const int q0 = narrow_first_row(b0, w) + ks * NKSR;
-    for (int idx = threadIdx.x; idx < NKSR; idx += THREADS) {
-        const int q = q0 + idx;
-        const bool ok = q >= b0 + w && q < mp && (q < k || q >= kp);
-        const int64_t g = ok ? rows[q < k ? q : q - (kp - k)] : 0;
-#pragma unroll
-        for (int c = 0; c < NR; ++c) xs[c * NKSR + idx] = ok && c < nrhs ? Y[g + (int64_t)c * n] : T(0);
-    }
-    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T *F = front + d.foff[s] + (int64_t)j0 * ld;
     constexpr int CW = NARROW_COLS / NWARP;
-    for (int c0 = 0; c0 < CW; c0 += CG) {
-        VT x[CG][H];
+    VT x[CG][H];
+    auto fetch = [&](int c0) {
 #pragma unroll
         for (int u = 0; u < CG; ++u)
 #pragma unroll
@@ -646,6 +678,20 @@ __global__ void __launch_bounds__(THREADS) rnarrow_kernel(DevSym d, const T *__r
                 // q < mp: the 16 bytes lie inside the column (ld is a multiple of 32)
                 if (c0 + u < CW && cl < nb && q < mp) x[u][h] = *reinterpret_cast<const VT *>(F + (int64_t)cl * ld + q);
             }
+    };
+    fetch(0);
+    allow_dependents();
+    wait_prerequisites();
+    for (int idx = threadIdx.x; idx < NKSR; idx += THREADS) {
+        const int q = q0 + idx;
+        const bool ok = q >= b0 + w && q < mp && (q < k || q >= kp);
+        const int64_t g = ok ? rows[q < k ? q : q - (kp - k)] : 0;
+#pragma unroll
+        for (int c = 0; c < NR; ++c) xs[c * NKSR + idx] = ok && c < nrhs ? Y[g + (int64_t)c * n] : T(0);
+    }
+    __syncthreads();
+    for (int c0 = 0; c0 < CW; c0 += CG) {
+        if (c0 > 0) fetch(c0);
 #pragma unroll
         for (int u = 0; u < CG; ++u) {
             const int cl = warp * CW + c0 + u;
@@ -741,38 +787,50 @@ void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const
     else finish_go<T, t32::TT, t32::TT>(d, Y, Tt, P, items, count, nrhs, st);
 }
 
-// f<NR>() for nrhs <= 8
+template <class... P, class... A>
+static void launch_narrow(void (*kernel)(P...), int count, bool deep, cudaStream_t st, A... args) {
+    if (deep) launch_dependent(kernel, count, THREADS, 0, st, args...);
+    else kernel<<<count, THREADS, 0, st>>>(args...);
+}
+// f<NR, DEEP>() for nrhs <= 8
 template <class F>
-static void by_width(int nrhs, F f) {
-    if (nrhs == 1) f(std::integral_constant<int, 1>());
-    else if (nrhs == 2) f(std::integral_constant<int, 2>());
-    else if (nrhs <= 4) f(std::integral_constant<int, 4>());
-    else f(std::integral_constant<int, 8>());
+static void by_width(int nrhs, int count, F f) {
+    auto nr = [&](auto deep) {
+        if (nrhs == 1) f(std::integral_constant<int, 1>(), deep);
+        else if (nrhs == 2) f(std::integral_constant<int, 2>(), deep);
+        else if (nrhs <= 4) f(std::integral_constant<int, 4>(), deep);
+        else f(std::integral_constant<int, 8>(), deep);
+    };
+    if (count <= NARROW_DEEP) nr(std::true_type());
+    else nr(std::false_type());
 }
 template <class T>
 void launch_xnarrow(const DevSym &d, const T *xp, const int64_t *xsoff, T *Y, T *Tt, const T *W, const T *P,
                     const int4 *items, int count, bool forward, int nrhs, cudaStream_t st) {
     if (count <= 0) return;
-    by_width(nrhs, [&](auto nr) {
+    by_width(nrhs, count, [&](auto nr, auto deep) {
         if (forward)
-            xnarrow_kernel<T, nr.value, true><<<count, THREADS, 0, st>>>(d, xp, xsoff, Y, Tt, W, P, items, nrhs);
-        else xnarrow_kernel<T, nr.value, false><<<count, THREADS, 0, st>>>(d, xp, xsoff, Y, Tt, W, P, items, nrhs);
+            launch_narrow(xnarrow_kernel<T, nr.value, deep.value, true>, count, deep.value, st, d, xp, xsoff, Y, Tt, W, P,
+                          items, nrhs);
+        else
+            launch_narrow(xnarrow_kernel<T, nr.value, deep.value, false>, count, deep.value, st, d, xp, xsoff, Y, Tt, W,
+                          P, items, nrhs);
     });
 }
 template <class T>
 void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, const int4 *items, int count, int nrhs,
                     cudaStream_t st) {
     if (count <= 0) return;
-    by_width(nrhs, [&](auto nr) {
-        bnarrow_kernel<T, nr.value><<<count, THREADS, 0, st>>>(d, front, Y, Tt, W, items, nrhs);
+    by_width(nrhs, count, [&](auto nr, auto deep) {
+        launch_narrow(bnarrow_kernel<T, nr.value, deep.value>, count, deep.value, st, d, front, Y, Tt, W, items, nrhs);
     });
 }
 template <class T>
 void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
                     cudaStream_t st) {
     if (count <= 0) return;
-    by_width(nrhs, [&](auto nr) {
-        rnarrow_kernel<T, nr.value><<<count, THREADS, 0, st>>>(d, front, Y, P, items, nrhs);
+    by_width(nrhs, count, [&](auto nr, auto deep) {
+        launch_narrow(rnarrow_kernel<T, nr.value, deep.value>, count, deep.value, st, d, front, Y, P, items, nrhs);
     });
 }
 

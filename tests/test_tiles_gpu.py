@@ -171,3 +171,20 @@ def test_residual_chunks(wdlib, cuda, ncols):
         X = o.solve(B) * (1.0 + 1e-7 * rng.standard_normal(B.shape))
         ref = oracle.backward_error(cp, ri, v, X, B).max()
         assert abs(s.backward_error(X, B) - ref) <= 5e-15 + 1e-9 * ref
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("nrhs", [1, 2, 4, 8])
+def test_narrow_solve_large_launches(wdlib, cuda, prec, nrhs):
+    """Enough fronts in one level that its launches take the shallow form: a
+    forest of 700 small dense blocks, each column solved as alone."""
+    rng = np.random.default_rng(nrhs)
+    k, cnt = 5, 700
+    M = rng.standard_normal((cnt, k, k))
+    A = M @ M.transpose(0, 2, 1) + k * np.eye(k)
+    cp = np.concatenate([[0], np.cumsum(np.tile(np.arange(k, 0, -1), cnt))]).astype(np.int64)
+    ri = np.concatenate([np.arange(c * k + j, (c + 1) * k) for c in range(cnt) for j in range(k)]).astype(np.int32)
+    v = np.concatenate([A[c, j:, j] for c in range(cnt) for j in range(k)])
+    B = rhs(cnt * k, nrhs, seed=nrhs)
+    s = wdlib.Solver(relax_k=0, relax_pct=0).analyze(cp, ri).factor(v, prec)
+    assert oracle.backward_error(cp, ri, v, s.solve(B), B).max() <= 1e-12
