@@ -139,6 +139,8 @@ __global__ void __launch_bounds__(THREADS) bfwd_gather_kernel(DevSym d, const T 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = it.y * 32 + lane;
     const int m = d.sm[s], k = d.sk[s];
+    allow_dependents();
+    wait_prerequisites();
     if (r >= m) return;
     const int64_t n = d.n;
     const int f = d.sfirst[s];
@@ -364,6 +366,8 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
     const int f = d.sfirst[s];
     const int idx = (blockIdx.x % PER) * THREADS + threadIdx.x;
     const int cl = idx % ROWS, c = idx / ROWS;
+    allow_dependents();
+    wait_prerequisites();
     if (cl >= nb || c >= nc) return;
     T sum = T(0);
     for (int q = 0; q < nsplit; ++q) sum += P[((int64_t)(it.w + q) * RHS + c) * ROWS + cl];
@@ -751,14 +755,14 @@ template <class T>
 void launch_bfwd_gather(const DevSym &d, const T *Y, T *Tt, T *W, const int4 *items, int count, int rgt,
                         int nrhs, cudaStream_t st) {
     if (count <= 0) return;
-    if (rgt == 64) bfwd_gather_kernel<T, 64><<<count, THREADS, 0, st>>>(d, Y, Tt, W, items, nrhs);
-    else bfwd_gather_kernel<T, 16><<<count, THREADS, 0, st>>>(d, Y, Tt, W, items, nrhs);
+    if (rgt == 64) launch_dependent(bfwd_gather_kernel<T, 64>, count, THREADS, 0, st, d, Y, Tt, W, items, nrhs);
+    else launch_dependent(bfwd_gather_kernel<T, 16>, count, THREADS, 0, st, d, Y, Tt, W, items, nrhs);
 }
 template <class T, int ROWS, int RHS>
 static void finish_go(const DevSym &d, const T *Y, T *Tt, const T *P, const int4 *items, int count, int nrhs,
                       cudaStream_t st) {
     constexpr int PER = ROWS * RHS / THREADS;
-    breduce_finish_kernel<T, ROWS, RHS><<<count * PER, THREADS, 0, st>>>(d, Y, Tt, P, items, nrhs);
+    launch_dependent(breduce_finish_kernel<T, ROWS, RHS>, count * PER, THREADS, 0, st, d, Y, Tt, P, items, nrhs);
 }
 
 template <class T>
