@@ -182,9 +182,21 @@ __device__ __forceinline__ void issue_a(const DevSym &d, const TcSolveArgs &a, c
         const int rblk = (g.r0 + r) / NB;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int kblk = (kk0 + kh + 4 * q) / NB;
+            const int kq0 = kk0 + kh + 4 * q, kblk = kq0 / NB;
             const bool side = OP != OP_XAPPLY || (a.upper ? kblk >= rblk : kblk <= rblk);
-            const bool v = ok && side && kk0 + kh + 4 * q < lim;
+            const bool v = ok && side && kq0 < lim;
+            if (OP == OP_BREDUCE && kq0 < g.b0 + g.w) {
+                // rows of the super-block itself, ahead of the first row below
+                // it: above its diagonal the front holds anything (values of
+                // an FP64 factor in the same memory, say), and a NaN there
+                // would survive the zero it is multiplied with
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const bool ve = v && kq0 + e >= g.b0 + g.w;
+                    cp_async4(Ah + tc::sw128_offset(r, kh + 4 * q) + 4 * e, ve ? src + 4 * q + e : a.front, ve ? 4 : 0);
+                }
+                continue;
+            }
             cp_async16(Ah + tc::sw128_offset(r, kh + 4 * q), v ? src + 4 * q : a.front, v ? 16 : 0);
         }
     }

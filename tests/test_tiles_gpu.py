@@ -176,15 +176,37 @@ def test_residual_chunks(wdlib, cuda, ncols):
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("nrhs", [1, 2, 4, 8])
 def test_narrow_solve_large_launches(wdlib, cuda, prec, nrhs):
-    """Enough fronts in one level that its launches take the shallow form: a
-    forest of 700 small dense blocks, each column solved as alone."""
+    """Enough fronts in one level that its launches take the shallow form: 700
+    small dense blocks, each coupled to the same three unknowns."""
     rng = np.random.default_rng(nrhs)
-    k, cnt = 5, 700
+    k, cnt, b = 5, 700, 3
+    n = k * cnt + b
     M = rng.standard_normal((cnt, k, k))
     A = M @ M.transpose(0, 2, 1) + k * np.eye(k)
-    cp = np.concatenate([[0], np.cumsum(np.tile(np.arange(k, 0, -1), cnt))]).astype(np.int64)
-    ri = np.concatenate([np.arange(c * k + j, (c + 1) * k) for c in range(cnt) for j in range(k)]).astype(np.int32)
-    v = np.concatenate([A[c, j:, j] for c in range(cnt) for j in range(k)])
-    B = rhs(cnt * k, nrhs, seed=nrhs)
+    border = np.arange(k * cnt, n)
+    rows, vals = [], []
+    for c in range(cnt):
+        for j in range(k):
+            rows.append(np.concatenate([np.arange(c * k + j, (c + 1) * k), border]))
+            vals.append(np.concatenate([A[c, j:, j], 0.3 * rng.standard_normal(b)]))
+    for j in range(b):
+        rows.append(border[j:])
+        vals.append(np.concatenate([[float(n)], np.ones(b - 1 - j)]))
+    cp = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+    ri, v = np.concatenate(rows).astype(np.int32), np.concatenate(vals)
+    B = rhs(n, nrhs, seed=nrhs)
     s = wdlib.Solver(relax_k=0, relax_pct=0).analyze(cp, ri).factor(v, prec)
     assert oracle.backward_error(cp, ri, v, s.solve(B), B).max() <= 1e-12
+
+
+@pytest.mark.parametrize("dim,J", [(2, 4), (2, 5)])
+def test_solve_after_fp64_factor(wdlib, cuda, dim, J):
+    """The FP64 factor leaves words in the shared front pool that are NaN as
+    FP32 above the diagonals of a later mixed factor; a reduction that starts
+    inside a super-block (its end no multiple of 32) must not see them."""
+    b, cp, ri, v, o = _case(dim, J)
+    B = rhs(o.n, 40, seed=5)
+    s = wdlib.Solver().analyze(cp, ri, b)
+    s.factor(v, "fp64")
+    X = s.factor(v, "mixed").solve(B)
+    assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
