@@ -711,10 +711,11 @@ __global__ void xupdate_kernel(const float *__restrict__ Y, double *__restrict__
 // lanes it is three for four rows: 256 x 256 problem, one right-hand side, 93
 // -> 84 us; a batch of 64 instances 427 -> 278), NR (the
 // number of right-hand sides rounded up to 1, 2, 4 or 8) accumulators per
-// lane and U = 4 entries per lane in flight (their values, columns and x loads
-// are all issued before the first product), which hides the dependent
-// column -> x latency that one entry at a time leaves exposed.  Each lane adds
-// its entries in the same order as one entry per step would.  Every address
+// lane and U = 4 entries per lane in flight: their x loads are all issued
+// before the first product, and after them the loads of the next U values and
+// columns, so that a step waits for one memory latency, not for the column's
+// and then x's (16 theta steps at 128 x 128, 48 products, 7.90 -> 7.17 ms).  Each lane adds its entries in the
+// same order as one entry per step would.  Every address
 // formed is in range: lanes past the end of the chunk re-read the lane's
 // first entry with weight 0, accumulators past nrhs read right-hand side 0
 // (never written out), and a column index outside [0, n) is skipped and its
@@ -738,31 +739,35 @@ __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const in
     double acc[NR];
 #pragma unroll
     for (int c = 0; c < NR; ++c) acc[c] = 0.0;
-    for (int e0 = it.y + lane; e0 < it.z; e0 += SPL * U) {
-        double v[U];
-        int64_t xo[U];
+    double v[U];
+    int col[U];
+    auto fetch = [&](int e0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ec = e0 + SPL * u < it.z ? e0 + SPL * u : e0;
+            v[u] = __ldcs(d.csr_val + ec);
+            col[u] = __ldcs(d.csr_col + ec);
+        }
+    };
+    int e0 = it.y + lane;
+    if (e0 < it.z) fetch(e0);
+    for (; e0 < it.z; e0 += SPL * U) {
+        double x[U][NR], vv[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int e = e0 + SPL * u;
-            const bool in = e < it.z;
-            const int ec = in ? e : e0;
-            double val = __ldcs(d.csr_val + ec);
-            const int col = __ldcs(d.csr_col + ec);
-            const bool col_ok = (int64_t)(uint32_t)col < d.n;
+            const bool in = e < it.z, col_ok = (int64_t)(uint32_t)col[u] < d.n;
             if (!col_ok && in) atomicMin(bad, (unsigned long long)e);
-            if (!in || !col_ok) val = 0.0;
-            v[u] = val;
-            xo[u] = col_ok ? (int64_t)col * nrhs : 0;
+            vv[u] = in && col_ok ? v[u] : 0.0;
+            const double *xp = X + (col_ok ? (int64_t)col[u] * nrhs : 0);
+#pragma unroll
+            for (int c = 0; c < NR; ++c) x[u][c] = xp[c < nrhs ? c : 0];
         }
-        double x[U][NR];
+        if (e0 + SPL * U < it.z) fetch(e0 + SPL * U);
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int c = 0; c < NR; ++c) x[u][c] = X[xo[u] + (c < nrhs ? c : 0)];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int c = 0; c < NR; ++c) acc[c] += v[u] * x[u][c];
+            for (int c = 0; c < NR; ++c) acc[c] += vv[u] * x[u][c];
     }
 #pragma unroll
     for (int c = 0; c < NR; ++c) {
