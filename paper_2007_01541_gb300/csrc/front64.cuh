@@ -189,8 +189,9 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
     const int64_t o = d.foff[s] + (int64_t)kb * ld + kb, gcol0 = (int64_t)d.sfirst[s] + kb;
     const bool lu = a.g != nullptr, nonsym = lu && !a.sym;
     if (tid < NB) inv[tid] = 1.0;
-    // eight loads in flight per thread
-    constexpr int U = 8;
+    // sixteen loads in flight per thread (eight: LDL^T on the sphere 8.92 ms,
+    // 1D 1,024 unknowns 0.861; sixteen 8.70 and 0.851)
+    constexpr int U = 16;
     for (int i0 = tid; i0 < NB * NB; i0 += U * NT) {
         double v[U], w[U];
 #pragma unroll
