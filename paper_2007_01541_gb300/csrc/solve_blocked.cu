@@ -400,14 +400,15 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // 0.490 ms, the batch of 64 instances 12.47 -> 11.72.
 // ---------------------------------------------------------------------------
 constexpr int NRW = 32;
-// DEEP launches, at most NARROW_DEEP CTAs (four per SM): sixteen loads in flight
+// DEEP launches, at most NARROW_DEEP CTAs (two per SM): sixteen loads in flight
 // per lane, the first of them before the wait.  Larger launches (the lower
 // levels of large trees and of batches) have other CTAs to overlap with: four
 // loads (eight in the reduction), two to four CTAs per SM, ordinary launches.
-// All launches deep / up to 2,432 CTAs / up to 608: 256 x 256, one right-hand
-// side 1.17 / 1.08 / 1.05 ms; 16 theta steps at 128 x 128 8.01 / 7.92 / 7.85;
-// batch of 64 instances 12.87 / 11.83 / 11.72.  The arithmetic is the same.
-constexpr int NARROW_DEEP = 608;
+// The arithmetic is the same.  Limit 2,432 / 608 / 304 / 152 against each other
+// (and all launches deep first): 256 x 256, one right-hand side 1.17; 1.08 /
+// 1.05 / 1.03 / 1.07 ms; 16 theta steps at 128 x 128 8.01; 7.92 / 7.85 / 7.70 /
+// 7.94; batch of 64 instances 12.87; 11.83 / 11.72 / 11.72 / 11.74.
+constexpr int NARROW_DEEP = 304;
 template <bool DEEP, int NR>
 constexpr int narrow_ctas() { return DEEP ? 1 : (NR <= 2 ? 4 : NR == 4 ? 3 : 2); }
 constexpr int NWARP = THREADS / 32;
