@@ -1220,6 +1220,8 @@ static wd_status finish_analysis(wd_handle h, std::chrono::steady_clock::time_po
             CK(cudaMemcpy(h->d_spmv_fin, fin.data(), fin.size() * sizeof(int4), cudaMemcpyHostToDevice), "upload");
         CK(h->mem.alloc((void **)&h->d_norm_part, std::max(slots, 1) * sizeof(double)), "norm partials");
         CK(h->mem.alloc((void **)&h->d_spmv_bad, sizeof(unsigned long long)), "spmv check");
+        const unsigned long long none = ~0ULL;     // stays so unless a product meets a bad column
+        CK(cudaMemcpy(h->d_spmv_bad, &none, sizeof(none), cudaMemcpyHostToDevice), "spmv check");
     }
     d.csr_val = h->d_csr_val;
     CK(h->mem.alloc((void **)&h->d_status, sizeof(status_t)), "status alloc");
@@ -1791,10 +1793,9 @@ static wd_status launch_residual(wd_handle h, const double *X, int64_t nrhs, cud
         prof_single(h, "spmv_residual_df", 2.0 * nf * nrhs, 12.0 * nf + 24.0 * n * nrhs, st, false);
         h->launches += h->n_spmv_fin > 0 ? 3 : 2;
     } else {
-        CK(cudaMemsetAsync(h->d_spmv_bad, 0xff, sizeof(unsigned long long), st), "spmv check");
         prof_single(h, "spmv_residual_fp64", 0, 0, st, true);
         wd::launch_spmv_residual(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin,
-                                 h->n_spmv_fin, X, h->d_Bp, h->d_R, h->d_P, nrhs, h->d_spmv_bad, st);
+                                 h->n_spmv_fin, X, h->d_Bp, h->d_R, h->d_P, nrhs, h->d_spmv_bad, h->d_cm, st);
         prof_single(h, "spmv_residual_fp64", 2.0 * nf * nrhs, 12.0 * nf + 24.0 * n * nrhs, st, false);
         h->launches += h->n_spmv_fin > 0 ? 2 : 1;
     }
@@ -1803,6 +1804,8 @@ static wd_status launch_residual(wd_handle h, const double *X, int64_t nrhs, cud
 }
 
 static wd_status bad_column(wd_handle h, status_t at) {
+    const unsigned long long none = ~0ULL;
+    CK(cudaMemcpy(h->d_spmv_bad, &none, sizeof(none), cudaMemcpyHostToDevice), "spmv check");
     return fail(h, WD_ERR_CUDA, "residual: column index out of range at CSR position " + std::to_string(at));
 }
 

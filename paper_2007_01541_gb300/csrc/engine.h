@@ -216,11 +216,12 @@ void launch_transpose(Tc *C, double *Rm, int64_t n, int64_t nrhs, int dir, int a
                       cudaStream_t st);
 // chunks: (row, first entry, end, slot or -1); fin: (row, first slot, slots);
 // bad: smallest CSR position whose column index is outside [0, n) (atomic
-// minimum; the caller sets it to UINT64_MAX first; used for nrhs <= 8)
+// minimum on a word that was UINT64_MAX), zero: 3 nrhs doubles set to zero for
+// launch_colmax3 after it; both used for nrhs <= 8
 constexpr int SPMV_CHUNK = 512;
 void launch_spmv_residual(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, const double *X, const double *Bp, double *R, double *P,
-                          int64_t nrhs, unsigned long long *bad, cudaStream_t st);
+                          int64_t nrhs, unsigned long long *bad, double *zero, cudaStream_t st);
 // the same residual in double-float arithmetic (vh + vl = the CSR values;
 // Xp: n x nrhs scratch for the split of X as (hi, lo) pairs)
 void launch_spmv_residual_df(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin, int nfin,
@@ -237,6 +238,7 @@ void launch_xupdate(const float *Y, double *X, float *Xf, int64_t n, int64_t nrh
                     cudaStream_t st);
 void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, double *partial, double *out, cudaStream_t st);
+// nrhs <= 8: out3 holds zeros already
 void launch_colmax3(const double *R, const double *X, const double *Bp, int64_t n,
                     int64_t nrhs, double *out3, cudaStream_t st);
 template <class T>

@@ -719,7 +719,10 @@ __global__ void xupdate_kernel(const float *__restrict__ Y, double *__restrict__
 // formed is in range: lanes past the end of the chunk re-read the lane's
 // first entry with weight 0, accumulators past nrhs read right-hand side 0
 // (never written out), and a column index outside [0, n) is skipped and its
-// CSR position recorded in *bad (atomic minimum; the host clears and reads it).
+// CSR position recorded in *bad (atomic minimum; the host reads it, and clears it if
+// it was written).  zero: the 3 nrhs column maxima that follow the product
+// start from zero (instead of five memsets per theta step; 16 steps 6.98 ->
+// 6.88 ms).
 constexpr int SPL = 8;
 template <int NR>
 __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const int4 *__restrict__ items,
@@ -727,8 +730,10 @@ __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const in
                                                               const double *__restrict__ Bp,
                                                               double *__restrict__ R,
                                                               double *__restrict__ P, int nrhs,
-                                                              unsigned long long *__restrict__ bad) {
+                                                              unsigned long long *__restrict__ bad,
+                                                              double *__restrict__ zero) {
     const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / SPL;
+    if (blockIdx.x == 0 && threadIdx.x < 3 * nrhs) zero[threadIdx.x] = 0.0;
     const int lane = threadIdx.x % SPL;
     const unsigned mask = (0xFFu << (threadIdx.x & 24));    // this chunk's lanes
     if (w >= count) return;
@@ -1041,18 +1046,18 @@ void launch_transpose(Tc *C, double *Rm, int64_t n, int64_t nrhs, int dir, int a
 
 void launch_spmv_residual(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, const double *X, const double *Bp, double *R, double *P,
-                          int64_t nrhs, unsigned long long *bad, cudaStream_t st) {
+                          int64_t nrhs, unsigned long long *bad, double *zero, cudaStream_t st) {
     const int lanes = nrhs <= 8 ? SPL : 32;    // per chunk
     const int blocks = (int)(((int64_t)nchunks * lanes + THREADS - 1) / THREADS);
     const int nr = (int)nrhs;
     if (nrhs == 1)
-        spmv_narrow_kernel<1><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad);
+        spmv_narrow_kernel<1><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad, zero);
     else if (nrhs == 2)
-        spmv_narrow_kernel<2><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad);
+        spmv_narrow_kernel<2><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad, zero);
     else if (nrhs <= 4)
-        spmv_narrow_kernel<4><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad);
+        spmv_narrow_kernel<4><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad, zero);
     else if (nrhs <= 8)
-        spmv_narrow_kernel<8><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad);
+        spmv_narrow_kernel<8><<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, nr, bad, zero);
     else
         spmv_wide_kernel<<<blocks, THREADS, 0, st>>>(d, chunks, nchunks, X, Bp, R, P, (int)nrhs);
     if (nfin > 0 && nrhs <= 8)
@@ -1097,12 +1102,12 @@ void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, cons
 
 void launch_colmax3(const double *R, const double *X, const double *Bp, int64_t n, int64_t nrhs,
                     double *out3, cudaStream_t st) {
-    cudaMemsetAsync(out3, 0, 3 * nrhs * sizeof(double), st);
-    if (nrhs <= 8) {
+    if (nrhs <= 8) {    // out3 zeroed by the product before
         const int blocks = (int)std::min<int64_t>((n + 1023) / 1024, 152);
         colmax3_narrow_kernel<<<blocks, 256, 0, st>>>(R, X, Bp, n, (int)nrhs, out3);
         return;
     }
+    cudaMemsetAsync(out3, 0, 3 * nrhs * sizeof(double), st);
     const int64_t rpb = std::max<int64_t>(16, (n + 607) / 608);    // four blocks per SM
     colmax3_rm_kernel<<<(int)((n + rpb - 1) / rpb), 256, 0, st>>>(R, X, Bp, n, (int)nrhs, rpb, out3);
 }

@@ -210,3 +210,27 @@ def test_solve_after_fp64_factor(wdlib, cuda, dim, J):
     s.factor(v, "fp64")
     X = s.factor(v, "mixed").solve(B)
     assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("cnt", [1, 2, 4, 5, 6, 9, 10])
+def test_extend_add_children(wdlib, cuda, prec, cnt):
+    """A dense front of 140 unknowns (more than one slice of rows) with cnt - 1
+    children, fewer and more than one group of them."""
+    rng = np.random.default_rng(cnt)
+    k, b = 7, 140
+    n = k * cnt + b
+    A = np.zeros((n, n))
+    for c in range(cnt):
+        M = rng.standard_normal((k, k))
+        A[c * k:(c + 1) * k, c * k:(c + 1) * k] = M @ M.T + k * np.eye(k)
+        A[k * cnt:, c * k:(c + 1) * k] = 0.3 * rng.standard_normal((b, k))
+    M = rng.standard_normal((b, b))
+    A[k * cnt:, k * cnt:] = M @ M.T + n * np.eye(b)
+    A = np.tril(A)
+    cp = np.concatenate([[0], np.cumsum((A != 0).sum(0))]).astype(np.int64)
+    ri = np.nonzero(A.T)[1].astype(np.int32)
+    v = A.T[A.T != 0]
+    B = rhs(n, 3, seed=cnt)
+    s = wdlib.Solver(relax_k=0, relax_pct=0).analyze(cp, ri).factor(v, prec)
+    assert oracle.backward_error(cp, ri, v, s.solve(B), B).max() <= (1e-14 if prec == "fp64" else 1e-12)
