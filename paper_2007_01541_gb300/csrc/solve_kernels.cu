@@ -714,8 +714,8 @@ __global__ void xupdate_kernel(const float *__restrict__ Y, double *__restrict__
 // lane and U = 4 entries per lane in flight: their x loads are all issued
 // before the first product, and after them the loads of the next U values and
 // columns, so that a step waits for one memory latency, not for the column's
-// and then x's (16 theta steps at 128 x 128, 48 products, 7.90 -> 7.17 ms).  Each lane adds its entries in the
-// same order as one entry per step would.  Every address
+// and then x's (16 theta steps at 128 x 128, 48 products, 7.90 -> 7.17 ms).
+// Each lane adds its entries in the same order as one entry per step would.  Every address
 // formed is in range: lanes past the end of the chunk re-read the lane's
 // first entry with weight 0, accumulators past nrhs read right-hand side 0
 // (never written out), and a column index outside [0, n) is skipped and its
