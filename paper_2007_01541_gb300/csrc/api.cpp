@@ -1546,7 +1546,10 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
     const int64_t nnzl = h->S.pcp[h->S.n];
     if (!h->d_front) {
         CK(h->mem.alloc(&h->d_front, h->front_elems * sizeof(double)), "front pool alloc");
-        // padding rows stay zero forever: no kernel writes them
+        // (zero once, so that nothing is uninitialized.  A factor writes the
+        // lower parts of its fronts up to row mp, padding rows included; FP32
+        // and FP64 fronts share the pool, so what lies above the diagonals and
+        // past row mp is whatever an earlier factor left: no reader may use it)
         CK(cudaMemsetAsync(h->d_front, 0, h->front_elems * sizeof(double), st), "front pool clear");
     }
     if (!h->d_dinv) CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");

@@ -197,7 +197,9 @@ __device__ __forceinline__ void issue_a(const DevSym &d, const TcSolveArgs &a, c
                 }
                 continue;
             }
-            cp_async16(Ah + tc::sw128_offset(r, kh + 4 * q), v ? src + 4 * q : a.front, v ? 16 : 0);
+            // the front's last row need not end a vector: past it the pool
+            // holds anything too
+            cp_async16(Ah + tc::sw128_offset(r, kh + 4 * q), v ? src + 4 * q : a.front, v ? 4 * min(4, lim - kq0) : 0);
         }
     }
 }
