@@ -293,6 +293,12 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
         a.f[o + (int64_t)c * ld + r] = A[r][c];
         if (lu) a.g[o + (int64_t)c * ld + r] = A[c][r];
     }
+    // LDL^T does not assemble U^T's fronts, and no panel covers the padding
+    // rows of the last block: the solves multiply them by zero
+    if (lu && a.sym && kb + nb == k) {
+        const int pad = d.skp[s] - k;
+        for (int idx = tid; idx < nb * pad; idx += NT) a.g[o + (int64_t)(idx / pad) * ld + nb + idx % pad] = 0.0;
+    }
 }
 
 }  // namespace f64

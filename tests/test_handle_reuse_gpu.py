@@ -64,7 +64,7 @@ def _results(s, kind, n, ncols):
 
 
 @pytest.mark.parametrize("name", list(CASES))
-@pytest.mark.parametrize("later", ["mixed", "mixed_simt", "mixed_step", "fp64", "fp64_tc", "lu"])
+@pytest.mark.parametrize("later", ["mixed", "mixed_simt", "mixed_step", "fp64", "fp64_tc", "lu", "ldlt"])
 def test_factor_after_another_kind(wdlib, cuda, name, later):
     if name not in _made:
         _made[name] = CASES[name]()
