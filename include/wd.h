@@ -142,7 +142,9 @@ typedef struct {
     int32_t iterations;         /* refinement steps taken (0 in WD_FP64)       */
     double backward_error;      /* max over columns of
                                    ||b - A x||_inf / (||A||_inf ||x||_inf + ||b||_inf),
-                                   residual in FP64; -1 if not computed        */
+                                   residual in FP64; -1 if not computed;
+                                   infinity if x or the residual is not finite
+                                   in a column whose b is                     */
 } wd_solve_info;
 
 /* Fill *opt with the defaults listed above. */
@@ -203,7 +205,9 @@ wd_status wd_factor(wd_handle h, const double *values, int values_on_device, wd_
 /* B := A^-1 B for nrhs columns of leading dimension ldb >= n, original
    order.  B on the device (B_on_device = 1) or the host (0).  In WD_MIXED the
    solve is refined in FP64 until the backward error is <= ir_tol
-   (WD_ERR_NO_CONVERGENCE after ir_max_iter steps).  In WD_FP64 the backward
+   (WD_ERR_NO_CONVERGENCE after ir_max_iter steps, or if a finite column of B
+   has no finite result; columns of B that are not finite themselves do not
+   count).  In WD_FP64 the backward
    error is computed only if info is not NULL.  Synchronous. */
 wd_status wd_solve(wd_handle h, double *B, int64_t nrhs, int64_t ldb, int B_on_device,
                    void *stream, wd_solve_info *info);
@@ -240,7 +244,8 @@ wd_status wd_theta_step(wd_handle h, double *U, const double *F, int64_t nrhs, i
      ||b - A x||_inf / (||A||_inf ||x||_inf + ||b||_inf)
    X, B: n x nrhs, column-major, leading dimension ld, original order, device
    (1) or host (0).  The residual is formed from A's FP64 values: in FP64 for
-   up to 8 columns, in double-float arithmetic (about 48 bits) for more.  For
+   up to 8 columns, in double-float arithmetic (about 48 bits, FP32's range) for
+   more; infinity where x or the residual is not finite although b is.  For
    a batch, the largest of the instances' own backward errors.  Needs a
    successful wd_factor (for ||A||_inf).  Synchronous. */
 wd_status wd_backward_error(wd_handle h, const double *X, const double *B, int64_t nrhs, int64_t ld,

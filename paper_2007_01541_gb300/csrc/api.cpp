@@ -846,7 +846,7 @@ static wd_status ensure_pin(wd_handle h, int64_t elems) {
     h->pin_elems = elems;
     return WD_OK;
 }
-static status_t pin_word(wd_handle h, int i) {
+static status_t pin_word(wd_handle h, int64_t i) {
     status_t v;
     std::memcpy(&v, h->pin + i, sizeof(v));
     return v;
@@ -1252,7 +1252,7 @@ static wd_status finish_analysis(wd_handle h, std::chrono::steady_clock::time_po
     }
     {
         // enough for the column maxima of 128 right-hand sides (and instances)
-        const wd_status ps = ensure_pin(h, 3 * 128);
+        const wd_status ps = ensure_pin(h, 4 * 128);
         if (ps != WD_OK) return ps;
     }
     fill_info(h, nnzl, maxm, maxk, t0);
@@ -1651,15 +1651,15 @@ static wd_status ensure_solve_ws(wd_handle h, int64_t nrhs) {
     CK(h->work.alloc((void **)&h->d_X, n * nrhs * sizeof(double)), "solve ws");
     CK(h->work.alloc((void **)&h->d_Xp, n * nrhs * sizeof(float2)), "solve ws");
     CK(h->work.alloc((void **)&h->d_R, n * nrhs * sizeof(double)), "solve ws");
-    CK(h->work.alloc((void **)&h->d_cm, 3 * nrhs * sizeof(double)), "solve ws");
+    CK(h->work.alloc((void **)&h->d_cm, 4 * nrhs * sizeof(double)), "solve ws");
     CK(h->work.alloc((void **)&h->d_P, std::max(h->n_spmv_slots, 1) * nrhs * sizeof(double)), "solve ws");
     h->d_batch_cm = nullptr;
     if (h->batch_count > 0)
-        CK(h->work.alloc((void **)&h->d_batch_cm, 3 * (int64_t)h->batch_count * nrhs * sizeof(double)),
+        CK(h->work.alloc((void **)&h->d_batch_cm, 4 * (int64_t)h->batch_count * nrhs * sizeof(double)),
            "solve ws");
     {
         // before anything of the call is in flight
-        const wd_status ps = ensure_pin(h, 3 * (int64_t)std::max(1, h->batch_count) * nrhs);
+        const wd_status ps = ensure_pin(h, 4 * (int64_t)std::max(1, h->batch_count) * nrhs);
         if (ps != WD_OK) return ps;
     }
     h->ws_cols = nrhs;
@@ -1821,19 +1821,21 @@ static wd_status enqueue_backward_errors(wd_handle h, const double *X, int64_t n
     if (s != WD_OK) return s;
     double *cm = h->batch_count > 0 ? h->d_batch_cm : h->d_cm;
     if (h->batch_count > 0)
-        wd::launch_seg_colmax3(h->d_R, X, h->d_Bp, h->d_batch_coff, (int)cnt, (int)nrhs, cm, st);
+        wd::launch_seg_colmax(h->d_R, X, h->d_Bp, h->d_batch_coff, (int)cnt, (int)nrhs, cm, st);
     else
-        wd::launch_colmax3(h->d_R, X, h->d_Bp, h->S.n, nrhs, cm, st);
+        wd::launch_colmax(h->d_R, X, h->d_Bp, h->S.n, nrhs, cm, st);
     h->launches += 2;
     if (nrhs <= 8)
         CK(cudaMemcpyAsync(h->pin + PIN_BAD, h->d_spmv_bad, sizeof(status_t), cudaMemcpyDeviceToHost, st),
            "spmv check");
-    CK(cudaMemcpyAsync(h->pin + PIN_CM, cm, 3 * cnt * nrhs * sizeof(double), cudaMemcpyDeviceToHost, st), "be D2H");
+    CK(cudaMemcpyAsync(h->pin + PIN_CM, cm, 4 * cnt * nrhs * sizeof(double), cudaMemcpyDeviceToHost, st), "be D2H");
     return WD_OK;
 }
 
 // the largest normwise backward error over columns (and instances), after the
-// copies have landed
+// copies have landed: infinite where x or the residual is not finite although
+// b is.  (A column whose b is not finite has no finite solution; what of it is
+// NaN does not count.)
 static wd_status read_backward_errors(wd_handle h, int64_t nrhs, double *be_max) {
     if (nrhs <= 8 && pin_word(h, PIN_BAD) != ~0ULL) return bad_column(h, pin_word(h, PIN_BAD));
     const int64_t cnt = h->batch_count > 0 ? h->batch_count : 1;
@@ -1841,9 +1843,11 @@ static wd_status read_backward_errors(wd_handle h, int64_t nrhs, double *be_max)
     for (int64_t i = 0; i < cnt; ++i) {
         const double nrm = h->batch_count > 0 ? h->batch_normA[i] : h->normA;
         for (int64_t c = 0; c < nrhs; ++c) {
-            const double *q = h->pin + PIN_CM + (i * nrhs + c) * 3;
+            const int64_t o = PIN_CM + (i * nrhs + c) * 4;
+            const double *q = h->pin + o;
             const double den = nrm * q[1] + q[2];
-            mx = std::max(mx, den > 0 ? q[0] / den : 0.0);
+            const bool bad = (pin_word(h, o + 3) & (wd::CM_BAD_X | wd::CM_BAD_B)) == wd::CM_BAD_X;
+            mx = std::max(mx, bad ? HUGE_VAL : (den > 0 ? q[0] / den : 0.0));
         }
     }
     *be_max = mx;
@@ -1956,7 +1960,7 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
             CK(cudaStreamSynchronize(st), "backward error");
             s = read_backward_errors(h, nrhs, &be);
             if (s != WD_OK) return s;
-            if (be <= h->opt.ir_tol || it >= h->opt.ir_max_iter) {
+            if (be <= h->opt.ir_tol || it >= h->opt.ir_max_iter || pin_word(h, PIN_TSTATUS) != 0) {
                 if (!last) {
                     wd::launch_permute_out_rm(h->d_X, Bd, ld, h->dsym.perm, n, nrhs, st);
                     h->launches += 1;

@@ -82,31 +82,28 @@ __global__ void seg_norm_finish_kernel(const int4 *__restrict__ fin, int nfin, c
     atomic_max_nonneg(out + instance_of(coff, count, fin[i].x), acc);
 }
 
-// out[(inst * nrhs + c) * 3 + {0, 1, 2}] = max |R|, |X|, |B| over the
-// instance's rows of column c (row-major n x nrhs arrays)
-__global__ void __launch_bounds__(THREADS) seg_colmax3_kernel(const double *__restrict__ R,
-                                                              const double *__restrict__ X,
-                                                              const double *__restrict__ B,
-                                                              const int64_t *__restrict__ coff, int nrhs,
-                                                              double *__restrict__ out) {
+// out[(inst * nrhs + c) * 4 + {0, 1, 2, 3}] = max |R|, |X|, |B| and the flags
+// (ColMax) over the instance's rows of column c (row-major n x nrhs arrays)
+__global__ void __launch_bounds__(THREADS) seg_colmax_kernel(const double *__restrict__ R,
+                                                             const double *__restrict__ X,
+                                                             const double *__restrict__ B,
+                                                             const int64_t *__restrict__ coff, int nrhs,
+                                                             double *__restrict__ out) {
     __shared__ unsigned long long red[THREADS / 32];
     const int inst = blockIdx.x;
     for (int c = 0; c < nrhs; ++c) {
-        unsigned long long a = 0, b = 0, e = 0;
+        ColMax v;
 #pragma unroll 4
-        for (int64_t r = coff[inst] + threadIdx.x; r < coff[inst + 1]; r += THREADS) {
-            a = max(a, abs_key(R[r * nrhs + c]));
-            b = max(b, abs_key(X[r * nrhs + c]));
-            e = max(e, abs_key(B[r * nrhs + c]));
-        }
-        a = block_max(a, red);
-        b = block_max(b, red);
-        e = block_max(e, red);
+        for (int64_t r = coff[inst] + threadIdx.x; r < coff[inst + 1]; r += THREADS)
+            v.add(R[r * nrhs + c], X[r * nrhs + c], B[r * nrhs + c]);
+        const unsigned long long a = block_max(v.m[0], red), b = block_max(v.m[1], red), e = block_max(v.m[2], red);
+        const int bad_x = __syncthreads_or(v.flags & CM_BAD_X), bad_b = __syncthreads_or(v.flags & CM_BAD_B);
         if (threadIdx.x == 0) {
-            double *o = out + ((int64_t)inst * nrhs + c) * 3;
+            double *o = out + ((int64_t)inst * nrhs + c) * 4;
             o[0] = __longlong_as_double((long long)a);
             o[1] = __longlong_as_double((long long)b);
             o[2] = __longlong_as_double((long long)e);
+            o[3] = __longlong_as_double((long long)((bad_x ? CM_BAD_X : 0) | (bad_b ? CM_BAD_B : 0)));
         }
     }
 }
@@ -148,9 +145,9 @@ void launch_seg_norm_inf(const DevSym &d, const int4 *chunks, int nchunks, const
     if (nfin > 0) seg_norm_finish_kernel<<<(nfin + 127) / 128, 128, 0, st>>>(fin, nfin, partial, coff, count, out);
 }
 
-void launch_seg_colmax3(const double *R, const double *X, const double *B, const int64_t *coff, int count,
-                        int nrhs, double *out, cudaStream_t st) {
-    seg_colmax3_kernel<<<count, THREADS, 0, st>>>(R, X, B, coff, nrhs, out);
+void launch_seg_colmax(const double *R, const double *X, const double *B, const int64_t *coff, int count,
+                       int nrhs, double *out, cudaStream_t st) {
+    seg_colmax_kernel<<<count, THREADS, 0, st>>>(R, X, B, coff, nrhs, out);
 }
 
 template <class T>

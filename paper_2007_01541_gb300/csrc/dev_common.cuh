@@ -54,11 +54,23 @@ inline void launch_dependent(void (*kernel)(P...), unsigned blocks, unsigned thr
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
-// |x| as a key that orders like the value; NaN counts as 0 (fmax ignores it)
-__device__ __forceinline__ unsigned long long abs_key(double x) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-    return u > 0x7FF0000000000000ull ? 0ull : u;
-}
+// Column maxima of the backward error: max |r|, |x| and |b| (NaN does not
+// count), then a word of flags: r or x, and b, held a value that is not finite
+struct ColMax {
+    unsigned long long m[3] = {0, 0, 0};
+    unsigned flags = 0;
+    __device__ __forceinline__ void add(double r, double x, double b) {
+        const unsigned long long inf = 0x7FF0000000000000ull, u[3] = {bits(r), bits(x), bits(b)};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            m[q] = max(m[q], u[q] > inf ? 0ull : u[q]);
+            if (u[q] >= inf) flags |= q < 2 ? CM_BAD_X : CM_BAD_B;
+        }
+    }
+    static __device__ __forceinline__ unsigned long long bits(double x) {
+        return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;   // |x|, ordered like the value
+    }
+};
 
 // the supernode of column j
 __device__ __forceinline__ int supernode_of(const DevSym &d, int j) {

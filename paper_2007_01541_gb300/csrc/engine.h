@@ -216,8 +216,8 @@ void launch_transpose(Tc *C, double *Rm, int64_t n, int64_t nrhs, int dir, int a
                       cudaStream_t st);
 // chunks: (row, first entry, end, slot or -1); fin: (row, first slot, slots);
 // bad: smallest CSR position whose column index is outside [0, n) (atomic
-// minimum on a word that was UINT64_MAX), zero: 3 nrhs doubles set to zero for
-// launch_colmax3 after it; both used for nrhs <= 8
+// minimum on a word that was UINT64_MAX), zero: 4 nrhs doubles set to zero for
+// launch_colmax after it; both used for nrhs <= 8
 constexpr int SPMV_CHUNK = 512;
 void launch_spmv_residual(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, const double *X, const double *Bp, double *R, double *P,
@@ -238,9 +238,12 @@ void launch_xupdate(const float *Y, double *X, float *Xf, int64_t n, int64_t nrh
                     cudaStream_t st);
 void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, double *partial, double *out, cudaStream_t st);
-// nrhs <= 8: out3 holds zeros already
-void launch_colmax3(const double *R, const double *X, const double *Bp, int64_t n,
-                    int64_t nrhs, double *out3, cudaStream_t st);
+// per column four words: max |R|, |X| and |B| (NaN does not count), and as an
+// integer CM_BAD_X (R or X held a value that is not finite) | CM_BAD_B (B did);
+// nrhs <= 8: out holds zeros already
+constexpr unsigned CM_BAD_X = 1, CM_BAD_B = 2;
+void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n,
+                   int64_t nrhs, double *out, cudaStream_t st);
 template <class T>
 void launch_axpy_into(double *X, const T *D, int64_t count, int accumulate, cudaStream_t st);
 template <class T>
@@ -372,8 +375,9 @@ void launch_tc_breduce(const DevSym &d, const TcSolveArgs &a, const int4 *items,
 // scratch of one double per slot)
 void launch_seg_norm_inf(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin, int nfin,
                          double *partial, const int64_t *coff, int count, double *out, cudaStream_t st);
-void launch_seg_colmax3(const double *R, const double *X, const double *B, const int64_t *coff, int count,
-                        int nrhs, double *out, cudaStream_t st);
+// the words of launch_colmax per instance and column
+void launch_seg_colmax(const double *R, const double *X, const double *B, const int64_t *coff, int count,
+                       int nrhs, double *out, cudaStream_t st);
 // out[i] = log det A_i (sdl: scratch of one double per supernode)
 template <class T>
 void launch_seg_logdet(const DevSym &d, const T *front, const int32_t *soff, int count, double *sdl,

@@ -720,8 +720,8 @@ __global__ void xupdate_kernel(const float *__restrict__ Y, double *__restrict__
 // first entry with weight 0, accumulators past nrhs read right-hand side 0
 // (never written out), and a column index outside [0, n) is skipped and its
 // CSR position recorded in *bad (atomic minimum; the host reads it, and clears it if
-// it was written).  zero: the 3 nrhs column maxima that follow the product
-// start from zero (instead of five memsets per theta step; 16 steps 6.98 ->
+// it was written).  zero: the 4 nrhs words of column maxima that follow the
+// product start from zero (instead of five memsets per theta step; 16 steps 6.98 ->
 // 6.88 ms).
 constexpr int SPL = 8;
 template <int NR>
@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(THREADS) spmv_narrow_kernel(DevSym d, const in
                                                               unsigned long long *__restrict__ bad,
                                                               double *__restrict__ zero) {
     const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / SPL;
-    if (blockIdx.x == 0 && threadIdx.x < 3 * nrhs) zero[threadIdx.x] = 0.0;
+    if (blockIdx.x == 0 && threadIdx.x < 4 * nrhs) zero[threadIdx.x] = 0.0;
     const int lane = threadIdx.x % SPL;
     const unsigned mask = (0xFFu << (threadIdx.x & 24));    // this chunk's lanes
     if (w >= count) return;
@@ -853,64 +853,62 @@ __global__ void norm_inf_finish_kernel(const int4 *__restrict__ fin, int nfin,
     atomic_max_nonneg(out, acc);
 }
 
-// per column c: out[3c] = max|R|, out[3c+1] = max|X|, out[3c+2] = max|B|
-// (row-major arrays; out must be zeroed; blocks take chunks of rows), on the
-// bits of |x| (abs_key: NaN does not count): an FP64 comparison takes the FP64
-// pipe.  256 threads are 64 columns x 4 rows; one atomic per block and column
+// per column c: out[4c] = max|R|, out[4c+1] = max|X|, out[4c+2] = max|B|,
+// out[4c+3] = the flags (row-major arrays; out must be zeroed; blocks take
+// chunks of rows), on the bits of |x| (ColMax): an FP64 comparison takes the
+// FP64 pipe.  256 threads are 64 columns x 4 rows; one atomic per block and column
 // (a block of 32 rows with its own atomics spent its time on them: 65,536
 // rows, 64 columns, with it the 256 x
 // 256 step 11.70 -> 11.56 ms).
-__global__ void __launch_bounds__(256) colmax3_rm_kernel(const double *__restrict__ R, const double *__restrict__ X,
-                                                         const double *__restrict__ B, int64_t n, int nrhs,
-                                                         int64_t rows_per_block, double *out) {
+__global__ void __launch_bounds__(256) colmax_rm_kernel(const double *__restrict__ R, const double *__restrict__ X,
+                                                        const double *__restrict__ B, int64_t n, int nrhs,
+                                                        int64_t rows_per_block, double *out) {
     __shared__ unsigned long long red[3][4][64];
+    __shared__ unsigned redf[4][64];
     const int64_t r0 = blockIdx.x * rows_per_block;
     const int64_t r1 = min(n, r0 + rows_per_block);
     const int cl = threadIdx.x & 63, g = threadIdx.x >> 6;
     for (int c0 = 0; c0 < nrhs; c0 += 64) {
         const int c = c0 + cl;
-        unsigned long long a = 0, b = 0, e = 0;
+        ColMax v;
         if (c < nrhs) {
 #pragma unroll 4
-            for (int64_t i = r0 + g; i < r1; i += 4) {
-                a = max(a, abs_key(R[i * nrhs + c]));
-                b = max(b, abs_key(X[i * nrhs + c]));
-                e = max(e, abs_key(B[i * nrhs + c]));
-            }
+            for (int64_t i = r0 + g; i < r1; i += 4) v.add(R[i * nrhs + c], X[i * nrhs + c], B[i * nrhs + c]);
         }
-        red[0][g][cl] = a;
-        red[1][g][cl] = b;
-        red[2][g][cl] = e;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) red[q][g][cl] = v.m[q];
+        redf[g][cl] = v.flags;
         __syncthreads();
-        for (int t = threadIdx.x; t < 192; t += 256) {
-            const int q = t / 64, cc = t % 64;
-            const unsigned long long v = max(max(red[q][0][cc], red[q][1][cc]), max(red[q][2][cc], red[q][3][cc]));
-            if (c0 + cc < nrhs)
-                atomicMax(reinterpret_cast<unsigned long long *>(out + 3 * (int64_t)(c0 + cc) + q), v);
+        // group q: word q of every column
+        unsigned long long *o = reinterpret_cast<unsigned long long *>(out + 4 * (int64_t)c + g);
+        if (c < nrhs && g < 3) {
+            atomicMax(o, max(max(red[g][0][cl], red[g][1][cl]), max(red[g][2][cl], red[g][3][cl])));
+        } else if (c < nrhs) {
+            const unsigned f = redf[0][cl] | redf[1][cl] | redf[2][cl] | redf[3][cl];
+            if (f) atomicOr(o, (unsigned long long)f);
         }
         __syncthreads();
     }
 }
 // few right-hand sides: lanes over rows
-__global__ void __launch_bounds__(256) colmax3_narrow_kernel(const double *__restrict__ R,
-                                                             const double *__restrict__ X,
-                                                             const double *__restrict__ B, int64_t n, int nrhs,
-                                                             double *out) {
+__global__ void __launch_bounds__(256) colmax_narrow_kernel(const double *__restrict__ R,
+                                                            const double *__restrict__ X,
+                                                            const double *__restrict__ B, int64_t n, int nrhs,
+                                                            double *out) {
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     for (int c = 0; c < nrhs; ++c) {
-        unsigned long long m[3] = {0, 0, 0};
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += step) {
-            m[0] = max(m[0], abs_key(R[i * nrhs + c]));
-            m[1] = max(m[1], abs_key(X[i * nrhs + c]));
-            m[2] = max(m[2], abs_key(B[i * nrhs + c]));
-        }
+        unsigned long long *w = reinterpret_cast<unsigned long long *>(out + 4 * (int64_t)c);
+        ColMax v;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += step)
+            v.add(R[i * nrhs + c], X[i * nrhs + c], B[i * nrhs + c]);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m[q] = max(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
-            if ((threadIdx.x & 31) == 0)
-                atomicMax(reinterpret_cast<unsigned long long *>(out + 3 * (int64_t)c + q), m[q]);
+            for (int o = 16; o > 0; o >>= 1) v.m[q] = max(v.m[q], __shfl_xor_sync(0xffffffffu, v.m[q], o));
+            if ((threadIdx.x & 31) == 0) atomicMax(w + q, v.m[q]);
         }
+        const unsigned f = __reduce_or_sync(0xffffffffu, v.flags);
+        if ((threadIdx.x & 31) == 0 && f) atomicOr(w + 3, (unsigned long long)f);
     }
 }
 
@@ -1100,16 +1098,16 @@ void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, cons
     if (nfin > 0) norm_inf_finish_kernel<<<(nfin + 127) / 128, 128, 0, st>>>(fin, nfin, partial, out);
 }
 
-void launch_colmax3(const double *R, const double *X, const double *Bp, int64_t n, int64_t nrhs,
-                    double *out3, cudaStream_t st) {
-    if (nrhs <= 8) {    // out3 zeroed by the product before
+void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n, int64_t nrhs,
+                   double *out, cudaStream_t st) {
+    if (nrhs <= 8) {    // out zeroed by the product before
         const int blocks = (int)std::min<int64_t>((n + 1023) / 1024, 152);
-        colmax3_narrow_kernel<<<blocks, 256, 0, st>>>(R, X, Bp, n, (int)nrhs, out3);
+        colmax_narrow_kernel<<<blocks, 256, 0, st>>>(R, X, Bp, n, (int)nrhs, out);
         return;
     }
-    cudaMemsetAsync(out3, 0, 3 * nrhs * sizeof(double), st);
+    cudaMemsetAsync(out, 0, 4 * nrhs * sizeof(double), st);
     const int64_t rpb = std::max<int64_t>(16, (n + 607) / 608);    // four blocks per SM
-    colmax3_rm_kernel<<<(int)((n + rpb - 1) / rpb), 256, 0, st>>>(R, X, Bp, n, (int)nrhs, rpb, out3);
+    colmax_rm_kernel<<<(int)((n + rpb - 1) / rpb), 256, 0, st>>>(R, X, Bp, n, (int)nrhs, rpb, out);
 }
 
 template <class T>
