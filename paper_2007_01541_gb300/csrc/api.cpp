@@ -1871,6 +1871,7 @@ static wd_status prepare_solve(wd_handle h, int64_t nrhs, bool mixed) {
     // matrix-vector shaped kernels, lanes over rows
     const int large = nrhs <= 8 ? 2 : (mixed && !h->opt.solve_simt ? 1 : 0);
     if (h->splan_nrhs != nrhs || h->splan.large != large) {
+        h->splan_nrhs = -1;     // no plan until all of its buffers are there
         build_solve_plan(h->S, (int)nrhs, large, h->sms, h->splan);
         s = upload_plan(h, h->work, h->splan);
         if (s != WD_OK) return s;

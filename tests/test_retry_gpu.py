@@ -1,0 +1,63 @@
+"""Calls repeated after WD_ERR_OOM (needs a GB300; memory runs out on the host
+side of the allocator): nothing half made is taken for ready.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from wdgen import Kernel, compressed_pattern, compressed_values, haar_basis, rhs
+
+pytestmark = pytest.mark.gpu
+
+_c = {}
+
+
+def _small():
+    if not _c:
+        b = haar_basis(2, 5)
+        cp, ri = compressed_pattern(b)
+        _c.update(b=b, cp=cp, ri=ri, v=compressed_values(b, cp, ri, Kernel("matern32", 0.1), 1e-3))
+    return _c["b"], _c["cp"], _c["ri"], _c["v"]
+
+
+def _each_allocation(wdlib, call, **opts):
+    """call(solver, attempt) with the k-th device allocation failing, for every
+    k; attempt(f, ...) is f(...), done again if it ran out of memory."""
+    failures = 0
+    for k in range(1, 300):
+        s = wdlib.Solver(test_fail_alloc=k, **opts)
+        failed = []
+
+        def attempt(f, *args, between=None):
+            try:
+                return f(*args)
+            except wdlib.WdError as e:
+                assert e.status == wdlib.WD_ERR_OOM, (k, str(e))
+                failed.append(1)
+                if between:
+                    between()
+                return f(*args)
+
+        call(s, attempt)
+        s.close()
+        assert len(failed) <= 1
+        failures += len(failed)
+        if not failed:
+            return failures
+    pytest.fail("more than 299 device allocations")
+
+
+def test_solve_of_another_kind(wdlib, cuda):
+    """The same number of right-hand sides in another precision: the plan is
+    made anew, and its buffers with it."""
+    b, cp, ri, v = _small()
+    B = rhs(b.N, 40, seed=0)
+
+    def call(s, attempt):
+        attempt(s.analyze, cp, ri, b)
+        for prec in ("mixed", "fp64", "mixed"):
+            attempt(s.factor, v, prec)
+            X = attempt(s.solve, B)
+            assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
+
+    assert _each_allocation(wdlib, call) >= 10
