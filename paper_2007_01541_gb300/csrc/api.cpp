@@ -1630,6 +1630,7 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
 // ---------------------------------------------------------------------------
 static wd_status ensure_solve_ws(wd_handle h, int64_t nrhs) {
     if (h->ws_cols >= nrhs) return WD_OK;
+    h->ws_cols = 0;             // none, until all of them are there
     h->work.free_all();
     h->d_Y = h->d_W = h->d_T = h->d_part = nullptr;
     h->part_elems = 0;

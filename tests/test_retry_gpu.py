@@ -61,3 +61,27 @@ def test_solve_of_another_kind(wdlib, cuda):
             assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
 
     assert _each_allocation(wdlib, call) >= 10
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_fewer_columns_after_a_failed_solve(wdlib, cuda, prec):
+    """A wider solve that runs out of memory gives the workspaces back; the
+    next, narrower one makes its own."""
+    b, cp, ri, v = _small()
+    B = rhs(b.N, 70, seed=0)
+
+    def call(s, attempt):
+        attempt(s.analyze, cp, ri, b)
+        attempt(s.factor, v, prec)
+
+        def narrow():
+            X = s.solve(B[:, :3])
+            assert oracle.backward_error(cp, ri, v, X, B[:, :3]).max() <= 1e-12
+            s.apply_L(B[:, :3])
+
+        for c in (3, 40, 70):
+            X = attempt(s.solve, B[:, :c], between=narrow)
+            assert oracle.backward_error(cp, ri, v, X, B[:, :c]).max() <= 1e-12
+            attempt(s.apply_L, B[:, :c], between=narrow)
+
+    assert _each_allocation(wdlib, call) >= 10
