@@ -1555,8 +1555,8 @@ extern "C" wd_status wd_factor(wd_handle h, const double *values, int values_on_
     if (!h->d_dinv) CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
     if (!h->d_xs) CK(h->mem.alloc(&h->d_xs, h->xs_elems * sizeof(double)), "super-block inverse alloc");
     if (!h->d_xts) CK(h->mem.alloc(&h->d_xts, h->xs_elems * sizeof(double)), "super-block inverse alloc");
-    if (prec == WD_FP64 && h->opt.fp64_tc_schur && !h->d_oz_sl) {
-        CK(h->mem.alloc((void **)&h->d_oz_sl, h->oz_sl_bytes), "slice planes alloc");
+    if (prec == WD_FP64 && h->opt.fp64_tc_schur && !(h->d_oz_sl && h->d_oz_ex)) {
+        if (!h->d_oz_sl) CK(h->mem.alloc((void **)&h->d_oz_sl, h->oz_sl_bytes), "slice planes alloc");
         CK(h->mem.alloc((void **)&h->d_oz_ex, h->oz_ex_elems * sizeof(int16_t)), "slice scales alloc");
         // rows no slicing writes (padding, the window past the front) stay zero
         CK(cudaMemsetAsync(h->d_oz_sl, 0, h->oz_sl_bytes, st), "slice planes clear");

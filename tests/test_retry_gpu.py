@@ -85,3 +85,17 @@ def test_fewer_columns_after_a_failed_solve(wdlib, cuda, prec):
             attempt(s.apply_L, B[:, :c], between=narrow)
 
     assert _each_allocation(wdlib, call) >= 10
+
+
+def test_factor_with_slices(wdlib, cuda):
+    """FP64 updates on the tensor cores: the slices' planes and their scales."""
+    b, cp, ri, v = _small()
+    B = rhs(b.N, 3, seed=0)
+
+    def call(s, attempt):
+        attempt(s.analyze, cp, ri, b)
+        attempt(s.factor, v, "fp64")
+        X = attempt(s.solve, B)
+        assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
+
+    assert _each_allocation(wdlib, call, fp64_tc_schur=True) >= 10
