@@ -2287,10 +2287,12 @@ extern "C" wd_status wd_export_L(wd_handle h, double *panels) {
 // ---------------------------------------------------------------------------
 static wd_status upload_pattern_maps(wd_handle h) {
     const wd::Symbolic &S = h->S;
+    const int32_t *p = nullptr;
     if (!h->d_prow) {
-        const int32_t *p = nullptr;
         UP(S.prow, p);
         h->d_prow = const_cast<int32_t *>(p);
+    }
+    if (!h->d_psrc) {
         UP(S.psrc, p);
         h->d_psrc = const_cast<int32_t *>(p);
     }

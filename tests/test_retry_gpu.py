@@ -99,3 +99,21 @@ def test_factor_with_slices(wdlib, cuda):
         assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
 
     assert _each_allocation(wdlib, call, fp64_tc_schur=True) >= 10
+
+
+def test_selected_inverse_and_gradient(wdlib, cuda):
+    """The pattern's maps are made by whichever call needs them first."""
+    b, cp, ri, v = _small()
+    U = rhs(b.N, 2, seed=0)
+    col = np.repeat(np.arange(b.N), np.diff(cp))
+    outer = 2.0 * (U[ri] * U[col]).sum(1) * np.where(ri == col, 0.5, 1.0)
+    ref = wdlib.Solver().analyze(cp, ri, b).factor(v, "fp64").selinv()
+
+    def call(s, attempt):
+        attempt(s.analyze, cp, ri, b)
+        assert np.abs(attempt(s.sym_pattern_outer, U, U) - outer).max() <= 1e-12 * np.abs(outer).max()
+        attempt(s.factor, v, "fp64")
+        np.testing.assert_array_equal(attempt(s.selinv), ref)
+        assert np.abs(attempt(s.sym_pattern_outer, U, U) - outer).max() <= 1e-12 * np.abs(outer).max()
+
+    assert _each_allocation(wdlib, call) >= 10
