@@ -2756,16 +2756,19 @@ extern "C" wd_status wd_set_level_schedule(wd_handle h, const int8_t *step, int3
     if (nlevels != h->S.nlevels) return fail(h, WD_ERR_INVALID_ARG, "one flag per level of the analysis");
     for (int32_t l = 0; l < nlevels; ++l)
         if (step[l] != 0 && step[l] != 1) return fail(h, WD_ERR_INVALID_ARG, "level flags are 0 or 1");
-    h->level_step.assign(step, step + nlevels);
-    build_factor_plan(h->S, h->fplan_tc, true, false, h->chain, h->level_step.data());
+    Plan plan;      // takes the old one's place (and its graph's) when it is there
+    build_factor_plan(h->S, plan, true, false, h->chain, step);
     if (!h->opt.symbolic_only) {
         CK(cudaSetDevice(h->device), "set device");
         wait_export(h);
-        const wd_status us = upload_plan(h, h->mem, h->fplan_tc);
+        const wd_status us = upload_plan(h, h->mem, plan);
         if (us != WD_OK) return us;
         h->g_factor.reset();
+        h->mem.release(h->fplan_tc.d_items);
         h->factored = false;
     }
+    h->fplan_tc = std::move(plan);
+    h->level_step.assign(step, step + nlevels);
     return WD_OK;
 }
 

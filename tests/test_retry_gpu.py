@@ -117,3 +117,30 @@ def test_selected_inverse_and_gradient(wdlib, cuda):
         assert np.abs(attempt(s.sym_pattern_outer, U, U) - outer).max() <= 1e-12 * np.abs(outer).max()
 
     assert _each_allocation(wdlib, call) >= 10
+
+
+def test_level_schedule(wdlib, cuda):
+    """A schedule that does not fit leaves the one before in place."""
+    b, cp, ri, v = _small()
+    B = rhs(b.N, 3, seed=0)
+
+    def call(s, attempt):
+        attempt(s.analyze, cp, ri, b)
+
+        def solved():
+            X = attempt(s.factor, v, "mixed").solve(B)
+            assert oracle.backward_error(cp, ri, v, X, B).max() <= 1e-12
+
+        attempt(s.factor, v, "mixed")
+        attempt(s.solve, B)
+        flags = [1] * len(s.level_schedule())
+
+        def before():
+            assert s.level_schedule() == [0] * len(flags)
+            solved()
+
+        attempt(s.set_level_schedule, flags, between=before)
+        assert s.level_schedule() == flags
+        solved()
+
+    assert _each_allocation(wdlib, call) >= 10
