@@ -109,13 +109,15 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
         cp_async16(Xs + p * PXL + r, valid ? C + (int64_t)(kb + p) * z.ld + r0 + r : Dv, 8 * valid);
     }
     cp_async_commit();
+    int extreme = 0;        // some pivot is: divisions
     if (a.sym && tid < nb) {
         const double dv = T[(int64_t)tid * z.ld + tid];
         rd[tid] = 1.0 / dv;
         rd[NB + tid] = dv;
+        extreme = f64::extreme(dv);
     }
     cp_async_wait<0>();
-    __syncthreads();
+    extreme = __syncthreads_or(extreme);
     const int c = tid % 16, ra = tid / 16;      // rows ra, ra + 8
     const int nblk = (nb + 15) / 16;
     for (int b = 0; b < nblk; ++b) {
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
             // v / d to half an ulp, by the reciprocal and one correction
             const double r = rd[p], x = v * r;
             a.g[d.foff[s] + o] = v;
-            C[o] = fma(fma(-x, rd[NB + p], v), r, x);
+            C[o] = extreme ? v / rd[NB + p] : fma(fma(-x, rd[NB + p], v), r, x);
         } else {
             C[o] = v;
         }

@@ -37,12 +37,16 @@ constexpr int OFF_INV = NB * LDB, OFF_U = OFF_INV + NB, BLOCK_ELEMS = OFF_U + 3 
 // integer operations on the bits (conversions run on the FP64 pipe), then one
 // step of Householder's third-order iteration r (1 + e + e^2), e = 1 - d r:
 // three FP64 instructions instead of a division's seven on the serial chain.
-// e is below 2^-21, so the iteration's own error is below 2^-63.  Values
-// whose reciprocal leaves the normal range take the division.
+// e is below 2^-21, so the iteration's own error is below 2^-63.  Not for
+// extreme d: there the reciprocal is near the ends of the normal range or
+// beyond it (a subnormal pivot's may be infinite where its quotients are not).
+__device__ __forceinline__ bool extreme(double d) {
+    const int e = (int)(((uint32_t)__double2hiint(d) >> 20) & 0x7FFu) - 1023;
+    return e < -1000 || e > 1000;       // infinity and NaN too
+}
 __device__ __forceinline__ double reciprocal(double d) {
     const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
     const int e = (int)((hi >> 20) & 0x7FFu) - 1023;
-    if (e < -1000 || e > 1000) return 1.0 / d;
     const float m = __uint_as_float(0x3F800000u | ((hi & 0xFFFFFu) << 3) | (lo >> 29));   // in [1, 2)
     float rf;
     asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(rf) : "f"(m));
@@ -63,11 +67,16 @@ __device__ __forceinline__ bool bad_pivot(double d, bool lu) {
     return zero || (!lu && (nan || (hi >> 31)));
 }
 
-// the block's elimination in A (see above); UNSYM: A's upper part is its own
-template <int NT, bool UNSYM>
-__device__ __forceinline__ void eliminate(double (*A)[LDB], double *inv, double *ubuf, int nb, bool lu, int64_t gcol0,
+// the block's elimination in A (see above); UNSYM: A's upper part is its own.
+// Quotients by reciprocals, or, DIVIDE, by divisions.  Returns whether it met
+// an extreme pivot and has to be done again with divisions (a test of the
+// exponent beside the chain; on the chain itself, scaled operands cost the 1D
+// case 4.7% and LDL^T on the sphere 4.0%, calls of a division 0 and 1.6%).
+template <int NT, bool UNSYM, bool DIVIDE>
+__device__ __forceinline__ bool eliminate(double (*A)[LDB], double *inv, double *ubuf, int nb, bool lu, int64_t gcol0,
                                           status_t *status) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int first_bad = -1, ext = 0;
 #pragma unroll 1
     for (int jb = 0; jb < nb; jb += S8) {
         const int t0 = jb + S8;
@@ -99,14 +108,15 @@ __device__ __forceinline__ void eliminate(double (*A)[LDB], double *inv, double 
                     bad = bad < 0 && jb + c < nb ? c : bad;
                     dc = 1.0;
                 }
-                const double r = reciprocal(dc);
+                if (!DIVIDE) ext |= extreme(dc) ? 1 : 0;
+                const double r = DIVIDE ? 1.0 / dc : reciprocal(dc);
                 if (lane == c) rl = r, v[c] = dc;
                 __syncwarp();
                 if (lane > c) {
                     const double w = v[c];
-                    double x = w * r;
+                    double x = DIVIDE ? w / dc : w * r;
                     // LU: the quotient to half an ulp, x stays in the factor
-                    if (lu) x = fma(fma(-x, dc, w), r, x);
+                    if (!DIVIDE && lu) x = fma(fma(-x, dc, w), r, x);
                     if (!UNSYM && lane >= S8 && act) A[jb + c][row] = w;
                     v[c] = x;
 #pragma unroll
@@ -114,7 +124,7 @@ __device__ __forceinline__ void eliminate(double (*A)[LDB], double *inv, double 
                 }
                 __syncwarp();
             }
-            if (bad >= 0 && tid == 0) atomicMin(status, (status_t)(gcol0 + jb + bad));
+            if (bad >= 0 && first_bad < 0) first_bad = jb + bad;
             if (tid < S8) inv[jb + tid] = rl;
             if (lane >= S8 && act) {
 #pragma unroll
@@ -175,19 +185,17 @@ __device__ __forceinline__ void eliminate(double (*A)[LDB], double *inv, double 
         }
         __syncthreads();
     }
+    if (!DIVIDE && __syncthreads_or(ext)) return true;
+    if (first_bad >= 0 && tid == 0) atomicMin(status, (status_t)(gcol0 + first_bad));
+    return false;
 }
-
-// Diagonal block kb of front s; all NT >= 128 threads of the CTA; sm holds
-// BLOCK_ELEMS doubles.  The block's values in global memory are final and
-// visible (read past the L1 cache: another CTA may have written them).
+// diagonal block kb of front s into A, the reciprocal pivots set to 1
 template <int NT>
-__device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, double *sm) {
-    double(*A)[LDB] = reinterpret_cast<double(*)[LDB]>(sm);
-    double *inv = sm + OFF_INV;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int k = d.sk[s], ld = d.sld[s], nb = min(NB, k - kb);
-    const int64_t o = d.foff[s] + (int64_t)kb * ld + kb, gcol0 = (int64_t)d.sfirst[s] + kb;
-    const bool lu = a.g != nullptr, nonsym = lu && !a.sym;
+__device__ __forceinline__ void load_block(const DevSym &d, const F64Args &a, int s, int kb, double (*A)[LDB],
+                                           double *inv) {
+    const int tid = threadIdx.x, ld = d.sld[s], nb = min(NB, d.sk[s] - kb);
+    const int64_t o = d.foff[s] + (int64_t)kb * ld + kb;
+    const bool nonsym = a.g != nullptr && !a.sym;
     if (tid < NB) inv[tid] = 1.0;
     // sixteen loads in flight per thread (eight: LDL^T on the sphere 8.92 ms,
     // 1D 1,024 unknowns 0.861; sixteen 8.70 and 0.851)
@@ -210,8 +218,34 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
         }
     }
     __syncthreads();
-    if (nonsym) eliminate<NT, true>(A, inv, sm + OFF_U, nb, true, gcol0, a.status);
-    else eliminate<NT, false>(A, inv, sm + OFF_U, nb, lu, gcol0, a.status);
+}
+
+// the block once more from the front, which still holds its values
+template <int NT>
+__device__ __noinline__ void eliminate_by_division(const DevSym &d, const F64Args &a, int s, int kb, double *sm) {
+    double(*A)[LDB] = reinterpret_cast<double(*)[LDB]>(sm);
+    load_block<NT>(d, a, s, kb, A, sm + OFF_INV);
+    const int nb = min(NB, d.sk[s] - kb);
+    const int64_t gcol0 = (int64_t)d.sfirst[s] + kb;
+    if (a.g != nullptr && !a.sym) eliminate<NT, true, true>(A, sm + OFF_INV, sm + OFF_U, nb, true, gcol0, a.status);
+    else eliminate<NT, false, true>(A, sm + OFF_INV, sm + OFF_U, nb, a.g != nullptr, gcol0, a.status);
+}
+
+// Diagonal block kb of front s; all NT >= 128 threads of the CTA; sm holds
+// BLOCK_ELEMS doubles.  The block's values in global memory are final and
+// visible (read past the L1 cache: another CTA may have written them).
+template <int NT>
+__device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, double *sm) {
+    double(*A)[LDB] = reinterpret_cast<double(*)[LDB]>(sm);
+    double *inv = sm + OFF_INV;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int k = d.sk[s], ld = d.sld[s], nb = min(NB, k - kb);
+    const int64_t o = d.foff[s] + (int64_t)kb * ld + kb, gcol0 = (int64_t)d.sfirst[s] + kb;
+    const bool lu = a.g != nullptr, nonsym = lu && !a.sym;
+    load_block<NT>(d, a, s, kb, A, inv);
+    const bool again = nonsym ? eliminate<NT, true, false>(A, inv, sm + OFF_U, nb, true, gcol0, a.status)
+                              : eliminate<NT, false, false>(A, inv, sm + OFF_U, nb, lu, gcol0, a.status);
+    if (again) eliminate_by_division<NT>(d, a, s, kb, sm);
     if (!lu) {
         // L = x sqrt(d); the reciprocal roots, and the roots (one correction
         // step) on the diagonal
