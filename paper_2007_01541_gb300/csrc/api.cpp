@@ -121,11 +121,9 @@ struct wd_ctx {
     int32_t *d_csr_src = nullptr;
     double *d_csr_val = nullptr;
     // LU without pivoting (wd_factor_lu, FP64): position codes of the full
-    // CSR, both values per position, the fronts of U^T and the inverses of
-    // their diagonal blocks
+    // CSR, both values per position, the inverses of U^T's diagonal blocks
     bool lu_factored = false;
     bool ldlt = false;          // the LU factor is that of a symmetric matrix (wd_factor_ldlt)
-    void *d_front_u = nullptr;
     GraphCache g_lu;
     std::vector<int8_t> h_csr_code;
     int8_t *d_lu_code = nullptr;
@@ -887,7 +885,6 @@ static wd_status reset_analysis(wd_handle h) {
     h->d_dinv = nullptr;
     h->d_gcsr = h->mass_buf = nullptr;
     h->lu_factored = false;
-    h->d_front_u = nullptr;
     h->g_lu.reset();
     h->d_lu_code = nullptr;
     h->d_vrow = h->d_vcol = h->d_uinv = h->d_lu_part = h->d_upper_stage = nullptr;
@@ -1043,7 +1040,7 @@ static wd_status finish_analysis(wd_handle h, std::chrono::steady_clock::time_po
         foff[s] = fo;
         woff[s] = wo;
         dioff[s] = dio;
-        fo += (int64_t)sld[s] * mp;
+        fo += sld[s] * wd::front_cols(mp);
         wo += sm[s] - sk[s];
         dio += (int64_t)((sk[s] + NB - 1) / NB) * NB * NB;
         pkoff[s] = pko;
@@ -1672,7 +1669,6 @@ static wd_status ensure_solve_ws(wd_handle h, int64_t nrhs) {
 template <class T>
 static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, bool prof, bool lu) {
     const T *F = static_cast<const T *>(h->d_front);
-    const T *Fb = lu ? static_cast<const T *>(h->d_front_u) : F;
     const T *Xs = static_cast<const T *>(h->d_xs);
     const T *XTs = static_cast<const T *>(h->d_xts);
     T *W = static_cast<T *>(h->d_W);
@@ -1736,9 +1732,9 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.ksr = L.arg;
                     wd::launch_tc_breduce(d, a, it, L.count, st);
                 } else if (lg == 2) {
-                    wd::launch_rnarrow<T>(d, Fb, Y, P, it, L.count, nrhs, st);
+                    wd::launch_rnarrow<T>(d, F, Y, P, it, L.count, nrhs, st, lu);
                 } else {
-                    wd::launch_breduce<T>(d, Fb, Y, P, it, L.count, nrhs, st);
+                    wd::launch_breduce<T>(d, F, Y, P, it, L.count, nrhs, st, lu);
                 }
                 break;
             case K_BWD_FINISH: wd::launch_breduce_finish<T>(d, Y, Tt, P, it, L.count, lg, nrhs, st); break;
@@ -2623,7 +2619,7 @@ static void enqueue_lu_plan(wd_handle h, cudaStream_t st, bool sym) {
     const Plan &P = h->fplan;
     wd::F64Args fa{};
     fa.f = static_cast<double *>(h->d_front);
-    fa.g = static_cast<double *>(h->d_front_u);
+    fa.lu = 1;
     fa.di = static_cast<double *>(h->d_dinv);
     fa.du = h->d_uinv;
     fa.sym = sym ? 1 : 0;
@@ -2639,7 +2635,7 @@ static void enqueue_lu_plan(wd_handle h, cudaStream_t st, bool sym) {
                 wd::launch_front_init<double>(dv, fa.f, it, L.count, st);
                 if (sym) break;
                 dv.csr_val = h->d_vrow;
-                wd::launch_front_init<double>(dv, fa.g, it, L.count, st);
+                wd::launch_front_init<double>(dv, fa.f, it, L.count, st, true);
                 break;
             }
             case K_DIAG: wd::launch_diag64(d, fa, it, L.count, st); break;
@@ -2653,13 +2649,14 @@ static void enqueue_lu_plan(wd_handle h, cudaStream_t st, bool sym) {
     for (int side = 1; side >= 0; --side)
         for (const Launch &L : P.launches) {
             const int4 *it = P.d_items + L.off;
-            const double *F = side ? fa.g : fa.f;
             double *D = side ? fa.du : fa.di;
             switch (L.kind) {
-                case K_SBINV_DIAG: wd::launch_sbinv_diag64(d, F, D, xs, h->d_xsoff, it, L.count, st); break;
+                case K_SBINV_DIAG:
+                    wd::launch_sbinv_diag64(d, fa.f, D, xs, h->d_xsoff, it, L.count, st, side != 0);
+                    break;
                 case K_SBINV_STAGE:
-                    wd::launch_sbinv_double<double>(d, F, xs, xts, h->d_xsoff, it, L.count, L.arg / 2, L.arg % 2,
-                                                    st);
+                    wd::launch_sbinv_double<double>(d, fa.f, xs, xts, h->d_xsoff, it, L.count, L.arg / 2, L.arg % 2,
+                                                    st, side != 0);
                     break;
                 case K_SBINV_T:
                     if (side) wd::launch_sbinv_transpose<double>(d, xs, xts, h->d_xsoff, it, L.count, st);
@@ -2706,10 +2703,6 @@ static wd_status factor_lu(wd_handle h, const double *lower, const double *upper
     if (!h->d_dinv) CK(h->mem.alloc(&h->d_dinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
     if (!h->d_xs) CK(h->mem.alloc(&h->d_xs, h->xs_elems * sizeof(double)), "super-block inverse alloc");
     if (!h->d_xts) CK(h->mem.alloc(&h->d_xts, h->xs_elems * sizeof(double)), "super-block inverse alloc");
-    if (!h->d_front_u) {
-        CK(h->mem.alloc(&h->d_front_u, h->front_elems * sizeof(double)), "front pool alloc");
-        CK(cudaMemsetAsync(h->d_front_u, 0, h->front_elems * sizeof(double), st), "front pool clear");
-    }
     if (!h->d_uinv) CK(h->mem.alloc((void **)&h->d_uinv, h->dinv_elems * sizeof(double)), "inverse blocks alloc");
     if (!h->d_vrow) CK(h->mem.alloc((void **)&h->d_vrow, h->nnz_full * sizeof(double)), "values alloc");
     if (!h->d_vcol) CK(h->mem.alloc((void **)&h->d_vcol, h->nnz_full * sizeof(double)), "values alloc");
@@ -2893,8 +2886,7 @@ extern "C" wd_status wd_export_LU(wd_handle h, double *lpanels, double *utpanels
         return cuda_fail(h, cudaErrorMemoryAllocation, "export alloc");
     }
     cudaMemcpy(d_poff, poff.data(), S.ns * sizeof(int64_t), cudaMemcpyHostToDevice);
-    wd::launch_lu_export(h->dsym, static_cast<const double *>(h->d_front),
-                         static_cast<const double *>(h->d_front_u), d_out, d_out + tot, d_poff, 0);
+    wd::launch_lu_export(h->dsym, static_cast<const double *>(h->d_front), d_out, d_out + tot, d_poff, 0);
     cudaError_t e = cudaMemcpy(lpanels, d_out, tot * sizeof(double), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(utpanels, d_out + tot, tot * sizeof(double), cudaMemcpyDeviceToHost);
     cudaFree(d_out);

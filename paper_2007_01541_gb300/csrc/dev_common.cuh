@@ -54,6 +54,29 @@ inline void launch_dependent(void (*kernel)(P...), unsigned blocks, unsigned thr
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// The columns of one triangular front (entries r >= c).  L's is column-major
+// with leading dimension ld in the front's place of the pool.  U^T's (LU, FP64)
+// fills the part above L's diagonal and two more columns (front_cols), column
+// after column backwards, every pair of columns two entries further up:
+//   L(r, c) at c ld + r,   U^T(r, c) at (mp + 1 - c) ld + r - 2 (c / 2):
+// column c of U^T takes rows 0 .. mp - c of column mp + 1 - c at most, which are
+// above L's diagonal, and starts on 16 bytes as L's do.  Offsets from an even
+// column c0 are those from column 0: col(c0 + p) = col(c0) + p ld - (p & cut).
+template <class T>
+struct FrontCols {
+    T *p;
+    int ld, cut;
+    __device__ __forceinline__ T *col(int c) const { return p + ((int64_t)c * ld - (c & cut)); }
+};
+template <bool UT, class T>
+__device__ __forceinline__ FrontCols<T> front_columns(const DevSym &d, T *pool, int s) {
+    const int ld = d.sld[s];
+    T *f = pool + d.foff[s];
+    if (!UT) return {f, ld, 0};
+    const int mp = d.skp[s] + d.sm[s] - d.sk[s];
+    return {f + (mp + (int64_t)1) * ld, -ld, ~1};
+}
+
 // Column maxima of the backward error: max |r|, |x| and |b| (NaN does not
 // count), then a word of flags: r or x, and b, held a value that is not finite
 struct ColMax {
@@ -90,14 +113,14 @@ __device__ __forceinline__ void cp_async_elem(T *smem, const T *gmem, bool valid
     else cp_async4(smem, valid ? gmem : smem, valid ? 4 : 0);
 }
 
-// Stage a tile of `rows` x `cols` elements, column c starting at g + c*ldg
-// (columns contiguous in global memory, 16-byte aligned, rows a multiple of
+// Stage a tile of `rows` x `cols` elements, column c starting at g + c*ldg - (c & cut)
+// (FrontCols; columns contiguous in global memory, 16-byte aligned, rows a multiple of
 // the vector width), into shared memory s + c*lds (lds a multiple of the
 // vector width).  Rows >= rvalid (and columns >= cvalid) are zero-filled.
 // Issues cp.async only; the caller commits and waits.
 template <class T, int THREADS>
 __device__ __forceinline__ void stage_tile(T *s, int lds, const T *g, int64_t ldg, int rows,
-                                           int cols, int rvalid, int cvalid) {
+                                           int cols, int rvalid, int cvalid, int cut = 0) {
     constexpr int V = 16 / sizeof(T);  // elements per 16-byte vector
     const int vpc = rows / V;          // vectors per column
     const int total = vpc * cols;
@@ -105,7 +128,7 @@ __device__ __forceinline__ void stage_tile(T *s, int lds, const T *g, int64_t ld
         const int c = idx / vpc, r = (idx % vpc) * V;
         int valid = (c < cvalid) ? rvalid - r : 0;
         valid = valid < 0 ? 0 : (valid > V ? V : valid);
-        const T *src = valid ? g + (int64_t)c * ldg + r : g;
+        const T *src = valid ? g + ((int64_t)c * ldg - (c & cut)) + r : g;
         cp_async16(s + c * lds + r, src, valid * (int)sizeof(T));
     }
 }

@@ -11,6 +11,10 @@ using status_t = unsigned long long;
 constexpr int NB = 64;        // pivot block width and Schur tile size
 constexpr int RB = 64;        // rows per panel (TRSM) block
 
+// Columns of the front pool per front of mp rows: the front's, and two more so
+// that the upper part holds a second triangle of the same order (U^T of LU)
+constexpr int64_t front_cols(int64_t mp) { return mp + 2; }
+
 // Device pointers of the analysis (all arrays are owned by the handle).
 struct DevSym {
     int64_t n;
@@ -20,7 +24,7 @@ struct DevSym {
     const int32_t *sm;          // ns: number of front rows m_s
     const int32_t *skp;         // ns: k_s rounded up to 32 (first row of R in the front)
     const int32_t *sld;         // ns: leading dimension of the front (multiple of 32)
-    const int64_t *foff;        // ns: offset of front s in the front pool
+    const int64_t *foff;        // ns: offset of front s in the front pool (front_cols(mp) columns of sld)
     const int64_t *rowptr;      // ns+1: offset of the rows of s
     const int32_t *rows;        // front rows (global permuted indices)
     const int32_t *child_ptr;   // ns+1
@@ -60,8 +64,9 @@ inline void init_kernel_attributes() {
 
 
 // ---- factorization (front_kernels.cu) ------------------------------------
+// ut (FP64): the fronts of U^T
 template <class T>
-void launch_front_init(const DevSym &d, T *front, const int4 *items, int count, cudaStream_t st);
+void launch_front_init(const DevSym &d, T *front, const int4 *items, int count, cudaStream_t st, bool ut = false);
 // diagonal block (s, kb) of each item: L11 into the front, L11^-1 into dinv
 // at dinvoff + (kb / NB) NB^2; FP32 fronts of width >= diag64_min_k (> 0)
 // factor the block in FP64
@@ -76,14 +81,14 @@ void launch_panel(const DevSym &d, T *front, const T *dinv, unsigned char *pk, c
 // tile of the plans' FP64 update items
 constexpr int SCHUR_BM = 128, SCHUR_BN = 64;
 
-// FP64 fronts (front64.cu): Cholesky (g = nullptr), or LU with the fronts of
-// U^T beside those of L
+// FP64 fronts (front64.cu): Cholesky, or LU with the fronts of U^T in the upper
+// parts of those of L (FrontCols)
 struct F64Args {
-    double *f;          // fronts: L
-    double *g;          // LU: fronts of U^T
+    double *f;          // fronts
+    int lu;
     double *di, *du;    // inverses of the diagonal blocks of L and U^T: the 16 x 16 diagonal sub-blocks
                         // (the diagonal's entries are the reciprocal pivots), completed by sbinv_diag64
-    int sym;            // LU of a symmetric matrix: U^T = L D comes out of L's panels, g is not assembled
+    int sym;            // LU of a symmetric matrix: U^T = L D comes out of L's panels, its fronts are not assembled
     int *cnt;           // per supernode: arrivals at the next diagonal block (zero between launches)
     status_t *status;
 };
@@ -95,7 +100,7 @@ void launch_panel64(const DevSym &d, const F64Args &a, const int4 *items, int co
 void launch_update64(const DevSym &d, const F64Args &a, const int4 *items, int count, int kb, int mode,
                      cudaStream_t st);
 void launch_sbinv_diag64(const DevSym &d, const double *front, double *dinv, double *xpool, const int64_t *xsoff,
-                         const int4 *items, int count, cudaStream_t st);
+                         const int4 *items, int count, cudaStream_t st, bool ut = false);
 
 // Packed tf32 operand lines of a supernode's L panel (FP32 fronts, tensor-core
 // Schur updates): for each chunk kc of 32 pivot columns and plane p (0 = hi,
@@ -293,7 +298,7 @@ void launch_sbinv_diag(const DevSym &d, const float *dinv, float *xpool, const i
 // columns in place; tpool: the transposes' store (scratch in its lower blocks)
 template <class T>
 void launch_sbinv_double(const DevSym &d, const T *front, T *xpool, T *tpool, const int64_t *xsoff,
-                         const int4 *items, int count, int hb, int phase, cudaStream_t st);
+                         const int4 *items, int count, int hb, int phase, cudaStream_t st, bool ut = false);
 template <class T>
 void launch_sbinv_transpose(const DevSym &d, const T *xpool, T *xtpool, const int64_t *xsoff,
                             const int4 *items, int count, cudaStream_t st);
@@ -330,13 +335,13 @@ void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, co
                     cudaStream_t st);
 template <class T>
 void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
-                    cudaStream_t st);
+                    cudaStream_t st, bool ut = false);
 // split reduction of the backward pass: partial sums of KSR-row splits into
 // P (rows x rhs of the tile per slot), then Tt = y - sum over the splits in order
 constexpr int SOLVE_KSR = 128;
 template <class T>
 void launch_breduce(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count,
-                    int nrhs, cudaStream_t st);
+                    int nrhs, cudaStream_t st, bool ut = false);
 template <class T>
 void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const int4 *items, int count,
                            int large, int nrhs, cudaStream_t st);
@@ -392,8 +397,8 @@ void launch_lu_gather(const int32_t *src, const int8_t *code, const double *lowe
 // partial[nblocks + b] = the number of negative pivots there
 void launch_lu_logdet(const DevSym &d, const double *front, double *partial, int nblocks, cudaStream_t st);
 // factor panels for export: L with its unit diagonal, and U^T, each m_s x k_s per supernode
-void launch_lu_export(const DevSym &d, const double *front, const double *ufront, double *lpan, double *upan,
-                      const int64_t *poff, cudaStream_t st);
+void launch_lu_export(const DevSym &d, const double *front, double *lpan, double *upan, const int64_t *poff,
+                      cudaStream_t st);
 
 // ---- allocation-free export of the factor (noalloc.cu) ---------------------
 // the panel offsets sit in a static device array of NOALLOC_MAX_SUPERNODES + 1

@@ -3,8 +3,9 @@
 //
 // Both keep triangular fronts (column-major, lower part; rows: k_s pivot rows,
 // zero padding to kp_s, the rows below).  Cholesky has one, F, which becomes
-// L.  LU has two of the same layout: F becomes L (unit lower; its diagonal
-// holds U's) and G becomes U^T.  With A^T's fronts beside A's, every step of
+// L.  LU has two of the same shape: F becomes L (unit lower; its diagonal
+// holds U's) and G, in the upper part of F's square (FrontCols), becomes U^T:
+// one pool, as for Cholesky.  With A^T's fronts in reach of A's, every step of
 // LU has the form of a Cholesky step with the operands taken from both:
 //   diagonal   F11 = L11 U11
 //   panel      L21 = F21 U11^-1 = F21 (U^T)11^-T,   (U^T)21 = G21 L11^-T
@@ -75,6 +76,7 @@ constexpr int PLD = NB + 2;      // row stride of the staged T (16-byte multiple
 constexpr int PXL = PR + 2;      // column stride of the staged rows
 constexpr int PANEL_ELEMS = NB * PLD + NB * PXL + PR * (PR + 1) + 2 * NB;
 
+template <bool LU>
 __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const int4 *__restrict__ items, int kb,
                                                       int sides) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -91,33 +93,36 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
     const int r0 = (t0 == z.k ? z.kp : t0) + rb * RB + q * PR;
     if (r0 >= z.mp) return;
     // Cholesky and the symmetric case read T from F; LU from the other side
-    const bool lu = a.g != nullptr && !a.sym;
-    double *C = (side == 0 ? a.f : a.g) + d.foff[s];
-    const double *T = (lu && side == 0 ? a.g : a.f) + d.foff[s] + (int64_t)kb * z.ld + kb;
+    const bool lu = LU && !a.sym;
+    const FrontCols<double> f = front_columns<false>(d, a.f, s), g = front_columns<LU>(d, a.f, s);
+    const FrontCols<double> C = side == 0 ? f : g;
+    FrontCols<double> T = lu && side == 0 ? g : f;
+    T.p = T.col(kb) + kb;
     const double *Dv = (lu && side == 0 ? a.du : a.di) + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB;
     const int tid = threadIdx.x;
     for (int idx = tid; idx < NB * (NB / 2); idx += T64) {
         const int p = idx / (NB / 2), c = (idx % (NB / 2)) * 2;   // two rows c, c + 1 of column p
         const int bp = p / 16, bc = c / 16;
-        const double *src = bc == bp ? Dv + p * NB + c : T + (int64_t)p * z.ld + c;
+        const double *src = bc == bp ? Dv + p * NB + c : T.col(p) + c;
         const int valid = (p < nb && bc >= bp && c < nb) ? min(2, nb - c) : 0;
         cp_async16(Ts + p * PLD + c, valid ? src : Dv, 8 * valid);
     }
     for (int idx = tid; idx < NB * (PR / 2); idx += T64) {
         const int p = idx / (PR / 2), r = (idx % (PR / 2)) * 2;
         const int valid = p < nb ? max(0, min(2, z.mp - (r0 + r))) : 0;
-        cp_async16(Xs + p * PXL + r, valid ? C + (int64_t)(kb + p) * z.ld + r0 + r : Dv, 8 * valid);
+        cp_async16(Xs + p * PXL + r, valid ? C.col(kb + p) + r0 + r : Dv, 8 * valid);
     }
     cp_async_commit();
     int extreme = 0;        // some pivot is: divisions
-    if (a.sym && tid < nb) {
-        const double dv = T[(int64_t)tid * z.ld + tid];
+    if (LU && a.sym && tid < nb) {
+        const double dv = T.col(tid)[tid];
         rd[tid] = 1.0 / dv;
         rd[NB + tid] = dv;
         extreme = f64::extreme(dv);
     }
     cp_async_wait<0>();
-    extreme = __syncthreads_or(extreme);
+    if (LU) extreme = __syncthreads_or(extreme);
+    else __syncthreads();
     const int c = tid % 16, ra = tid / 16;      // rows ra, ra + 8
     const int nblk = (nb + 15) / 16;
     for (int b = 0; b < nblk; ++b) {
@@ -145,17 +150,16 @@ __global__ void __launch_bounds__(T64) panel64_kernel(DevSym d, F64Args a, const
         __syncthreads();
     }
     for (int idx = tid; idx < nb * PR; idx += T64) {
-        const int r = idx % PR, p = idx / PR;
-        if (r0 + r >= z.mp) continue;
-        const double v = Xs[p * PXL + r];
-        const int64_t o = (int64_t)(kb + p) * z.ld + r0 + r;
-        if (a.sym) {
+        const int row = idx % PR, p = idx / PR;
+        if (r0 + row >= z.mp) continue;
+        const double v = Xs[p * PXL + row];
+        if (LU && a.sym) {
             // v / d to half an ulp, by the reciprocal and one correction
             const double r = rd[p], x = v * r;
-            a.g[d.foff[s] + o] = v;
-            C[o] = extreme ? v / rd[NB + p] : fma(fma(-x, rd[NB + p], v), r, x);
+            g.col(kb + p)[r0 + row] = v;
+            C.col(kb + p)[r0 + row] = extreme ? v / rd[NB + p] : fma(fma(-x, rd[NB + p], v), r, x);
         } else {
-            C[o] = v;
+            C.col(kb + p)[r0 + row] = v;
         }
     }
 }
@@ -175,6 +179,7 @@ constexpr int UT = 32, UK = 32;
 constexpr int SUBR = SCHUR_BM / UT, SUBS = SUBR * (SCHUR_BN / UT);
 constexpr size_t UPDATE_BYTES = sizeof(double) * (2 * UK * 2 * UT > f64::BLOCK_ELEMS ? 2 * UK * 2 * UT : f64::BLOCK_ELEMS);
 
+template <bool LU>
 __global__ void __launch_bounds__(T64) update64_kernel(DevSym d, F64Args a, const int4 *__restrict__ items, int kb,
                                                        int mode, int sides) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -194,13 +199,12 @@ __global__ void __launch_bounds__(T64) update64_kernel(DevSym d, F64Args a, cons
     const bool live = r0 < z.mp && c0 < cmax && r0 + UT > c0;
     const int tid = threadIdx.x;
     if (live) {
-        const double *A = (side == 0 ? a.f : a.g) + d.foff[s] + (int64_t)ka * z.ld + r0;
-        const double *B = (side == 0 && a.g != nullptr ? a.g : a.f) + d.foff[s] + (int64_t)ka * z.ld + c0;
-        double *C = (side == 0 ? a.f : a.g) + d.foff[s];
+        const FrontCols<double> f = front_columns<false>(d, a.f, s), g = front_columns<LU>(d, a.f, s);
+        const FrontCols<double> A = side == 0 ? f : g, B = LU && side == 0 ? g : f, C = A;
         const int tx = tid % 8, ty = tid / 8;
         auto stage = [&](int buf, int k0) {
-            stage_tile<double, T64>(As[buf], UT, A + (int64_t)k0 * z.ld, z.ld, UT, UK, z.mp - r0, K - k0);
-            stage_tile<double, T64>(Bs[buf], UT, B + (int64_t)k0 * z.ld, z.ld, UT, UK, cmax - c0, K - k0);
+            stage_tile<double, T64>(As[buf], UT, A.col(ka + k0) + r0, A.ld, UT, UK, z.mp - r0, K - k0, A.cut);
+            stage_tile<double, T64>(Bs[buf], UT, B.col(ka + k0) + c0, B.ld, UT, UK, cmax - c0, K - k0, B.cut);
             cp_async_commit();
         };
         stage(0, 0);
@@ -239,14 +243,14 @@ __global__ void __launch_bounds__(T64) update64_kernel(DevSym d, F64Args a, cons
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const bool v = r + i < z.mp && c + j < cmax && r + i >= c + j;
-                old[i][j] = v ? C[(int64_t)(c + j) * z.ld + r + i] : 0.0;
+                old[i][j] = v ? C.col(c + j)[r + i] : 0.0;
             }
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (r + i < z.mp && c + j < cmax && r + i >= c + j)
-                    C[(int64_t)(c + j) * z.ld + r + i] = old[i][j] - acc[i][j];
+                    C.col(c + j)[r + i] = old[i][j] - acc[i][j];
     }
     if (diag) {
         __threadfence();
@@ -272,6 +276,7 @@ __global__ void __launch_bounds__(T64) update64_kernel(DevSym d, F64Args a, cons
 // matrix in one launch, off the factorization's serial chain.
 // ---------------------------------------------------------------------------
 constexpr int SI_THREADS = 256;
+template <bool UT>
 __global__ void __launch_bounds__(SI_THREADS) sbinv_diag64_kernel(DevSym d, const double *__restrict__ front,
                                                                   double *__restrict__ dinv,
                                                                   double *__restrict__ xpool,
@@ -281,13 +286,14 @@ __global__ void __launch_bounds__(SI_THREADS) sbinv_diag64_kernel(DevSym d, cons
     double *sm = reinterpret_cast<double *>(smem_raw);
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y, t = it.z;
-    const int k = d.sk[s], ld = d.sld[s], kb = sb * SB + t * NB;
+    const int k = d.sk[s], kb = sb * SB + t * NB;
     const int nb = min(NB, k - kb);
     const int w = min(SB, k - sb * SB), wp = (w + NB - 1) / NB * NB;
     double *Dv = dinv + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB;
     double *XT = sm + blk::BP_XT, *invd = sm + blk::BP_INVD;
     if (threadIdx.x < nb) invd[threadIdx.x] = Dv[threadIdx.x * (NB + 1)];
-    blk::block_load<double, double, SI_THREADS>(front + d.foff[s] + (int64_t)kb * ld + kb, ld, nb, sm);
+    const FrontCols<const double> f = front_columns<UT>(d, front, s);
+    blk::block_load<double, double, SI_THREADS>(f.col(kb) + kb, f.ld, nb, sm, f.cut);
     blk::block_inverse<double, SI_THREADS>(nb, reinterpret_cast<const double(*)[NB + 1]>(sm), XT, invd);
     double *X = xpool + xsoff[s] + (int64_t)sb * SB * SB + (int64_t)(t * NB) * wp + t * NB;
     for (int idx = threadIdx.x; idx < NB * NB; idx += SI_THREADS) {
@@ -303,14 +309,16 @@ __global__ void __launch_bounds__(SI_THREADS) sbinv_diag64_kernel(DevSym d, cons
 void init_front64_attributes() {
     static bool done = false;
     if (done) return;
-    cudaFuncSetAttribute(panel64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(PANEL_ELEMS * sizeof(double)));
-    cudaFuncSetAttribute(sbinv_diag64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)blk::block_smem_bytes<double>());
+    for (auto *kernel : {panel64_kernel<false>, panel64_kernel<true>})
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(PANEL_ELEMS * sizeof(double)));
+    for (auto *kernel : {sbinv_diag64_kernel<false>, sbinv_diag64_kernel<true>})
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)blk::block_smem_bytes<double>());
     done = true;
 }
 
-static int sides_of(const F64Args &a) { return a.g != nullptr && !a.sym ? 2 : 1; }
+static int sides_of(const F64Args &a) { return a.lu && !a.sym ? 2 : 1; }
 
 void launch_diag64(const DevSym &d, const F64Args &a, const int4 *items, int count, cudaStream_t st) {
     if (count > 0) diag64_kernel<<<count, T64, f64::BLOCK_ELEMS * sizeof(double), st>>>(d, a, items);
@@ -319,20 +327,22 @@ void launch_panel64(const DevSym &d, const F64Args &a, const int4 *items, int co
     if (count <= 0) return;
     init_front64_attributes();
     const int sides = sides_of(a);
-    panel64_kernel<<<count * sides * (RB / PR), T64, PANEL_ELEMS * sizeof(double), st>>>(d, a, items, kb, sides);
+    auto *kernel = a.lu ? panel64_kernel<true> : panel64_kernel<false>;
+    kernel<<<count * sides * (RB / PR), T64, PANEL_ELEMS * sizeof(double), st>>>(d, a, items, kb, sides);
 }
 void launch_update64(const DevSym &d, const F64Args &a, const int4 *items, int count, int kb, int mode,
                      cudaStream_t st) {
     if (count <= 0) return;
     const int sides = sides_of(a);
-    update64_kernel<<<count * sides * SUBS, T64, UPDATE_BYTES, st>>>(d, a, items, kb, mode, sides);
+    auto *kernel = a.lu ? update64_kernel<true> : update64_kernel<false>;
+    kernel<<<count * sides * SUBS, T64, UPDATE_BYTES, st>>>(d, a, items, kb, mode, sides);
 }
 void launch_sbinv_diag64(const DevSym &d, const double *front, double *dinv, double *xpool, const int64_t *xsoff,
-                         const int4 *items, int count, cudaStream_t st) {
+                         const int4 *items, int count, cudaStream_t st, bool ut) {
     if (count <= 0) return;
     init_front64_attributes();
-    sbinv_diag64_kernel<<<count, SI_THREADS, blk::block_smem_bytes<double>(), st>>>(d, front, dinv, xpool, xsoff,
-                                                                                  items);
+    auto *kernel = ut ? sbinv_diag64_kernel<true> : sbinv_diag64_kernel<false>;
+    kernel<<<count, SI_THREADS, blk::block_smem_bytes<double>(), st>>>(d, front, dinv, xpool, xsoff, items);
 }
 
 }  // namespace wd

@@ -21,6 +21,7 @@
 // A pivot that is not positive (LU: that is zero) records its column in
 // *status (smallest wins) and is replaced by 1.
 #pragma once
+#include "dev_common.cuh"
 #include "engine.h"
 
 namespace wd {
@@ -193,9 +194,11 @@ __device__ __forceinline__ bool eliminate(double (*A)[LDB], double *inv, double 
 template <int NT>
 __device__ __forceinline__ void load_block(const DevSym &d, const F64Args &a, int s, int kb, double (*A)[LDB],
                                            double *inv) {
-    const int tid = threadIdx.x, ld = d.sld[s], nb = min(NB, d.sk[s] - kb);
-    const int64_t o = d.foff[s] + (int64_t)kb * ld + kb;
-    const bool nonsym = a.g != nullptr && !a.sym;
+    const int tid = threadIdx.x, nb = min(NB, d.sk[s] - kb);
+    const bool nonsym = a.lu && !a.sym;
+    FrontCols<double> f = front_columns<false>(d, a.f, s), g = front_columns<true>(d, a.f, s);
+    f.p = f.col(kb) + kb;
+    g.p = g.col(kb) + kb;
     if (tid < NB) inv[tid] = 1.0;
     // sixteen loads in flight per thread (eight: LDL^T on the sphere 8.92 ms,
     // 1D 1,024 unknowns 0.861; sixteen 8.70 and 0.851)
@@ -206,8 +209,8 @@ __device__ __forceinline__ void load_block(const DevSym &d, const F64Args &a, in
         for (int u = 0; u < U; ++u) {
             const int idx = i0 + u * NT, r = idx % NB, c = idx / NB;
             const bool in = c <= r && r < nb;
-            v[u] = in ? __ldcg(a.f + o + (int64_t)c * ld + r) : (r == c ? 1.0 : 0.0);
-            w[u] = in && nonsym ? __ldcg(a.g + o + (int64_t)c * ld + r) : 0.0;
+            v[u] = in ? __ldcg(f.col(c) + r) : (r == c ? 1.0 : 0.0);
+            w[u] = in && nonsym ? __ldcg(g.col(c) + r) : 0.0;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -227,8 +230,8 @@ __device__ __noinline__ void eliminate_by_division(const DevSym &d, const F64Arg
     load_block<NT>(d, a, s, kb, A, sm + OFF_INV);
     const int nb = min(NB, d.sk[s] - kb);
     const int64_t gcol0 = (int64_t)d.sfirst[s] + kb;
-    if (a.g != nullptr && !a.sym) eliminate<NT, true, true>(A, sm + OFF_INV, sm + OFF_U, nb, true, gcol0, a.status);
-    else eliminate<NT, false, true>(A, sm + OFF_INV, sm + OFF_U, nb, a.g != nullptr, gcol0, a.status);
+    if (a.lu && !a.sym) eliminate<NT, true, true>(A, sm + OFF_INV, sm + OFF_U, nb, true, gcol0, a.status);
+    else eliminate<NT, false, true>(A, sm + OFF_INV, sm + OFF_U, nb, a.lu, gcol0, a.status);
 }
 
 // Diagonal block kb of front s; all NT >= 128 threads of the CTA; sm holds
@@ -239,9 +242,9 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
     double(*A)[LDB] = reinterpret_cast<double(*)[LDB]>(sm);
     double *inv = sm + OFF_INV;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int k = d.sk[s], ld = d.sld[s], nb = min(NB, k - kb);
-    const int64_t o = d.foff[s] + (int64_t)kb * ld + kb, gcol0 = (int64_t)d.sfirst[s] + kb;
-    const bool lu = a.g != nullptr, nonsym = lu && !a.sym;
+    const int k = d.sk[s], nb = min(NB, k - kb);
+    const int64_t gcol0 = (int64_t)d.sfirst[s] + kb;
+    const bool lu = a.lu, nonsym = lu && !a.sym;
     load_block<NT>(d, a, s, kb, A, inv);
     const bool again = nonsym ? eliminate<NT, true, false>(A, inv, sm + OFF_U, nb, true, gcol0, a.status)
                               : eliminate<NT, false, false>(A, inv, sm + OFF_U, nb, lu, gcol0, a.status);
@@ -321,17 +324,20 @@ __device__ void factor_block(const DevSym &d, const F64Args &a, int s, int kb, d
             X21[r + 4] = t1;
         }
     }
+    FrontCols<double> f = front_columns<false>(d, a.f, s), g = front_columns<true>(d, a.f, s);
+    f.p = f.col(kb) + kb;
+    g.p = g.col(kb) + kb;
     for (int idx = tid; idx < NB * NB; idx += NT) {
         const int r = idx % NB, c = idx / NB;
         if (r < c || r >= nb) continue;
-        a.f[o + (int64_t)c * ld + r] = A[r][c];
-        if (lu) a.g[o + (int64_t)c * ld + r] = A[c][r];
+        f.col(c)[r] = A[r][c];
+        if (lu) g.col(c)[r] = A[c][r];
     }
     // LDL^T does not assemble U^T's fronts, and no panel covers the padding
     // rows of the last block: the solves multiply them by zero
     if (lu && a.sym && kb + nb == k) {
         const int pad = d.skp[s] - k;
-        for (int idx = tid; idx < nb * pad; idx += NT) a.g[o + (int64_t)(idx / pad) * ld + nb + idx % pad] = 0.0;
+        for (int idx = tid; idx < nb * pad; idx += NT) g.col(idx / pad)[nb + idx % pad] = 0.0;
     }
 }
 

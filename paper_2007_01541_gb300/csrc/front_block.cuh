@@ -103,12 +103,12 @@ constexpr int BP_ELEMS = BP_COL + SB;
 template <class TC>
 constexpr size_t block_smem_bytes() { return sizeof(TC) * BP_ELEMS; }
 
-// Loads the lower part of the nb x nb block at F (column-major, ld) into A
-// (converted to TC, zero outside the block) and zeroes XT.  All of a thread's
+// Loads the lower part of the nb x nb block at F (column c at c ld - (c & cut),
+// FrontCols) into A (converted to TC, zero outside the block) and zeroes XT.  All of a thread's
 // loads are issued before the first store, so their latencies overlap.  Ends
 // with a block barrier.
 template <class TC, class TF, int NT>
-__device__ void block_load(const TF *F, int ld, int nb, TC *smem) {
+__device__ void block_load(const TF *F, int ld, int nb, TC *smem, int cut = 0) {
     TC(*A)[NB + 1] = reinterpret_cast<TC(*)[NB + 1]>(smem);
     TC *XT = smem + BP_XT;
     constexpr int PER = (NB * NB + NT - 1) / NT;
@@ -117,7 +117,7 @@ __device__ void block_load(const TF *F, int ld, int nb, TC *smem) {
     for (int u = 0; u < PER; ++u) {
         const int idx = threadIdx.x + u * NT;
         const int r = idx % NB, c = idx / NB;
-        v[u] = (idx < NB * NB && r >= c && r < nb && c < nb) ? F[(int64_t)c * ld + r] : TF(0);
+        v[u] = (idx < NB * NB && r >= c && r < nb && c < nb) ? F[(int64_t)c * ld - (c & cut) + r] : TF(0);
     }
 #pragma unroll
     for (int u = 0; u < PER; ++u) {

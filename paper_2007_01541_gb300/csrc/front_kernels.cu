@@ -73,7 +73,7 @@ __device__ __forceinline__ Dims dims(const DevSym &d, int s) {
 constexpr int INIT_ROWS = 128;
 constexpr int INIT_MAXCH = 16;   // children staged at once (more are taken in groups)
 
-template <class T>
+template <class T, bool UT>
 __global__ void __launch_bounds__(THREADS) front_init_kernel(DevSym d, T *__restrict__ front,
                                                              const int4 *__restrict__ items,
                                                              int count) {
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(THREADS) front_init_kernel(DevSym d, T *__rest
     const Dims z = dims(d, s);
     const int pad = z.kp - z.k;
     const int qc = q < 0 ? -1 : (q < z.k ? q : (q < z.kp ? -1 : q - pad));   // local column
-    T *F = front + d.foff[s] + (int64_t)max(q, 0) * z.ld;
+    T *F = front_columns<UT>(d, front, s).col(max(q, 0));
     const int cb = d.child_ptr[s], ce = d.child_ptr[s + 1];
     // first row slice of the CTA: its smallest column
     const int qmin = items[blockIdx.x * (THREADS / 32)].y;
@@ -112,8 +112,8 @@ __global__ void __launch_bounds__(THREADS) front_init_kernel(DevSym d, T *__rest
                     const int c = sch[gi];
                     const int ic = d.relmap[d.mapoff[c] + qc];
                     if (ic < 0) continue;
-                    const int kpc = d.skp[c], ldc = d.sld[c];
-                    const T *U = front + d.foff[c] + (int64_t)(kpc + ic) * ldc + kpc;
+                    const int kpc = d.skp[c];
+                    const T *U = front_columns<UT>(d, front, c).col(kpc + ic) + kpc;
 #pragma unroll
                     for (int u = 0; u < INIT_ROWS / 32; ++u) {
                         const int ir = smap[gi][u * 32 + lane];
@@ -275,10 +275,16 @@ void init_front_attributes() {
 }
 
 template <class T>
-void launch_front_init(const DevSym &d, T *front, const int4 *items, int count, cudaStream_t st) {
+void launch_front_init(const DevSym &d, T *front, const int4 *items, int count, cudaStream_t st, bool ut) {
     if (count <= 0) return;
-    const int warps = THREADS / 32;
-    front_init_kernel<T><<<(count + warps - 1) / warps, THREADS, 0, st>>>(d, front, items, count);
+    const int warps = THREADS / 32, blocks = (count + warps - 1) / warps;
+    if constexpr (sizeof(T) == 8) {
+        if (ut) {
+            front_init_kernel<T, true><<<blocks, THREADS, 0, st>>>(d, front, items, count);
+            return;
+        }
+    }
+    front_init_kernel<T, false><<<blocks, THREADS, 0, st>>>(d, front, items, count);
 }
 
 template <class T>
@@ -300,8 +306,8 @@ void launch_panel(const DevSym &d, T *front, const T *dinv, unsigned char *pk, c
     panel_kernel<T><<<count, THREADS, panel_smem<T>(), st>>>(d, front, dinv, pk, items, kb);
 }
 
-template void launch_front_init<double>(const DevSym &, double *, const int4 *, int, cudaStream_t);
-template void launch_front_init<float>(const DevSym &, float *, const int4 *, int, cudaStream_t);
+template void launch_front_init<double>(const DevSym &, double *, const int4 *, int, cudaStream_t, bool);
+template void launch_front_init<float>(const DevSym &, float *, const int4 *, int, cudaStream_t, bool);
 template void launch_diag_factor<float>(const DevSym &, float *, float *, const int4 *, int, int, status_t *,
                                         cudaStream_t);
 template void launch_panel<float>(const DevSym &, float *, const float *, unsigned char *, const int4 *, int, int,

@@ -4,8 +4,8 @@
 // factorizations share the ordering; U has the pattern of L transposed).
 //
 // The factorization itself runs on the FP64 front kernels (front64.cu), with
-// the fronts of L and of U^T side by side in the layout of the Cholesky
-// fronts, and the substitutions on the Cholesky path's kernels and plan
+// the fronts of L in the layout of the Cholesky fronts and those of U^T in the
+// upper parts of the same squares (FrontCols), and the substitutions on the Cholesky path's kernels and plan
 // (solve_blocked.cu): forward with L, backward with U^T in the place of L.
 // Against the kernels of its own that LU had before (a full-square front
 // updated at every 64-column step, a one-CTA diagonal block of 235 us, one
@@ -68,18 +68,17 @@ __global__ void lu_gather_kernel(const int32_t *__restrict__ src, const int8_t *
 
 // export: supernode s (one CTA), entry (r, c) of its m x k panels (r local
 // row, c local pivot column): L with unit diagonal, and U^T (U[c][row r])
-__global__ void lu_export_kernel(DevSym d, const double *__restrict__ front, const double *__restrict__ ufront,
-                                 double *__restrict__ lpan, double *__restrict__ upan,
-                                 const int64_t *__restrict__ poff) {
+__global__ void lu_export_kernel(DevSym d, const double *__restrict__ front, double *__restrict__ lpan,
+                                 double *__restrict__ upan, const int64_t *__restrict__ poff) {
     const int s = blockIdx.x;
-    const int k = d.sk[s], m = d.sm[s], kp = d.skp[s], ld = d.sld[s];
-    const double *F = front + d.foff[s], *G = ufront + d.foff[s];
+    const int k = d.sk[s], m = d.sm[s], kp = d.skp[s];
+    const FrontCols<const double> F = front_columns<false>(d, front, s), G = front_columns<true>(d, front, s);
     double *Lp = lpan + poff[s], *Up = upan + poff[s];
     for (int64_t idx = threadIdx.x; idx < (int64_t)m * k; idx += THREADS) {
         const int r = (int)(idx % m), c = (int)(idx / m);
-        const int64_t o = (int64_t)c * ld + (r < k ? r : r + kp - k);
-        Lp[idx] = r > c ? F[o] : (r == c ? 1.0 : 0.0);
-        Up[idx] = r >= c ? G[o] : 0.0;
+        const int fr = r < k ? r : r + kp - k;
+        Lp[idx] = r > c ? F.col(c)[fr] : (r == c ? 1.0 : 0.0);
+        Up[idx] = r >= c ? G.col(c)[fr] : 0.0;
     }
 }
 
@@ -98,9 +97,9 @@ void launch_lu_gather(const int32_t *src, const int8_t *code, const double *lowe
 void launch_lu_logdet(const DevSym &d, const double *front, double *partial, int nblocks, cudaStream_t st) {
     lu_logdet_kernel<<<nblocks, THREADS, 0, st>>>(d, front, partial);
 }
-void launch_lu_export(const DevSym &d, const double *front, const double *ufront, double *lpan, double *upan,
-                      const int64_t *poff, cudaStream_t st) {
-    lu_export_kernel<<<d.ns, THREADS, 0, st>>>(d, front, ufront, lpan, upan, poff);
+void launch_lu_export(const DevSym &d, const double *front, double *lpan, double *upan, const int64_t *poff,
+                      cudaStream_t st) {
+    lu_export_kernel<<<d.ns, THREADS, 0, st>>>(d, front, lpan, upan, poff);
 }
 
 }  // namespace wd

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(THREADS) sbinv_diag_kernel(DevSym d, const flo
 // the other are seven launches with an inner dimension of up to 448 and, at
 // the end of each, a product with D_t by one thread per entry.  Square, 16,384
 // unknowns, FP64: 2.54 -> 0.68 ms; 11,003 unknowns, FP32: 0.43 -> 0.06 ms.
-template <class T>
+template <class T, bool UT>
 __global__ void __launch_bounds__(t32::TH) sbinv_double_kernel(DevSym d, const T *__restrict__ front,
                                                                T *__restrict__ xpool, T *__restrict__ tpool,
                                                                const int64_t *__restrict__ xsoff,
@@ -74,10 +74,10 @@ __global__ void __launch_bounds__(t32::TH) sbinv_double_kernel(DevSym d, const T
     T acc[4][2] = {};
     if (phase == 0) {
         // X11 is lower triangular: its rows from the tile's first column on
-        const int ld = d.sld[s];
-        const T *L = front + d.foff[s] + (int64_t)c0 * ld + c0;
+        FrontCols<const T> L = front_columns<UT>(d, front, s);
+        L.p = L.col(c0) + c0;
         t32::product(acc, As, Bs, j0, mid, [&](int buf, int p) {
-            t32::stage_rows(As[buf], L + (int64_t)p * ld + i0, ld, w - i0, mid - p);
+            t32::stage_rows(As[buf], L.col(p) + i0, L.ld, w - i0, mid - p, L.cut);
             t32::stage_inner(Bs[buf], X + (int64_t)j0 * wp + p, wp, t32::TT, mid - p);
         });
     } else {
@@ -312,24 +312,25 @@ constexpr int KSR = SOLVE_KSR;    // rows below B per split of the reduction
 // zero padding, the rows of R; x of a front row read at its global row), 32
 // columns from j0 = b0 + 32 cb: P[slot] ([rhs][c]) = sum_i L(i, j0 + c) x(i,
 // rhs).  item = (s, sb * 16 + cb, tile + 65536 * ks, slot)
-template <class T>
+template <class T, bool UT>
 __global__ void __launch_bounds__(t32::TH) breduce_kernel(DevSym d, const T *__restrict__ front,
                                                           const T *__restrict__ Y, T *__restrict__ P,
                                                           const int4 *__restrict__ items, int nrhs) {
     __shared__ T As[2][t32::TK * t32::LD], Bs[2][t32::TK * t32::LD];
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y >> 4, cb = it.y & 15, g = it.z & 0xFFFF, ks = it.z >> 16;
-    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s], mp = kp + m - k;
+    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], mp = kp + m - k;
     const int b0 = sb * SB, w = min(SB, k - b0);
     const int j0 = b0 + cb * t32::TT, nb = min(t32::TT, b0 + w - j0);
     const int c0 = g * t32::TT, nc = min(t32::TT, nrhs - c0);
     const int64_t n = d.n;
-    const T *F = front + d.foff[s] + (int64_t)j0 * ld;
+    FrontCols<const T> F = front_columns<UT>(d, front, s);
+    F.p = F.col(j0);
     const int32_t *rows = d.rows + d.rowptr[s];
     const int q0 = b0 + w + ks * KSR, q1 = min(mp, q0 + KSR);
     T acc[4][2] = {};
     t32::product(acc, As, Bs, q0, q1, [&](int buf, int q) {
-        t32::stage_inner(As[buf], F + q, ld, nb, q1 - q);
+        t32::stage_inner(As[buf], F.p + q, F.ld, nb, q1 - q, F.cut);
         // a thread's rows of x are the same for all its right-hand sides
         const int pp = threadIdx.x % t32::TK, row = q + pp;
         const bool vr = row < q1 && (row < k || row >= kp);
@@ -653,25 +654,31 @@ __global__ void __launch_bounds__(THREADS, narrow_ctas<DEEP, NR>()) bnarrow_kern
 // storage rows [q0, q0 + NKSR) from the 32-row boundary at or above the super-
 // block's end, for the 64 columns b0 + 64 cb ...: 8 columns per warp, lanes
 // over rows (x zero at rows that do not count); P[slot] ([rhs][column]).
-// item = (s, sb * 16 + cb, 65536 * ks, slot)
+// item = (s, sb * 16 + cb, 65536 * ks, slot).  ut (FP64): the fronts of U^T.
+// (The FP64 deep form takes more than 128 registers, so one CTA per SM.  With
+// 128 two fit; dependent launches then crowd some SMs, whose FP64 pipe is the
+// bound, and LDL^T on the sphere, 8 right-hand sides, takes 9.03 instead of
+// 8.60 ms.)
 template <class T, int NR, bool DEEP>
 __global__ void __launch_bounds__(THREADS, narrow_ctas<DEEP, NR>()) rnarrow_kernel(DevSym d, const T *__restrict__ front,
                                                           const T *__restrict__ Y, T *__restrict__ P,
-                                                          const int4 *__restrict__ items, int nrhs) {
+                                                          const int4 *__restrict__ items, int nrhs, int ut) {
     using VT = typename Vec16<T>::type;
     constexpr int VR = 16 / sizeof(T), H = NKSR / (32 * VR);   // vectors of a lane per column
     constexpr int CG = (DEEP ? 16 : 8) / H;                    // columns whose loads are in flight together
     __shared__ T xs[NKSR * NR];
     const int4 it = items[blockIdx.x];
     const int s = it.x, sb = it.y >> 4, cb = it.y & 15, ks = it.z >> 16;
-    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], ld = d.sld[s], mp = kp + m - k;
+    const int m = d.sm[s], k = d.sk[s], kp = d.skp[s], mp = kp + m - k;
     const int b0 = sb * SB, w = min(SB, k - b0);
     const int j0 = b0 + cb * NARROW_COLS, nb = min(NARROW_COLS, b0 + w - j0);
     const int64_t n = d.n;
     const int32_t *rows = d.rows + d.rowptr[s];
     const int q0 = narrow_first_row(b0, w) + ks * NKSR;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const T *F = front + d.foff[s] + (int64_t)j0 * ld;
+    FrontCols<const T> F = front_columns<false>(d, front, s);
+    if (sizeof(T) == 8 && ut) F = front_columns<true>(d, front, s);
+    F.p = F.col(j0);
     constexpr int CW = NARROW_COLS / NWARP;
     VT x[CG][H];
     auto fetch = [&](int c0) {
@@ -681,7 +688,7 @@ __global__ void __launch_bounds__(THREADS, narrow_ctas<DEEP, NR>()) rnarrow_kern
             for (int h = 0; h < H; ++h) {
                 const int cl = warp * CW + c0 + u, q = q0 + (h * 32 + lane) * VR;
                 // q < mp: the 16 bytes lie inside the column (ld is a multiple of 32)
-                if (c0 + u < CW && cl < nb && q < mp) x[u][h] = *reinterpret_cast<const VT *>(F + (int64_t)cl * ld + q);
+                if (c0 + u < CW && cl < nb && q < mp) x[u][h] = *reinterpret_cast<const VT *>(F.col(cl) + q);
             }
     };
     fetch(0);
@@ -743,9 +750,12 @@ void launch_sbinv_diag(const DevSym &d, const float *dinv, float *xpool, const i
 }
 template <class T>
 void launch_sbinv_double(const DevSym &d, const T *front, T *xpool, T *tpool, const int64_t *xsoff,
-                         const int4 *items, int count, int hb, int phase, cudaStream_t st) {
-    if (count > 0)
-        sbinv_double_kernel<T><<<count, t32::TH, 0, st>>>(d, front, xpool, tpool, xsoff, items, hb, phase);
+                         const int4 *items, int count, int hb, int phase, cudaStream_t st, bool ut) {
+    if (count <= 0) return;
+    auto *kernel = sbinv_double_kernel<T, false>;
+    if constexpr (sizeof(T) == 8)
+        if (ut) kernel = sbinv_double_kernel<T, true>;
+    kernel<<<count, t32::TH, 0, st>>>(d, front, xpool, tpool, xsoff, items, hb, phase);
 }
 template <class T>
 void launch_sbinv_transpose(const DevSym &d, const T *xpool, T *xtpool, const int64_t *xsoff,
@@ -780,9 +790,12 @@ void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, T 
 }
 template <class T>
 void launch_breduce(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count,
-                    int nrhs, cudaStream_t st) {
+                    int nrhs, cudaStream_t st, bool ut) {
     if (count <= 0) return;
-    breduce_kernel<T><<<count, t32::TH, 0, st>>>(d, front, Y, P, items, nrhs);
+    auto *kernel = breduce_kernel<T, false>;
+    if constexpr (sizeof(T) == 8)
+        if (ut) kernel = breduce_kernel<T, true>;
+    kernel<<<count, t32::TH, 0, st>>>(d, front, Y, P, items, nrhs);
 }
 template <class T>
 void launch_breduce_finish(const DevSym &d, const T *Y, T *Tt, const T *P, const int4 *items, int count,
@@ -832,16 +845,17 @@ void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, co
 }
 template <class T>
 void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
-                    cudaStream_t st) {
+                    cudaStream_t st, bool ut) {
     if (count <= 0) return;
     by_width(nrhs, count, [&](auto nr, auto deep) {
-        launch_narrow(rnarrow_kernel<T, nr.value, deep.value>, count, deep.value, st, d, front, Y, P, items, nrhs);
+        launch_narrow(rnarrow_kernel<T, nr.value, deep.value>, count, deep.value, st, d, front, Y, P, items, nrhs,
+                      (int)ut);
     });
 }
 
 #define WD_BLOCKED_INST(T)                                                                              \
     template void launch_sbinv_double<T>(const DevSym &, const T *, T *, T *, const int64_t *,           \
-                                         const int4 *, int, int, int, cudaStream_t);                    \
+                                         const int4 *, int, int, int, cudaStream_t, bool);              \
     template void launch_sbinv_transpose<T>(const DevSym &, const T *, T *, const int64_t *, const int4 *, \
                                             int, cudaStream_t);                                         \
     template void launch_bfwd_gather<T>(const DevSym &, const T *, T *, T *, const int4 *, int, int, int, \
@@ -855,9 +869,9 @@ void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int
     template void launch_bnarrow<T>(const DevSym &, const T *, T *, const T *, T *, const int4 *, int,   \
                                     int, cudaStream_t);                                                 \
     template void launch_rnarrow<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
-                                    cudaStream_t);                                                      \
+                                    cudaStream_t, bool);                                                      \
     template void launch_breduce<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
-                                    cudaStream_t);                                                 \
+                                    cudaStream_t, bool);                                                 \
     template void launch_breduce_finish<T>(const DevSym &, const T *, T *, const T *, const int4 *, int, \
                                            int, int, cudaStream_t);
 WD_BLOCKED_INST(float)

@@ -11,24 +11,24 @@ namespace t32 {
 
 constexpr int TT = 32, TK = 32, LD = 33, TH = 128;   // odd stride: no bank conflicts either way
 
-// chunk [p][r] of an operand whose element (r, p) is at g[p * ld + r]
+// chunk [p][r] of an operand whose element (r, p) is at g[p * ld - (p & cut) + r]
 template <class T>
-__device__ __forceinline__ void stage_rows(T *s, const T *g, int64_t ld, int rvalid, int pvalid) {
+__device__ __forceinline__ void stage_rows(T *s, const T *g, int64_t ld, int rvalid, int pvalid, int cut = 0) {
 #pragma unroll
     for (int u = 0; u < TT * TK / TH; ++u) {
         const int idx = threadIdx.x + u * TH, r = idx % TT, p = idx / TT;
         const bool v = r < rvalid && p < pvalid;
-        cp_async_elem(s + p * LD + r, v ? g + (int64_t)p * ld + r : g, v);
+        cp_async_elem(s + p * LD + r, v ? g + ((int64_t)p * ld - (p & cut)) + r : g, v);
     }
 }
-// element (r, p) at g[r * ld + p]
+// element (r, p) at g[r * ld - (r & cut) + p]
 template <class T>
-__device__ __forceinline__ void stage_inner(T *s, const T *g, int64_t ld, int rvalid, int pvalid) {
+__device__ __forceinline__ void stage_inner(T *s, const T *g, int64_t ld, int rvalid, int pvalid, int cut = 0) {
 #pragma unroll
     for (int u = 0; u < TT * TK / TH; ++u) {
         const int idx = threadIdx.x + u * TH, p = idx % TK, r = idx / TK;
         const bool v = r < rvalid && p < pvalid;
-        cp_async_elem(s + p * LD + r, v ? g + (int64_t)r * ld + p : g, v);
+        cp_async_elem(s + p * LD + r, v ? g + ((int64_t)r * ld - (r & cut)) + p : g, v);
     }
 }
 

@@ -86,3 +86,24 @@ def test_factor_after_another_kind(wdlib, cuda, name, later):
         for c, r in ref.items():
             for got, want in zip(_results(s, kind, n, c), r):
                 np.testing.assert_array_equal(got, want, err_msg=f"{later} after {earlier}, {c} columns")
+
+
+@pytest.mark.parametrize("kind", ["lu", "ldlt"])
+def test_lu_keeps_one_front_pool(wdlib, cuda, kind):
+    """U^T lies in the upper parts of L's fronts: next to a Cholesky factor's
+    memory LU takes the values once more per triangle and U's block inverses,
+    here an eighth of the fronts, and no second pool."""
+    cp, ri, v, basis = _tree(7)
+
+    def used(k):
+        cuda.cuda.synchronize()
+        before = cuda.cuda.mem_get_info()[0]
+        s = wdlib.Solver().analyze(cp, ri, basis)
+        _factor(wdlib, s, k, v)
+        return before - cuda.cuda.mem_get_info()[0], s.info()["front_bytes"]
+
+    used("fp64")                            # module loading
+    chol, fronts = used("fp64")
+    lu, _ = used(kind)
+    assert fronts > 400 << 20
+    assert lu - chol <= fronts / 4
