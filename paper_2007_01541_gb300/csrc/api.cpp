@@ -2820,12 +2820,17 @@ extern "C" wd_status wd_solve_lu(wd_handle h, double *B, int64_t nrhs, int64_t l
     if (nrhs == 0) return WD_OK;
     CK(cudaSetDevice(h->device), "set device");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // passes of at most CH columns, cut evenly, all with the plan (and graph)
+    // passes of at most 64 columns (half as many, down to 16, where the
+    // workspaces of more do not fit), cut evenly, all with the plan (and graph)
     // of the first; a shorter last pass solves zero columns beside its own
-    constexpr int64_t CH = 64;
-    const int64_t npass = (nrhs + CH - 1) / CH;
-    const int nc = (int)((nrhs + npass - 1) / npass);
-    wd_status s = prepare_solve(h, nc, false);
+    int nc = 0;
+    wd_status s = WD_OK;
+    for (int64_t ch = 64;; ch = std::max(16, (nc + 1) / 2)) {
+        const int64_t npass = (nrhs + ch - 1) / ch;
+        nc = (int)((nrhs + npass - 1) / npass);
+        s = prepare_solve(h, nc, false);
+        if (s != WD_ERR_OOM || nc <= 16) break;
+    }
     if (s != WD_OK) return s;
     double *Y = static_cast<double *>(h->d_Y);
     const DevSym &d = h->dsym;

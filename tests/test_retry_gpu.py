@@ -144,3 +144,29 @@ def test_level_schedule(wdlib, cuda):
         solved()
 
     assert _each_allocation(wdlib, call) >= 10
+
+
+@pytest.mark.parametrize("nrhs", [5, 16, 17, 130])
+def test_lu_solve_takes_fewer_columns_at_a_time(wdlib, cuda, nrhs):
+    """Where the workspaces of 64 columns do not fit those of 32 or 16 do: with
+    more than 16 columns one allocation that fails does not fail the call."""
+    b, cp, ri, v = _small()
+    B = rhs(b.N, nrhs, seed=0)
+    in_solve = []
+
+    def call(s, attempt):
+        attempt(s.analyze, cp, ri, b)
+        attempt(s.factor_lu, v, v)
+
+        def solve():
+            try:
+                return s.solve_lu(B)
+            except wdlib.WdError:
+                in_solve.append(1)
+                raise
+
+        assert oracle.backward_error(cp, ri, v, attempt(solve), B).max() <= 1e-12
+        assert oracle.backward_error(cp, ri, v, attempt(solve), B).max() <= 1e-12
+
+    _each_allocation(wdlib, call)
+    assert (len(in_solve) == 0) == (nrhs > 16)
