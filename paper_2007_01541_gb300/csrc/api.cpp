@@ -1442,13 +1442,13 @@ static void enqueue_factor_plan(wd_handle h, cudaStream_t st, bool prof) {
             case K_INIT: wd::launch_front_init<T>(d, F, it, L.count, st); break;
             case K_DIAG:
                 if (fp32)
-                    wd::launch_diag_factor<float>(d, reinterpret_cast<float *>(F), ta.dinv, it, L.count,
-                                                  h->opt.diag64_min_k, h->d_status, st);
+                    wd::launch_diag_factor(d, reinterpret_cast<float *>(F), ta.dinv, it, L.count,
+                                           h->opt.diag64_min_k, h->d_status, st);
                 else wd::launch_diag64(d, fa, it, L.count, st);
                 break;
             case K_PANEL:
                 if (fp32)
-                    wd::launch_panel<float>(d, reinterpret_cast<float *>(F), ta.dinv, pk, it, L.count, L.arg, st);
+                    wd::launch_panel(d, reinterpret_cast<float *>(F), ta.dinv, pk, it, L.count, L.arg, st);
                 else wd::launch_panel64(d, fa, it, L.count, L.arg, st);
                 break;
             case K_UPDATE: wd::launch_update64(d, fa, it, L.count, L.arg, 0, st); break;

@@ -46,7 +46,6 @@ struct DevSym {
 // Set the dynamic shared-memory limits of all kernels (once per process,
 // before any stream capture).
 void init_front_attributes();
-void init_solve_attributes();
 void init_tc_attributes();
 void init_tc_solve_attributes();
 void init_oz_attributes();
@@ -54,7 +53,6 @@ void init_chain_attributes();
 void init_front64_attributes();
 inline void init_kernel_attributes() {
     init_front_attributes();
-    init_solve_attributes();
     init_tc_attributes();
     init_tc_solve_attributes();
     init_oz_attributes();
@@ -64,19 +62,17 @@ inline void init_kernel_attributes() {
 
 
 // ---- factorization (front_kernels.cu) ------------------------------------
-// ut (FP64): the fronts of U^T
+// assembly; ut (FP64): the fronts of U^T
 template <class T>
 void launch_front_init(const DevSym &d, T *front, const int4 *items, int count, cudaStream_t st, bool ut = false);
-// diagonal block (s, kb) of each item: L11 into the front, L11^-1 into dinv
-// at dinvoff + (kb / NB) NB^2; FP32 fronts of width >= diag64_min_k (> 0)
+// FP32 fronts: diagonal block (s, kb) of each item, L11 into the front, L11^-1
+// into dinv at dinvoff + (kb / NB) NB^2; fronts of width >= diag64_min_k (> 0)
 // factor the block in FP64
-template <class T>
-void launch_diag_factor(const DevSym &d, T *front, T *dinv, const int4 *items, int count, int diag64_min_k,
+void launch_diag_factor(const DevSym &d, float *front, float *dinv, const int4 *items, int count, int diag64_min_k,
                         status_t *status, cudaStream_t st);
 // panel of pivot block kb (L11^-1 in dinv): L21 = F21 L11^-T for the items'
-// 64-row blocks; pk != nullptr (FP32 only): also write the packed tf32 lines
-template <class T>
-void launch_panel(const DevSym &d, T *front, const T *dinv, unsigned char *pk, const int4 *items, int count,
+// 64-row blocks; pk != nullptr: also write the packed tf32 lines
+void launch_panel(const DevSym &d, float *front, const float *dinv, unsigned char *pk, const int4 *items, int count,
                   int kb, cudaStream_t st);
 // tile of the plans' FP64 update items
 constexpr int SCHUR_BM = 128, SCHUR_BN = 64;
@@ -249,8 +245,6 @@ void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, cons
 constexpr unsigned CM_BAD_X = 1, CM_BAD_B = 2;
 void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n,
                    int64_t nrhs, double *out, cudaStream_t st);
-template <class T>
-void launch_axpy_into(double *X, const T *D, int64_t count, int accumulate, cudaStream_t st);
 template <class T>
 void launch_cast(const double *src, T *dst, int64_t count, cudaStream_t st);
 template <class T>

@@ -33,14 +33,9 @@ namespace {
 constexpr int THREADS = 256;
 
 using blk::load4;
-// four consecutive shared-memory elements (16-byte aligned for float,
-// two 16-byte halves for double)
+// four consecutive shared-memory elements, 16-byte aligned
 __device__ __forceinline__ void store4(float *p, const float (&v)[4]) {
     *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ void store4(double *p, const double (&v)[4]) {
-    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
 }
 
 // x = hi + lo, hi = x rounded to tf32 (cvt.rna), lo = (x - hi) rounded to tf32
@@ -144,18 +139,18 @@ __global__ void __launch_bounds__(THREADS) front_init_kernel(DevSym d, T *__rest
 // update launch of the step before).  FP32 fronts whose width is at least
 // diag64_min_k (> 0) factor the block in FP64.
 // ---------------------------------------------------------------------------
-template <class T, bool HAS64>
-__global__ void __launch_bounds__(THREADS) diag_factor_kernel(DevSym d, T *__restrict__ front,
-                                                              T *__restrict__ dinv,
+template <bool HAS64>
+__global__ void __launch_bounds__(THREADS) diag_factor_kernel(DevSym d, float *__restrict__ front,
+                                                              float *__restrict__ dinv,
                                                               const int4 *__restrict__ items,
                                                               int diag64_min_k, status_t *status) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int4 it = items[blockIdx.x];
     const int s = it.x, kb = it.y;
-    if (HAS64 && sizeof(T) == 4 && diag64_min_k > 0 && d.sk[s] >= diag64_min_k)
-        blk::factor_diag_block<double, T, THREADS>(d, front, dinv, s, kb, status, smem_raw);
+    if (HAS64 && diag64_min_k > 0 && d.sk[s] >= diag64_min_k)
+        blk::factor_diag_block<double, float, THREADS>(d, front, dinv, s, kb, status, smem_raw);
     else
-        blk::factor_diag_block<T, T, THREADS>(d, front, dinv, s, kb, status, smem_raw);
+        blk::factor_diag_block<float, float, THREADS>(d, front, dinv, s, kb, status, smem_raw);
 }
 
 // ---------------------------------------------------------------------------
@@ -165,33 +160,32 @@ __global__ void __launch_bounds__(THREADS) diag_factor_kernel(DevSym d, T *__res
 // have no rows.
 // ---------------------------------------------------------------------------
 constexpr int XLD = blk::XLD;
-template <class T>
-__global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2) panel_kernel(DevSym d, T *__restrict__ front,
-                                                        const T *__restrict__ dinv,
-                                                        unsigned char *__restrict__ pk,
-                                                        const int4 *__restrict__ items, int kb) {
+__global__ void __launch_bounds__(THREADS, 4) panel_kernel(DevSym d, float *__restrict__ front,
+                                                           const float *__restrict__ dinv,
+                                                           unsigned char *__restrict__ pk,
+                                                           const int4 *__restrict__ items, int kb) {
     static_assert(RB == 64 && NB == 64 && THREADS == 256, "4 x 4 register tiles cover the 64 x 64 panel block");
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    T *LT = reinterpret_cast<T *>(smem_raw);         // LT[p * XLD + c] = Linv(c, p)
-    T *Xs = LT + NB * XLD;                            // [p][r], ld RB
+    float *LT = reinterpret_cast<float *>(smem_raw);         // LT[p * XLD + c] = Linv(c, p)
+    float *Xs = LT + NB * XLD;                            // [p][r], ld RB
     const int4 it = items[blockIdx.x];
     const int s = it.x, rb = it.y;
     const Dims z = dims(d, s);
     const int nb = min(NB, z.k - kb);
     const int t0 = kb + nb;
     const int r0 = (t0 == z.k ? z.kp : t0) + rb * RB;
-    T *F = front + d.foff[s];
+    float *F = front + d.foff[s];
     {
         // Linv is stored column-major (Dv[c + p NB] = Linv(c, p)), so LT's rows
         // are Dv's columns: 16-byte copies
-        const T *Dv = dinv + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB;
-        constexpr int V = 16 / sizeof(T);
+        const float *Dv = dinv + d.dinvoff[s] + (int64_t)(kb / NB) * NB * NB;
+        constexpr int V = 16 / sizeof(float);
         for (int idx = threadIdx.x; idx < NB * NB / V; idx += THREADS) {
             const int p = idx / (NB / V), c = (idx % (NB / V)) * V;
             cp_async16(LT + p * XLD + c, Dv + p * NB + c, 16);
         }
     }
-    stage_tile<T, THREADS>(Xs, RB, F + (int64_t)kb * z.ld + r0, z.ld, RB, NB, z.mp - r0, nb);
+    stage_tile<float, THREADS>(Xs, RB, F + (int64_t)kb * z.ld + r0, z.ld, RB, NB, z.mp - r0, nb);
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
@@ -201,15 +195,15 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2) panel_kernel(
     // thread's last column (Linv is lower triangular).
     const int tid = threadIdx.x;
     const int rq = tid % (RB / 4), cq = tid / (RB / 4);
-    T acc[4][4];
+    float acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     const int pend = min(nb, 4 * cq + 4);
 #pragma unroll 4
     for (int pp = 0; pp < pend; ++pp) {
-        T xv[4], lv[4];
+        float xv[4], lv[4];
         load4(xv, Xs + pp * RB + 4 * rq);
         load4(lv, LT + pp * XLD + 4 * cq);
 #pragma unroll
@@ -219,10 +213,10 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2) panel_kernel(
     }
     // through shared memory ([c][r], ld RB) for whole-column stores
     __syncthreads();
-    T *Os = Xs;
+    float *Os = Xs;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        T o[4] = {acc[0][j], acc[1][j], acc[2][j], acc[3][j]};
+        float o[4] = {acc[0][j], acc[1][j], acc[2][j], acc[3][j]};
         store4(Os + (4 * cq + j) * RB + 4 * rq, o);
     }
     __syncthreads();
@@ -241,7 +235,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2) panel_kernel(
             const int kc = kb / 32 + g / 8, gg = g % 8;
             uint32_t hi[4], lo[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) split_tf32_bits((float)Os[(4 * g + j) * RB + rr], hi[j], lo[j]);
+            for (int j = 0; j < 4; ++j) split_tf32_bits(Os[(4 * g + j) * RB + rr], hi[j], lo[j]);
             const int64_t sw = (int64_t)((gg ^ (row & 7)) * 16);
             *reinterpret_cast<uint4 *>(P + pack_offset(kc, 0, row, prow) + sw) =
                 make_uint4(hi[0], hi[1], hi[2], hi[3]);
@@ -251,27 +245,18 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2) panel_kernel(
     }
 }
 
-template <class T>
-constexpr size_t panel_smem() { return sizeof(T) * (NB * XLD + NB * RB); }
+constexpr size_t panel_smem() { return sizeof(float) * (NB * XLD + NB * RB); }
 constexpr size_t diag_smem() { return blk::block_smem_bytes<double>(); }
-
-template <class T>
-void set_smem_attrs() {
-    static bool done = false;  // per instantiation and process
-    if (done) return;
-    cudaFuncSetAttribute(panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)panel_smem<T>());
-    cudaFuncSetAttribute(diag_factor_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)diag_smem());
-    cudaFuncSetAttribute(diag_factor_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)diag_smem());
-    done = true;
-}
 
 }  // namespace
 
 void init_front_attributes() {
-    set_smem_attrs<float>();
+    static bool done = false;
+    if (done) return;
+    cudaFuncSetAttribute(panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem());
+    cudaFuncSetAttribute(diag_factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem());
+    cudaFuncSetAttribute(diag_factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem());
+    done = true;
 }
 
 template <class T>
@@ -287,30 +272,22 @@ void launch_front_init(const DevSym &d, T *front, const int4 *items, int count, 
     front_init_kernel<T, false><<<blocks, THREADS, 0, st>>>(d, front, items, count);
 }
 
-template <class T>
-void launch_diag_factor(const DevSym &d, T *front, T *dinv, const int4 *items, int count, int diag64_min_k,
+void launch_diag_factor(const DevSym &d, float *front, float *dinv, const int4 *items, int count, int diag64_min_k,
                         status_t *status, cudaStream_t st) {
     if (count <= 0) return;
-    set_smem_attrs<T>();
-    if (sizeof(T) == 4 && diag64_min_k > 0)
-        diag_factor_kernel<T, true><<<count, THREADS, diag_smem(), st>>>(d, front, dinv, items, diag64_min_k, status);
-    else
-        diag_factor_kernel<T, false><<<count, THREADS, diag_smem(), st>>>(d, front, dinv, items, diag64_min_k, status);
+    init_front_attributes();
+    auto *kernel = diag64_min_k > 0 ? diag_factor_kernel<true> : diag_factor_kernel<false>;
+    kernel<<<count, THREADS, diag_smem(), st>>>(d, front, dinv, items, diag64_min_k, status);
 }
 
-template <class T>
-void launch_panel(const DevSym &d, T *front, const T *dinv, unsigned char *pk, const int4 *items, int count,
+void launch_panel(const DevSym &d, float *front, const float *dinv, unsigned char *pk, const int4 *items, int count,
                   int kb, cudaStream_t st) {
     if (count <= 0) return;
-    set_smem_attrs<T>();
-    panel_kernel<T><<<count, THREADS, panel_smem<T>(), st>>>(d, front, dinv, pk, items, kb);
+    init_front_attributes();
+    panel_kernel<<<count, THREADS, panel_smem(), st>>>(d, front, dinv, pk, items, kb);
 }
 
 template void launch_front_init<double>(const DevSym &, double *, const int4 *, int, cudaStream_t, bool);
 template void launch_front_init<float>(const DevSym &, float *, const int4 *, int, cudaStream_t, bool);
-template void launch_diag_factor<float>(const DevSym &, float *, float *, const int4 *, int, int, status_t *,
-                                        cudaStream_t);
-template void launch_panel<float>(const DevSym &, float *, const float *, unsigned char *, const int4 *, int, int,
-                                  cudaStream_t);
 
 }  // namespace wd

@@ -913,14 +913,6 @@ __global__ void __launch_bounds__(256) colmax_narrow_kernel(const double *__rest
 }
 
 template <class T>
-__global__ void axpy_into_kernel(double *__restrict__ X, const T *__restrict__ D, int64_t cnt,
-                                 int acc) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt;
-         t += (int64_t)gridDim.x * blockDim.x)
-        X[t] = acc ? X[t] + (double)D[t] : (double)D[t];
-}
-
-template <class T>
 __global__ void cast_kernel(const double *__restrict__ src, T *__restrict__ dst, int64_t cnt) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt;
          t += (int64_t)gridDim.x * blockDim.x)
@@ -980,8 +972,6 @@ inline int grid_for(int64_t work) {
 }
 
 }  // namespace
-
-void init_solve_attributes() {}
 
 void launch_gather_values(const int32_t *src, const double *values, double *out, float *hi, float *lo,
                           int64_t nnz, cudaStream_t st) {
@@ -1111,11 +1101,6 @@ void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n
 }
 
 template <class T>
-void launch_axpy_into(double *X, const T *D, int64_t cnt, int acc, cudaStream_t st) {
-    axpy_into_kernel<T><<<grid_for(cnt), THREADS, 0, st>>>(X, D, cnt, acc);
-}
-
-template <class T>
 void launch_cast(const double *src, T *dst, int64_t cnt, cudaStream_t st) {
     cast_kernel<T><<<grid_for(cnt), THREADS, 0, st>>>(src, dst, cnt);
 }
@@ -1143,7 +1128,6 @@ void launch_export_panels(const DevSym &d, const T *front, double *panels, const
                                         int64_t, cudaStream_t);                                  \
     template void launch_apply_L<T>(const DevSym &, const T *, const T *, T *, T *,              \
                                     const int4 *, int, int, cudaStream_t);                       \
-    template void launch_axpy_into<T>(double *, const T *, int64_t, int, cudaStream_t);          \
     template void launch_transpose<T>(T *, double *, int64_t, int64_t, int, int, cudaStream_t);  \
     template void launch_cast<T>(const double *, T *, int64_t, cudaStream_t);                    \
     template void launch_logdet_partial<T>(const DevSym &, const T *, double *, int,             \
