@@ -1707,7 +1707,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.upper = 0;
                     wd::launch_tc_xapply(d, a, it, L.count, st);
                 } else if (lg == 2) {
-                    wd::launch_xnarrow<T>(d, Xs, h->d_xsoff, Y, Tt, W, P, it, L.count, true, nrhs, st);
+                    wd::launch_xnarrow<T>(d, Xs, h->d_xsoff, Y, Tt, W, P, it, L.count, true, nrhs, h->sms, st);
                 } else {
                     wd::launch_xapply<T>(d, Xs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 0, nrhs, st);
                 }
@@ -1719,7 +1719,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.out = reinterpret_cast<float *>(Tt);
                     wd::launch_tc_bupdate(d, a, it, L.count, st);
                 } else if (lg == 2) {
-                    wd::launch_bnarrow<T>(d, F, Y, Tt, W, it, L.count, nrhs, st);
+                    wd::launch_bnarrow<T>(d, F, Y, Tt, W, it, L.count, nrhs, h->sms, st);
                 } else {
                     wd::launch_bupdate<T>(d, F, Y, Tt, W, ksw, h->d_kcnt, it, L.count, nrhs, st);
                 }
@@ -1732,7 +1732,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.ksr = L.arg;
                     wd::launch_tc_breduce(d, a, it, L.count, st);
                 } else if (lg == 2) {
-                    wd::launch_rnarrow<T>(d, F, Y, P, it, L.count, nrhs, st, lu);
+                    wd::launch_rnarrow<T>(d, F, Y, P, it, L.count, nrhs, h->sms, st, lu);
                 } else {
                     wd::launch_breduce<T>(d, F, Y, P, it, L.count, nrhs, st, lu);
                 }
@@ -1747,7 +1747,7 @@ static void enqueue_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, boo
                     a.upper = 1;
                     wd::launch_tc_xapply(d, a, it, L.count, st);
                 } else if (lg == 2) {
-                    wd::launch_xnarrow<T>(d, XTs, h->d_xsoff, Y, Tt, W, P, it, L.count, false, nrhs, st);
+                    wd::launch_xnarrow<T>(d, XTs, h->d_xsoff, Y, Tt, W, P, it, L.count, false, nrhs, h->sms, st);
                 } else {
                     wd::launch_xapply<T>(d, XTs, h->d_xsoff, Tt, Y, ksw, h->d_kcnt, it, L.count, 1, nrhs, st);
                 }
@@ -1820,7 +1820,7 @@ static wd_status enqueue_backward_errors(wd_handle h, const double *X, int64_t n
     if (h->batch_count > 0)
         wd::launch_seg_colmax(h->d_R, X, h->d_Bp, h->d_batch_coff, (int)cnt, (int)nrhs, cm, st);
     else
-        wd::launch_colmax(h->d_R, X, h->d_Bp, h->S.n, nrhs, cm, st);
+        wd::launch_colmax(h->d_R, X, h->d_Bp, h->S.n, nrhs, cm, h->sms, st);
     h->launches += 2;
     if (nrhs <= 8)
         CK(cudaMemcpyAsync(h->pin + PIN_BAD, h->d_spmv_bad, sizeof(status_t), cudaMemcpyDeviceToHost, st),

@@ -244,7 +244,7 @@ void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, cons
 // nrhs <= 8: out holds zeros already
 constexpr unsigned CM_BAD_X = 1, CM_BAD_B = 2;
 void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n,
-                   int64_t nrhs, double *out, cudaStream_t st);
+                   int64_t nrhs, double *out, int sms, cudaStream_t st);
 template <class T>
 void launch_cast(const double *src, T *dst, int64_t count, cudaStream_t st);
 template <class T>
@@ -319,17 +319,18 @@ template <class T>
 void launch_bupdate(const DevSym &d, const T *front, const T *Y, T *Tt, T *W, T *ksw, int *kcnt,
                     const int4 *items, int count, int nrhs, cudaStream_t st);
 // mode 2: y_B (forward: Y and the children's into Tt) or x_B (backward: Tt and
-// the partial sums P into Y); the rows below; the partial sums
+// the partial sums P into Y); the rows below; the partial sums;
+// sms: the device's SMs, which set what a large launch is
 constexpr int SOLVE_KSR_NARROW = 256;
 template <class T>
 void launch_xnarrow(const DevSym &d, const T *xp, const int64_t *xsoff, T *Y, T *Tt, const T *W, const T *P,
-                    const int4 *items, int count, bool forward, int nrhs, cudaStream_t st);
+                    const int4 *items, int count, bool forward, int nrhs, int sms, cudaStream_t st);
 template <class T>
 void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, const int4 *items, int count, int nrhs,
-                    cudaStream_t st);
+                    int sms, cudaStream_t st);
 template <class T>
 void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
-                    cudaStream_t st, bool ut = false);
+                    int sms, cudaStream_t st, bool ut = false);
 // split reduction of the backward pass: partial sums of KSR-row splits into
 // P (rows x rhs of the tile per slot), then Tt = y - sum over the splits in order
 constexpr int SOLVE_KSR = 128;

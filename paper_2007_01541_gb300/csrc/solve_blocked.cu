@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // L once per direction, would take a tenth of the time).  So
 //   * a CTA covers 32 rows and all its columns (or 64 columns and 256 rows) with
 //     16-byte loads, up to sixteen of them in flight per lane, most often all;
-//   * the kernels of launches that are not large (NARROW_DEEP) are launched
+//   * the kernels of launches that are not large (narrow_deep) are launched
 //     dependent on one another programmatically: while one finishes, the next
 //     one's CTAs start, read their items and sizes and load their part of L or
 //     X, which no solve writes, and only then wait;
@@ -398,18 +398,19 @@ __global__ void __launch_bounds__(THREADS) breduce_finish_kernel(DevSym d, const
 // their own for the gather and the sum: 256 x 256, one right-hand side against
 // a kept factor 2.30 -> 1.67 ms; 128 x 128, a theta step 0.84 -> 0.68 ms.
 // Dependent launches and the deep and shallow forms: 1.57 -> 1.03 ms, 0.655 ->
-// 0.481 ms, the batch of 64 instances 12.47 -> 11.72.
+// 0.481 ms, the batch of 64 instances 12.47 -> 11.72.  With the faster
+// residuals of solve_kernels.cu the two are 0.98 and 0.43 ms.
 // ---------------------------------------------------------------------------
 constexpr int NRW = 32;
-// DEEP launches, at most NARROW_DEEP CTAs (two per SM): sixteen loads in flight
+// DEEP launches, at most two CTAs per SM: sixteen loads in flight
 // per lane, the first of them before the wait.  Larger launches (the lower
 // levels of large trees and of batches) have other CTAs to overlap with: four
 // loads (eight in the reduction), two to four CTAs per SM, ordinary launches.
-// The arithmetic is the same.  Limit 2,432 / 608 / 304 / 152 against each other
-// (and all launches deep first): 256 x 256, one right-hand side 1.17; 1.08 /
+// The arithmetic is the same.  Limit 2,432 / 608 / 304 / 152 CTAs on 152 SMs
+// against each other (and all launches deep first): 256 x 256, one right-hand side 1.17; 1.08 /
 // 1.05 / 1.03 / 1.07 ms; 16 theta steps at 128 x 128 8.01; 7.92 / 7.85 / 7.70 /
 // 7.94; batch of 64 instances 12.87; 11.83 / 11.72 / 11.72 / 11.74.
-constexpr int NARROW_DEEP = 304;
+inline bool narrow_deep(int count, int sms) { return count <= 2 * sms; }
 template <bool DEEP, int NR>
 constexpr int narrow_ctas() { return DEEP ? 1 : (NR <= 2 ? 4 : NR == 4 ? 3 : 2); }
 constexpr int NWARP = THREADS / 32;
@@ -810,23 +811,23 @@ static void launch_narrow(void (*kernel)(P...), int count, bool deep, cudaStream
     if (deep) launch_dependent(kernel, count, THREADS, 0, st, args...);
     else kernel<<<count, THREADS, 0, st>>>(args...);
 }
-// f<NR, DEEP>() for nrhs <= 8
+// f(NR, DEEP) for nrhs <= 8
 template <class F>
-static void by_width(int nrhs, int count, F f) {
+static void by_width(int nrhs, bool deep_launch, F f) {
     auto nr = [&](auto deep) {
         if (nrhs == 1) f(std::integral_constant<int, 1>(), deep);
         else if (nrhs == 2) f(std::integral_constant<int, 2>(), deep);
         else if (nrhs <= 4) f(std::integral_constant<int, 4>(), deep);
         else f(std::integral_constant<int, 8>(), deep);
     };
-    if (count <= NARROW_DEEP) nr(std::true_type());
+    if (deep_launch) nr(std::true_type());
     else nr(std::false_type());
 }
 template <class T>
 void launch_xnarrow(const DevSym &d, const T *xp, const int64_t *xsoff, T *Y, T *Tt, const T *W, const T *P,
-                    const int4 *items, int count, bool forward, int nrhs, cudaStream_t st) {
+                    const int4 *items, int count, bool forward, int nrhs, int sms, cudaStream_t st) {
     if (count <= 0) return;
-    by_width(nrhs, count, [&](auto nr, auto deep) {
+    by_width(nrhs, narrow_deep(count, sms), [&](auto nr, auto deep) {
         if (forward)
             launch_narrow(xnarrow_kernel<T, nr.value, deep.value, true>, count, deep.value, st, d, xp, xsoff, Y, Tt, W, P,
                           items, nrhs);
@@ -837,17 +838,17 @@ void launch_xnarrow(const DevSym &d, const T *xp, const int64_t *xsoff, T *Y, T 
 }
 template <class T>
 void launch_bnarrow(const DevSym &d, const T *front, T *Y, const T *Tt, T *W, const int4 *items, int count, int nrhs,
-                    cudaStream_t st) {
+                    int sms, cudaStream_t st) {
     if (count <= 0) return;
-    by_width(nrhs, count, [&](auto nr, auto deep) {
+    by_width(nrhs, narrow_deep(count, sms), [&](auto nr, auto deep) {
         launch_narrow(bnarrow_kernel<T, nr.value, deep.value>, count, deep.value, st, d, front, Y, Tt, W, items, nrhs);
     });
 }
 template <class T>
 void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int4 *items, int count, int nrhs,
-                    cudaStream_t st, bool ut) {
+                    int sms, cudaStream_t st, bool ut) {
     if (count <= 0) return;
-    by_width(nrhs, count, [&](auto nr, auto deep) {
+    by_width(nrhs, narrow_deep(count, sms), [&](auto nr, auto deep) {
         launch_narrow(rnarrow_kernel<T, nr.value, deep.value>, count, deep.value, st, d, front, Y, P, items, nrhs,
                       (int)ut);
     });
@@ -865,11 +866,11 @@ void launch_rnarrow(const DevSym &d, const T *front, const T *Y, T *P, const int
     template void launch_bupdate<T>(const DevSym &, const T *, const T *, T *, T *, T *, int *,          \
                                     const int4 *, int, int, cudaStream_t);                              \
     template void launch_xnarrow<T>(const DevSym &, const T *, const int64_t *, T *, T *, const T *,     \
-                                    const T *, const int4 *, int, bool, int, cudaStream_t);             \
+                                    const T *, const int4 *, int, bool, int, int, cudaStream_t);        \
     template void launch_bnarrow<T>(const DevSym &, const T *, T *, const T *, T *, const int4 *, int,   \
-                                    int, cudaStream_t);                                                 \
+                                    int, int, cudaStream_t);                                            \
     template void launch_rnarrow<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
-                                    cudaStream_t, bool);                                                      \
+                                    int, cudaStream_t, bool);                                                    \
     template void launch_breduce<T>(const DevSym &, const T *, const T *, T *, const int4 *, int, int,   \
                                     cudaStream_t, bool);                                                 \
     template void launch_breduce_finish<T>(const DevSym &, const T *, T *, const T *, const int4 *, int, \

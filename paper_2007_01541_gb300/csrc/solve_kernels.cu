@@ -1089,14 +1089,14 @@ void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, cons
 }
 
 void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n, int64_t nrhs,
-                   double *out, cudaStream_t st) {
+                   double *out, int sms, cudaStream_t st) {
     if (nrhs <= 8) {    // out zeroed by the product before
-        const int blocks = (int)std::min<int64_t>((n + 1023) / 1024, 152);
+        const int blocks = (int)std::min<int64_t>((n + 1023) / 1024, sms);
         colmax_narrow_kernel<<<blocks, 256, 0, st>>>(R, X, Bp, n, (int)nrhs, out);
         return;
     }
     cudaMemsetAsync(out, 0, 4 * nrhs * sizeof(double), st);
-    const int64_t rpb = std::max<int64_t>(16, (n + 607) / 608);    // four blocks per SM
+    const int64_t rpb = std::max<int64_t>(16, (n + 4 * sms - 1) / (4 * sms));    // four blocks per SM
     colmax_rm_kernel<<<(int)((n + rpb - 1) / rpb), 256, 0, st>>>(R, X, Bp, n, (int)nrhs, rpb, out);
 }
 
