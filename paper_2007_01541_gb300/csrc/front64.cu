@@ -21,12 +21,13 @@
 //     SM, and a step has to cut into many tiles to use all SMs (the 128 x 64
 //     tiles before took 126 us each, whatever the step);
 //   * the diagonal block, the serial part, spends no FP64 instruction it can
-//     avoid: one warp chain per 16 columns carries the 16 x 16 diagonal
-//     sub-block (lanes 0-15) and 16 more rows (lanes 16-31) through the same
-//     instructions, without square roots or divisions on the chain, and no
-//     64 x 64 inverse is formed: the panels only need the inverses of the four
-//     16 x 16 sub-blocks, and the 64 x 64 ones that the solves use are
-//     completed for all blocks at once after the factorization (sbinv_diag64).
+//     avoid: by sub-blocks of 8 columns, three warps carry the 8 x 8 diagonal
+//     sub-block (lanes 0-7) and 24 more rows each (lanes 8-31) through the same
+//     instructions, without square roots or divisions on the chain
+//     (front64.cuh), and no 64 x 64 inverse is formed: the panels only need the
+//     inverses of the four 16 x 16 sub-blocks, and the 64 x 64 ones that the
+//     solves use are completed for all blocks at once after the factorization
+//     (sbinv_diag64).
 // A step is two dependent launches: panel, then update; the update CTA that
 // finishes the last of the next diagonal block's tiles factors that block.
 // Measured against the 128 x 64 tiles, 64-row panels and 64 x 64 inverses on

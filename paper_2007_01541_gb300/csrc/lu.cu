@@ -10,9 +10,9 @@
 // Against the kernels of its own that LU had before (a full-square front
 // updated at every 64-column step, a one-CTA diagonal block of 235 us, one
 // substitution launch per 64 columns with one CTA per block row): square,
-// 16,384 unknowns, 16 right-hand sides, 69.7 -> 25.5 ms (backward
+// 16,384 unknowns, 16 right-hand sides, 69.7 -> 25.1 ms (backward
 // substitution 31.3 ms of it before); LDL^T on the sphere, 6,144 unknowns, 8
-// right-hand sides, 32.0 -> 8.7 ms.
+// right-hand sides, 32.0 -> 8.6 ms.
 // Here: the values, the determinant and the export.
 #include "dev_common.cuh"
 #include "engine.h"
