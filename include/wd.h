@@ -244,8 +244,8 @@ wd_status wd_theta_step(wd_handle h, double *U, const double *F, int64_t nrhs, i
      ||b - A x||_inf / (||A||_inf ||x||_inf + ||b||_inf)
    X, B: n x nrhs, column-major, leading dimension ld, original order, device
    (1) or host (0).  The residual is formed from A's FP64 values: in FP64 for
-   up to 8 columns, in double-float arithmetic (about 48 bits, FP32's range) for
-   more; infinity where x or the residual is not finite although b is.  For
+   up to 8 columns, in double-float arithmetic (about 48 bits; where that leaves
+   FP32's range, in FP64) for more; infinity where x or the residual is not finite although b is.  For
    a batch, the largest of the instances' own backward errors.  Needs a
    successful wd_factor (for ||A||_inf).  Synchronous. */
 wd_status wd_backward_error(wd_handle h, const double *X, const double *B, int64_t nrhs, int64_t ld,

@@ -1772,19 +1772,20 @@ static wd_status run_solve_plan(wd_handle h, T *Y, int nrhs, cudaStream_t st, bo
 
 // R = Bp - A X (row-major n x nrhs, factor order) to FP64 accuracy: FP64 up
 // to 8 columns (with the device check of the column indices, read back by the
-// caller from d_spmv_bad), double-float arithmetic beyond
+// caller from d_spmv_bad), double-float arithmetic beyond unless fp64 says
+// otherwise
 static wd_status launch_residual(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st,
-                                 const float *Xf = nullptr, const double *S = nullptr) {
+                                 const float *Xf = nullptr, const double *S = nullptr, bool fp64 = false) {
     const int64_t n = h->S.n;
     const double nf = (double)h->nnz_full;
-    if (nrhs > 8 && Xf != nullptr) {
+    if (nrhs > 8 && !fp64 && Xf != nullptr) {
         // x exactly FP32: R = S - A x (S = b, or R itself for the recurrence)
         prof_single(h, "spmv_residual_df32", 0, 0, st, true);
         wd::launch_spmv_residual_df32(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin,
                                       h->n_spmv_fin, h->d_csr_vh, h->d_csr_vl, Xf, S, h->d_R, h->d_P, nrhs, st);
         prof_single(h, "spmv_residual_df32", 2.0 * nf * nrhs, 12.0 * nf + 20.0 * n * nrhs, st, false);
         h->launches += h->n_spmv_fin > 0 ? 2 : 1;
-    } else if (nrhs > 8) {
+    } else if (nrhs > 8 && !fp64) {
         // many right-hand sides: double-float arithmetic on the FP32 pipes
         prof_single(h, "spmv_residual_df", 0, 0, st, true);
         wd::launch_spmv_residual_df(h->dsym, h->d_spmv_chunks, h->n_spmv_chunks, h->d_spmv_fin,
@@ -1812,9 +1813,9 @@ static wd_status bad_column(wd_handle h, status_t at) {
 // R = Bp - A X (FP64, row-major n x nrhs) and its column maxima (per instance
 // for a batch, each its own system), enqueued with their copies to h->pin
 static wd_status enqueue_backward_errors(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st,
-                                         const float *Xf = nullptr, const double *S = nullptr) {
+                                         const float *Xf = nullptr, const double *S = nullptr, bool fp64 = false) {
     const int64_t cnt = h->batch_count > 0 ? h->batch_count : 1;
-    wd_status s = launch_residual(h, X, nrhs, st, Xf, S);
+    wd_status s = launch_residual(h, X, nrhs, st, Xf, S, fp64);
     if (s != WD_OK) return s;
     double *cm = h->batch_count > 0 ? h->d_batch_cm : h->d_cm;
     if (h->batch_count > 0)
@@ -1832,30 +1833,45 @@ static wd_status enqueue_backward_errors(wd_handle h, const double *X, int64_t n
 // the largest normwise backward error over columns (and instances), after the
 // copies have landed: infinite where x or the residual is not finite although
 // b is.  (A column whose b is not finite has no finite solution; what of it is
-// NaN does not count.)
-static wd_status read_backward_errors(wd_handle h, int64_t nrhs, double *be_max) {
+// NaN does not count.)  *range: a residual is not finite although x and b are.
+static wd_status read_backward_errors(wd_handle h, int64_t nrhs, double *be_max, bool *range) {
     if (nrhs <= 8 && pin_word(h, PIN_BAD) != ~0ULL) return bad_column(h, pin_word(h, PIN_BAD));
     const int64_t cnt = h->batch_count > 0 ? h->batch_count : 1;
     double mx = 0.0;
+    *range = false;
     for (int64_t i = 0; i < cnt; ++i) {
         const double nrm = h->batch_count > 0 ? h->batch_normA[i] : h->normA;
         for (int64_t c = 0; c < nrhs; ++c) {
             const int64_t o = PIN_CM + (i * nrhs + c) * 4;
             const double *q = h->pin + o;
             const double den = nrm * q[1] + q[2];
-            const bool bad = (pin_word(h, o + 3) & (wd::CM_BAD_X | wd::CM_BAD_B)) == wd::CM_BAD_X;
+            const status_t f = pin_word(h, o + 3);
+            const bool bad = f != 0 && !(f & wd::CM_BAD_B);
             mx = std::max(mx, bad ? HUGE_VAL : (den > 0 ? q[0] / den : 0.0));
+            if (f == wd::CM_BAD_R) *range = true;
         }
     }
     *be_max = mx;
     return WD_OK;
 }
 
+// the same; where the double-float residual left FP32's range it is formed once
+// more in FP64 (and R is that one)
+static wd_status settle_backward_errors(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st, double *be_max) {
+    bool range = false;
+    wd_status s = read_backward_errors(h, nrhs, be_max, &range);
+    if (s != WD_OK || !range || nrhs <= 8) return s;
+    s = enqueue_backward_errors(h, X, nrhs, st, nullptr, nullptr, true);
+    if (s != WD_OK) return s;
+    CK(cudaStreamSynchronize(st), "backward error");
+    return read_backward_errors(h, nrhs, be_max, &range);
+}
+
 static wd_status backward_errors(wd_handle h, const double *X, int64_t nrhs, cudaStream_t st, double *be_max) {
     wd_status s = enqueue_backward_errors(h, X, nrhs, st);
     if (s != WD_OK) return s;
     CK(cudaStreamSynchronize(st), "backward error");
-    return read_backward_errors(h, nrhs, be_max);
+    return settle_backward_errors(h, X, nrhs, st, be_max);
 }
 
 // workspaces and the launch plan of solves with nrhs right-hand sides
@@ -1956,7 +1972,7 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
             CK(cudaMemcpyAsync(h->pin + PIN_TSTATUS, h->d_tstatus, sizeof(status_t), cudaMemcpyDeviceToHost, st),
                "status D2H");
             CK(cudaStreamSynchronize(st), "backward error");
-            s = read_backward_errors(h, nrhs, &be);
+            s = settle_backward_errors(h, h->d_X, nrhs, st, &be);
             if (s != WD_OK) return s;
             if (be <= h->opt.ir_tol || it >= h->opt.ir_max_iter || pin_word(h, PIN_TSTATUS) != 0) {
                 if (!last) {
@@ -1995,7 +2011,7 @@ static wd_status solve_core(wd_handle h, double *Bd, int64_t ld, double *B, int6
                              cudaMemcpyDeviceToHost, st),
            "B D2H");
     if (h->prec == WD_FP64 || !B_on_device) CK(cudaStreamSynchronize(st), "solve");
-    if (h->prec == WD_FP64 && info) return read_backward_errors(h, nrhs, &info->backward_error);
+    if (h->prec == WD_FP64 && info) return settle_backward_errors(h, h->d_X, nrhs, st, &info->backward_error);
     return WD_OK;
 }
 

@@ -97,13 +97,14 @@ __global__ void __launch_bounds__(THREADS) seg_colmax_kernel(const double *__res
         for (int64_t r = coff[inst] + threadIdx.x; r < coff[inst + 1]; r += THREADS)
             v.add(R[r * nrhs + c], X[r * nrhs + c], B[r * nrhs + c]);
         const unsigned long long a = block_max(v.m[0], red), b = block_max(v.m[1], red), e = block_max(v.m[2], red);
-        const int bad_x = __syncthreads_or(v.flags & CM_BAD_X), bad_b = __syncthreads_or(v.flags & CM_BAD_B);
+        unsigned flags = 0;
+        for (unsigned f : {CM_BAD_R, CM_BAD_X, CM_BAD_B}) flags |= __syncthreads_or(v.flags & f) ? f : 0;
         if (threadIdx.x == 0) {
             double *o = out + ((int64_t)inst * nrhs + c) * 4;
             o[0] = __longlong_as_double((long long)a);
             o[1] = __longlong_as_double((long long)b);
             o[2] = __longlong_as_double((long long)e);
-            o[3] = __longlong_as_double((long long)((bad_x ? CM_BAD_X : 0) | (bad_b ? CM_BAD_B : 0)));
+            o[3] = __longlong_as_double((long long)flags);
         }
     }
 }

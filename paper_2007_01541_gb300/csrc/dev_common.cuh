@@ -78,7 +78,7 @@ __device__ __forceinline__ FrontCols<T> front_columns(const DevSym &d, T *pool, 
 }
 
 // Column maxima of the backward error: max |r|, |x| and |b| (NaN does not
-// count), then a word of flags: r or x, and b, held a value that is not finite
+// count), then a word of flags: which of them held a value that is not finite
 struct ColMax {
     unsigned long long m[3] = {0, 0, 0};
     unsigned flags = 0;
@@ -87,7 +87,7 @@ struct ColMax {
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             m[q] = max(m[q], u[q] > inf ? 0ull : u[q]);
-            if (u[q] >= inf) flags |= q < 2 ? CM_BAD_X : CM_BAD_B;
+            if (u[q] >= inf) flags |= CM_BAD_R << q;
         }
     }
     static __device__ __forceinline__ unsigned long long bits(double x) {

@@ -240,9 +240,9 @@ void launch_xupdate(const float *Y, double *X, float *Xf, int64_t n, int64_t nrh
 void launch_norm_inf_rows(const DevSym &d, const int4 *chunks, int nchunks, const int4 *fin,
                           int nfin, double *partial, double *out, cudaStream_t st);
 // per column four words: max |R|, |X| and |B| (NaN does not count), and as an
-// integer CM_BAD_X (R or X held a value that is not finite) | CM_BAD_B (B did);
-// nrhs <= 8: out holds zeros already
-constexpr unsigned CM_BAD_X = 1, CM_BAD_B = 2;
+// integer CM_BAD_R | CM_BAD_X | CM_BAD_B (R, X, B held a value that is not
+// finite); nrhs <= 8: out holds zeros already
+constexpr unsigned CM_BAD_R = 1, CM_BAD_X = 2, CM_BAD_B = 4;
 void launch_colmax(const double *R, const double *X, const double *Bp, int64_t n,
                    int64_t nrhs, double *out, int sms, cudaStream_t st);
 template <class T>

@@ -78,3 +78,23 @@ def test_right_hand_side_not_finite_is_taken(wdlib, cuda, prec, ncols):
     assert np.isnan(X[:, 1]).any()
     keep = np.arange(ncols) != 1
     assert oracle.backward_error(cp, ri, v, X[:, keep], B[:, keep]).max() <= 1e-12
+
+
+@pytest.mark.parametrize("batch", [False, True])
+@pytest.mark.parametrize("ncols", [8, 9, 70])
+@pytest.mark.parametrize("scale", [1e50, 1e-300])
+def test_backward_error_beyond_fp32(wdlib, cuda, batch, ncols, scale):
+    """Values that FP64 holds and FP32 does not: the residual of more than 8
+    columns takes FP64 where double-float arithmetic overflows (1e50; 1e-300
+    vanishes in it)."""
+    s, n, v = _solver(wdlib, batch)
+    s.factor(v, "fp64")
+    B = scale * rhs(n, ncols, seed=4)
+    X = s.solve(B)
+    if scale > 1.0 or ncols <= 8:
+        assert s.last_solve["backward_error"] <= 1e-12
+        assert s.backward_error(X, B) <= 1e-12
+    assert np.isfinite(X).all()
+    for i in range(0, n, _one()[0].N):
+        b, cp, ri, one = _one()
+        assert oracle.backward_error(cp, ri, one, X[i:i + b.N], B[i:i + b.N]).max() <= 1e-12
