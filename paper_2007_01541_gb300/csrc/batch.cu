@@ -97,8 +97,9 @@ __global__ void __launch_bounds__(THREADS) seg_colmax_kernel(const double *__res
         for (int64_t r = coff[inst] + threadIdx.x; r < coff[inst + 1]; r += THREADS)
             v.add(R[r * nrhs + c], X[r * nrhs + c], B[r * nrhs + c]);
         const unsigned long long a = block_max(v.m[0], red), b = block_max(v.m[1], red), e = block_max(v.m[2], red);
+        const unsigned mine = v.flags();
         unsigned flags = 0;
-        for (unsigned f : {CM_BAD_R, CM_BAD_X, CM_BAD_B}) flags |= __syncthreads_or(v.flags & f) ? f : 0;
+        for (unsigned f : {CM_BAD_R, CM_BAD_X, CM_BAD_B}) flags |= __syncthreads_or(mine & f) ? f : 0;
         if (threadIdx.x == 0) {
             double *o = out + ((int64_t)inst * nrhs + c) * 4;
             o[0] = __longlong_as_double((long long)a);

@@ -81,14 +81,20 @@ __device__ __forceinline__ FrontCols<T> front_columns(const DevSym &d, T *pool, 
 // count), then a word of flags: which of them held a value that is not finite
 struct ColMax {
     unsigned long long m[3] = {0, 0, 0};
-    unsigned flags = 0;
+    unsigned top[3] = {0, 0, 0};    // largest leading word, NaN included
     __device__ __forceinline__ void add(double r, double x, double b) {
         const unsigned long long inf = 0x7FF0000000000000ull, u[3] = {bits(r), bits(x), bits(b)};
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             m[q] = max(m[q], u[q] > inf ? 0ull : u[q]);
-            if (u[q] >= inf) flags |= CM_BAD_R << q;
+            top[q] = max(top[q], (unsigned)(u[q] >> 32));
         }
+    }
+    __device__ __forceinline__ unsigned flags() const {
+        unsigned f = 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) f |= top[q] >= 0x7FF00000u ? CM_BAD_R << q : 0u;
+        return f;
     }
     static __device__ __forceinline__ unsigned long long bits(double x) {
         return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;   // |x|, ordered like the value

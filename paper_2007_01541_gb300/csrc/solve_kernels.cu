@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(256) colmax_rm_kernel(const double *__restrict
         }
 #pragma unroll
         for (int q = 0; q < 3; ++q) red[q][g][cl] = v.m[q];
-        redf[g][cl] = v.flags;
+        redf[g][cl] = v.flags();
         __syncthreads();
         // group q: word q of every column
         unsigned long long *o = reinterpret_cast<unsigned long long *>(out + 4 * (int64_t)c + g);
@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(256) colmax_narrow_kernel(const double *__rest
             for (int o = 16; o > 0; o >>= 1) v.m[q] = max(v.m[q], __shfl_xor_sync(0xffffffffu, v.m[q], o));
             if ((threadIdx.x & 31) == 0) atomicMax(w + q, v.m[q]);
         }
-        const unsigned f = __reduce_or_sync(0xffffffffu, v.flags);
+        const unsigned f = __reduce_or_sync(0xffffffffu, v.flags());
         if ((threadIdx.x & 31) == 0 && f) atomicOr(w + 3, (unsigned long long)f);
     }
 }

@@ -199,7 +199,8 @@ __device__ __forceinline__ void issue_a(const DevSym &d, const TcSolveArgs &a, c
             }
             // the front's last row need not end a vector: past it the pool
             // holds anything too
-            cp_async16(Ah + tc::sw128_offset(r, kh + 4 * q), v ? src + 4 * q : a.front, v ? 4 * min(4, lim - kq0) : 0);
+            const int bytes = OP == OP_BREDUCE ? 4 * min(4, lim - kq0) : 16;
+            cp_async16(Ah + tc::sw128_offset(r, kh + 4 * q), v ? src + 4 * q : a.front, v ? bytes : 0);
         }
     }
 }
